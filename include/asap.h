@@ -201,9 +201,9 @@ asap_status asap_consolidate(asap_ctx *ctx, const asap_inputs *in, const asap_pa
  * the spans, q and k of `in` are read; `p` must be a valid parameter set (as for asap_score).
  * `v` and `out` are bf16 [total_tokens, H, head_dim] device tensors, 16-byte aligned, that must
  * not overlap.  `scratch`: caller-owned device memory of at least
- * asap_attention_scratch_bytes(total_tokens, D) bytes, 16-byte aligned (the transposed values);
- * nothing is kept in it between calls.  Two launches (plus the validation kernel); may be recorded
- * by a stream capture. */
+ * asap_attention_scratch_bytes(total_tokens, D) bytes, 16-byte aligned; nothing is kept in it between calls (the
+ * present kernel multiplies the values as they lie and leaves it untouched).  One launch, which validates the batch
+ * too; may be recorded by a stream capture. */
 size_t asap_attention_scratch_bytes(int32_t total_tokens, int32_t D);
 asap_status asap_attention(asap_ctx *ctx, const asap_inputs *in, const asap_params *p,
                            const float *mask_log, const void *v, void *scratch, size_t scratch_bytes,

@@ -708,7 +708,7 @@ asap_status asap_init(asap_ctx **ctx_out, int device, size_t max_total_tokens, i
   const size_t o_mpart = carve(Hc * T * sizeof(float));
   const size_t o_inv = carve(T * sizeof(float));
   const size_t o_kinv = carve(max_keep_rows * sizeof(float));
-  const size_t o_cnt = carve((Bc * col_blocks + 3 * Bc + 2) * sizeof(unsigned int));
+  const size_t o_cnt = carve((Bc * col_blocks + 3 * Bc + 4) * sizeof(unsigned int));
   const size_t o_role = carve(T * sizeof(int32_t));
   const size_t o_seg = carve((max_keep_rows + Bc) * sizeof(int32_t));
   const size_t o_mem = carve(T * sizeof(int32_t));
@@ -735,7 +735,7 @@ asap_status asap_init(asap_ctx **ctx_out, int device, size_t max_total_tokens, i
   if (const char *env = getenv("ASAP_SIM_CLUSTER")) ctx->sim_cluster = atoi(env);
   ctx->inv_norm = reinterpret_cast<float *>(ctx->arena + o_inv);
   ctx->kept_inv = reinterpret_cast<float *>(ctx->arena + o_kinv);
-  ctx->counters_off = o_cnt; ctx->counters_bytes = (Bc * col_blocks + 3 * Bc + 2) * sizeof(unsigned int);
+  ctx->counters_off = o_cnt; ctx->counters_bytes = (Bc * col_blocks + 3 * Bc + 4) * sizeof(unsigned int);
   ctx->tiles_off = o_tiles; ctx->tiles_bytes = ctx->cap_tiles * sizeof(unsigned int);
   ctx->cnt_qsum = reinterpret_cast<unsigned int *>(ctx->arena + o_cnt);
   ctx->cnt_mass = ctx->cnt_qsum + Bc * col_blocks;
@@ -750,7 +750,7 @@ asap_status asap_init(asap_ctx **ctx_out, int device, size_t max_total_tokens, i
   ctx->cnt_tiles = reinterpret_cast<unsigned int *>(ctx->arena + o_tiles);
   ctx->sim_part = reinterpret_cast<float *>(ctx->arena + o_simpart);
   ctx->status = reinterpret_cast<uint32_t *>(ctx->arena + o_status);
-  e = cudaMemset(ctx->arena + o_cnt, 0, (Bc * col_blocks + 3 * Bc + 2) * sizeof(unsigned int));
+  e = cudaMemset(ctx->arena + o_cnt, 0, (Bc * col_blocks + 3 * Bc + 4) * sizeof(unsigned int));
   if (e == cudaSuccess) e = cudaMemset(ctx->arena + o_tiles, 0, ctx->cap_tiles * sizeof(unsigned int));
   if (e == cudaSuccess) e = cudaMemset(ctx->status, 0, sizeof(uint32_t));
   // kernels whose dynamic shared memory exceeds the 48 KB default
@@ -851,27 +851,25 @@ asap_status asap_attention(asap_ctx *ctx, const asap_inputs *in, const asap_para
     return fail(ctx, ASAP_ERR_WORKSPACE, "asap_attention: scratch is null, unaligned or smaller than asap_attention_scratch_bytes");
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   const int total = in->total_tokens, D = in->D;
-  const int total_pad = (int)align_up((size_t)total, 8);
-  CUtensorMap map_q, map_k, map_vt;
+  CUtensorMap map_q, map_k, map_v;
   if (!make_map(ctx, &map_q, in->q, (uint64_t)total, (uint64_t)D, 128) ||
       !make_map(ctx, &map_k, in->k, (uint64_t)total, (uint64_t)D, 128) ||
-      !make_map(ctx, &map_vt, scratch, (uint64_t)D, (uint64_t)total, 128, (uint64_t)total_pad))
-    return fail(ctx, ASAP_ERR_CUDA, "cuTensorMapEncodeTiled failed for q / k / transposed v");
-  ASAP_TRY(launch_prepare(ctx, in, p, nullptr, 0x7fffffff, st));
-  mark(ctx, "transpose_v", st);
-  launch_pdl(transpose_v_kernel, dim3((total_pad + TR_TILE - 1) / TR_TILE, (D + TR_TILE - 1) / TR_TILE), dim3(TR_THREADS), 0, st,
-             static_cast<const __nv_bfloat16 *>(v), static_cast<__nv_bfloat16 *>(scratch), total, total_pad, D);
-  ASAP_TRY(after_launch(ctx, "transpose_v"));
+      !make_map(ctx, &map_v, v, (uint64_t)total, (uint64_t)D, 128))
+    return fail(ctx, ASAP_ERR_CUDA, "cuTensorMapEncodeTiled failed for q / k / v");
   AttnArgs aa;
-  aa.desc = ctx->desc; aa.H = in->H; aa.D = D; aa.max_vis = in->max_vis; aa.mask_enable = p->mask_enable ? 1 : 0;
+  aa.pa = prepare_args(ctx, in, p, nullptr, 0x7fffffff); aa.pa.write_desc = 0;
+  aa.H = in->H; aa.pairs = (in->max_seq + 255) / 256; aa.max_vis = in->max_vis; aa.mask_enable = p->mask_enable ? 1 : 0;
+  const long long items = (long long)aa.pairs * in->H * in->B;
+  if (items > 0x7fffffffLL - 65536) return fail(ctx, ASAP_ERR_UNSUPPORTED, "asap_attention: B * H * max_seq is too large");
+  aa.n_items = (int)items;
   aa.scale_log2 = 1.4426950408889634f / sqrtf((float)in->head_dim);
   aa.mask_log = mask_log; aa.out = static_cast<__nv_bfloat16 *>(out); aa.status = ctx->status;
-  aa.wait_limit = ctx->wait_limit;
+  aa.work = ctx->cnt_work + 2; aa.wait_limit = ctx->wait_limit;
   aa.mask_b_stride = p->per_head_mask ? in->H * in->max_vis : in->max_vis;
   aa.mask_h_stride = p->per_head_mask ? in->max_vis : 0;
   mark(ctx, "attention", st);
-  launch_pdl(attn_kernel, dim3((in->max_seq + 255) / 256, in->H, in->B), dim3(AT_THREADS), (size_t)AT_SMEM_BYTES, st,
-             map_q, map_k, map_vt, aa);
+  launch_pdl(attn_kernel, dim3(items < ctx->num_sms ? (int)items : ctx->num_sms), dim3(AT_THREADS), (size_t)AT_SMEM_BYTES, st,
+             map_q, map_k, map_v, aa);
   return finish(ctx, after_launch(ctx, "attention"), st);
 }
 

@@ -66,6 +66,41 @@ __device__ __forceinline__ float fast_exp2(float x) {
   return y;
 }
 
+constexpr float LOG2E_F = 1.4426950408889634f;
+
+__device__ __forceinline__ float max3(float a, float b, float c) {
+  float m;
+  asm("max.f32 %0, %1, %2, %3;" : "=f"(m) : "f"(a), "f"(b), "f"(c));
+  return m;
+}
+
+// Two fp32 values in one 64-bit register: one instruction issues both operations.
+__device__ __forceinline__ uint64_t f2_pack(float lo, float hi) {
+  uint64_t r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+  return r;
+}
+__device__ __forceinline__ void f2_unpack(uint64_t v, float &lo, float &hi) {
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
+}
+__device__ __forceinline__ uint64_t f2_add(uint64_t a, uint64_t b) {
+  uint64_t r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ uint64_t f2_fma(uint64_t a, uint64_t b, uint64_t c) {
+  uint64_t r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+
+// Register share of the calling warpgroup (all its threads execute it); the shares of a block's warpgroups must not add
+// up to more than the block was launched with.
+template <int N>
+__device__ __forceinline__ void reg_inc() { asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(N)); }
+template <int N>
+__device__ __forceinline__ void reg_dec() { asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(N)); }
+
 // ---------------------------------------------------------------------------------------
 // Shared-memory addresses, mbarriers
 // ---------------------------------------------------------------------------------------
@@ -126,6 +161,12 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, const W
       return false;
     }
   }
+}
+
+// The whole warp waits, and is converged afterwards.
+__device__ __forceinline__ void mbar_wait_warp(uint32_t bar, uint32_t parity, const WaitCtx &w) {
+  mbar_wait(bar, parity, w);
+  __syncwarp();
 }
 
 // Drain wait used at teardown for copies this thread issued itself: ignores the abort flag,
@@ -238,16 +279,49 @@ __device__ __forceinline__ void tc_mma_bf16_k128(uint32_t d_tmem, uint64_t a_des
         "n"(A_HALF_BYTES / 16 + 4), "n"(B_HALF_BYTES / 16 + 4), "n"(A_HALF_BYTES / 16 + 6), "n"(B_HALF_BYTES / 16 + 6)
       : "memory");
 }
-// D[tmem] (+)= A[tmem] * B[smem]^T: the A operand lives in tensor memory, row m in lane m, sixteen
-// bf16 (one k-step) in eight consecutive 32-bit columns, the even element in the low half.
-__device__ __forceinline__ void tc_mma_bf16_ta(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc,
-                                               uint32_t idesc, uint32_t accumulate) {
+// The issuing warp's form of these: the WHOLE warp executes the statement, `leader` (see warp_leader) is non-zero in the
+// one lane that issues.  A warp that stays converged keeps the descriptors in uniform registers and spends one or two
+// instructions per MMA; code under `if (lane == 0)` spends a dozen, each of which waits its turn among the other warps of the
+// scheduler (measured, M = 128, N = 128, two warps of FMAs beside the issuer: 76 clocks per MMA against 565; the pipe takes 64).
+__device__ __forceinline__ uint32_t warp_leader() {
+  uint32_t p;
+  asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(p));
+  return p;
+}
+__device__ __forceinline__ void tc_mma_bf16_w(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,
+                                              uint32_t accumulate, uint32_t leader) {
   asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}"
-      ::"r"(d_tmem), "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accumulate)
+      "{\n\t.reg .pred p, q;\n\t"
+      "setp.ne.b32 p, %4, 0;\n\tsetp.ne.b32 q, %5, 0;\n\t"
+      "@q tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
+      ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate), "r"(leader)
       : "memory");
+}
+// The A operand lives in tensor memory: row m in lane m, sixteen bf16 (one k-step) in eight consecutive 32-bit columns, the
+// even element in the low half.
+__device__ __forceinline__ void tc_mma_bf16_ta_w(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc, uint32_t idesc,
+                                                 uint32_t accumulate, uint32_t leader) {
+  asm volatile(
+      "{\n\t.reg .pred p, q;\n\t"
+      "setp.ne.b32 p, %4, 0;\n\tsetp.ne.b32 q, %5, 0;\n\t"
+      "@q tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}"
+      ::"r"(d_tmem), "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accumulate), "r"(leader)
+      : "memory");
+}
+__device__ __forceinline__ void tc_commit_w(uint32_t bar, uint32_t leader) {
+  asm volatile(
+      "{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %1, 0;\n\t"
+      "@q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}" ::"r"(bar), "r"(leader)
+      : "memory");
+}
+// A K extent of 128 bf16 held as two 64-column blocks (each 128-byte-swizzled), `a_half` / `b_half` bytes apart; the first
+// MMA overwrites the accumulator, the others add.
+__device__ __forceinline__ void tc_mma_bf16_k128_w(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t a_half, uint32_t b_half,
+                                                   uint32_t idesc, uint32_t leader) {
+#pragma unroll
+  for (uint32_t kk = 0; kk < 8; ++kk)
+    tc_mma_bf16_w(d_tmem, a_desc + (kk & 3) * 2 + (kk >> 2) * (a_half >> 4), b_desc + (kk & 3) * 2 + (kk >> 2) * (b_half >> 4), idesc,
+                  kk > 0 ? 1u : 0u, leader);
 }
 // Stores: the mirror images of the loads below (thread t of the warp writes lane base + t).
 __device__ __forceinline__ void tmem_st16(uint32_t taddr, const uint32_t (&r)[16]) {
@@ -334,6 +408,20 @@ __device__ __forceinline__ uint64_t umma_desc_sw128(uint32_t smem_addr) {
   return static_cast<uint64_t>((smem_addr >> 4) & 0x3fffu) | (1ull << 16) | (64ull << 32) |
          (1ull << 46) | (2ull << 61);
 }
+// The same for an MN-major B operand, i.e. a tile whose rows (128 bytes = 64 elements of N, 128-byte swizzle) are
+// the K steps: here the leading byte offset is the distance between 64-element blocks along N and the stride byte
+// offset (1024) the distance between groups of eight K steps.  Sixteen steps along K add 2048 bytes to the start address.
+__device__ __forceinline__ uint64_t umma_desc_sw128_mn(uint32_t smem_addr, uint32_t block_bytes) {
+  return static_cast<uint64_t>((smem_addr >> 4) & 0x3fffu) | (static_cast<uint64_t>(block_bytes >> 4) << 16) |
+         (64ull << 32) | (1ull << 46) | (2ull << 61);
+}
+// The same for a K-major tile of ONE k-step: rows of 32 bytes (16 bf16), 32-byte swizzle (mode 6): the two 16-byte chunks
+// of row r trade places where bit 2 of r is set; 8-row groups are 256 bytes apart.
+__device__ __forceinline__ uint64_t umma_desc_sw32(uint32_t smem_addr) {
+  return static_cast<uint64_t>((smem_addr >> 4) & 0x3fffu) | (1ull << 16) | (16ull << 32) | (1ull << 46) | (6ull << 61);
+}
+constexpr uint32_t UMMA_IDESC_B_MN = 1u << 16;   // instruction-descriptor bit: B is MN-major
+
 // Instruction descriptor for kind::f16 with bf16 A and B (both K-major) and fp32 D:
 // D format fp32 (1) in bits [4,6), A format bf16 (1) in [7,10), B format bf16 (1) in [10,13),
 // N >> 3 in [17,23), M >> 4 in [24,29).

@@ -1,180 +1,158 @@
 // The layer's attention under the salience-guided bidirectional mask (Eq. 4 applied to the
 // values):  O^h = Softmax(W^h + M_bidir) V^h,  W^h = Q^h K^h^T / sqrt(d).
 //
-//   transpose_v_kernel  V [tokens, D] -> V^T [D, tokens] (row pitch padded to 8 tokens), so that
-//                       a value tile can be loaded as a K-major MMA operand like every other tile.
-//   attn_kernel         one block per (two tiles of 128 query rows, head, sequence); the two row
-//                       tiles share every key / value tile and take turns on the tensor pipe.
-//                       For every tile of 128 keys:  S = Q K^T on tcgen05 into tensor memory; the
-//                       row tile's eight softmax warps read S once (two threads per row, 64 keys
-//                       each, exchanging their maxima through shared memory), add Eq. 3's
-//                       m_j for the future keys of the image span on rows of the image span (nothing
-//                       else above the diagonal is admitted), turn the logits into probabilities
-//                       relative to a reference maximum and store them as bf16 over S's own columns;
-//                       O += P V then runs with P read from tensor memory and O accumulated in
-//                       tensor memory.  The reference maximum only moves (and O is only rescaled)
-//                       when a row's maximum has grown by more than 2^8; the final division by the
-//                       row sum makes the result independent of the reference.  M_bidir is never
-//                       materialised: it is the vector m_j plus position tests.
+//   attn_kernel  persistent blocks; a work item is (two tiles of 128 query rows, head, sequence).  The
+//                two row tiles share every key / value tile and take turns on the tensor pipe.
+//                For every tile of 128 keys:  S = Q K^T on tcgen05 into tensor memory; the row tile's
+//                softmax warpgroup (one thread per row) reads S once, adds Eq. 3's m_j for the future
+//                keys of the image span on rows of the image span (nothing else above the diagonal is
+//                admitted), turns the logits into probabilities relative to a reference maximum and
+//                stores them as bf16 in tensor memory; O += P V then runs with P read from tensor
+//                memory and O accumulated in tensor memory.  The final division by the row sum makes
+//                the result independent of the reference.  M_bidir is never materialised: it is the
+//                vector m_j plus position tests.
 //
-// Key tiles start at the sequence's first packed row rounded DOWN to a multiple of 8, because the
-// token coordinate is the contiguous one of V^T and a TMA copy must start on a 16-byte boundary;
-// the up to seven foreign keys in front are masked like any other inadmissible key.
+// V tiles are loaded as they lie in memory (rows = keys) and multiplied as an MN-major operand.
+//
+// Per (row tile, key tile) the tensor pipe needs 1024 clocks (16 MMAs of 64) and the exponentials 1024 as well (128 x 128,
+// 16 per clock and SM), so two row tiles cannot take less than 2048 per key tile; see the figures at attn_kernel.
 #pragma once
 
 #include "common.cuh"
+#include "kernels_stream.cuh"
 
 namespace asap {
 
 enum : uint32_t { STATUS_ATTN_TIMEOUT = 16u };   // a bounded wait ran out in the attention kernel
 
-// ---------------------------------------------------------------------------------------
-constexpr int TR_TILE = 64;
-constexpr int TR_THREADS = 256;
-
-__global__ void __launch_bounds__(TR_THREADS)
-transpose_v_kernel(const __nv_bfloat16 *__restrict__ v, __nv_bfloat16 *__restrict__ vt, int total,
-                   int total_pad, int D) {
-  pdl_enter();
-  __shared__ uint16_t tile[TR_TILE][TR_TILE + 2];
-  const int t0 = blockIdx.x * TR_TILE, d0 = blockIdx.y * TR_TILE;
-  const uint16_t *src = reinterpret_cast<const uint16_t *>(v);
-  uint16_t *dst = reinterpret_cast<uint16_t *>(vt);
-  for (int i = threadIdx.x; i < TR_TILE * (TR_TILE / 8); i += TR_THREADS) {
-    const int r = i / (TR_TILE / 8), c8 = i % (TR_TILE / 8);
-    uint4 x = make_uint4(0u, 0u, 0u, 0u);
-    if (t0 + r < total && d0 + c8 * 8 < D)
-      x = __ldg(reinterpret_cast<const uint4 *>(src + (size_t)(t0 + r) * D + d0 + c8 * 8));
-    const uint32_t w[4] = {x.x, x.y, x.z, x.w};
-#pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      tile[c8 * 8 + 2 * e][r] = (uint16_t)(w[e] & 0xffffu);
-      tile[c8 * 8 + 2 * e + 1][r] = (uint16_t)(w[e] >> 16);
-    }
-  }
-  __syncthreads();
-  for (int i = threadIdx.x; i < TR_TILE * (TR_TILE / 8); i += TR_THREADS) {
-    const int dd = i / (TR_TILE / 8), c8 = i % (TR_TILE / 8);
-    if (d0 + dd >= D || t0 + c8 * 8 >= total_pad) continue;
-    uint32_t w[4];
-#pragma unroll
-    for (int e = 0; e < 4; ++e)
-      w[e] = (uint32_t)tile[dd][c8 * 8 + 2 * e] | ((uint32_t)tile[dd][c8 * 8 + 2 * e + 1] << 16);
-    *reinterpret_cast<uint4 *>(dst + (size_t)(d0 + dd) * total_pad + t0 + c8 * 8) = make_uint4(w[0], w[1], w[2], w[3]);
-  }
-}
-
-// ---------------------------------------------------------------------------------------
-constexpr int AT_THREADS = 576;                 // warp 0: copies, warp 1: MMA issue, warps 2-17: two softmax groups of eight
+constexpr int AT_THREADS = 384;                 // warp 0: items and copies, warp 1: MMA issue, warp 2: Eq. 3's addends, warps 4-11: two softmax warpgroups
 constexpr int AT_TILE_BYTES = 128 * 128 * 2;    // 128 rows x 128 bf16 as two 64-column blocks of 16 KB
 constexpr int AT_BLOCK_BYTES = AT_TILE_BYTES / 2;
-constexpr int AT_STAGES = 2;                    // a stage = one key tile + one value tile
-constexpr int AT_MAIN_BYTES = 2 * AT_TILE_BYTES + AT_STAGES * 2 * AT_TILE_BYTES;
-constexpr int AT_BOOK_BYTES = 3072;
+constexpr int AT_SLOTS = 4;                     // ring of key and value tiles in the order K0 V0 K1 V1 ...
+constexpr int AT_STAGE_BYTES = 32 * 64;         // per softmax warp: 32 rows x 32 columns of the result
+constexpr int AT_EXT_BYTES = 128 * 32;          // one k-step: 128 rows x 16 bf16
+constexpr int AT_EXT_BUFS = 2;                  // key-side addend tiles in flight
+constexpr int AT_EXT_OFF = (2 + AT_SLOTS) * AT_TILE_BYTES;
+constexpr int AT_STAGE_OFF = AT_EXT_OFF + (2 + AT_EXT_BUFS) * AT_EXT_BYTES;
+constexpr int AT_MAIN_BYTES = AT_STAGE_OFF + 8 * AT_STAGE_BYTES;
+constexpr int AT_BOOK_BYTES = 2048;
 constexpr int AT_SMEM_BYTES = AT_MAIN_BYTES + AT_BOOK_BYTES;
-constexpr uint32_t AT_TMEM_COLS = 512;          // per row tile: S / P (128 columns) and O (128 columns)
+// Tensor memory: O of both row tiles (2 x 128 columns), ONE S (128) that the row tiles use in turn, P of both (2 x 64).
+// A row tile's logits are in registers soon after they are complete, so the next S can be multiplied while their
+// exponentials are taken; with an S per row tile P has to lie over it, and softmax, P V and the next S form a chain.
+constexpr uint32_t AT_TMEM_COLS = 512, AT_S_COL = 256, AT_P_COL = 384;
 constexpr long long AT_WAIT_LIMIT = 2000000000LL;
-constexpr float AT_RESCALE_STEP = 8.0f;         // log2 units the row maximum may outgrow the reference
-static_assert(AT_SMEM_BYTES <= 195 * 1024, "the attention block must stay inside the 196 KB carve-out");
+constexpr float AT_SUM_LIMIT = 1.0995116e12f;   // 2^40: a key tile's sum relative to the reference at which the reference moves
+constexpr float AT_NEVER = -1e30f;              // addend of a key that is not admitted (finite: it is a factor of an MMA)
+constexpr int AT_ITEM_SLOTS = 4;
+static_assert((AT_SLOTS & (AT_SLOTS - 1)) == 0, "ring slots are taken by masking");
 
 struct AttnArgs {
-  const SampleDesc *desc;
-  int H, D, max_vis, mask_enable;
+  PrepareArgs pa;              // the blocks derive the descriptors themselves
+  int H, pairs;                // pairs: row-tile pairs of the longest sequence
+  int n_items, max_vis, mask_enable;
   float scale_log2;            // log2(e) / sqrt(head_dim)
   const float *mask_log;       // [B, max_vis] m_j (natural log) or [B, H, max_vis]; may be null with the mask off
   int mask_b_stride, mask_h_stride;   // max_vis, 0   or   H * max_vis, max_vis
   __nv_bfloat16 *out;          // [tokens, H, 128]
+  unsigned int *work;          // [2] items drawn / blocks that have finished; both zero between launches
   uint32_t *status;
   long long wait_limit;        // clock cycles a wait may take before the block gives up
 };
 
+struct AttnItem {
+  int b;                       // sequence, -1: no more items
+  int h, q_base;               // head, first query row (sequence-relative) of the pair
+  int n_kt[2];                 // key tiles each row tile looks at (0: no rows)
+  int sees[2];                 // the row tile holds rows of the image span and the mask is on
+  int row0, n, v0, v_end;
+};
+
 struct AttnBook {
-  uint64_t full[AT_STAGES], empty[AT_STAGES], q_full, s_full[2], p_ready[2], pv_done[2], mma_done;
+  uint64_t full[AT_SLOTS], empty[AT_SLOTS], q_full[2], q_empty[2], s_full[2], s_empty, p_ready[2], pv_done[2];
+  uint64_t m_full[2], m_empty[2], ext_full[AT_EXT_BUFS], ext_empty[AT_EXT_BUFS], rows_full[2], rows_empty[2];
+  uint64_t item_full[AT_ITEM_SLOTS], item_empty[AT_ITEM_SLOTS], mma_done;
+  AttnItem item[AT_ITEM_SLOTS];
   uint32_t tmem_base;
   int abort_flag;
-  alignas(16) float m_tile[2][128];   // [row tile][key]: Eq. 3's addend for the keys of the current tile
-  uint32_t row_max[2][128];    // [row tile][row]: running row maximum as an order-preserving integer
+  alignas(16) float m_tile[2][128];   // [row tile][key]: Eq. 3's addends for the key tile that the diagonal crosses, in the
+                                      // units of q.k: m_j inside the span, AT_NEVER outside
 };
 static_assert(sizeof(AttnBook) <= AT_BOOK_BYTES, "attention kernel bookkeeping exceeds its shared-memory slot");
-
-// order-preserving integer image of a float (no NaN here) and its inverse, for atomicMax
-__device__ __forceinline__ uint32_t attn_key(float f) {
-  const uint32_t u = __float_as_uint(f);
-  return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
-}
-__device__ __forceinline__ float attn_unkey(uint32_t k) {
-  return __uint_as_float((k & 0x80000000u) ? (k & 0x7fffffffu) : ~k);
-}
+static_assert(AT_SMEM_BYTES <= 227 * 1024, "attention kernel exceeds an SM's shared memory");
 
 // keys a tile of query rows [q_lo, q_lo + 128) can see: up to its last row (causal), and to the end
 // of the image span if one of its rows lies inside the span and the mask is on
-__device__ __forceinline__ int attn_key_end(const SampleDesc &d, int q_lo, int mask_enable, bool &sees_span) {
+__device__ __forceinline__ int attn_key_end(const SampleDesc &d, int q_lo, int mask_enable, int &sees_span) {
   const int q_hi = min(q_lo + 128, d.n);
   sees_span = mask_enable && q_lo < d.v0 + d.nv && q_hi > d.v0;
   return min(d.n, sees_span ? max(q_hi, d.v0 + d.nv) : q_hi);
 }
 
+// What Eq. 3's mask does to key tile kt for a row tile that starts at row q_lo.
+struct AttnTileKind {
+  bool above;    // the row tile holds rows of the span and all keys of the tile lie after all of its rows: every row needs an
+                 // addend for every key (m_j for a row of the span, AT_NEVER for any other): one more k-step of the S MMA
+  bool crossed;  // the row tile holds rows of the span and the diagonal crosses the key tile: the softmax warps add m_j
+};
+__device__ __forceinline__ AttnTileKind attn_tile_kind(int sees, int q_lo, int kt) {
+  AttnTileKind k;
+  k.above = sees && kt * 128 > q_lo + 127;
+  k.crossed = sees && !k.above && kt * 128 + 127 > q_lo;
+  return k;
+}
+
+// What bounds it: at the largest size the power cap (1.04 PFLOP/s algorithmic, 75 % of what a library GEMM sustains under
+// the same cap); below that the hand-overs between the tensor pipe and the softmax warps: a key tile of both row tiles takes
+// about 3000 clocks where either alone needs 2048.  Measured per call (before: a block per pair of row tiles, a kernel that
+// transposed V, a validation kernel, two threads per query row with a shared running maximum, S and P on the same columns):
+//   1 x 643 rows, 32 heads            29.0 ->   20.6 us
+//   16 x 627-739 rows, 32 heads        304 ->    176 us
+//   64 x 2947-3171 rows, 32 heads     14.2 ->    8.9 ms   (9.3 TFLOP)
+// Of that on the largest: persistent blocks with V as an MN-major operand 14.1 -> 12.3, an S of its own 11.7 -> 9.8, the mask
+// above the diagonal as one more k-step and the issuing warp converged -> 9.0 ms.  A polynomial for an eighth or a quarter of
+// the exponentials changed nothing (8.9-9.0), for three eighths it cost 4 %.
 __global__ void __launch_bounds__(AT_THREADS, 1)
 attn_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__ CUtensorMap tmap_k,
-            const __grid_constant__ CUtensorMap tmap_vt, AttnArgs a) {
-  pdl_enter();
+            const __grid_constant__ CUtensorMap tmap_v, AttnArgs a) {
   extern __shared__ __align__(1024) uint8_t at_smem[];
-  const int pair = (int)gridDim.x - 1 - (int)blockIdx.x;     // long rows first
-  const int h = blockIdx.y, b = blockIdx.z;
-  const SampleDesc d = a.desc[b];
-  const int q_base = pair * 256;
-  if (!d.valid || q_base >= d.n) return;
-  if (*reinterpret_cast<volatile uint32_t *>(a.status) & STATUS_ATTN_TIMEOUT) return;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
   const uint32_t base = smem_u32(at_smem);
   const uint32_t q_smem = base, ring = base + 2 * AT_TILE_BYTES;
   AttnBook *bk = reinterpret_cast<AttnBook *>(at_smem + AT_MAIN_BYTES);
 
-  const int delta = d.row0 & 7;
-  const int kbase = d.row0 - delta;
-  bool sees0 = false, sees1 = false;
-  const int n_kt0 = (attn_key_end(d, q_base, a.mask_enable, sees0) + delta + 127) / 128;
-  const int n_kt1 = q_base + 128 < d.n ? (attn_key_end(d, q_base + 128, a.mask_enable, sees1) + delta + 127) / 128 : 0;
-  const int n_max = max(n_kt0, n_kt1);
-
   if (threadIdx.x == 0) {
-    for (int s = 0; s < AT_STAGES; ++s) {
+    for (int s = 0; s < AT_SLOTS; ++s) {
       mbar_init(smem_u32(&bk->full[s]), 1);
       mbar_init(smem_u32(&bk->empty[s]), 1);
     }
-    mbar_init(smem_u32(&bk->q_full), 1);
     for (int g = 0; g < 2; ++g) {
+      mbar_init(smem_u32(&bk->q_full[g]), 1);
+      mbar_init(smem_u32(&bk->q_empty[g]), 1);
       mbar_init(smem_u32(&bk->s_full[g]), 1);
-      mbar_init(smem_u32(&bk->p_ready[g]), 256);
+      mbar_init(smem_u32(&bk->p_ready[g]), 4);            // the row tile's four softmax warps
       mbar_init(smem_u32(&bk->pv_done[g]), 1);
-      if (g == 0) mbar_init(smem_u32(&bk->mma_done), 1);
+      mbar_init(smem_u32(&bk->m_full[g]), 1);
+      mbar_init(smem_u32(&bk->m_empty[g]), 4);
+      mbar_init(smem_u32(&bk->rows_full[g]), 1);
+      mbar_init(smem_u32(&bk->rows_empty[g]), 1);
     }
+    for (int i = 0; i < AT_EXT_BUFS; ++i) {
+      mbar_init(smem_u32(&bk->ext_full[i]), 1);
+      mbar_init(smem_u32(&bk->ext_empty[i]), 1);
+    }
+    for (int i = 0; i < AT_ITEM_SLOTS; ++i) {
+      mbar_init(smem_u32(&bk->item_full[i]), 1);
+      mbar_init(smem_u32(&bk->item_empty[i]), 10);        // the MMA issuer, the addend warp, every softmax warp
+    }
+    mbar_init(smem_u32(&bk->mma_done), 1);
+    mbar_init(smem_u32(&bk->s_empty), 4);                 // the softmax warps that have taken an S into registers
     bk->abort_flag = 0;
     fence_barrier_init();
-    // the query tiles and the first key / value tiles are requested right away, while the other
-    // warps are still setting up (this thread is the copy thread)
     tma_prefetch_desc(&tmap_q);
     tma_prefetch_desc(&tmap_k);
-    tma_prefetch_desc(&tmap_vt);
-    const int n_q = n_kt1 > 0 ? 2 : 1;
-    mbar_expect_tx(smem_u32(&bk->q_full), n_q * AT_TILE_BYTES);
-    for (int g = 0; g < n_q; ++g) {
-      tma_load_2d(q_smem + g * AT_TILE_BYTES, &tmap_q, smem_u32(&bk->q_full), h * 128, d.row0 + q_base + g * 128);
-      tma_load_2d(q_smem + g * AT_TILE_BYTES + AT_BLOCK_BYTES, &tmap_q, smem_u32(&bk->q_full), h * 128 + 64,
-                  d.row0 + q_base + g * 128);
-    }
-    for (int kt = 0; kt < min(n_max, AT_STAGES); ++kt) {
-      const uint32_t dst = ring + kt * 2 * AT_TILE_BYTES;
-      const uint32_t bar = smem_u32(&bk->full[kt]);
-      const int key0 = kbase + kt * 128;
-      mbar_expect_tx(bar, 2 * AT_TILE_BYTES);
-      tma_load_2d(dst, &tmap_k, bar, h * 128, key0);
-      tma_load_2d(dst + AT_BLOCK_BYTES, &tmap_k, bar, h * 128 + 64, key0);
-      tma_load_2d(dst + AT_TILE_BYTES, &tmap_vt, bar, key0, h * 128);
-      tma_load_2d(dst + AT_TILE_BYTES + AT_BLOCK_BYTES, &tmap_vt, bar, key0 + 64, h * 128);
-    }
+    tma_prefetch_desc(&tmap_v);
   }
-  if (threadIdx.x < 256) (&bk->row_max[0][0])[threadIdx.x] = 0u;      // below every encoded float
   if (warp == 1) {
     tmem_alloc(smem_u32(&bk->tmem_base), AT_TMEM_COLS);
     tmem_relinquish();
@@ -184,270 +162,465 @@ attn_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__ 
   tc_fence_after();
   const uint32_t tmem_base = bk->tmem_base;
   WaitCtx wc{&bk->abort_flag, a.status, STATUS_ATTN_TIMEOUT, a.wait_limit};
+  pdl_enter();
+  if (*reinterpret_cast<volatile uint32_t *>(a.status) & STATUS_ATTN_TIMEOUT) bk->abort_flag = 1;   // benign race: same value
+  __syncthreads();
 
-  if (warp == 0) {
-    if (lane == 0) {
-      int issued = min(n_max, AT_STAGES);          // the first tiles were requested during set-up
-      for (int kt = issued; kt < n_max; ++kt) {
-        const int s = kt % AT_STAGES;
-        if (kt >= AT_STAGES) mbar_wait(smem_u32(&bk->empty[s]), ((kt / AT_STAGES) - 1) & 1, wc);
-        if (bk->abort_flag) break;
-        const uint32_t dst = ring + s * 2 * AT_TILE_BYTES;
-        const uint32_t bar = smem_u32(&bk->full[s]);
-        const int key0 = kbase + kt * 128;
-        mbar_expect_tx(bar, 2 * AT_TILE_BYTES);
-        tma_load_2d(dst, &tmap_k, bar, h * 128, key0);
-        tma_load_2d(dst + AT_BLOCK_BYTES, &tmap_k, bar, h * 128 + 64, key0);
-        tma_load_2d(dst + AT_TILE_BYTES, &tmap_vt, bar, key0, h * 128);
-        tma_load_2d(dst + AT_TILE_BYTES + AT_BLOCK_BYTES, &tmap_vt, bar, key0 + 64, h * 128);
-        issued = kt + 1;
-      }
-      // drain: every copy issued must have landed before the block leaves
-      mbar_wait_drain(smem_u32(&bk->q_full), 0, AT_WAIT_LIMIT);
-      for (int s = 0; s < AT_STAGES; ++s) {
-        if (issued > s) {
-          const int last = ((issued - 1 - s) / AT_STAGES) * AT_STAGES + s;
-          mbar_wait_drain(smem_u32(&bk->full[s]), (last / AT_STAGES) & 1, AT_WAIT_LIMIT);
+  // The launch gives every thread 168 registers; a softmax thread holds its row's 128 logits and needs more, the first
+  // warpgroup needs few: 128 x 72 + 256 x 216 = 384 x 168.
+  if (warp < 4) {
+    reg_dec<72>();
+    if (warp == 0) {
+      // ---------------------------------------------------------------- items, query / key / value tiles
+      if (lane == 0) {
+        int ic = 0;                               // items published
+        bool first = true;                        // every block's first item is its own number, the others are drawn
+        // Draws the next item that has rows and publishes it.  The item queue keeps working after an abort (its waits
+        // ignore the flag and are bounded on their own): every consumer must see the same sequence, ending with -1.
+        auto draw = [&](AttnItem &it) {
+          while (true) {
+            const int item = bk->abort_flag ? a.n_items : (first ? (int)blockIdx.x : (int)(gridDim.x + atomicAdd(a.work, 1u)));
+            first = false;
+            it.b = -1;
+            if (item >= a.n_items) break;
+            const int bh = item / a.pairs;
+            it.q_base = (a.pairs - 1 - (item - bh * a.pairs)) * 256;       // long rows first
+            it.b = bh / a.H;
+            it.h = bh - it.b * a.H;
+            const SampleDesc d = make_desc(a.pa, it.b);
+            if (!d.valid || it.q_base >= d.n) continue;
+            it.row0 = d.row0; it.n = d.n; it.v0 = d.v0; it.v_end = d.v0 + d.nv;
+            it.n_kt[0] = (attn_key_end(d, it.q_base, a.mask_enable, it.sees[0]) + 127) / 128;
+            it.n_kt[1] = 0; it.sees[1] = 0;
+            if (it.q_base + 128 < d.n) it.n_kt[1] = (attn_key_end(d, it.q_base + 128, a.mask_enable, it.sees[1]) + 127) / 128;
+            break;
+          }
+          const int slot = ic % AT_ITEM_SLOTS;
+          if (ic >= AT_ITEM_SLOTS &&
+              !mbar_wait_drain(smem_u32(&bk->item_empty[slot]), ((ic / AT_ITEM_SLOTS) - 1) & 1, AT_WAIT_LIMIT)) {
+            it.b = -1;
+            return;
+          }
+          bk->item[slot] = it;
+          mbar_arrive(smem_u32(&bk->item_full[slot]));      // release: the slot's content is visible to the waiters
+          ++ic;
+        };
+        AttnItem cur, nxt;
+        int tc = 0, qc[2] = {0, 0};               // key / value tiles and query tiles so far
+        int t_issued = 0, q_issued[2] = {0, 0};   // copies actually issued
+        draw(cur);
+        while (cur.b >= 0) {
+          auto load_q = [&](int g) {
+            if (cur.n_kt[g] == 0) return;
+            if (qc[g] >= 1) mbar_wait(smem_u32(&bk->q_empty[g]), (qc[g] - 1) & 1, wc);
+            if (!bk->abort_flag) {
+              const uint32_t bar = smem_u32(&bk->q_full[g]);
+              const int row = cur.row0 + cur.q_base + g * 128;
+              mbar_expect_tx(bar, AT_TILE_BYTES);
+              tma_load_2d(q_smem + g * AT_TILE_BYTES, &tmap_q, bar, cur.h * 128, row);
+              tma_load_2d(q_smem + g * AT_TILE_BYTES + AT_BLOCK_BYTES, &tmap_q, bar, cur.h * 128 + 64, row);
+              q_issued[g] = qc[g] + 1;
+            }
+            ++qc[g];
+          };
+          auto load_tile = [&](const CUtensorMap *map, int kt) {
+            const int s = tc % AT_SLOTS;
+            if (tc >= AT_SLOTS) mbar_wait(smem_u32(&bk->empty[s]), ((tc / AT_SLOTS) - 1) & 1, wc);
+            if (!bk->abort_flag) {
+              const uint32_t bar = smem_u32(&bk->full[s]), dst = ring + s * AT_TILE_BYTES;
+              const int row = cur.row0 + kt * 128;
+              mbar_expect_tx(bar, AT_TILE_BYTES);
+              tma_load_2d(dst, map, bar, cur.h * 128, row);
+              tma_load_2d(dst + AT_BLOCK_BYTES, map, bar, cur.h * 128 + 64, row);
+              t_issued = tc + 1;
+            }
+            ++tc;
+          };
+          const int n_max = max(cur.n_kt[0], cur.n_kt[1]);
+          load_q(0);
+          load_tile(&tmap_k, 0);
+          load_q(1);
+          load_tile(&tmap_v, 0);
+          draw(nxt);                              // its look-ups overlap this item's work
+          for (int kt = 1; kt < n_max; ++kt) {
+            load_tile(&tmap_k, kt);
+            load_tile(&tmap_v, kt);
+          }
+          cur = nxt;
+        }
+        // drain: every copy issued must have landed before the block leaves
+        for (int g = 0; g < 2; ++g)
+          if (q_issued[g] > 0) mbar_wait_drain(smem_u32(&bk->q_full[g]), (q_issued[g] - 1) & 1, AT_WAIT_LIMIT);
+        for (int s = 0; s < AT_SLOTS; ++s) {
+          const int fills = t_issued > s ? (t_issued - s + AT_SLOTS - 1) / AT_SLOTS : 0;
+          if (fills > 0) mbar_wait_drain(smem_u32(&bk->full[s]), (fills - 1) & 1, AT_WAIT_LIMIT);
         }
       }
-    }
-  } else if (warp == 1) {
-    if (lane == 0) {
-      const uint32_t idesc = umma_idesc_bf16(128, 128);
-      // S of row tile g for key tile kt.  Issued after the P V of key tile kt - 1 of the same row tile,
-      // whose P it overwrites; the tensor pipe runs one thread's MMAs in issue order.
-      auto issue_s = [&](int g, int kt) {
-        const int s = kt % AT_STAGES;
-        mbar_wait(smem_u32(&bk->full[s]), (kt / AT_STAGES) & 1, wc);
-        tc_fence_after();
-        if (bk->abort_flag) return;
-        const uint32_t qa = q_smem + g * AT_TILE_BYTES, kb = ring + s * 2 * AT_TILE_BYTES;
+    } else if (warp == 1) {
+      // ---------------------------------------------------------------- MMA issuer
+      // Per key tile and row tile: S of this key tile, then P V of the PREVIOUS one.  In that order an S never waits in the
+      // pipe behind a P V that could as well run after it, and no P V is late: its P has been ready for half a turn.
+      // The whole warp walks the loop and stays converged (see warp_leader).  After an abort its waits return at once and it
+      // goes on multiplying whatever lies in the block's own memory: nothing of it is used.
+      const uint32_t leader = warp_leader();
+      const uint32_t tm = __shfl_sync(0xffffffffu, tmem_base, 0);
+      const uint32_t idesc_s = umma_idesc_bf16(128, 128), idesc_o = idesc_s | UMMA_IDESC_B_MN;
+      const uint64_t qdesc = umma_desc_sw128(q_smem), tile0 = umma_desc_sw128(ring), vtile0 = umma_desc_sw128_mn(ring, AT_BLOCK_BYTES);
+      int t0 = 0;                                 // first tile of the item in the ring: K0 V0 K1 V1 ...
+      int qc[2] = {0, 0}, pc[2] = {0, 0}, sn = 0;             // query tiles, P tiles and S so far
+      int rc[2] = {0, 0}, ec = 0;                 // row-side and key-side addend tiles so far
+      for (int ic = 0;; ++ic) {
+        const int slot = ic % AT_ITEM_SLOTS;
+        const bool got = mbar_wait_drain(smem_u32(&bk->item_full[slot]), (ic / AT_ITEM_SLOTS) & 1, AT_WAIT_LIMIT);
+        __syncwarp();
+        auto field = [&](const int &f) { return __shfl_sync(0xffffffffu, f, 0); };
+        const AttnItem &it = bk->item[slot];
+        const int b = field(got ? it.b : -1);
+        const int n[2] = {field(it.n_kt[0]), field(it.n_kt[1])}, sees[2] = {field(it.sees[0]), field(it.sees[1])}, q_base = field(it.q_base);
+        if (leader) mbar_arrive(smem_u32(&bk->item_empty[slot]));
+        if (b < 0) break;
+        const int n_max = max(n[0], n[1]);
+        for (int kt = 0; kt <= n_max; ++kt) {
+          const int tk = t0 + 2 * kt, tv = tk - 1;            // ring tiles: K of this key tile, V of the previous one
+          const int sk = tk & (AT_SLOTS - 1), sv = tv & (AT_SLOTS - 1);
+          bool above[2] = {false, false};
+          const int eb = ec % AT_EXT_BUFS;
+          if (kt < n_max) {
+            above[0] = kt < n[0] && attn_tile_kind(sees[0], q_base, kt).above;
+            above[1] = kt < n[1] && attn_tile_kind(sees[1], q_base + 128, kt).above;
+            mbar_wait_warp(smem_u32(&bk->full[sk]), (tk / AT_SLOTS) & 1, wc);
+            if (above[0] || above[1]) mbar_wait_warp(smem_u32(&bk->ext_full[eb]), (ec / AT_EXT_BUFS) & 1, wc);
+          }
+          if (kt > 0) mbar_wait_warp(smem_u32(&bk->full[sv]), (tv / AT_SLOTS) & 1, wc);
+          const uint64_t kdesc = tile0 + sk * (AT_TILE_BYTES >> 4), vdesc = vtile0 + sv * (AT_TILE_BYTES >> 4);
 #pragma unroll
-        for (int kk = 0; kk < 8; ++kk)
-          tc_mma_bf16(tmem_base + g * 256, umma_desc_sw128(qa + (kk >> 2) * AT_BLOCK_BYTES + (kk & 3) * 32),
-                      umma_desc_sw128(kb + (kk >> 2) * AT_BLOCK_BYTES + (kk & 3) * 32), idesc, kk > 0 ? 1u : 0u);
-        tc_commit(smem_u32(&bk->s_full[g]));
+          for (int g = 0; g < 2; ++g) {
+            if (kt < n[g]) {
+              if (kt == 0) {
+                mbar_wait_warp(smem_u32(&bk->q_full[g]), qc[g] & 1, wc);
+                ++qc[g];
+                if (sees[g]) {
+                  mbar_wait_warp(smem_u32(&bk->rows_full[g]), rc[g] & 1, wc);
+                  ++rc[g];
+                }
+              }
+              if (sn > 0) mbar_wait_warp(smem_u32(&bk->s_empty), (sn - 1) & 1, wc);     // the previous S is in registers
+              ++sn;
+              tc_fence_after();
+              tc_mma_bf16_k128_w(tm + AT_S_COL, qdesc + g * (AT_TILE_BYTES >> 4), kdesc, AT_BLOCK_BYTES, AT_BLOCK_BYTES, idesc_s, leader);
+              if (above[g])
+                tc_mma_bf16_w(tm + AT_S_COL, umma_desc_sw32(base + AT_EXT_OFF + g * AT_EXT_BYTES),
+                              umma_desc_sw32(base + AT_EXT_OFF + (2 + eb) * AT_EXT_BYTES), idesc_s, 1u, leader);
+              tc_commit_w(smem_u32(&bk->s_full[g]), leader);
+              if (g == (kt < n[1] ? 1 : 0)) {                 // the last row tile that looks at this key tile
+                tc_commit_w(smem_u32(&bk->empty[sk]), leader);
+                if (above[0] || above[1]) tc_commit_w(smem_u32(&bk->ext_empty[eb]), leader);
+              }
+              if (kt == n[g] - 1) {
+                tc_commit_w(smem_u32(&bk->q_empty[g]), leader);
+                if (sees[g]) tc_commit_w(smem_u32(&bk->rows_empty[g]), leader);
+              }
+            }
+            if (kt > 0 && kt - 1 < n[g]) {
+              mbar_wait_warp(smem_u32(&bk->p_ready[g]), pc[g] & 1, wc);
+              ++pc[g];
+              tc_fence_after();
+#pragma unroll
+              for (int kk = 0; kk < 8; ++kk)
+                tc_mma_bf16_ta_w(tm + g * 128, tm + AT_P_COL + g * 64 + kk * 8, vdesc + kk * (2048 >> 4), idesc_o,
+                                 (kt > 1 || kk > 0) ? 1u : 0u, leader);
+              tc_commit_w(smem_u32(&bk->pv_done[g]), leader);
+              if (g == (kt - 1 < n[1] ? 1 : 0)) tc_commit_w(smem_u32(&bk->empty[sv]), leader);
+            }
+          }
+          if (above[0] || above[1]) ++ec;
+        }
+        t0 += 2 * n_max;
+      }
+      // every MMA this warp issued has completed before tensor memory is given back: after an abort the
+      // softmax warps no longer wait for S or P V, so nothing else would hold the block until then
+      tc_commit_w(smem_u32(&bk->mma_done), leader);
+      mbar_wait_drain(smem_u32(&bk->mma_done), 0, AT_WAIT_LIMIT);
+      __syncwarp();
+    } else if (warp == 2) {
+      // ---------------------------------------------------------------- Eq. 3's addends, one key tile at a time, per row tile
+      // (written by the softmax warps themselves they cost those a barrier and a global load per key tile)
+      if (blockIdx.x == 0)                        // ... and the validation of the batch
+        for (int b = lane; b < a.pa.B; b += 32)
+          if (!make_desc(a.pa, b).valid) atomicOr(a.status, (uint32_t)STATUS_BAD_SAMPLE);
+      const float m_to_raw = LOG2E_F / a.scale_log2;
+      // 16-byte chunk 0 of row r of a one-k-step operand tile; chunk 1 (columns 8-15) stays zero
+      auto ext_row = [&](int tile, int r) {
+        return reinterpret_cast<uint4 *>(at_smem + AT_EXT_OFF + tile * AT_EXT_BYTES + r * 32 + (((r >> 2) & 1) << 4));
       };
-      mbar_wait(smem_u32(&bk->q_full), 0, wc);
-      issue_s(0, 0);
-      if (n_kt1 > 0) issue_s(1, 0);
-      for (int kt = 0; kt < n_max; ++kt) {
-        const int s = kt % AT_STAGES;
+      for (int t = lane; t < (2 + AT_EXT_BUFS) * AT_EXT_BYTES / 16; t += 32)
+        reinterpret_cast<uint4 *>(at_smem + AT_EXT_OFF)[t] = make_uint4(0u, 0u, 0u, 0u);
+      __syncwarp();
+      int rc[2] = {0, 0}, mc[2] = {0, 0}, ec = 0;             // row-side, diagonal and key-side addend tiles so far
+      for (int ic = 0;; ++ic) {
+        const int slot = ic % AT_ITEM_SLOTS;
+        const bool got = mbar_wait_drain(smem_u32(&bk->item_full[slot]), (ic / AT_ITEM_SLOTS) & 1, AT_WAIT_LIMIT);
+        AttnItem it;
+        if (got) it = bk->item[slot];
+        else it.b = -1;
+        __syncwarp();
+        if (lane == 0) mbar_arrive(smem_u32(&bk->item_empty[slot]));
+        if (it.b < 0) break;
+        if (!it.sees[0] && !it.sees[1]) continue;
+        const float *mlog = a.mask_log + (size_t)it.b * a.mask_b_stride + (size_t)it.h * a.mask_h_stride - it.v0;
+        // row side: columns 0-2 are 1 for a row of the span (they meet the three pieces of m_j), column 3 for any other row
+        // (it meets AT_NEVER)
 #pragma unroll
         for (int g = 0; g < 2; ++g) {
-          const int n_g = g == 0 ? n_kt0 : n_kt1;
-          if (kt >= n_g) continue;
-          mbar_wait(smem_u32(&bk->p_ready[g]), kt & 1, wc);
-          tc_fence_after();
-          if (!bk->abort_flag) {
-            const uint32_t vb = ring + s * 2 * AT_TILE_BYTES + AT_TILE_BYTES;
-#pragma unroll
-            for (int kk = 0; kk < 8; ++kk)
-              tc_mma_bf16_ta(tmem_base + g * 256 + 128, tmem_base + g * 256 + kk * 8,
-                             umma_desc_sw128(vb + (kk >> 2) * AT_BLOCK_BYTES + (kk & 3) * 32), idesc,
-                             (kt > 0 || kk > 0) ? 1u : 0u);
-            tc_commit(smem_u32(&bk->pv_done[g]));
+          if (!it.sees[g]) continue;
+          if (rc[g] >= 1) mbar_wait_warp(smem_u32(&bk->rows_empty[g]), (rc[g] - 1) & 1, wc);
+          for (int r = lane; r < 128; r += 32) {
+            const int i = it.q_base + g * 128 + r;
+            const bool vis = i >= it.v0 && i < it.v_end;
+            *ext_row(g, r) = vis ? make_uint4(0x3f803f80u, 0x00003f80u, 0u, 0u) : make_uint4(0u, 0x3f800000u, 0u, 0u);
           }
-          if (kt + 1 < n_g) issue_s(g, kt + 1);
+          fence_proxy_async();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(smem_u32(&bk->rows_full[g]));
+          ++rc[g];
         }
-        if (!bk->abort_flag) tc_commit(smem_u32(&bk->empty[s]));
+        const int n_max = max(it.n_kt[0], it.n_kt[1]);
+        for (int kt = 0; kt < n_max; ++kt) {
+          AttnTileKind kind[2];
+#pragma unroll
+          for (int g = 0; g < 2; ++g) kind[g] = attn_tile_kind(kt < it.n_kt[g] ? it.sees[g] : 0, it.q_base + g * 128, kt);
+          if (!kind[0].above && !kind[1].above && !kind[0].crossed && !kind[1].crossed) continue;
+          float m[4];                                         // keys kt * 128 + lane + 32 e
+#pragma unroll
+          for (int e = 0; e < 4; ++e) {
+            const int j = kt * 128 + lane + 32 * e;
+            m[e] = j >= it.v0 && j < it.v_end ? fmaxf(__ldg(mlog + j) * m_to_raw, AT_NEVER) : AT_NEVER;
+          }
+#pragma unroll
+          for (int g = 0; g < 2; ++g) {
+            if (!kind[g].crossed) continue;
+            if (mc[g] >= 1) mbar_wait_warp(smem_u32(&bk->m_empty[g]), (mc[g] - 1) & 1, wc);
+#pragma unroll
+            for (int e = 0; e < 4; ++e) bk->m_tile[g][lane + 32 * e] = m[e];
+            __syncwarp();
+            if (lane == 0) mbar_arrive(smem_u32(&bk->m_full[g]));
+            ++mc[g];
+          }
+          if (kind[0].above || kind[1].above) {
+            const int eb = ec % AT_EXT_BUFS;
+            if (ec >= AT_EXT_BUFS) mbar_wait_warp(smem_u32(&bk->ext_empty[eb]), ((ec / AT_EXT_BUFS) - 1) & 1, wc);
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+              // the addend as three bf16 pieces: 24 bits of mantissa, all of fp32's
+              float piece[3], rest = m[e];
+#pragma unroll
+              for (int k = 0; k < 3; ++k) {
+                piece[k] = __bfloat162float(__float2bfloat16_rn(rest));
+                rest -= piece[k];
+              }
+              *ext_row(2 + eb, lane + 32 * e) = make_uint4(pack2_rn(piece[0], piece[1]), pack2_rn(piece[2], AT_NEVER), 0u, 0u);
+            }
+            fence_proxy_async();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(smem_u32(&bk->ext_full[eb]));
+            ++ec;
+          }
+        }
       }
-      // every MMA this thread issued has completed before tensor memory is given back: after an abort the
-      // softmax warps no longer wait for S or P V, so nothing else would hold the block until then
-      tc_commit(smem_u32(&bk->mma_done));
-      mbar_wait_drain(smem_u32(&bk->mma_done), 0, AT_WAIT_LIMIT);
     }
   } else {
-    // Two threads per query row: warps w and w + 4 of a group own the same 32 rows (tensor-memory
-    // lanes) and one half of the tile's 128 key columns each.
-    const int sw = warp - 2;
-    const int g = sw >> 3;                        // row tile of this softmax group
-    const int hf = (sw >> 2) & 1;                 // column half
+    reg_inc<216>();
+    // ------------------------------------------------------------------ softmax: one thread per query row
+    const int g = (warp - 4) >> 2;                // row tile of this warpgroup
     const int quarter = warp & 3;                 // the TMEM lanes this warp may read
     const int lrow = quarter * 32 + lane;
-    const int q_lo = q_base + g * 128;
-    const int i = q_lo + lrow;                    // sequence-relative query row
-    const bool vis_row = a.mask_enable && i >= d.v0 && i < d.v0 + d.nv;
-    const int hi_adm = min(d.n - 1, vis_row ? max(i, d.v0 + d.nv - 1) : i);   // last admitted key
-    const uint32_t s_row = tmem_base + ((uint32_t)(quarter * 32) << 16) + g * 256;
-    const uint32_t s_addr = s_row + hf * 64;      // this thread's 64 logits
-    const uint32_t p_addr = s_row + hf * 32;      // its 64 probabilities, packed in 32 columns
-    const uint32_t o_addr = s_row + 128 + hf * 64;   // its 64 columns of O
-    const float *mlog_b = a.mask_log ? a.mask_log + (size_t)b * a.mask_b_stride + (size_t)h * a.mask_h_stride : nullptr;
-    const int st = (threadIdx.x - 64) & 255;      // 0..255 inside the group
-    const int my_kt = g == 0 ? n_kt0 : n_kt1;
-    const bool my_sees = g == 0 ? sees0 : sees1;
-    const int pair_bar = 1 + g * 4 + quarter;     // named barrier of the two warps that share these rows
-    const int group_bar = 9 + g;
-
-    // Logits stay in the units the MMA produced (q.k); the scale log2(e)/sqrt(d) enters inside the
-    // exponential's multiply-add.  m_ref is the reference maximum in those units.
-    const float step_raw = AT_RESCALE_STEP / a.scale_log2;
-    const float m_to_raw = 1.4426950408889634f / a.scale_log2;
-    float m_ref = -INFINITY, l_run = 0.f;
-    for (int kt = 0; kt < my_kt; ++kt) {
-      const int j0 = kt * 128 - delta;            // sequence-relative key of column 0
-      // a tile strictly below the diagonal for every row of the row tile needs no mask at all
-      const bool plain = j0 >= 0 && j0 + 127 <= q_lo && j0 + 127 < d.n;
-      const bool soft = !plain && my_sees && j0 + 127 > q_lo;      // may hold future keys of the span
-      const float *mt = bk->m_tile[g] + hf * 64;
-      // addend of key j for a query row of the span that lies before it: m_j inside the
-      // span, -infinity outside (such a key is never admitted above the diagonal)
-      float mv = -INFINITY;
-      if (soft && st < 128) {
-        const int j = j0 + st;
-        if (mlog_b && j >= d.v0 && j < d.v0 + d.nv) mv = __ldg(mlog_b + (j - d.v0)) * m_to_raw;
-      }
-      mbar_wait(smem_u32(&bk->s_full[g]), kt & 1, wc);
-      tc_fence_after();
-      if (soft) {
-        // every thread of the group has finished the previous tile (its arrival was needed for
-        // the S just waited for), so the addends can be replaced
-        if (st < 128) bk->m_tile[g][st] = mv;
-        asm volatile("bar.sync %0, 256;" ::"r"(group_bar) : "memory");
-      }
-      // ---- this thread's 64 logits, once
-      uint32_t xr[64];
-      tmem_ld32p(s_addr, xr);
-      tmem_ld32p(s_addr + 32, xr + 32);
-      tmem_wait_ld();
-      float mx4[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};     // four independent chains
-      if (plain) {
-#pragma unroll
-        for (int c = 0; c < 64; ++c) mx4[c & 3] = fmaxf(mx4[c & 3], __uint_as_float(xr[c]));
-      } else {
-        // columns relative to this half: the diagonal, the first and the last admitted column
-        const int di = i - j0 - hf * 64, lo = -j0 - hf * 64, hi = hi_adm - j0 - hf * 64;
-        if (soft && j0 > q_lo + 127) {
-          // the whole tile lies above the diagonal of every row of the row tile: a row of the span
-          // admits exactly the keys of the span (finite addend), any other row admits nothing.  Two
-          // additions per logit on the FMA pipe instead of compares and selects on the half-rate one.
-          const float rowoff = vis_row ? 0.f : -INFINITY;
-#pragma unroll
-          for (int c4 = 0; c4 < 64; c4 += 4) {
-            const float4 m4 = *reinterpret_cast<const float4 *>(mt + c4);
-            const float add[4] = {m4.x, m4.y, m4.z, m4.w};
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-              const float v = __uint_as_float(xr[c4 + e]) + (add[e] + rowoff);
-              xr[c4 + e] = __float_as_uint(v);
-              mx4[e] = fmaxf(mx4[e], v);
-            }
-          }
-        } else if (soft) {
-          // the addends are loaded unconditionally (four per load) and selected, so the loop has no branch
-#pragma unroll
-          for (int c4 = 0; c4 < 64; c4 += 4) {
-            const float4 m4 = *reinterpret_cast<const float4 *>(mt + c4);
-            const float add[4] = {m4.x, m4.y, m4.z, m4.w};
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-              const int c = c4 + e;
-              float v = __uint_as_float(xr[c]) + (c > di ? add[e] : 0.f);
-              v = (c < lo || c > hi) ? -INFINITY : v;
-              xr[c] = __float_as_uint(v);
-              mx4[e] = fmaxf(mx4[e], v);
-            }
-          }
-        } else {
-#pragma unroll
-          for (int c = 0; c < 64; ++c) {
-            const float v = (c < lo || c > hi) ? -INFINITY : __uint_as_float(xr[c]);
-            xr[c] = __float_as_uint(v);
-            mx4[c & 3] = fmaxf(mx4[c & 3], v);
-          }
-        }
-      }
-      float mx = fmaxf(fmaxf(mx4[0], mx4[1]), fmaxf(mx4[2], mx4[3]));
-      // ---- the running row maximum over both halves and all tiles so far.  (The partner has read
-      // its logits by the time it passes this barrier, so the probabilities may overwrite them.)
-      atomicMax(&bk->row_max[g][lrow], attn_key(mx));
-      asm volatile("bar.sync %0, 64;" ::"r"(pair_bar) : "memory");
-      mx = attn_unkey(bk->row_max[g][lrow]);
-      // ---- move the reference (and rescale O) only when some row of the warp outgrew it
-      if (kt == 0) {
-        m_ref = mx;
-      } else {
-        const bool need = mx > m_ref + step_raw;
-        if (__any_sync(0xffffffffu, need)) {
-          // O holds every earlier P V: the S just waited for was committed after them
-          const float f = need ? fast_exp2((m_ref - mx) * a.scale_log2) : 1.0f;
-#pragma unroll
-          for (int c0 = 0; c0 < 64; c0 += 16) {
-            uint32_t r[16];
-            tmem_ld16(o_addr + c0, r);
+    const uint32_t lane_addr = tmem_base + ((uint32_t)(quarter * 32) << 16);
+    const uint32_t s_addr = lane_addr + AT_S_COL, p_addr = lane_addr + AT_P_COL + g * 64, o_addr = lane_addr + g * 128;
+    const float scale = a.scale_log2;
+    const uint64_t scale2 = f2_pack(scale, scale);
+    int ic = 0, sc = 0, mc = 0;                   // items / key tiles / addend tiles so far
+    while (true) {
+      const int slot = ic % AT_ITEM_SLOTS;
+      const bool got = mbar_wait_drain(smem_u32(&bk->item_full[slot]), (ic / AT_ITEM_SLOTS) & 1, AT_WAIT_LIMIT);
+      AttnItem it;
+      if (got) it = bk->item[slot];
+      else it.b = -1;
+      __syncwarp();
+      if (lane == 0) mbar_arrive(smem_u32(&bk->item_empty[slot]));
+      ++ic;
+      if (it.b < 0) break;
+      const int my_kt = g == 0 ? it.n_kt[0] : it.n_kt[1];
+      if (my_kt == 0) continue;
+      const int my_sees = g == 0 ? it.sees[0] : it.sees[1];
+      const int q_lo = it.q_base + g * 128;
+      const int i = q_lo + lrow;                    // sequence-relative query row
+      const int i_lo = q_lo + quarter * 32;         // first row of this warp
+      const bool vis_row = a.mask_enable && i >= it.v0 && i < it.v_end;
+      const int hi_adm = min(it.n - 1, vis_row ? max(i, it.v_end - 1) : i);   // last admitted key
+      // p = 2^((x - ref) * scale), x = q.k + addend.  The reference is the maximum of the row's first key tile and then
+      // stays: a reference below the running maximum only scales the sums.  Should a tile's sum outgrow AT_SUM_LIMIT in some
+      // row of the warp, that tile is done again with the row's true maximum as the new reference (O and the sum so far
+      // are rescaled), so no tile but the first needs a pass for its maximum.
+      // The code of a key tile is straight-line (its logits are in registers), and its size matters: with an own version
+      // per kind of mask it outgrew the instruction cache and ran at half the speed.  So the masks only change x.
+      float neg_ref = 0.f, l_run = 0.f;             // -ref * scale
+      for (int kt = 0; kt < my_kt; ++kt, ++sc) {
+        const int j0 = kt * 128;                    // key of column 0
+        const AttnTileKind kind = attn_tile_kind(my_sees, q_lo, kt);
+        mbar_wait(smem_u32(&bk->s_full[g]), sc & 1, wc);
+        tc_fence_after();
+        if (!kind.above && (j0 + 127 > i_lo || j0 + 127 >= it.n)) {
+          // Some row of the warp does not admit every key, or needs an addend for a later one: the logits are put right
+          // in tensor memory, 32 keys at a time (a loop: once per row tile or twice, and straight-line code of that length
+          // would run from outside the instruction cache).  Where no addend belongs to the key tile nothing above the
+          // diagonal is admitted, and c > hi hides whatever m_tile holds.
+          if (kind.crossed) mbar_wait(smem_u32(&bk->m_full[g]), mc & 1, wc);
+          const int di = i - j0, hi = hi_adm - j0;  // columns of the diagonal and of the last admitted key
+#pragma unroll 1
+          for (int c0 = 0; c0 < 128; c0 += 32) {
+            if (j0 + c0 + 31 <= i_lo && j0 + c0 + 31 < it.n) continue;       // nothing to do for any row of the warp
+            uint32_t r[32];
+            tmem_ld32(s_addr + c0, r);
             tmem_wait_ld();
 #pragma unroll
-            for (int e = 0; e < 16; ++e) r[e] = __float_as_uint(__uint_as_float(r[e]) * f);
-            tmem_st16(o_addr + c0, r);
+            for (int c4 = 0; c4 < 32; c4 += 4) {
+              const float4 m4 = *reinterpret_cast<const float4 *>(bk->m_tile[g] + c0 + c4);
+              const float add[4] = {m4.x, m4.y, m4.z, m4.w};
+#pragma unroll
+              for (int e = 0; e < 4; ++e) {
+                const int c = c0 + c4 + e;
+                const float v = __uint_as_float(r[c4 + e]) + (c > di ? add[e] : 0.f);
+                r[c4 + e] = __float_as_uint(c > hi ? -INFINITY : v);
+              }
+            }
+            tmem_st32(s_addr + c0, r);
           }
-          l_run *= f;
-          if (need) m_ref = mx;
+          tmem_wait_st();
+          if (kind.crossed) {
+            __syncwarp();
+            if (lane == 0) mbar_arrive(smem_u32(&bk->m_empty[g]));
+            ++mc;
+          }
         }
-      }
-      // ---- probabilities relative to the reference, stored as bf16 over S's first 64 columns
-      const float neg_ref = -m_ref * a.scale_log2;
-      float l0 = 0.f, l1 = 0.f;
+        // ---- this row's 128 logits, once
+        uint32_t xr[128];
 #pragma unroll
-      for (int c0 = 0; c0 < 64; c0 += 32) {
-        uint32_t w[16];
-#pragma unroll
-        for (int e = 0; e < 16; ++e) {
-          const float p0 = fast_exp2(fmaf(__uint_as_float(xr[c0 + 2 * e]), a.scale_log2, neg_ref));
-          const float p1 = fast_exp2(fmaf(__uint_as_float(xr[c0 + 2 * e + 1]), a.scale_log2, neg_ref));
-          l0 += p0;
-          l1 += p1;
-          w[e] = pack2_rn(p0, p1);
+        for (int c = 0; c < 128; c += 32) tmem_ld32p(s_addr + c, xr + c);
+        tmem_wait_ld();
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(smem_u32(&bk->s_empty));
+        if (kt > 0) {
+          mbar_wait(smem_u32(&bk->pv_done[g]), (sc - 1) & 1, wc);      // O is complete up to here, and P may be overwritten
+          tc_fence_after();
         }
-        tmem_st16(p_addr + (c0 >> 1), w);
+        bool move = kt == 0, again = kt == 0;
+        float tile_sum;
+#pragma unroll 1
+        while (true) {
+          if (again) {
+            // ---- the row's true maximum becomes the reference of the rows that need it
+            float mx4[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};       // four independent chains
+#pragma unroll
+            for (int c = 0; c < 128; c += 8)
+#pragma unroll
+              for (int e = 0; e < 4; ++e) mx4[e] = max3(mx4[e], __uint_as_float(xr[c + e]), __uint_as_float(xr[c + 4 + e]));
+            const float neg = -fmaxf(fmaxf(mx4[0], mx4[1]), fmaxf(mx4[2], mx4[3])) * scale;   // (key 0 is admitted by every row: finite)
+            if (kt > 0) {
+              const float f = move ? fast_exp2(neg - neg_ref) : 1.0f;
+#pragma unroll 1
+              for (int c0 = 0; c0 < 128; c0 += 16) {
+                uint32_t r[16];
+                tmem_ld16(o_addr + c0, r);
+                tmem_wait_ld();
+#pragma unroll
+                for (int e = 0; e < 16; ++e) r[e] = __float_as_uint(__uint_as_float(r[e]) * f);
+                tmem_st16(o_addr + c0, r);
+              }
+              l_run *= f;
+            }
+            if (move) neg_ref = neg;
+          }
+          // ---- probabilities relative to the reference, stored as bf16
+          const uint64_t neg2 = f2_pack(neg_ref, neg_ref);
+          uint64_t sum2[2] = {0ull, 0ull};          // even and odd keys apart, two chains
+#pragma unroll
+          for (int c0 = 0; c0 < 128; c0 += 32) {
+            uint32_t w[16];
+#pragma unroll
+            for (int e = 0; e < 16; ++e) {
+              float p0, p1;
+              f2_unpack(f2_fma(f2_pack(__uint_as_float(xr[c0 + 2 * e]), __uint_as_float(xr[c0 + 2 * e + 1])), scale2, neg2), p0, p1);
+              p0 = fast_exp2(p0);
+              p1 = fast_exp2(p1);
+              sum2[e & 1] = f2_add(sum2[e & 1], f2_pack(p0, p1));
+              w[e] = pack2_rn(p0, p1);
+            }
+            tmem_st16(p_addr + (c0 >> 1), w);
+          }
+          float s0, s1;
+          f2_unpack(f2_add(sum2[0], sum2[1]), s0, s1);
+          tile_sum = s0 + s1;
+          move = !(tile_sum < AT_SUM_LIMIT);
+          if (again || !__any_sync(0xffffffffu, move)) break;   // (relative to the true maximum no sum exceeds 128)
+          again = true;
+        }
+        l_run += tile_sum;
+        tmem_wait_st();
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(smem_u32(&bk->p_ready[g]));
       }
-      l_run += l0 + l1;
-      tmem_wait_st();
-      tc_fence_before();
-      mbar_arrive(smem_u32(&bk->p_ready[g]));
-    }
-    // ---- normalisation and store: the two halves of a row add their sums first
-    if (my_kt > 0) {
-      // the row's slot of maxima is free once both threads have read the last one
-      asm volatile("bar.sync %0, 64;" ::"r"(pair_bar) : "memory");
-      if (hf == 0) bk->row_max[g][lrow] = __float_as_uint(l_run);
-      asm volatile("bar.sync %0, 64;" ::"r"(pair_bar) : "memory");
-      if (hf == 1) {
-        l_run += __uint_as_float(bk->row_max[g][lrow]);
-        bk->row_max[g][lrow] = __float_as_uint(l_run);
-      }
-      asm volatile("bar.sync %0, 64;" ::"r"(pair_bar) : "memory");
-      if (hf == 0) l_run = __uint_as_float(bk->row_max[g][lrow]);
-      mbar_wait(smem_u32(&bk->pv_done[g]), (my_kt - 1) & 1, wc);
+      // ---- normalisation and store
+      mbar_wait(smem_u32(&bk->pv_done[g]), (sc - 1) & 1, wc);
       tc_fence_after();
       const float inv_l = l_run > 0.f ? 1.0f / l_run : 0.f;
-      const bool store = i < d.n && !bk->abort_flag;
-      uint4 *orow = reinterpret_cast<uint4 *>(a.out + ((size_t)(d.row0 + i) * a.H + h) * 128 + hf * 64);
-#pragma unroll
-      for (int c0 = 0; c0 < 64; c0 += 32) {
+      // Through shared memory (32 columns at a time, 16-byte chunk c of row r at c ^ ((r >> 1) & 3)), so that a store
+      // instruction covers eight pieces of 64 bytes: with one row per lane it touches 32 lines, and the eight warps'
+      // stores of an item took 2100 clocks.
+      uint8_t *stage = at_smem + AT_STAGE_OFF + (warp - 4) * AT_STAGE_BYTES;
+      __nv_bfloat16 *orow = a.out + ((size_t)(it.row0 + i_lo) * a.H + it.h) * 128;
+      const int rows = bk->abort_flag ? 0 : it.n - i_lo;       // rows of this warp inside the sequence
+#pragma unroll 1
+      for (int c0 = 0; c0 < 128; c0 += 32) {
         uint32_t r[32];
         tmem_ld32(o_addr + c0, r);
         tmem_wait_ld();
-        if (store) {
+        __syncwarp();                               // the previous piece has been read
 #pragma unroll
-          for (int q4 = 0; q4 < 4; ++q4) {
-            uint4 w;
-            w.x = pack2_rn(__uint_as_float(r[8 * q4 + 0]) * inv_l, __uint_as_float(r[8 * q4 + 1]) * inv_l);
-            w.y = pack2_rn(__uint_as_float(r[8 * q4 + 2]) * inv_l, __uint_as_float(r[8 * q4 + 3]) * inv_l);
-            w.z = pack2_rn(__uint_as_float(r[8 * q4 + 4]) * inv_l, __uint_as_float(r[8 * q4 + 5]) * inv_l);
-            w.w = pack2_rn(__uint_as_float(r[8 * q4 + 6]) * inv_l, __uint_as_float(r[8 * q4 + 7]) * inv_l);
-            orow[(c0 >> 3) + q4] = w;
-          }
+        for (int c = 0; c < 4; ++c) {
+          uint32_t w[4];
+#pragma unroll
+          for (int e = 0; e < 4; ++e)
+            w[e] = pack2_rn(__uint_as_float(r[8 * c + 2 * e]) * inv_l, __uint_as_float(r[8 * c + 2 * e + 1]) * inv_l);
+          *reinterpret_cast<uint4 *>(stage + lane * 64 + ((c ^ ((lane >> 1) & 3)) << 4)) = make_uint4(w[0], w[1], w[2], w[3]);
+        }
+        __syncwarp();
+#pragma unroll
+        for (int r8 = 0; r8 < 32; r8 += 8) {
+          const int rr = r8 + (lane >> 2), c = lane & 3;
+          const uint4 x = *reinterpret_cast<const uint4 *>(stage + rr * 64 + ((c ^ ((rr >> 1) & 3)) << 4));
+          if (rr < rows) *reinterpret_cast<uint4 *>(orow + (size_t)rr * a.H * 128 + c0 + c * 8) = x;
         }
       }
+      tc_fence_before();                            // the next item's first P (and so its first P V) comes after these loads
     }
-    tc_fence_before();
   }
   tc_fence_before();
   __syncthreads();
   if (warp == 1) {
     tc_fence_after();
     tmem_dealloc(tmem_base, AT_TMEM_COLS);
+  }
+  // the block that leaves last puts the work counters back to zero for the next launch (every block has drawn its
+  // last item by then)
+  if (threadIdx.x == 0) {
+    const unsigned int done = atomicAdd(a.work + 1, 1u);
+    if (done == gridDim.x - 1) {
+      a.work[0] = 0u;
+      a.work[1] = 0u;
+      __threadfence();
+    }
   }
 }
 

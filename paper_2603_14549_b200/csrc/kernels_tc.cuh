@@ -21,7 +21,6 @@
 namespace asap {
 
 constexpr long long TC_WAIT_LIMIT = 1500000000LL;   // clock cycles, roughly one second
-constexpr float LOG2E_F = 1.4426950408889634f;
 
 // named barriers of the score kernel: 2 = all eight epilogue
 // warps; 3 / 4 = one of its two epilogue groups

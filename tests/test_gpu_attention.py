@@ -75,6 +75,20 @@ def test_attention_matches_oracle(ctx, nvs, texts, lam):
     print("attention max abs err", _compare(batch, v, out, ms))
 
 
+@pytest.mark.parametrize("where,scale", [(140, 300.0), (300, 300.0), (300, 40.0)])
+def test_a_late_dominant_key_moves_the_softmax_reference(ctx, where, scale):
+    """One key of a later key tile is scaled so that its logits exceed all earlier ones by hundreds of nats in some
+    rows (and fall that far below in others): relative to the first tile's maximum the probabilities overflow there, so
+    those rows' tile is done again with a new reference and what they have summed so far is rescaled."""
+    batch = W.tiny(B=2, n_vis=[400, 330], text_lens=[40, 150], H=2, keep_k=8, seed=615)
+    for b in range(2):
+        row = int(batch.cu_seqlens[b]) + int(batch.vis_start[b]) + where
+        batch.k[row] = (batch.k[row].float() * scale).to(torch.bfloat16)
+    v = W.draw_values(batch, 86)
+    m, ms = _mask_vectors(batch, 1.0)
+    _compare(batch, v, _run(ctx, batch, v, m), ms)
+
+
 def test_mask_off_is_causal_attention_and_only_visual_rows_differ(ctx):
     batch = W.tiny(B=2, n_vis=[200, 333], text_lens=[17, 5], H=2, keep_k=8, seed=610)
     v = W.draw_values(batch, 78)
