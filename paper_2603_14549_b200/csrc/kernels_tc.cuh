@@ -93,11 +93,11 @@ struct ScoreArgs {
 };
 
 struct ScoreBook {             // bookkeeping block placed after the tiles in shared memory
-  uint64_t full[SC_STAGES], empty[SC_STAGES], q_full, q_empty, acc_full[2], acc_empty[2];
+  uint64_t full[SC_STAGES], empty[SC_STAGES], q_full, q_empty, acc_full[4], acc_empty[4];
   uint64_t item_full[SC_ITEM_SLOTS], item_empty[SC_ITEM_SLOTS], mma_done, qbar_ready;
   int item_q[SC_ITEM_SLOTS];   // items drawn by the producer, -1 = no more
-  alignas(16) float off[256];  // per ranking row of the pair: max + log2(sum), +inf for rows past its end
-                               // (with one row tile, off[128..255] carries group 1's partial sums)
+  alignas(16) float noff[256]; // per ranking row of the pair: -(max + log2(sum)), -inf for rows past its end
+                               // (with one row tile, noff[128..255] carries group 1's partial sums)
   alignas(16) float soft[2][128];   // per epilogue group, per key of its current tile: m_j*log2(e) or -inf
                                // (soft[1] also carries group 1's partial maxima at the end of pass 1)
   uint32_t tmem_base;
@@ -157,9 +157,9 @@ score_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__
     }
     mbar_init(smem_u32(&bk->q_full), 1);
     mbar_init(smem_u32(&bk->q_empty), 1);
-    for (int i = 0; i < 2; ++i) {
+    for (int i = 0; i < 4; ++i) {
       mbar_init(smem_u32(&bk->acc_full[i]), 1);
-      mbar_init(smem_u32(&bk->acc_empty[i]), 8);          // every epilogue warp
+      mbar_init(smem_u32(&bk->acc_empty[i]), 4);          // the epilogue warps of the group that owns the buffer
     }
     for (int i = 0; i < SC_ITEM_SLOTS; ++i) {
       mbar_init(smem_u32(&bk->item_full[i]), 1);
@@ -248,7 +248,8 @@ score_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__
     // goes on multiplying whatever lies in the block's own memory: nothing of it is used)
     const uint32_t leader = warp_leader();
     const uint32_t tm = __shfl_sync(0xffffffffu, tmem_base, 0);
-    int kc = 0, qc = 0, g = 0, ic = 0, mc = 0;        // mc: items whose summed-query rows were waited for
+    int kc = 0, qc = 0, ic = 0, mc = 0;               // mc: items whose summed-query rows were waited for
+    int ops0 = 0, ops1 = 0;                           // operations given to either epilogue group
     const uint32_t idesc1 = umma_idesc_bf16(128, 128);
     const uint64_t qdesc = umma_desc_sw128(q_smem), kdesc0 = umma_desc_sw128(k_smem);   // (every tile lies below 256 KB: offsets never carry out of the address field)
     while (true) {
@@ -267,28 +268,39 @@ score_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__
       for (int rp = 0; rp < n_rp; ++rp, ++qc) {
         const RowPair T = score_row_pair(d, rp, a.mask_enable, pair_rows);
         const bool mass_here = with_mass && rp == 0;         // three more columns (16 with padding): the summed query
-        const uint32_t idesc2 = umma_idesc_bf16(128, T.n2 + (mass_here ? 16 : 0));
+        const int n2 = T.n2 + (mass_here ? 16 : 0);          // columns of a pass-2 accumulator
         mbar_wait_warp(smem_u32(&bk->q_full), qc & 1, wc);
-        for (int u = 0; u < T.n_kt + T.n_p2; ++u, ++kc, ++g) {
-          const bool pass1 = u < T.n_kt;
+        // the accumulator of group gr's next operation, once the group has given it back
+        auto acc = [&](int gr) -> int {
+          const int n = gr ? ops1 : ops0, buf = 2 * gr + (n & 1);
+          if (gr) ++ops1;
+          else ++ops0;
+          if (n >= 2) mbar_wait_warp(smem_u32(&bk->acc_empty[buf]), ((n >> 1) - 1) & 1, wc);
+          tc_fence_after();
+          return buf;
+        };
+        for (int u = 0; u < T.n_kt + T.n_p2; ++u, ++kc) {
+          const int s = kc % SC_STAGES;
           if (mass_here && u == T.n_kt) {                    // an epilogue warp has written the summed-query rows
             mbar_wait_warp(smem_u32(&bk->qbar_ready), mc & 1, wc);
             ++mc;
           }
-          const int s = kc % SC_STAGES, hh = g & 1;
           mbar_wait_warp(smem_u32(&bk->full[s]), (kc / SC_STAGES) & 1, wc);
-          if (g >= 2) mbar_wait_warp(smem_u32(&bk->acc_empty[hh]), ((g >> 1) - 1) & 1, wc);
-          tc_fence_after();
-          const uint32_t dcol = tm + hh * 256;
           const uint64_t kdesc = kdesc0 + s * (SC_TILE_BYTES >> 4);
-          if (pass1) {
-            tc_mma_bf16_k128_w(dcol, qdesc, kdesc, SC_Q_HALF_BYTES, SC_HALF_BYTES, idesc1, leader);
-            if (T.nrt == 2)
-              tc_mma_bf16_k128_w(dcol + 128, qdesc + (SC_HALF_BYTES >> 4), kdesc, SC_Q_HALF_BYTES, SC_HALF_BYTES, idesc1, leader);
+          if (u < T.n_kt) {
+            for (int rt = 0; rt < T.nrt; ++rt) {
+              const int buf = acc(T.nrt == 2 ? rt : u & 1);
+              tc_mma_bf16_k128_w(tm + buf * 128, qdesc + rt * (SC_HALF_BYTES >> 4), kdesc, SC_Q_HALF_BYTES, SC_HALF_BYTES, idesc1, leader);
+              tc_commit_w(smem_u32(&bk->acc_full[buf]), leader);
+            }
           } else {
-            tc_mma_bf16_k128_w(dcol, kdesc, qdesc, SC_HALF_BYTES, SC_Q_HALF_BYTES, idesc2, leader);
+            for (int c0 = 0; c0 < n2; c0 += 128) {
+              const int buf = acc((u - T.n_kt + 1) & 1);
+              tc_mma_bf16_k128_w(tm + buf * 128, kdesc, qdesc + (c0 >> 7) * (SC_HALF_BYTES >> 4), SC_HALF_BYTES, SC_Q_HALF_BYTES,
+                                 umma_idesc_bf16(128, min(128, n2 - c0)), leader);
+              tc_commit_w(smem_u32(&bk->acc_full[buf]), leader);
+            }
           }
-          tc_commit_w(smem_u32(&bk->acc_full[hh]), leader);
           tc_commit_w(smem_u32(&bk->empty[s]), leader);
         }
         if (mass_here && T.n_p2 == 0) {                      // (no visual key tile: keep the barrier's phases in step)
@@ -313,8 +325,9 @@ score_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__
     const float scale = a.scale_log2;
     const uint32_t tlane0 = tmem_base + ((uint32_t)(quarter * 32) << 16);
     float *soft = bk->soft[group];
-    float *pm = bk->soft[1], *pl = bk->off + 128;  // group 1's (max, sum) when both groups share one row tile
-    int g = 0, ic = 0, qc = 0;
+    float *pm = bk->soft[1], *pl = bk->noff + 128; // group 1's (max, sum) when both groups share one row tile
+    const uint64_t scale2 = f2_pack(scale, scale);
+    int ops = 0, ic = 0, qc = 0;                   // ops: operations of this group so far
     while (true) {
       const int slot = ic % SC_ITEM_SLOTS;
       const bool got = mbar_wait_drain(smem_u32(&bk->item_full[slot]), (ic / SC_ITEM_SLOTS) & 1, TC_WAIT_LIMIT);
@@ -385,21 +398,20 @@ score_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__
         const int p_i = T.R0 + my_row;
         const bool row_vis = T.use_soft && p_i >= d.v0 && p_i < v_end;
         float m = -INFINITY, l = 0.f;
-        for (int t = 0; t < T.n_kt; ++t, ++g) {
-          const int hh = g & 1;
-          const bool mine = two || hh == group;
+        for (int t = two ? 0 : group; t < T.n_kt; t += two ? 1 : 2, ++ops) {
+          const int buf = 2 * group + (ops & 1);
           const int j0 = t * 128;
           const bool fast = (j0 + 127 <= T.R0 + (two ? group * 128 : 0));
-          const bool stage_soft = mine && T.use_soft && !fast;
+          const bool stage_soft = T.use_soft && !fast;
           if (stage_soft) {
             const int j = j0 + lrow;
             soft[lrow] = (j >= d.v0 && j < v_end) ? __ldg(mlog + (j - d.v0)) * LOG2E_F : -INFINITY;
             group_bar_sync(group);
           }
-          const uint32_t tlane = tlane0 + hh * 256 + (two ? group * 128 : 0);
-          mbar_wait(smem_u32(&bk->acc_full[hh]), (g >> 1) & 1, wc);
+          const uint32_t tlane = tlane0 + buf * 128;
+          mbar_wait(smem_u32(&bk->acc_full[buf]), (ops >> 1) & 1, wc);
           tc_fence_after();
-          if (mine && warp_rows && !bk->abort_flag) {
+          if (warp_rows && !bk->abort_flag) {
 #pragma unroll 1
             for (int c = 0; c < 128; c += 64) {
               uint32_t r[64];
@@ -412,10 +424,17 @@ score_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__
                 // exp2(dot * scale - m) without looking for a new maximum (a stale reference only scales
                 // the sum; off_i = m + log2(l) comes out the same).  Should a term outgrow fp32's range
                 // the chunk is done again below, with its true maximum as the new reference.
-                float sm[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+                const uint64_t negm2 = f2_pack(-m, -m);
+                uint64_t sm2[4] = {0ull, 0ull, 0ull, 0ull};
 #pragma unroll
-                for (int e = 0; e < 64; ++e) sm[e & 7] += fast_exp2(fmaf(__uint_as_float(r[e]), scale, -m));
-                const float cs = ((sm[0] + sm[1]) + (sm[2] + sm[3])) + ((sm[4] + sm[5]) + (sm[6] + sm[7]));
+                for (int e = 0; e < 64; e += 2) {
+                  float x0, x1;
+                  f2_unpack(f2_fma(f2_pack(__uint_as_float(r[e]), __uint_as_float(r[e + 1])), scale2, negm2), x0, x1);
+                  sm2[(e >> 1) & 3] = f2_add(sm2[(e >> 1) & 3], f2_pack(fast_exp2(x0), fast_exp2(x1)));
+                }
+                float cs, c1;
+                f2_unpack(f2_add(f2_add(sm2[0], sm2[1]), f2_add(sm2[2], sm2[3])), cs, c1);
+                cs += c1;
                 if (cs < 1e30f) {
                   if (row_ok) l += cs;
                   summed = true;
@@ -478,16 +497,15 @@ score_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__
           }
           tc_fence_before();
           __syncwarp();
-          if (lane == 0) mbar_arrive(smem_u32(&bk->acc_empty[hh]));
+          if (lane == 0) mbar_arrive(smem_u32(&bk->acc_empty[buf]));
           if (stage_soft) group_bar_sync(group);   // soft[] is rewritten by this group's next masked tile
         }
         // off_i = max_i + log2(sum_i), so that exp2(x - off_i) = exp2(x - max_i) / sum_i.  With one row
         // tile the two groups saw disjoint key tiles: their (max, sum) per row are merged first
+        epi_bar_sync();                             // both groups are past the previous row pair's offsets and the last soft[1]
         if (two) {
-          bk->off[my_row] = row_ok ? (m + __log2f(l)) : INFINITY;
-          epi_bar_sync();
+          bk->noff[my_row] = row_ok ? -(m + __log2f(l)) : -INFINITY;
         } else {
-          epi_bar_sync();                           // group 0 is past its last use of soft[1] and off[128..]
           if (group == 1) { pm[lrow] = m; pl[lrow] = l; }
           epi_bar_sync();
           if (group == 0) {
@@ -496,77 +514,88 @@ score_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__
             float ll = 0.f;
             if (m > -INFINITY) ll += l * fast_exp2(m - mm);
             if (m1 > -INFINITY) ll += l1 * fast_exp2(m1 - mm);
-            bk->off[lrow] = row_ok ? (mm + __log2f(ll)) : INFINITY;
+            bk->noff[lrow] = row_ok ? -(mm + __log2f(ll)) : -INFINITY;
           }
-          epi_bar_sync();
         }
+        epi_bar_sync();
         // ---------------- pass 2: thread = key; the groups take alternate visual key tiles
-        for (int u = 0; u < T.n_p2; ++u, ++g) {
-          const int hh = g & 1;
-          const bool mine = hh == group;
+        const int n2 = T.n2 + (with_mass && rp == 0 ? 16 : 0);
+        for (int u = group ^ 1; u < T.n_p2; u += 2) {
           const int t = T.t_hi - u, j0 = t * 128;
           const int j = j0 + lrow;
           const bool key_ok = j >= d.v0 && j < v_end;
           const bool fast = (j0 + 127 <= T.R0);
           const bool warp_keys = (j0 + quarter * 32 + 31 >= d.v0) && (j0 + quarter * 32 < v_end);
-          const float soft_j = (mine && T.use_soft && key_ok) ? __ldg(mlog + (j - d.v0)) * LOG2E_F : -INFINITY;
-          const uint32_t tlane = tlane0 + hh * 256;
-          mbar_wait(smem_u32(&bk->acc_full[hh]), (g >> 1) & 1, wc);
-          tc_fence_after();
-          if (mine && warp_keys && !bk->abort_flag) {
-            float sm[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+          const float soft_j = (T.use_soft && key_ok) ? __ldg(mlog + (j - d.v0)) * LOG2E_F : -INFINITY;
+          uint64_t sm2[4] = {0ull, 0ull, 0ull, 0ull};
 #pragma unroll 1
-            for (int c = 0; c < T.n2; c += 32) {
-              uint32_t r[32];
-              const bool full = c + 32 <= T.n2;       // n2 is a multiple of 16: the last chunk may be half
-              if (full) tmem_ld32p(tlane + c, r);
-              else {
-                tmem_ld16p(tlane + c, r);
+          for (int h0 = 0; h0 < n2; h0 += 128, ++ops) {
+            const int buf = 2 * group + (ops & 1);
+            const uint32_t tlane = tlane0 + buf * 128;
+            mbar_wait(smem_u32(&bk->acc_full[buf]), (ops >> 1) & 1, wc);
+            tc_fence_after();
+            if (warp_keys && !bk->abort_flag) {
+              const int n_here = min(128, T.n2 - h0);
+#pragma unroll 1
+              for (int c = 0; c < n_here; c += 32) {
+                uint32_t r[32];
+                if (c + 32 <= n_here) tmem_ld32p(tlane + c, r);
+                else {                                // n2 is a multiple of 16: the last chunk may be half
+                  tmem_ld16p(tlane + c, r);
 #pragma unroll
-                for (int e = 16; e < 32; ++e) r[e] = 0u;
-              }
-              tmem_wait_ld();
-              // rows past the pair's end have off = +inf (every entry up to the next multiple of 128 is
-              // written), so their terms vanish; four offsets per shared-memory load
-              float o32[32];
+                  for (int e = 16; e < 32; ++e) r[e] = 0u;
+                }
+                tmem_wait_ld();
+                // rows past the pair's end have the offset -inf (every entry up to the next multiple of 128 is
+                // written), so their terms vanish; four offsets per shared-memory load
+                if (fast) {
 #pragma unroll
-              for (int e = 0; e < 32; e += 4)
-                *reinterpret_cast<float4 *>(o32 + e) = *reinterpret_cast<const float4 *>(bk->off + c + e);
-              if (fast) {
+                  for (int e = 0; e < 32; e += 4) {
+                    const ulonglong2 o = *reinterpret_cast<const ulonglong2 *>(bk->noff + h0 + c + e);
+                    float x0, x1, x2, x3;
+                    f2_unpack(f2_fma(f2_pack(__uint_as_float(r[e]), __uint_as_float(r[e + 1])), scale2, o.x), x0, x1);
+                    f2_unpack(f2_fma(f2_pack(__uint_as_float(r[e + 2]), __uint_as_float(r[e + 3])), scale2, o.y), x2, x3);
+                    sm2[(e >> 1) & 3] = f2_add(sm2[(e >> 1) & 3], f2_pack(fast_exp2(x0), fast_exp2(x1)));
+                    sm2[((e >> 1) + 1) & 3] = f2_add(sm2[((e >> 1) + 1) & 3], f2_pack(fast_exp2(x2), fast_exp2(x3)));
+                  }
+                } else {
 #pragma unroll
-                for (int e = 0; e < 32; ++e) sm[e & 7] += fast_exp2(fmaf(__uint_as_float(r[e]), scale, -o32[e]));
-              } else {
+                  for (int e = 0; e < 32; e += 2) {
+                    const float2 o = *reinterpret_cast<const float2 *>(bk->noff + h0 + c + e);
+                    float x[2];
 #pragma unroll
-                for (int e = 0; e < 32; ++e) {
-                  const int p = T.R0 + c + e;
-                  const float o = o32[e];
-                  const float above = (p >= d.v0 && p < v_end) ? soft_j : -INFINITY;
-                  const float add = (j <= p) ? 0.f : above;
-                  sm[e & 7] += fast_exp2(fmaf(__uint_as_float(r[e]), scale, add) - o);
+                    for (int k = 0; k < 2; ++k) {
+                      const int p = T.R0 + h0 + c + e + k;
+                      const float above = (p >= d.v0 && p < v_end) ? soft_j : -INFINITY;
+                      x[k] = fast_exp2(fmaf(__uint_as_float(r[e + k]), scale, (j <= p) ? 0.f : above) + (k ? o.y : o.x));
+                    }
+                    sm2[(e >> 1) & 3] = f2_add(sm2[(e >> 1) & 3], f2_pack(x[0], x[1]));
+                  }
                 }
               }
+              if (with_mass && rp == 0 && T.n2 - h0 >= 0 && T.n2 - h0 < 128) {
+                // columns n2 .. n2 + 2: the three pieces of the summed query against this key
+                uint32_t r[16];
+                tmem_ld16(tlane + (T.n2 - h0), r);
+                tmem_wait_ld();
+                if (key_ok)
+                  a.mass_heads[((size_t)b * a.H + h) * a.max_vis + (j - d.v0)] =
+                      (__uint_as_float(r[0]) + __uint_as_float(r[1])) + __uint_as_float(r[2]);
+              }
             }
-            if (key_ok) {
-              const float sum = ((sm[0] + sm[1]) + (sm[2] + sm[3])) + ((sm[4] + sm[5]) + (sm[6] + sm[7]));
-              // the first row pair initialises the slots it covers; later row pairs add
-              if (rp == 0) part[j - d.v0] = sum;
-              else part[j - d.v0] += sum;
-            }
-            if (with_mass && rp == 0) {
-              // columns n2 .. n2 + 2: the three pieces of the summed query against this key
-              uint32_t r[16];
-              tmem_ld16(tlane + T.n2, r);
-              tmem_wait_ld();
-              if (key_ok)
-                a.mass_heads[((size_t)b * a.H + h) * a.max_vis + (j - d.v0)] =
-                    (__uint_as_float(r[0]) + __uint_as_float(r[1])) + __uint_as_float(r[2]);
-            }
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(smem_u32(&bk->acc_empty[buf]));
           }
-          tc_fence_before();
-          __syncwarp();
-          if (lane == 0) mbar_arrive(smem_u32(&bk->acc_empty[hh]));
+          if (key_ok && !bk->abort_flag) {
+            float s0, s1;
+            f2_unpack(f2_add(f2_add(sm2[0], sm2[1]), f2_add(sm2[2], sm2[3])), s0, s1);
+            // the first row pair initialises the slots it covers; later row pairs add (the barriers between their passes
+            // make the earlier pair's sums visible, whichever group wrote them)
+            if (rp == 0) part[j - d.v0] = s0 + s1;
+            else part[j - d.v0] += s0 + s1;
+          }
         }
-        epi_bar_sync();   // off[] is rewritten by the next row pair; its sums are visible to the next pair's adds
       }
     }
     __threadfence();
