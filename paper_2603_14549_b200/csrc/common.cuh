@@ -129,6 +129,17 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
       : "memory");
   return ok != 0;
 }
+__device__ __forceinline__ bool mbar_test_wait(uint32_t bar, uint32_t parity) {
+  uint32_t ok;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(ok)
+      : "r"(bar), "r"(parity)
+      : "memory");
+  return ok != 0;
+}
 __device__ __forceinline__ void fence_barrier_init() {
   asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
 }
@@ -148,18 +159,19 @@ struct WaitCtx {
 };
 
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, const WaitCtx &w) {
-  if (mbar_try_wait(bar, parity)) return true;
+  if (mbar_test_wait(bar, parity)) return true;
   const long long t0 = clock64();
   while (true) {
     // (a try_wait that fails has itself waited for a while inside the hardware, so looking at the
-    // flag and the clock after every one costs nothing that matters)
-    if (mbar_try_wait(bar, parity)) return true;
+    // flag and the clock before every one costs nothing that matters; and a limit of a clock or two
+    // gives up at every wait that is not satisfied at once, however short)
     if (*w.abort_flag) return false;
     if (clock64() - t0 > w.limit) {
       *w.abort_flag = 1;
       atomicOr(w.status, w.status_bit);
       return false;
     }
+    if (mbar_try_wait(bar, parity)) return true;
   }
 }
 
@@ -233,61 +245,16 @@ __device__ __forceinline__ void tc_fence_before() {
 __device__ __forceinline__ void tc_fence_after() {
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 }
-// The mbarrier gets one arrival once every MMA issued so far by this thread has finished.
-__device__ __forceinline__ void tc_commit(uint32_t bar) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar)
-               : "memory");
-}
-// D[tmem] (+)= A[smem] * B[smem]^T, bf16 operands, fp32 accumulator; one thread issues.
-__device__ __forceinline__ void tc_mma_bf16(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc,
-                                            uint32_t idesc, uint32_t accumulate) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
-      ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
-      : "memory");
-}
-// Eight MMAs over a K extent of 128 bf16 held as two 64-column blocks (each 128-byte-swizzled): k-steps 0-3
-// advance both start addresses by 32 bytes inside the first block, k-steps 4-7 do the same in the second
-// block, `a_half` / `b_half` bytes further on.  The first MMA overwrites the accumulator, the others add.
-// One statement with the descriptors stepped by immediate adds: the issuing thread's instruction stream per
-// MMA is two adds and the MMA instead of rebuilding both 64-bit descriptors (the single issuing thread is the
-// slowest stage of the score kernel for row pairs of one tile: measured 3 % on the whole kernel).
-template <int A_HALF_BYTES, int B_HALF_BYTES>
-__device__ __forceinline__ void tc_mma_bf16_k128(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc) {
-  asm volatile(
-      "{\n\t.reg .pred p0, p1;\n\t.reg .b64 a, b;\n\t"
-      "setp.ne.b32 p0, 0, 0;\n\tsetp.ne.b32 p1, 1, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p0;\n\t"
-      "add.u64 a, %1, 2;\n\tadd.u64 b, %2, 2;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %3, p1;\n\t"
-      "add.u64 a, %1, 4;\n\tadd.u64 b, %2, 4;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %3, p1;\n\t"
-      "add.u64 a, %1, 6;\n\tadd.u64 b, %2, 6;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %3, p1;\n\t"
-      "add.u64 a, %1, %4;\n\tadd.u64 b, %2, %5;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %3, p1;\n\t"
-      "add.u64 a, %1, %6;\n\tadd.u64 b, %2, %7;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %3, p1;\n\t"
-      "add.u64 a, %1, %8;\n\tadd.u64 b, %2, %9;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %3, p1;\n\t"
-      "add.u64 a, %1, %10;\n\tadd.u64 b, %2, %11;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %3, p1;\n\t}"
-      ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc),
-        "n"(A_HALF_BYTES / 16), "n"(B_HALF_BYTES / 16), "n"(A_HALF_BYTES / 16 + 2), "n"(B_HALF_BYTES / 16 + 2),
-        "n"(A_HALF_BYTES / 16 + 4), "n"(B_HALF_BYTES / 16 + 4), "n"(A_HALF_BYTES / 16 + 6), "n"(B_HALF_BYTES / 16 + 6)
-      : "memory");
-}
-// The issuing warp's form of these: the WHOLE warp executes the statement, `leader` (see warp_leader) is non-zero in the
-// one lane that issues.  A warp that stays converged keeps the descriptors in uniform registers and spends one or two
-// instructions per MMA; code under `if (lane == 0)` spends a dozen, each of which waits its turn among the other warps of the
-// scheduler (measured, M = 128, N = 128, two warps of FMAs beside the issuer: 76 clocks per MMA against 565; the pipe takes 64).
+// MMAs and their commits are statements of the WHOLE issuing warp; `leader` is non-zero in the one lane that issues.  A warp
+// that stays converged keeps the descriptors in uniform registers and spends one or two instructions per MMA; code under
+// `if (lane == 0)` spends a dozen, each of which waits its turn among the other warps of the scheduler (measured, M = 128,
+// N = 128, two warps of FMAs beside the issuer: 76 clocks per MMA against 565; the pipe takes 64).
 __device__ __forceinline__ uint32_t warp_leader() {
   uint32_t p;
   asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(p));
   return p;
 }
+// D[tmem] (+)= A[smem] * B[smem]^T, bf16 operands, fp32 accumulator.
 __device__ __forceinline__ void tc_mma_bf16_w(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,
                                               uint32_t accumulate, uint32_t leader) {
   asm volatile(
@@ -308,6 +275,7 @@ __device__ __forceinline__ void tc_mma_bf16_ta_w(uint32_t d_tmem, uint32_t a_tme
       ::"r"(d_tmem), "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accumulate), "r"(leader)
       : "memory");
 }
+// The mbarrier gets one arrival once every MMA issued so far by the leader has finished.
 __device__ __forceinline__ void tc_commit_w(uint32_t bar, uint32_t leader) {
   asm volatile(
       "{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %1, 0;\n\t"

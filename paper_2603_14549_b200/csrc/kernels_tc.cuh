@@ -771,7 +771,7 @@ sim_kernel(const __grid_constant__ CUtensorMap tmap_h, const __grid_constant__ C
   if (mt * 128 >= max(n_rows, 1)) return;
   // (in the cluster form the blocks of a cluster must leave together: decided below, by the cluster's first block)
   if (!a.cluster && (*reinterpret_cast<volatile uint32_t *>(a.status) & STATUS_SIM_TIMEOUT)) return;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
 
   const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
   uint8_t *base_ptr = smem_raw + (base - smem_u32(smem_raw));
@@ -820,15 +820,15 @@ sim_kernel(const __grid_constant__ CUtensorMap tmap_h, const __grid_constant__ C
   const uint32_t tmem_base = bk->tmem_base;
   WaitCtx wc{&bk->abort_flag, a.status, STATUS_SIM_TIMEOUT, a.wait_limit};
   // cluster form, in the tile ring once it is free: this slice's partial products [keep_k][128]; per quarter
-  // of this block's share of the slots the rows' best (value [4][128], slot [4][128]); and, filled by all
-  // blocks in the cluster's first block, every slice's partial squared norms and every block's best
-  // (value, slot) ([splits][128] each)
+  // of this block's share of the slots the rows' best (value [4][128], slot [4][128]); this slice's partial squared
+  // norms [128]; and, filled by all blocks in the cluster's first block, every block's best (value, slot)
+  // ([splits][128] each)
   const int cl_per = (a.keep_k + a.splits - 1) / a.splits;
   float *cl_p = reinterpret_cast<float *>(base_ptr);
   float *cl_wv = cl_p + (size_t)a.keep_k * 128;
   int *cl_ws = reinterpret_cast<int *>(cl_wv + 4 * 128);
   float *cl_ss = reinterpret_cast<float *>(cl_ws + 4 * 128);
-  float *cl_bv = cl_ss + a.splits * 128;
+  float *cl_bv = cl_ss + 128;
   int *cl_bs = reinterpret_cast<int *>(cl_bv + a.splits * 128);
   // steps of this slice: 128 columns each, or 64 in the one-pass layout
   const int n_kb = a.wide ? (a.D / 64) / a.splits : (a.D / 128) / a.splits;
@@ -928,54 +928,59 @@ sim_kernel(const __grid_constant__ CUtensorMap tmap_h, const __grid_constant__ C
       cp_async_wait<0>();                                 // nothing of this thread's is in flight when the block leaves
     }
   } else if (warp == 1) {
-    if (lane == 0) {
-      const uint32_t idesc = umma_idesc_bf16(128, a.n_tile);
-      int it = 0;
+    // ---- MMA issuer: the whole warp walks the loop and stays converged (see warp_leader).  After an abort its waits return
+    // at once and it goes on multiplying whatever lies in the block's own memory: nothing of it is used.
+    // With gathered rows one lane issues alone: there the shared-memory writes of the gather warps pace the kernel, and the
+    // converged warp, which issues a stage's MMAs in one burst, was slower (1152 of 2304 slots, 32 sequences: 880 -> 1000 us).
+    const uint32_t leader = GATHER ? (lane == 0 ? 1u : 0u) : warp_leader();
+    const uint32_t tm = __shfl_sync(0xffffffffu, tmem_base, 0);
+    const uint32_t idesc = umma_idesc_bf16(128, a.n_tile);
+    const uint64_t desc0 = umma_desc_sw128(base);
+    auto wait = [&](uint32_t bar, uint32_t parity) {
+      mbar_wait(bar, parity, wc);
+      if (!GATHER) __syncwarp();
+    };
+    int it = 0;
+    if (!GATHER || lane == 0) {
       if (a.wide) {
         for (int kb = 0; kb < n_kb; ++kb) {
           const int s = kb % a.stages;
-          mbar_wait(smem_u32(&bk->full[s]), (kb / a.stages) & 1, wc);
-          fence_proxy_async();       // the gathered rows were written by ordinary asynchronous copies
+          wait(smem_u32(&bk->full[s]), (kb / a.stages) & 1);
+          if (gather) fence_proxy_async();       // the gathered rows were written by ordinary asynchronous copies
           tc_fence_after();
-          if (!bk->abort_flag) {
-            const uint32_t sa = base + s * stage_bytes, sb = sa + SIM_A_BYTES;
-            for (int t = 0; t < a.n_nt; ++t)
-#pragma unroll
-              for (int kk = 0; kk < 4; ++kk)
-                tc_mma_bf16(tmem_base + t * a.n_tile, umma_desc_sw128(sa + kk * 32),
-                            umma_desc_sw128(sb + t * b_bytes + kk * 32), idesc, (kb > 0 || kk > 0) ? 1u : 0u);
-            tc_commit(smem_u32(&bk->empty[s]));
-            if (a.smat) mbar_arrive_n(smem_u32(&bk->empty[s]), 4);
-          }
+          const uint64_t da = desc0 + (uint32_t)(s * stage_bytes) / 16, db = da + SIM_A_BYTES / 16;
+          for (int t = 0; t < a.n_nt; ++t)
+  #pragma unroll
+            for (int kk = 0; kk < 4; ++kk)
+              tc_mma_bf16_w(tm + t * a.n_tile, da + kk * 2, db + t * (b_bytes / 16) + kk * 2, idesc, (kb > 0 || kk > 0) ? 1u : 0u, leader);
+          tc_commit_w(smem_u32(&bk->empty[s]), leader);
+          if (a.smat && leader) mbar_arrive_n(smem_u32(&bk->empty[s]), 4);
         }
-        if (!bk->abort_flag) tc_commit(smem_u32(&bk->acc_full[0]));
+        tc_commit_w(smem_u32(&bk->acc_full[0]), leader);
       }
       for (int nt = 0; nt < (a.wide ? 0 : a.n_nt); ++nt) {
         const int buf = nt & 1;
-        if (nt >= 2) mbar_wait(smem_u32(&bk->acc_empty[buf]), ((nt >> 1) - 1) & 1, wc);
-        const uint32_t dcol = tmem_base + buf * (a.tmem_cols >> 1);
+        if (nt >= 2) wait(smem_u32(&bk->acc_empty[buf]), ((nt >> 1) - 1) & 1);
+        const uint32_t dcol = tm + buf * (a.tmem_cols >> 1);
         for (int kb = 0; kb < n_kb; ++kb, ++it) {
           const int s = it % a.stages;
-          mbar_wait(smem_u32(&bk->full[s]), (it / a.stages) & 1, wc);
-          fence_proxy_async();
+          wait(smem_u32(&bk->full[s]), (it / a.stages) & 1);
+          if (gather) fence_proxy_async();
           tc_fence_after();
-          if (!bk->abort_flag) {
-            const uint32_t sa = base + s * stage_bytes, sb = sa + 2 * SIM_A_BYTES;
-#pragma unroll
-            for (int kk = 0; kk < 8; ++kk)
-              tc_mma_bf16(dcol, umma_desc_sw128(sa + (kk >> 2) * SIM_A_BYTES + (kk & 3) * 32),
-                          umma_desc_sw128(sb + (kk >> 2) * b_bytes + (kk & 3) * 32), idesc,
-                          (kb > 0 || kk > 0) ? 1u : 0u);
-            tc_commit(smem_u32(&bk->empty[s]));
-            // after the first accumulator the epilogue warps no longer read the stages
-            if (nt > 0 || a.smat) mbar_arrive_n(smem_u32(&bk->empty[s]), 4);
-          }
+          const uint64_t da = desc0 + (uint32_t)(s * stage_bytes) / 16, db = da + 2 * SIM_A_BYTES / 16;
+  #pragma unroll
+          for (int kk = 0; kk < 8; ++kk)
+            tc_mma_bf16_w(dcol, da + (kk >> 2) * (SIM_A_BYTES / 16) + (kk & 3) * 2, db + (kk >> 2) * (b_bytes / 16) + (kk & 3) * 2, idesc,
+                          (kb > 0 || kk > 0) ? 1u : 0u, leader);
+          tc_commit_w(smem_u32(&bk->empty[s]), leader);
+          // after the first accumulator the epilogue warps no longer read the stages
+          if ((nt > 0 || a.smat) && leader) mbar_arrive_n(smem_u32(&bk->empty[s]), 4);
         }
-        if (!bk->abort_flag) tc_commit(smem_u32(&bk->acc_full[buf]));
+        tc_commit_w(smem_u32(&bk->acc_full[buf]), leader);
       }
-      // every MMA this thread issued has completed before tensor memory is given back: after an abort the
+      // every MMA this warp issued has completed before tensor memory is given back: after an abort the
       // epilogue warps no longer wait for the accumulators, so nothing else would hold the block until then
-      tc_commit(smem_u32(&bk->mma_done));
+      tc_commit_w(smem_u32(&bk->mma_done), leader);
       mbar_wait_drain(smem_u32(&bk->mma_done), 0, TC_WAIT_LIMIT);
     }
     __syncwarp();
@@ -1095,8 +1100,13 @@ sim_kernel(const __grid_constant__ CUtensorMap tmap_h, const __grid_constant__ C
       // warps' bests per row are merged (larger value, lower slot among equals), handed to the cluster's
       // first block, and that block takes the maximum over the blocks in ascending slots.
       const int rank = (int)cluster_cta_rank(), S = a.splits;
-      st_cluster_f32(cluster_map(smem_u32(cl_ss), 0) + (uint32_t)(rank * 128 + lrow) * 4u, ss);
+      // (every block keeps its own norms until the barrier: the first block's ring may still be multiplied from)
+      cl_ss[lrow] = ss;
       cluster_sync_all();
+      if (rank == 0) {
+        ss_tot = 0.f;
+        for (int r2 = 0; r2 < S; ++r2) ss_tot += ld_cluster_f32(cluster_map(smem_u32(cl_ss), (uint32_t)r2) + (uint32_t)lrow * 4u);
+      }
       const int s_lo = min(a.keep_k, rank * cl_per), n_mine = min(a.keep_k, s_lo + cl_per) - s_lo;
       uint32_t pz[8];
 #pragma unroll
@@ -1143,8 +1153,6 @@ sim_kernel(const __grid_constant__ CUtensorMap tmap_h, const __grid_constant__ C
       cluster_sync_all();
       finalize = rank == 0;
       if (finalize) {
-        ss_tot = 0.f;
-        for (int r2 = 0; r2 < S; ++r2) ss_tot += cl_ss[r2 * 128 + lrow];
         best = -INFINITY;
         best_slot = 0;
         for (int r2 = 0; r2 < S; ++r2) {                    // ascending slots: the first maximum stays
@@ -1328,7 +1336,7 @@ sim_pair_kernel(const __grid_constant__ CUtensorMap tmap_h, const __grid_constan
   if (pr * 256 >= n_rows) return;
   if (*reinterpret_cast<volatile uint32_t *>(a.status) & STATUS_SIM_TIMEOUT) return;
   const bool two = pr * 256 + 128 < n_rows;              // the pair's second row tile holds visual rows
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
 
   const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
   uint8_t *base_ptr = smem_raw + (base - smem_u32(smem_raw));
@@ -1394,28 +1402,28 @@ sim_pair_kernel(const __grid_constant__ CUtensorMap tmap_h, const __grid_constan
       }
     }
   } else if (warp == 1) {
-    if (lane == 0) {
-      const uint32_t idesc = umma_idesc_bf16(128, a.n_tile);
-      const int n_t = two ? 2 : 1;
-      for (int it = 0; it < n_kb; ++it) {
-        const int s = it % a.stages;
-        mbar_wait(smem_u32(&bk->full[s]), (it / a.stages) & 1, wc);
-        tc_fence_after();
-        if (!bk->abort_flag) {
-          const uint32_t sa = base + s * stage_bytes, sb = sa + 2 * SIM_A_BYTES;
-          for (int t = 0; t < n_t; ++t)
+    // ---- MMA issuer (converged, as in sim_kernel)
+    const uint32_t leader = warp_leader();
+    const uint32_t tm = __shfl_sync(0xffffffffu, tmem_base, 0);
+    const uint32_t idesc = umma_idesc_bf16(128, a.n_tile);
+    const uint64_t desc0 = umma_desc_sw128(base);
+    const int n_t = two ? 2 : 1;
+    for (int it = 0; it < n_kb; ++it) {
+      const int s = it % a.stages;
+      mbar_wait_warp(smem_u32(&bk->full[s]), (it / a.stages) & 1, wc);
+      tc_fence_after();
+      const uint64_t da = desc0 + (uint32_t)(s * stage_bytes) / 16, db = da + 2 * SIM_A_BYTES / 16;
+      for (int t = 0; t < n_t; ++t)
 #pragma unroll
-            for (int kk = 0; kk < 4; ++kk)
-              tc_mma_bf16(tmem_base + t * a.n_tile, umma_desc_sw128(sa + t * SIM_A_BYTES + kk * 32),
-                          umma_desc_sw128(sb + kk * 32), idesc, (it > 0 || kk > 0) ? 1u : 0u);
-          tc_commit(smem_u32(&bk->empty[s]));
-        }
-      }
-      if (!bk->abort_flag) tc_commit(smem_u32(&bk->acc_full));
-      // every MMA this thread issued has completed before tensor memory is given back
-      tc_commit(smem_u32(&bk->mma_done));
-      mbar_wait_drain(smem_u32(&bk->mma_done), 0, TC_WAIT_LIMIT);
+        for (int kk = 0; kk < 4; ++kk)
+          tc_mma_bf16_w(tm + t * a.n_tile, da + t * (SIM_A_BYTES / 16) + kk * 2, db + kk * 2, idesc, (it > 0 || kk > 0) ? 1u : 0u, leader);
+      tc_commit_w(smem_u32(&bk->empty[s]), leader);
     }
+    tc_commit_w(smem_u32(&bk->acc_full), leader);
+    // every MMA this warp issued has completed before tensor memory is given back
+    tc_commit_w(smem_u32(&bk->mma_done), leader);
+    mbar_wait_drain(smem_u32(&bk->mma_done), 0, TC_WAIT_LIMIT);
+    __syncwarp();
   } else {
     const int grp = (warp - 2) >> 2;                     // row tile of the pair
     const int quarter = warp & 3;                        // the tensor-memory lanes a warp may read
