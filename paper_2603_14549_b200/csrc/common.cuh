@@ -191,6 +191,23 @@ __device__ __forceinline__ bool mbar_wait_drain(uint32_t bar, uint32_t parity, l
   return true;
 }
 
+// Non-zero in one lane of the (converged) calling warp.
+__device__ __forceinline__ uint32_t warp_leader() {
+  uint32_t p;
+  asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(p));
+  return p;
+}
+
+// A ring of buffers: slot and the parity of its barriers, stepped without divisions.
+struct RingPos {
+  int slot;
+  uint32_t phase;
+  __device__ __forceinline__ RingPos() : slot(0), phase(0u) {}
+  __device__ __forceinline__ void step(int n) {
+    if (++slot == n) { slot = 0; phase ^= 1u; }
+  }
+};
+
 // ---------------------------------------------------------------------------------------
 // TMA (tiled 2-D load, completion on an mbarrier)
 // ---------------------------------------------------------------------------------------
@@ -200,6 +217,23 @@ __device__ __forceinline__ void tma_load_2d(uint32_t smem_dst, const void *tmap,
       "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes "
       "[%0], [%1, {%3, %4}], [%2];"
       ::"r"(smem_dst), "l"(tmap), "r"(bar), "r"(x), "r"(y)
+      : "memory");
+}
+// The copying warp's form: the whole warp executes the statement and stays converged, `leader` (see warp_leader) issues.
+// One lane under a branch needs about 770 clocks per ring slot (wait, expectation, copy) whatever the copy's size; the
+// converged warp 360 (measured, 128 x 64 boxes out of L2 on all SMs, three per slot: 57 against 92 bytes per clock and SM).
+__device__ __forceinline__ void tma_load_2d_w(uint32_t smem_dst, const void *tmap, uint32_t bar, int32_t x, int32_t y, uint32_t leader) {
+  asm volatile(
+      "{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %5, 0;\n\t"
+      "@q cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes "
+      "[%0], [%1, {%3, %4}], [%2];\n\t}"
+      ::"r"(smem_dst), "l"(tmap), "r"(bar), "r"(x), "r"(y), "r"(leader)
+      : "memory");
+}
+__device__ __forceinline__ void mbar_expect_tx_w(uint32_t bar, uint32_t bytes, uint32_t leader) {
+  asm volatile(
+      "{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %2, 0;\n\t"
+      "@q mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n\t}" ::"r"(bar), "r"(bytes), "r"(leader)
       : "memory");
 }
 // Asynchronous 16-byte copies global -> shared issued by ordinary threads (used where the rows of a
@@ -249,11 +283,6 @@ __device__ __forceinline__ void tc_fence_after() {
 // that stays converged keeps the descriptors in uniform registers and spends one or two instructions per MMA; code under
 // `if (lane == 0)` spends a dozen, each of which waits its turn among the other warps of the scheduler (measured, M = 128,
 // N = 128, two warps of FMAs beside the issuer: 76 clocks per MMA against 565; the pipe takes 64).
-__device__ __forceinline__ uint32_t warp_leader() {
-  uint32_t p;
-  asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(p));
-  return p;
-}
 // D[tmem] (+)= A[smem] * B[smem]^T, bf16 operands, fp32 accumulator.
 __device__ __forceinline__ void tc_mma_bf16_w(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,
                                               uint32_t accumulate, uint32_t leader) {

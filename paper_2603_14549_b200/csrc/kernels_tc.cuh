@@ -185,62 +185,70 @@ score_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__
 
   if (warp == 0) {
     // ------------------------------------------------------------------ producer: items, queries, key tiles
-    if (lane == 0) {
+    // (converged, see tma_load_2d_w)
+    const uint32_t leader = warp_leader();
+    if (leader) {
       tma_prefetch_desc(&tmap_q);
       tma_prefetch_desc(&tmap_k);
-      int kc = 0, qc = 0, ic = 0;               // key tiles / row pairs / items so far
-      int k_issued = 0, q_issued = 0;           // copies actually issued (an abort is sticky, so
-                                                // these are prefixes of the two sequences)
-      while (true) {
-        const int slot = ic % SC_ITEM_SLOTS;
-        // The item queue keeps working after an abort (its waits ignore the flag and are bounded on their
-        // own): every consumer must see the same sequence of items, ending with -1, or the epilogue warps'
-        // named barriers would no longer match.  After an abort that sequence ends at once.
-        if (ic >= SC_ITEM_SLOTS &&
-            !mbar_wait_drain(smem_u32(&bk->item_empty[slot]), ((ic / SC_ITEM_SLOTS) - 1) & 1, TC_WAIT_LIMIT))
-          break;
-        int item = bk->abort_flag ? n_items : (int)atomicAdd(a.work, 1u);
+    }
+    int kc = 0, qc = 0, ic = 0;               // key tiles / row pairs / items so far
+    int k_issued = 0, q_issued = 0;           // copies actually issued (an abort is sticky, so
+                                              // these are prefixes of the two sequences)
+    while (true) {
+      const int slot = ic % SC_ITEM_SLOTS;
+      // The item queue keeps working after an abort (its waits ignore the flag and are bounded on their
+      // own): every consumer must see the same sequence of items, ending with -1, or the epilogue warps'
+      // named barriers would no longer match.  After an abort that sequence ends at once.
+      bool room = true;
+      if (ic >= SC_ITEM_SLOTS) room = mbar_wait_drain(smem_u32(&bk->item_empty[slot]), ((ic / SC_ITEM_SLOTS) - 1) & 1, TC_WAIT_LIMIT);
+      __syncwarp();
+      if (!__shfl_sync(0xffffffffu, room ? 1 : 0, 0)) break;
+      int item = 0;
+      if (lane == 0) {
+        item = bk->abort_flag ? n_items : (int)atomicAdd(a.work, 1u);
         if (item >= n_items) item = -1;
         bk->item_q[slot] = item;
         mbar_arrive(smem_u32(&bk->item_full[slot]));      // release: the slot's content is visible to the waiters
-        ++ic;
-        if (item < 0) break;
-        const int b = item / a.H, h = item - b * a.H;
-        const SampleDesc d = make_desc(a.pa, b);
-        if (!d.valid) continue;
-        const int n_rp = (d.nr + pair_rows - 1) / pair_rows;
-        for (int rp = 0; rp < n_rp; ++rp, ++qc) {
-          const RowPair T = score_row_pair(d, rp, a.mask_enable, pair_rows);
-          if (qc >= 1) mbar_wait(smem_u32(&bk->q_empty), (qc - 1) & 1, wc);
-          if (!bk->abort_flag) {
-            mbar_expect_tx(smem_u32(&bk->q_full), T.nrt * SC_TILE_BYTES);
-            for (int hf = 0; hf < 2; ++hf)
-              for (int rt = 0; rt < T.nrt; ++rt)
-                tma_load_2d(q_smem + hf * SC_Q_HALF_BYTES + rt * SC_HALF_BYTES, &tmap_q, smem_u32(&bk->q_full),
-                            h * 128 + hf * 64, d.row0 + T.R0 + rt * 128);
-            q_issued = qc + 1;
-          }
-          for (int u = 0; u < T.n_kt + T.n_p2; ++u, ++kc) {
-            const int t = u < T.n_kt ? u : T.t_hi - (u - T.n_kt);
-            const int s = kc % SC_STAGES;
-            if (kc >= SC_STAGES) mbar_wait(smem_u32(&bk->empty[s]), ((kc / SC_STAGES) - 1) & 1, wc);
-            if (!bk->abort_flag) {
-              const uint32_t dst = k_smem + s * SC_TILE_BYTES;
-              mbar_expect_tx(smem_u32(&bk->full[s]), SC_TILE_BYTES);
-              tma_load_2d(dst, &tmap_k, smem_u32(&bk->full[s]), h * 128, d.row0 + t * 128);
-              tma_load_2d(dst + SC_HALF_BYTES, &tmap_k, smem_u32(&bk->full[s]), h * 128 + 64, d.row0 + t * 128);
-              k_issued = kc + 1;
-            }
+      }
+      item = __shfl_sync(0xffffffffu, item, 0);
+      ++ic;
+      if (item < 0) break;
+      const int b = item / a.H, h = item - b * a.H;
+      const SampleDesc d = make_desc(a.pa, b);
+      if (!d.valid) continue;
+      const int n_rp = (d.nr + pair_rows - 1) / pair_rows;
+      for (int rp = 0; rp < n_rp; ++rp, ++qc) {
+        const RowPair T = score_row_pair(d, rp, a.mask_enable, pair_rows);
+        if (qc >= 1) mbar_wait_warp(smem_u32(&bk->q_empty), (qc - 1) & 1, wc);
+        if (!__shfl_sync(0xffffffffu, bk->abort_flag, 0)) {
+          mbar_expect_tx_w(smem_u32(&bk->q_full), T.nrt * SC_TILE_BYTES, leader);
+          for (int hf = 0; hf < 2; ++hf)
+            for (int rt = 0; rt < T.nrt; ++rt)
+              tma_load_2d_w(q_smem + hf * SC_Q_HALF_BYTES + rt * SC_HALF_BYTES, &tmap_q, smem_u32(&bk->q_full),
+                            h * 128 + hf * 64, d.row0 + T.R0 + rt * 128, leader);
+          q_issued = qc + 1;
+        }
+        for (int u = 0; u < T.n_kt + T.n_p2; ++u, ++kc) {
+          const int t = u < T.n_kt ? u : T.t_hi - (u - T.n_kt);
+          const int s = kc % SC_STAGES;
+          if (kc >= SC_STAGES) mbar_wait_warp(smem_u32(&bk->empty[s]), ((kc / SC_STAGES) - 1) & 1, wc);
+          if (!__shfl_sync(0xffffffffu, bk->abort_flag, 0)) {
+            const uint32_t dst = k_smem + s * SC_TILE_BYTES;
+            mbar_expect_tx_w(smem_u32(&bk->full[s]), SC_TILE_BYTES, leader);
+            tma_load_2d_w(dst, &tmap_k, smem_u32(&bk->full[s]), h * 128, d.row0 + t * 128, leader);
+            tma_load_2d_w(dst + SC_HALF_BYTES, &tmap_k, smem_u32(&bk->full[s]), h * 128 + 64, d.row0 + t * 128, leader);
+            k_issued = kc + 1;
           }
         }
       }
-      // every copy this thread issued must have landed before the block may leave
-      for (int s = 0; s < SC_STAGES; ++s) {
-        const int fills = k_issued > s ? (k_issued - s + SC_STAGES - 1) / SC_STAGES : 0;
-        if (fills > 0) mbar_wait_drain(smem_u32(&bk->full[s]), (fills - 1) & 1, TC_WAIT_LIMIT);
-      }
-      if (q_issued > 0) mbar_wait_drain(smem_u32(&bk->q_full), (q_issued - 1) & 1, TC_WAIT_LIMIT);
     }
+    // every copy this warp issued must have landed before the block may leave
+    for (int s = 0; s < SC_STAGES; ++s) {
+      const int fills = k_issued > s ? (k_issued - s + SC_STAGES - 1) / SC_STAGES : 0;
+      if (fills > 0) mbar_wait_drain(smem_u32(&bk->full[s]), (fills - 1) & 1, TC_WAIT_LIMIT);
+    }
+    if (q_issued > 0) mbar_wait_drain(smem_u32(&bk->q_full), (q_issued - 1) & 1, TC_WAIT_LIMIT);
+    __syncwarp();
   } else if (warp == 1) {
     // ------------------------------------------------------------------ MMA issuer
     // (the whole warp walks the loop and stays converged, see warp_leader: 64 sequences of 2880 visual tokens 1043 -> 1000 us,
@@ -836,47 +844,51 @@ sim_kernel(const __grid_constant__ CUtensorMap tmap_h, const __grid_constant__ C
   const int total_it = a.wide ? n_kb : a.n_nt * n_kb;
 
   if (warp == 0) {
-    // ---- copy warp: the kept-row tiles (and, in matrix mode, the row operand) by tiled copies
-    if (lane == 0) {
+    // ---- copy warp: the kept-row tiles (and, in matrix mode, the row operand) by tiled copies (converged, see tma_load_2d_w)
+    const uint32_t leader = warp_leader();
+    if (leader) {
       tma_prefetch_desc(&tmap_h);
       tma_prefetch_desc(&tmap_kept);
-      const int row_b = b * a.keep_k;
-      // tiled row operand: rows of the dense kept array (matrix mode) or of the image span
-      const int row_a = a.smat ? row_b + mt * 128 : d.row0 + d.v0 + mt * 128;
-      const int tx_bytes = gather ? stage_bytes - (a.wide ? 1 : 2) * SIM_A_BYTES : stage_bytes;
-      const int rot = (mt * 5 + b * 3) % n_kb;
-      int issued = 0;
-      for (int it = 0; it < total_it; ++it) {
-        // every block walks its k-blocks from a different starting point, so that at any moment
-        // the blocks read different 128-byte columns of the rows and spread over the memory channels
-        const int s = it % a.stages, nt = it / n_kb, kb = kb0 + (it - nt * n_kb + rot) % n_kb;
-        const uint32_t full = smem_u32(&bk->full[s]);
-        if (it >= a.stages) mbar_wait(smem_u32(&bk->empty[s]), ((it / a.stages) - 1) & 1, wc);
-        if (bk->abort_flag) break;
-        const uint32_t dst = base + s * stage_bytes;
-        mbar_expect_tx(full, tx_bytes);
-        if (a.wide) {
-          if (!gather) tma_load_2d(dst, &tmap_h, full, kb * 64, row_a);
-          for (int t = 0; t < a.n_nt; ++t)
-            tma_load_2d(dst + SIM_A_BYTES + t * b_bytes, &tmap_kept, full, kb * 64, row_b + (tile0 + t) * a.n_tile);
-        } else {
-          if (!gather) {
-            tma_load_2d(dst, &tmap_h, full, kb * 128, row_a);
-            tma_load_2d(dst + SIM_A_BYTES, &tmap_h, full, kb * 128 + 64, row_a);
-          }
-          tma_load_2d(dst + 2 * SIM_A_BYTES, &tmap_kept, full, kb * 128, row_b + nt * a.n_tile);
-          tma_load_2d(dst + 2 * SIM_A_BYTES + b_bytes, &tmap_kept, full, kb * 128 + 64, row_b + nt * a.n_tile);
+    }
+    const int row_b = b * a.keep_k;
+    // tiled row operand: rows of the dense kept array (matrix mode) or of the image span
+    const int row_a = a.smat ? row_b + mt * 128 : d.row0 + d.v0 + mt * 128;
+    const int tx_bytes = gather ? stage_bytes - (a.wide ? 1 : 2) * SIM_A_BYTES : stage_bytes;
+    // every block walks its k-blocks from a different starting point, so that at any moment
+    // the blocks read different 128-byte columns of the rows and spread over the memory channels
+    const int rot = (mt * 5 + b * 3) % n_kb;
+    int issued = 0, nt = 0, kr = 0, kb = kb0 + rot;           // slot tile, step of its pass, column step
+    RingPos r;
+    for (int it = 0; it < total_it; ++it) {
+      const uint32_t full = smem_u32(&bk->full[r.slot]);
+      if (it >= a.stages) mbar_wait_warp(smem_u32(&bk->empty[r.slot]), r.phase ^ 1u, wc);
+      if (__shfl_sync(0xffffffffu, bk->abort_flag, 0)) break;
+      const uint32_t dst = base + r.slot * stage_bytes;
+      mbar_expect_tx_w(full, tx_bytes, leader);
+      if (a.wide) {
+        if (!gather) tma_load_2d_w(dst, &tmap_h, full, kb * 64, row_a, leader);
+        for (int t = 0; t < a.n_nt; ++t)
+          tma_load_2d_w(dst + SIM_A_BYTES + t * b_bytes, &tmap_kept, full, kb * 64, row_b + (tile0 + t) * a.n_tile, leader);
+      } else {
+        if (!gather) {
+          tma_load_2d_w(dst, &tmap_h, full, kb * 128, row_a, leader);
+          tma_load_2d_w(dst + SIM_A_BYTES, &tmap_h, full, kb * 128 + 64, row_a, leader);
         }
-        issued = it + 1;
+        tma_load_2d_w(dst + 2 * SIM_A_BYTES, &tmap_kept, full, kb * 128, row_b + nt * a.n_tile, leader);
+        tma_load_2d_w(dst + 2 * SIM_A_BYTES + b_bytes, &tmap_kept, full, kb * 128 + 64, row_b + nt * a.n_tile, leader);
       }
-      // drain: the last fill of every stage must have landed before the block leaves
-      for (int s = 0; s < a.stages; ++s) {
-        if (issued > s) {
-          const int last = ((issued - 1 - s) / a.stages) * a.stages + s;
-          // after an abort the gather warps may not have handed their part of the stage over, so the
-          // barrier may never complete: the tiled copies themselves land within microseconds
-          mbar_wait_drain(smem_u32(&bk->full[s]), (last / a.stages) & 1, bk->abort_flag ? 400000LL : TC_WAIT_LIMIT);
-        }
+      issued = it + 1;
+      r.step(a.stages);
+      if (++kb == kb0 + n_kb) kb = kb0;
+      if (++kr == n_kb) { kr = 0; ++nt; kb = kb0 + rot; }
+    }
+    // drain: the last fill of every stage must have landed before the block leaves
+    for (int s = 0; s < a.stages; ++s) {
+      if (issued > s) {
+        const int last = ((issued - 1 - s) / a.stages) * a.stages + s;
+        // after an abort the gather warps may not have handed their part of the stage over, so the
+        // barrier may never complete: the tiled copies themselves land within microseconds
+        mbar_wait_drain(smem_u32(&bk->full[s]), (last / a.stages) & 1, bk->abort_flag ? 400000LL : TC_WAIT_LIMIT);
       }
     }
     __syncwarp();
@@ -1374,33 +1386,38 @@ sim_pair_kernel(const __grid_constant__ CUtensorMap tmap_h, const __grid_constan
   const int rot = (pr * 5 + b * 3) % n_kb;
 
   if (warp == 0) {
-    if (lane == 0) {
+    // ---- copy warp (converged, see tma_load_2d_w)
+    const uint32_t leader = warp_leader();
+    if (leader) {
       tma_prefetch_desc(&tmap_h);
       tma_prefetch_desc(&tmap_kept);
-      const int row_a = a.smat ? b * a.keep_k + pr * 256 : d.row0 + d.v0 + pr * 256;
-      const int row_b = b * a.keep_k + gz * a.n_tile;
-      const int tx_bytes = two ? stage_bytes : stage_bytes - SIM_A_BYTES;
-      int issued = 0;
-      for (int it = 0; it < n_kb; ++it) {
-        const int s = it % a.stages, kb = (it + rot) % n_kb;
-        const uint32_t full = smem_u32(&bk->full[s]);
-        if (it >= a.stages) mbar_wait(smem_u32(&bk->empty[s]), ((it / a.stages) - 1) & 1, wc);
-        if (bk->abort_flag) break;
-        const uint32_t dst = base + s * stage_bytes;
-        mbar_expect_tx(full, tx_bytes);
-        tma_load_2d(dst, &tmap_h, full, kb * 64, row_a);
-        if (two) tma_load_2d(dst + SIM_A_BYTES, &tmap_h, full, kb * 64, row_a + 128);
-        tma_load_2d(dst + 2 * SIM_A_BYTES, &tmap_kept, full, kb * 64, row_b);
-        issued = it + 1;
-      }
-      // drain: the last fill of every stage must have landed before the block leaves
-      for (int s = 0; s < a.stages; ++s) {
-        if (issued > s) {
-          const int last = ((issued - 1 - s) / a.stages) * a.stages + s;
-          mbar_wait_drain(smem_u32(&bk->full[s]), (last / a.stages) & 1, TC_WAIT_LIMIT);
-        }
+    }
+    const int row_a = a.smat ? b * a.keep_k + pr * 256 : d.row0 + d.v0 + pr * 256;
+    const int row_b = b * a.keep_k + gz * a.n_tile;
+    const int tx_bytes = two ? stage_bytes : stage_bytes - SIM_A_BYTES;
+    int issued = 0, kb = rot;
+    RingPos r;
+    for (int it = 0; it < n_kb; ++it) {
+      const uint32_t full = smem_u32(&bk->full[r.slot]);
+      if (it >= a.stages) mbar_wait_warp(smem_u32(&bk->empty[r.slot]), r.phase ^ 1u, wc);
+      if (__shfl_sync(0xffffffffu, bk->abort_flag, 0)) break;
+      const uint32_t dst = base + r.slot * stage_bytes;
+      mbar_expect_tx_w(full, tx_bytes, leader);
+      tma_load_2d_w(dst, &tmap_h, full, kb * 64, row_a, leader);
+      if (two) tma_load_2d_w(dst + SIM_A_BYTES, &tmap_h, full, kb * 64, row_a + 128, leader);
+      tma_load_2d_w(dst + 2 * SIM_A_BYTES, &tmap_kept, full, kb * 64, row_b, leader);
+      issued = it + 1;
+      r.step(a.stages);
+      if (++kb == n_kb) kb = 0;
+    }
+    // drain: the last fill of every stage must have landed before the block leaves
+    for (int s = 0; s < a.stages; ++s) {
+      if (issued > s) {
+        const int last = ((issued - 1 - s) / a.stages) * a.stages + s;
+        mbar_wait_drain(smem_u32(&bk->full[s]), (last / a.stages) & 1, TC_WAIT_LIMIT);
       }
     }
+    __syncwarp();
   } else if (warp == 1) {
     // ---- MMA issuer (converged, as in sim_kernel)
     const uint32_t leader = warp_leader();
@@ -1408,9 +1425,10 @@ sim_pair_kernel(const __grid_constant__ CUtensorMap tmap_h, const __grid_constan
     const uint32_t idesc = umma_idesc_bf16(128, a.n_tile);
     const uint64_t desc0 = umma_desc_sw128(base);
     const int n_t = two ? 2 : 1;
-    for (int it = 0; it < n_kb; ++it) {
-      const int s = it % a.stages;
-      mbar_wait_warp(smem_u32(&bk->full[s]), (it / a.stages) & 1, wc);
+    RingPos r;
+    for (int it = 0; it < n_kb; ++it, r.step(a.stages)) {
+      const int s = r.slot;
+      mbar_wait_warp(smem_u32(&bk->full[s]), r.phase, wc);
       tc_fence_after();
       const uint64_t da = desc0 + (uint32_t)(s * stage_bytes) / 16, db = da + 2 * SIM_A_BYTES / 16;
       for (int t = 0; t < n_t; ++t)
@@ -1435,9 +1453,10 @@ sim_pair_kernel(const __grid_constant__ CUtensorMap tmap_h, const __grid_constan
     // ---- squared norm of this thread's row (group 0 only; the other groups just free the stages)
     float ssq[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
     const bool norms = gz == 0 && active && !a.smat;
-    for (int it = 0; it < (norms ? n_kb : 0); ++it) {
-      const int s = it % a.stages;
-      mbar_wait(smem_u32(&bk->full[s]), (it / a.stages) & 1, wc);
+    RingPos r;
+    for (int it = 0; it < (norms ? n_kb : 0); ++it, r.step(a.stages)) {
+      const int s = r.slot;
+      mbar_wait(smem_u32(&bk->full[s]), r.phase, wc);
       if (!bk->abort_flag) {
         const uint4 *row = reinterpret_cast<const uint4 *>(base_ptr + (size_t)s * stage_bytes +
                                                            grp * SIM_A_BYTES + lrow * 128);
