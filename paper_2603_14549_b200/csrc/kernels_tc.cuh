@@ -756,6 +756,39 @@ __device__ __forceinline__ void mbar_arrive_n(uint32_t bar, uint32_t n) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(n) : "memory");
 }
 
+// Running first-argmax of one tensor-memory lane over 32 accumulator columns, column e scaled by kinv[e] (shared memory,
+// 16-byte aligned).  The chunk's maximum first (packed products, three-way maxima), then, only where some row of the warp has
+// a new maximum, the lowest column that attains it: about three instructions per column instead of a chain of four and a
+// global load (176 columns: 6000 -> 1600 clocks, on the path of a block that nothing overlaps).
+__device__ __forceinline__ void sim_scan32(uint32_t taddr, const float *kinv, int slot0, float &best, int &best_slot) {
+  uint32_t r[32];
+  tmem_ld32(taddr, r);
+  tmem_wait_ld();
+  float v[32];
+#pragma unroll
+  for (int e = 0; e < 32; e += 4) {
+    const ulonglong2 k = *reinterpret_cast<const ulonglong2 *>(kinv + e);
+    f2_unpack(f2_mul(f2_pack(__uint_as_float(r[e]), __uint_as_float(r[e + 1])), k.x), v[e], v[e + 1]);
+    f2_unpack(f2_mul(f2_pack(__uint_as_float(r[e + 2]), __uint_as_float(r[e + 3])), k.y), v[e + 2], v[e + 3]);
+  }
+  float m[4];
+#pragma unroll
+  for (int e = 0; e < 4; ++e) m[e] = max3(v[e], v[e + 4], v[e + 8]);
+#pragma unroll
+  for (int c = 12; c < 28; c += 8)
+#pragma unroll
+    for (int e = 0; e < 4; ++e) m[e] = max3(m[e], v[c + e], v[c + 4 + e]);
+#pragma unroll
+  for (int e = 0; e < 4; ++e) m[e] = fmaxf(m[e], v[28 + e]);
+  const float mx = fmaxf(max3(m[0], m[1], m[2]), m[3]);
+  if (__any_sync(0xffffffffu, mx > best)) {
+    int at = 31;
+#pragma unroll
+    for (int e = 30; e >= 0; --e) at = v[e] == mx ? e : at;
+    if (mx > best) { best = mx; best_slot = slot0 + at; }
+  }
+}
+
 constexpr int SIM_THREADS_TILED = 192;                  // without gather warps: two such blocks fit an SM
 
 template <bool GATHER>
@@ -1042,10 +1075,28 @@ sim_kernel(const __grid_constant__ CUtensorMap tmap_h, const __grid_constant__ C
       part = a.part + tile * (size_t)a.keep_k * 128;
       a.ss_part[tile * 128 + lrow] = ss;
     }
+    // one pass over the rows and no partial sums: the inverse norms of the slots wait in registers and go to the tile ring
+    // once the last MMA has read it
+    const bool scan_smem = !part && !a.smat && (a.wide || a.n_nt == 1);
+    float *sk = reinterpret_cast<float *>(base_ptr);
+    float kreg[4] = {0.f, 0.f, 0.f, 0.f};
+    if (scan_smem) {
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        const int c = e * 128 + lrow, slot = tile0 * a.n_tile + c;
+        if (c < a.n_nt * a.n_tile && slot < a.keep_k) kreg[e] = __ldg(kinv + slot);
+      }
+    }
     for (int nt = 0; nt < a.n_nt; ++nt) {
       const int buf = a.wide ? 0 : (nt & 1);
       mbar_wait(smem_u32(&bk->acc_full[buf]), a.wide ? 0 : ((nt >> 1) & 1), wc);
       tc_fence_after();
+      if (scan_smem && nt == 0) {
+        asm volatile("bar.sync 1, 128;" ::: "memory");     // the other warps have read their rows for the norms
+#pragma unroll
+        for (int e = 0; e < 4; ++e) sk[e * 128 + lrow] = kreg[e];
+        asm volatile("bar.sync 1, 128;" ::: "memory");
+      }
       const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) +
                              (a.wide ? nt * a.n_tile : buf * (a.tmem_cols >> 1));
       const int slot0 = (tile0 + nt) * a.n_tile;
@@ -1055,6 +1106,10 @@ sim_kernel(const __grid_constant__ CUtensorMap tmap_h, const __grid_constant__ C
         // 32 columns per tensor-memory wait while they last (see sim_pair_kernel)
 #pragma unroll 1
         for (; c0 + 32 <= ncol; c0 += 32) {
+          if (scan_smem) {
+            sim_scan32(taddr + c0, sk + nt * a.n_tile + c0, slot0 + c0, best, best_slot);
+            continue;
+          }
           uint32_t r[32];
           tmem_ld32(taddr + c0, r);
           tmem_wait_ld();
@@ -1330,6 +1385,7 @@ struct SimPairBook {
   int abort_flag;
   int is_last;
   int scan[33];
+  alignas(16) float kinv[256];   // 1/||kept row|| of this block's slots
 };
 
 static_assert(sizeof(SimPairBook) <= SIM_BOOK_BYTES, "pair kernel bookkeeping exceeds its shared-memory slot");
@@ -1476,10 +1532,12 @@ sim_pair_kernel(const __grid_constant__ CUtensorMap tmap_h, const __grid_constan
 
     float best = -INFINITY;
     int best_slot = 0;
-    mbar_wait(smem_u32(&bk->acc_full), 0, wc);
-    tc_fence_after();
     const int slot0 = gz * a.n_tile;
     const int ncol = max(0, min(a.n_tile, a.keep_k - slot0));
+    bk->kinv[prow] = prow < ncol ? __ldg(kinv + slot0 + prow) : 0.f;
+    asm volatile("bar.sync 1, 256;" ::: "memory");
+    mbar_wait(smem_u32(&bk->acc_full), 0, wc);
+    tc_fence_after();
     if (active && !bk->abort_flag) {
       const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + grp * a.n_tile;
       const float inv_p = (a.smat && v < a.keep_k) ? __ldg(kinv + v) : 0.f;
@@ -1488,17 +1546,7 @@ sim_pair_kernel(const __grid_constant__ CUtensorMap tmap_h, const __grid_constan
         // 32 columns per tensor-memory wait while they last: half as many waits on the path every block goes
         // through after its last MMA, which nothing overlaps (c4 881 -> 833 us; 64 columns per wait: the same)
 #pragma unroll 1
-        for (; c0 + 32 <= ncol; c0 += 32) {
-          uint32_t r[32];
-          tmem_ld32(taddr + c0, r);
-          tmem_wait_ld();
-#pragma unroll
-          for (int e = 0; e < 32; ++e) {
-            const int slot = slot0 + c0 + e;
-            const float val = __uint_as_float(r[e]) * __ldg(kinv + slot);
-            if (val > best) { best = val; best_slot = slot; }
-          }
-        }
+        for (; c0 + 32 <= ncol; c0 += 32) sim_scan32(taddr + c0, bk->kinv + c0, slot0 + c0, best, best_slot);
       }
 #pragma unroll 1
       for (int c = c0; c < ncol; c += 16) {
