@@ -329,6 +329,15 @@ asap_status launch_rank(asap_ctx *ctx, const asap_inputs *in, const asap_params 
 // dropped token itself)
 bool merging(const asap_inputs *in, const asap_params *p) { return p->merge_enable && in->max_vis > p->keep_k; }
 
+// true when the merge blocks find their members themselves instead of reading a grouping that the similarity kernel leaves
+// behind.  The grouping is a tail of about 5 us; the scan costs every wave of merge blocks about 1 us per 1024 dropped tokens.
+// Measured per step (grouped -> scanned): 1 x 192 slots of 576 50.5 -> 47.7 us, 16 x 64 of 576 133.0 -> 129.2 us; on the other
+// side of the line, 12 x 145 of 577-2881 286.9 -> 288.2 us, 32 x 576 of 1152 and 288 of 576 (5120 wide) merge 460 -> 500 us.
+bool merge_scans(const asap_ctx *ctx, const asap_inputs *in, const asap_params *p) {
+  const long long passes = (in->max_vis - p->keep_k + MERGE_SCAN - 1) / MERGE_SCAN;
+  return merging(in, p) && passes * p->keep_k * in->B <= 8LL * ctx->num_sms;
+}
+
 // `fused_head_sum`: the ranking scores are still per-head sums in scratch (the score kernel ran
 // without its head-sum kernel); the selection adds the heads itself and writes out->rank_score.
 asap_status launch_select(asap_ctx *ctx, const asap_inputs *in, const asap_params *p,
@@ -423,7 +432,7 @@ asap_status launch_merge_front(asap_ctx *ctx, const asap_inputs *in, const asap_
         sa.wide = 1; sa.groups = pg; sa.cluster = 0; sa.threshold = p->sim_threshold;
         sa.drop_idx = nullptr; sa.role = ctx->role;
         sa.hidden = static_cast<const __nv_bfloat16 *>(in->hidden); sa.kept_inv = ctx->kept_inv; sa.assign = out->assign;
-        sa.best_sim = out->best_sim; sa.seg = ctx->seg; sa.members = ctx->members; sa.counters = ctx->cnt_sim;
+        sa.best_sim = out->best_sim; sa.seg = merge_scans(ctx, in, p) ? nullptr : ctx->seg; sa.members = ctx->members; sa.counters = ctx->cnt_sim;
         sa.tile_counters = ctx->cnt_tiles; sa.part = ctx->sim_part; sa.ss_part = nullptr; sa.smat = nullptr;
         sa.drop_all = drop_idx; sa.salience = salience; sa.member_meta = salience ? ctx->member_meta : nullptr;
         sa.status = ctx->status; sa.wait_limit = ctx->wait_limit;
@@ -480,7 +489,7 @@ asap_status launch_merge_front(asap_ctx *ctx, const asap_inputs *in, const asap_
     sa.threshold = p->sim_threshold;
     sa.drop_idx = gather_rows ? drop_idx : nullptr; sa.role = ctx->role;
     sa.hidden = static_cast<const __nv_bfloat16 *>(in->hidden); sa.kept_inv = ctx->kept_inv; sa.assign = out->assign;
-    sa.best_sim = out->best_sim; sa.seg = ctx->seg; sa.members = ctx->members; sa.counters = ctx->cnt_sim;
+    sa.best_sim = out->best_sim; sa.seg = merge_scans(ctx, in, p) ? nullptr : ctx->seg; sa.members = ctx->members; sa.counters = ctx->cnt_sim;
     sa.tile_counters = ctx->cnt_tiles; sa.part = ctx->sim_part;
     sa.ss_part = ctx->sim_part + (size_t)B * max_mt * splits * (size_t)k * 128;
     sa.smat = nullptr;
@@ -502,7 +511,7 @@ asap_status launch_merge_front(asap_ctx *ctx, const asap_inputs *in, const asap_
 // Steps 4b-5: weighted merge and compaction (the first consumer of the salience).
 asap_status launch_merge_back(asap_ctx *ctx, const asap_inputs *in, const asap_params *p,
                               const float *salience, const int32_t *keep_idx, const int32_t *drop_idx,
-                              const asap_outputs *out, cudaStream_t st, bool grouped_with_weights = false) {
+                              const asap_outputs *out, cudaStream_t st, bool grouped_with_weights = false, bool scan = false) {
   const int B = in->B, D = in->D, k = p->keep_k;
   const bool do_merge = merging(in, p);
   MergeArgs ma;
@@ -510,12 +519,22 @@ asap_status launch_merge_back(asap_ctx *ctx, const asap_inputs *in, const asap_p
   ma.D = D; ma.max_vis = in->max_vis; ma.keep_k = k; ma.merge_enable = do_merge ? 1 : 0; ma.eps = p->eps;
   ma.salience = salience; ma.keep_idx = keep_idx; ma.drop_idx = drop_idx; ma.seg = ctx->seg;
   ma.members = ctx->members; ma.member_meta = (do_merge && grouped_with_weights) ? ctx->member_meta : nullptr;
+  ma.assign = out->assign;
   ma.out_hidden = static_cast<__nv_bfloat16 *>(out->out_hidden);
   ma.out_pos = out->out_pos; ma.src_row = out->src_row;
   const int copy_rows = in->max_seq - in->min_vis;   // prefix + suffix rows of the longest sequence, at most
   const dim3 grid(k + (copy_rows + MERGE_COPY_ROWS - 1) / MERGE_COPY_ROWS, B);
   const int nv = (D / 8 + MERGE_THREADS - 1) / MERGE_THREADS;
   mark(ctx, "merge_compact", st);
+  if (scan) {
+    switch (nv) {
+      case 1: launch_pdl(merge_compact_kernel<1, false, true>, dim3(grid), dim3(MERGE_THREADS), 0, st, ma); break;
+      case 2: launch_pdl(merge_compact_kernel<2, false, true>, dim3(grid), dim3(MERGE_THREADS), 0, st, ma); break;
+      case 3: launch_pdl(merge_compact_kernel<3, false, true>, dim3(grid), dim3(MERGE_THREADS), 0, st, ma); break;
+      default: launch_pdl(merge_compact_kernel<4, false, true>, dim3(grid), dim3(MERGE_THREADS), 0, st, ma); break;
+    }
+    return after_launch(ctx, "merge_compact");
+  }
   switch (nv) {
     case 1: launch_pdl(merge_compact_kernel<1>, dim3(grid), dim3(MERGE_THREADS), 0, st, ma); break;
     case 2:
@@ -534,7 +553,7 @@ asap_status launch_merge(asap_ctx *ctx, const asap_inputs *in, const asap_params
                          const float *salience, const int32_t *keep_idx, const int32_t *drop_idx,
                          const asap_outputs *out, cudaStream_t st) {
   ASAP_TRY(launch_merge_front(ctx, in, p, salience, keep_idx, drop_idx, out, st));
-  return launch_merge_back(ctx, in, p, salience, keep_idx, drop_idx, out, st, true);
+  return launch_merge_back(ctx, in, p, salience, keep_idx, drop_idx, out, st, true, merge_scans(ctx, in, p));
 }
 
 // Sec. 4.2 inside the kept set: kept rows gathered, their keep_k x keep_k cosine matrix, routing.
@@ -958,7 +977,7 @@ asap_status asap_prune_step(asap_ctx *ctx, const asap_inputs *in, const asap_par
   e = cudaStreamWaitEvent(st, ctx->ev_join, 0);
   if (e != cudaSuccess) return fail(ctx, ASAP_ERR_CUDA, "join with the side stream: %s", cudaGetErrorString(e));
   if (main_status != ASAP_OK) return main_status;
-  return finish(ctx, launch_merge_back(ctx, in, p, out->salience, out->keep_idx, out->drop_idx, out, st), st);
+  return finish(ctx, launch_merge_back(ctx, in, p, out->salience, out->keep_idx, out->drop_idx, out, st, false, merge_scans(ctx, in, p)), st);
 }
 
 asap_status asap_compact_kv(asap_ctx *ctx, const int32_t *src_row, const int32_t *n_rows, int32_t rows_capacity,

@@ -752,6 +752,8 @@ kept_gather_kernel(const __nv_bfloat16 *__restrict__ hidden, const SampleDesc *_
 // entry of `members`, the member's visual index and its merge weight (the salience, as bits): the
 // merge kernel then reaches a member's row in two dependent loads instead of four.
 // =======================================================================================
+constexpr int CSR_BATCH = 6;      // 2736 dropped tokens: one warp's chunk of 288 positions is two batches instead of nine round trips
+
 __device__ __forceinline__ void csr_block(const SampleDesc &d, int b, int max_vis, int keep_k,
                                           const int32_t *__restrict__ assign,
                                           int32_t *__restrict__ seg, int32_t *__restrict__ members,
@@ -770,9 +772,17 @@ __device__ __forceinline__ void csr_block(const SampleDesc &d, int b, int max_vi
   for (int i = threadIdx.x; i < (W + 1) * keep_k; i += blockDim.x) s_cnt[i] = 0;
   __syncthreads();
   const int p_lo = min(nd, warp * chunk), p_hi = min(nd, p_lo + chunk);
-  for (int p = p_lo + lane; p < p_hi; p += 32) {
-    const int a = __ldcg(as_b + p);
-    if (a >= 0 && a < keep_k) atomicAdd(&hist[warp * keep_k + a], 1);
+  // (CSR_BATCH groups of 32 positions at a time, here and below, so that their loads are in flight together)
+  for (int base = p_lo; base < p_hi; base += 32 * CSR_BATCH) {
+    int a[CSR_BATCH];
+#pragma unroll
+    for (int t = 0; t < CSR_BATCH; ++t) {
+      const int p = base + 32 * t + lane;
+      a[t] = p < p_hi ? __ldcg(as_b + p) : -1;
+    }
+#pragma unroll
+    for (int t = 0; t < CSR_BATCH; ++t)
+      if (a[t] >= 0 && a[t] < keep_k) atomicAdd(&hist[warp * keep_k + a[t]], 1);
   }
   __syncthreads();
   // per slot: turn the per-warp counts into per-warp offsets inside the slot, and total them
@@ -803,26 +813,40 @@ __device__ __forceinline__ void csr_block(const SampleDesc &d, int b, int max_vi
   __syncthreads();
   // stable fill: every warp walks its chunk 32 positions at a time in ascending order
   const bool meta = drop_idx && salience && member_meta;
-  for (int base = p_lo; base < p_hi; base += 32) {
-    const int p = base + lane;
-    int a = (p < p_hi) ? __ldcg(as_b + p) : -1;
-    if (a >= keep_k) a = -1;
-    int2 mm = make_int2(0, 0);
-    if (meta && a >= 0) {
-      mm.x = min(max(__ldg(drop_idx + (size_t)b * nd_max + p), 0), d.nv - 1);
-      mm.y = __float_as_int(__ldcg(salience + (size_t)b * max_vis + mm.x));
+  for (int base0 = p_lo; base0 < p_hi; base0 += 32 * CSR_BATCH) {
+    int av[CSR_BATCH];
+    int2 mv[CSR_BATCH];
+#pragma unroll
+    for (int t = 0; t < CSR_BATCH; ++t) {
+      const int p = base0 + 32 * t + lane;
+      av[t] = p < p_hi ? __ldcg(as_b + p) : -1;
+      mv[t] = make_int2((meta && p < p_hi) ? __ldg(drop_idx + (size_t)b * nd_max + p) : 0, 0);
     }
-    const unsigned peers = __match_any_sync(0xffffffffu, a);
-    const int rank = __popc(peers & ((1u << lane) - 1u));
-    int cur = 0;
-    if (a >= 0) cur = hist[warp * keep_k + a];
-    __syncwarp();
-    if (a >= 0) {
-      mem_b[tot[a] + cur + rank] = p;
-      if (meta) member_meta[(size_t)b * nd_max + tot[a] + cur + rank] = mm;
-      if (rank == 0) hist[warp * keep_k + a] = cur + __popc(peers);
+    if (meta) {
+#pragma unroll
+      for (int t = 0; t < CSR_BATCH; ++t) {
+        mv[t].x = min(max(mv[t].x, 0), d.nv - 1);
+        mv[t].y = __float_as_int(__ldcg(salience + (size_t)b * max_vis + mv[t].x));
+      }
     }
-    __syncwarp();
+#pragma unroll
+    for (int t = 0; t < CSR_BATCH; ++t) {
+      const int p = base0 + 32 * t + lane;
+      if (base0 + 32 * t >= p_hi) break;
+      int a = av[t];
+      if (a >= keep_k) a = -1;
+      const unsigned peers = __match_any_sync(0xffffffffu, a);
+      const int rank = __popc(peers & ((1u << lane) - 1u));
+      int cur = 0;
+      if (a >= 0) cur = hist[warp * keep_k + a];
+      __syncwarp();
+      if (a >= 0) {
+        mem_b[tot[a] + cur + rank] = p;
+        if (meta) member_meta[(size_t)b * nd_max + tot[a] + cur + rank] = mv[t];
+        if (rank == 0) hist[warp * keep_k + a] = cur + __popc(peers);
+      }
+      __syncwarp();
+    }
   }
 }
 
@@ -1204,6 +1228,7 @@ constexpr int MERGE_THREADS = 256;
 constexpr int MERGE_COPY_ROWS = MERGE_THREADS / 32;   // copy rows per block
 constexpr int MERGE_LIST = 256;                        // members listed per pass
 constexpr int MERGE_BATCH = 4;                         // member rows in flight per thread
+constexpr int MERGE_SCAN = 4 * MERGE_THREADS;          // destinations looked at per pass of a scan
 
 struct MergeArgs {
   const __nv_bfloat16 *hidden;
@@ -1214,6 +1239,7 @@ struct MergeArgs {
   const float *salience;
   const int32_t *keep_idx, *drop_idx, *seg, *members;
   const int2 *member_meta;   // [B, max_vis-keep_k] (visual index, weight bits) beside `members`, or nullptr
+  const int32_t *assign;     // [B, max_vis-keep_k] (SCAN only) destination slot of every dropped token
   __nv_bfloat16 *out_hidden;
   int32_t *out_pos, *src_row;
 };
@@ -1225,13 +1251,18 @@ struct MergeArgs {
 // few waves the shorter batches cost more than the occupancy gives (c2 24.8 -> 26.6 us), so those keep four rows.
 // Rows of 4097-6144 elements (NV = 3): one member row in flight, 64 registers, four blocks per SM as well
 // (D = 5120, 1152 of 2304 kept: 280 -> 241 us; 576 of 1152: 151 -> 133 us; 288 of 576: 85 -> 75 us).
-template <int NV, bool LEAN = false>
-__global__ void __launch_bounds__(MERGE_THREADS, NV >= 4 ? 2 : ((LEAN || NV == 3) ? 4 : 3))
+// SCAN: no grouping of the dropped tokens exists; the block finds its members itself, reading the destinations of all dropped
+// tokens of the sequence (MERGE_SCAN at a time, ascending, so the members come in the order the grouping would give).
+// Grouping is a chain of eight barriers at the end of the similarity kernel (10-12 thousand clocks with its hand-shake,
+// nothing beside it on a small batch); scanning costs every block 4 (n_v - k) bytes out of L2.
+template <int NV, bool LEAN = false, bool SCAN = false>
+__global__ void __launch_bounds__(MERGE_THREADS, NV >= 4 ? 2 : ((LEAN || (NV == 3 && !SCAN)) ? 4 : 3))
 merge_compact_kernel(MergeArgs a) {
   constexpr int BATCH = NV == 3 ? 1 : ((NV >= 4 || LEAN) ? 2 : MERGE_BATCH);
   pdl_enter();
-  __shared__ int s_j[MERGE_LIST];
-  __shared__ float s_w[MERGE_LIST];
+  __shared__ int s_j[SCAN ? MERGE_SCAN : MERGE_LIST];
+  __shared__ float s_w[SCAN ? MERGE_SCAN : MERGE_LIST];
+  __shared__ int s_tot[MERGE_THREADS / 32];
   const int b = blockIdx.y;
   const SampleDesc d = a.desc[b];
   if (!d.valid) return;
@@ -1275,7 +1306,9 @@ merge_compact_kernel(MergeArgs a) {
   uint4 *dst = reinterpret_cast<uint4 *>(a.out_hidden + (size_t)orow * a.D);
   const int nd_max = a.max_vis - k;
   int m_lo = 0, m_hi = 0;
-  if (a.merge_enable) {
+  if (SCAN) {
+    m_hi = d.nv - k;                      // every dropped token is looked at
+  } else if (a.merge_enable) {
     m_lo = min(max(a.seg[(size_t)b * (k + 1) + slot], 0), nd_max);
     m_hi = min(max(a.seg[(size_t)b * (k + 1) + slot + 1], m_lo), nd_max);
   }
@@ -1306,19 +1339,60 @@ merge_compact_kernel(MergeArgs a) {
     for (int e = 0; e < 8; ++e) acc[u][e] = w_self * f[e];
   }
   float den = w_self;
+  bool merged = !SCAN;
   const __nv_bfloat16 *vis0 = a.hidden + (size_t)(d.row0 + d.v0) * a.D;
-  for (int base = m_lo; base < m_hi; base += MERGE_LIST) {
-    const int cnt = min(MERGE_LIST, m_hi - base);
-    __syncthreads();                      // the previous list has been consumed
-    if ((int)threadIdx.x < cnt) {
-      if (a.member_meta) {
-        const int2 mm = __ldg(a.member_meta + (size_t)b * nd_max + base + threadIdx.x);
-        s_j[threadIdx.x] = min(max(mm.x, 0), d.nv - 1);
-        s_w[threadIdx.x] = __int_as_float(mm.y);
-      } else {
-        const int j = min(max(drop_b[min(max(mem_b[base + threadIdx.x], 0), nd_max - 1)], 0), d.nv - 1);
-        s_j[threadIdx.x] = j;
-        s_w[threadIdx.x] = sal_b[j];
+  for (int base = m_lo; base < m_hi; base += SCAN ? MERGE_SCAN : MERGE_LIST) {
+    int cnt;
+    if (SCAN) {
+      const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+      const int p0 = base + threadIdx.x * 4;
+      const int32_t *as = a.assign + (size_t)b * nd_max;
+      int dst[4];
+#pragma unroll
+      for (int e = 0; e < 4; ++e) dst[e] = p0 + e < m_hi ? __ldg(as + p0 + e) : -1;
+      int mine = 0;
+#pragma unroll
+      for (int e = 0; e < 4; ++e) mine += dst[e] == slot;
+      int inc = mine;
+      if (__any_sync(0xffffffffu, mine)) {
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+          const int t = __shfl_up_sync(0xffffffffu, inc, o);
+          if (lane >= o) inc += t;
+        }
+      }
+      __syncthreads();                    // the previous list has been consumed
+      if (lane == 31) s_tot[warp] = inc;
+      __syncthreads();
+      int at = inc - mine;
+      cnt = 0;
+#pragma unroll
+      for (int w = 0; w < MERGE_THREADS / 32; ++w) {
+        if (w < warp) at += s_tot[w];
+        cnt += s_tot[w];
+      }
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        if (dst[e] != slot) continue;
+        const int j = min(max(__ldg(drop_b + p0 + e), 0), d.nv - 1);
+        s_j[at] = j;
+        s_w[at] = __ldg(sal_b + j);
+        ++at;
+      }
+      merged = merged || cnt > 0;
+    } else {
+      cnt = min(MERGE_LIST, m_hi - base);
+      __syncthreads();                    // the previous list has been consumed
+      if ((int)threadIdx.x < cnt) {
+        if (a.member_meta) {
+          const int2 mm = __ldg(a.member_meta + (size_t)b * nd_max + base + threadIdx.x);
+          s_j[threadIdx.x] = min(max(mm.x, 0), d.nv - 1);
+          s_w[threadIdx.x] = __int_as_float(mm.y);
+        } else {
+          const int j = min(max(drop_b[min(max(mem_b[base + threadIdx.x], 0), nd_max - 1)], 0), d.nv - 1);
+          s_j[threadIdx.x] = j;
+          s_w[threadIdx.x] = sal_b[j];
+        }
       }
     }
     __syncthreads();
@@ -1351,7 +1425,7 @@ merge_compact_kernel(MergeArgs a) {
       }
     }
   }
-  if (den <= a.eps) {
+  if (den <= a.eps || !merged) {
 #pragma unroll
     for (int u = 0; u < NV; ++u) {
       const int v = threadIdx.x + u * MERGE_THREADS;

@@ -727,7 +727,7 @@ struct SimArgs {
   const float *kept_inv;     // [B*keep_k]   1/||kept row||, 0 for a zero row
   int32_t *assign;           // [B, max_vis-keep_k]
   float *best_sim;           // [B, max_vis-keep_k] or nullptr
-  int32_t *seg;              // [B, keep_k+1]       CSR of assign, built by the last block of a sample
+  int32_t *seg;              // [B, keep_k+1]       CSR of assign, built by the last block of a sample; nullptr: not wanted
   int32_t *members;          // [B, max_vis-keep_k]
   unsigned int *counters;    // [B]            finished row tiles per sample
   unsigned int *tile_counters;  // [B, max_mt] finished slices per row tile
@@ -789,6 +789,11 @@ __device__ __forceinline__ void sim_scan32(uint32_t taddr, const float *kinv, in
   }
 }
 
+template <int V>
+struct IntC {
+  static constexpr int value = V;
+};
+
 constexpr int SIM_THREADS_TILED = 192;                  // without gather warps: two such blocks fit an SM
 
 template <bool GATHER>
@@ -824,7 +829,7 @@ sim_kernel(const __grid_constant__ CUtensorMap tmap_h, const __grid_constant__ C
   if (n_rows <= 0) {
     // nothing was dropped in this sample: only the (empty) grouping has to be written
     pdl_enter();
-    if (z == 0 && gz == 0) csr_block(d, b, a.max_vis, a.keep_k, a.assign, a.seg, a.members, reinterpret_cast<int *>(base_ptr), bk->scan, a.drop_all, a.salience, a.member_meta);
+    if (z == 0 && gz == 0 && a.seg) csr_block(d, b, a.max_vis, a.keep_k, a.assign, a.seg, a.members, reinterpret_cast<int *>(base_ptr), bk->scan, a.drop_all, a.salience, a.member_meta);
     return;
   }
 
@@ -1181,29 +1186,47 @@ sim_kernel(const __grid_constant__ CUtensorMap tmap_h, const __grid_constant__ C
         pz[zz] = cluster_map(smem_u32(cl_p), (uint32_t)min(zz, S - 1)) + (uint32_t)lane * 16u;
       float wb[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
       int wsl[4] = {0, 0, 0, 0};
-      for (int i = quarter; i < n_mine; i += 4) {
-        const int slot = s_lo + i;
-        float4 x[8];
+      // (the loads of U slots are in flight together: with one slot's loads at a time the adding was a chain of round
+      // trips of 700 clocks, 6000-7000 in all)
+      auto add_slots = [&](auto uc, int i0) {
+        constexpr int U = decltype(uc)::value, Z = 8 / U;      // slots in flight, slices at most
+        float4 x[U][Z];
+        float ks[U];
 #pragma unroll
-        for (int zz = 0; zz < 8; ++zz)
-          if (zz < S) x[zz] = ld_cluster_v4f32(pz[zz] + (uint32_t)slot * 512u);
-        float acc[4] = {0.f, 0.f, 0.f, 0.f};
+        for (int u = 0; u < U; ++u) {
+          const int slot = min(s_lo + i0 + 4 * u, a.keep_k - 1);
+          ks[u] = __ldg(kinv + slot);
 #pragma unroll
-        for (int zz = 0; zz < 8; ++zz)
-          if (zz < S) { acc[0] += x[zz].x; acc[1] += x[zz].y; acc[2] += x[zz].z; acc[3] += x[zz].w; }
-        const float ks = __ldg(kinv + slot);
+          for (int zz = 0; zz < Z; ++zz)
+            if (zz < S) x[u][zz] = ld_cluster_v4f32(pz[zz] + (uint32_t)slot * 512u);
+        }
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          if (a.smat) {
-            const int vr = mt * 128 + lane * 4 + j;
-            if (vr < a.keep_k && !bk->abort_flag)
-              a.smat[((size_t)b * a.keep_k + vr) * a.keep_k + slot] = acc[j] * (__ldg(kinv + vr) * ks);
-          } else {
-            const float val = acc[j] * ks;
-            if (val > wb[j]) { wb[j] = val; wsl[j] = slot; }
+        for (int u = 0; u < U; ++u) {
+          if (i0 + 4 * u >= n_mine) continue;
+          const int slot = s_lo + i0 + 4 * u;
+          float acc[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+          for (int zz = 0; zz < Z; ++zz)
+            if (zz < S) { acc[0] += x[u][zz].x; acc[1] += x[u][zz].y; acc[2] += x[u][zz].z; acc[3] += x[u][zz].w; }
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            if (a.smat) {
+              const int vr = mt * 128 + lane * 4 + j;
+              if (vr < a.keep_k && !bk->abort_flag)
+                a.smat[((size_t)b * a.keep_k + vr) * a.keep_k + slot] = acc[j] * (__ldg(kinv + vr) * ks[u]);
+            } else {
+              const float val = acc[j] * ks[u];
+              if (val > wb[j]) { wb[j] = val; wsl[j] = slot; }
+            }
           }
         }
-      }
+      };
+      if (S <= 2)
+        for (int i = quarter; i < n_mine; i += 16) add_slots(IntC<4>(), i);
+      else if (S <= 4)
+        for (int i = quarter; i < n_mine; i += 8) add_slots(IntC<2>(), i);
+      else
+        for (int i = quarter; i < n_mine; i += 4) add_slots(IntC<1>(), i);
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
         cl_wv[quarter * 128 + lane * 4 + j] = wb[j];
@@ -1335,7 +1358,7 @@ sim_kernel(const __grid_constant__ CUtensorMap tmap_h, const __grid_constant__ C
     tmem_dealloc(tmem_base, a.tmem_cols);
   }
   if (a.smat) return;
-  if (!bk->is_last && (a.splits > 1 || a.groups > 1)) return;     // a slice / group that did not finalize its row tile
+  if (!a.seg || (!bk->is_last && (a.splits > 1 || a.groups > 1))) return;   // (or a slice / group that did not finalize its row tile)
   __syncthreads();
   // the block that finishes the sample's last row tile groups the dropped tokens by destination
   if (threadIdx.x == 0) {
@@ -1635,7 +1658,7 @@ sim_pair_kernel(const __grid_constant__ CUtensorMap tmap_h, const __grid_constan
     tc_fence_after();
     tmem_dealloc(tmem_base, a.tmem_cols);
   }
-  if (!bk->is_last) return;                              // a group that did not finalize its pair (or matrix mode)
+  if (!a.seg || !bk->is_last) return;                    // (or a group that did not finalize its pair, or matrix mode)
   __syncthreads();
   if (threadIdx.x == 0) {
     __threadfence();

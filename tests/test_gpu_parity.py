@@ -49,6 +49,16 @@ def test_two_slot_tiles_in_one_pass(ctx, k):
     run_step(ctx, batch, A.Params(keep_k=k))
 
 
+@pytest.mark.parametrize("nvs,k", [([1028, 1029], 4), ([2500, 1030], 3), ([40, 16], 16), ([2060], 7)],
+                         ids=["one_pass", "three_passes", "nothing_dropped", "three_passes_one"])
+def test_merge_blocks_that_scan_for_their_members(ctx, nvs, k):
+    """Few kept slots: the merge blocks look their members up among all dropped tokens, 1024 per pass -- exactly
+    one full pass, ragged later passes, far more members per slot than a list of the grouped form holds, and a
+    sequence without a dropped token."""
+    batch = W.tiny(B=len(nvs), n_vis=nvs, text_lens=[9 + b for b in range(len(nvs))], H=2, keep_k=k, seed=120 + k, centres=k + 1)
+    run_step(ctx, batch, A.Params(keep_k=k))
+
+
 def test_many_row_tiles_and_three_slot_tiles(ctx):
     """A batch large enough that the similarity kernel runs unsliced with more blocks than SMs
     (15 sequences x 19 row tiles) and three slot tiles (600 kept slots).  Odd and even numbers of row
