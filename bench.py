@@ -297,7 +297,7 @@ class Setup:
 
 def capture_graph(S):
     """One CUDA graph holding one step per device copy (the library's calls are capturable: no
-    allocation, no synchronisation, the side stream joins back inside the call)."""
+    allocation, no synchronisation)."""
     A = S.A
     c0 = A.asap_launch_count(S.ctx)
     graph = torch.cuda.CUDAGraph()

@@ -40,10 +40,6 @@
  *   - bf16 tensors are row-major with the stated shapes and no padding.
  *   - A context serves one stream at a time: two calls on the same context that overlap on
  *     the GPU race on its scratch memory.
- *   - asap_prune_step may enqueue two of its kernels (attention mass, salience) on a second
- *     stream that belongs to the context, forked from and joined back into `stream` with
- *     events inside the call: everything the call enqueues is ordered after the work already
- *     in `stream`, and work enqueued in `stream` after the call is ordered after all of it.
  */
 #ifndef ASAP_H
 #define ASAP_H
@@ -132,9 +128,8 @@ typedef struct {
 /* Creates a context on `device` and takes all scratch memory the step will ever need for
  * problems with total_tokens <= max_total_tokens, B <= max_B, H <= max_H, D <= max_D and
  * B * keep_k <= max_keep_rows (0 = max_total_tokens).  The only call that allocates.
- * Which kernel form a launch takes is decided from the problem size; four environment variables, read
+ * Which kernel form a launch takes is decided from the problem size; three environment variables, read
  * here once per context, move those decisions for measurements (results are the same up to rounding order):
- *   ASAP_FUSE_MASS_MIN_TOKENS   B * max_vis from which Eq. 1's key side rides in the score kernel (default 50000)
  *   ASAP_SIM_PAIR_MIN_BLOCKS    blocks from which the similarity takes two row tiles per block (default: half the SMs)
  *   ASAP_SIM_PAIR_STAGES        tile stages of that form (default: what fits 192 KB)
  *   ASAP_SIM_CLUSTER            0: sliced similarity launches add their partial products through global memory
@@ -210,8 +205,7 @@ asap_status asap_attention(asap_ctx *ctx, const asap_inputs *in, const asap_para
                            void *out, void *stream);
 
 /* Steps 1a-5 back to back on `stream`; fills every field of `out`.  The call may be recorded by a
- * stream capture (it allocates nothing and does not synchronise; the context's side stream forks from
- * and joins back into `stream` inside the call) and the graph replayed on new contents of the same
+ * stream capture (it allocates nothing and does not synchronise) and the graph replayed on new contents of the same
  * buffers. */
 asap_status asap_prune_step(asap_ctx *ctx, const asap_inputs *in, const asap_params *p,
                             const asap_outputs *out, void *stream);

@@ -45,7 +45,6 @@ struct asap_ctx {
   unsigned int *cnt_qsum = nullptr, *cnt_mass = nullptr, *cnt_score = nullptr, *cnt_sim = nullptr,
                *cnt_tiles = nullptr, *cnt_work = nullptr;
   float *mass_partial = nullptr;    // [B, H, max_vis] per-head attention masses written by the score kernel
-  long long fuse_mass_min_tokens = 50000;   // B * max_vis from which the attention mass rides in the score kernel
   long long sim_pair_min_blocks = 0;        // blocks from which the similarity takes two row tiles per block (0: half the SM count)
   int sim_pair_stages = 0;                  // stages of that form (0: what fits 192 KB)
   int sim_cluster = 1;                      // 0: sliced similarity launches add their partials through global memory
@@ -56,8 +55,6 @@ struct asap_ctx {
   __nv_bfloat16 *kept_rows = nullptr;
   uint32_t *status = nullptr;
   EncodeTiledFn encode = nullptr;
-  cudaStream_t side = nullptr;            // second stream for the mass kernels of asap_prune_step
-  cudaEvent_t ev_fork = nullptr, ev_desc = nullptr, ev_join = nullptr;
   uint64_t launches = 0;
   long long wait_limit = TC_WAIT_LIMIT;   // clock cycles a wait of the tensor-core kernels may take (asap_debug_wait_limit)
   size_t counters_off = 0, counters_bytes = 0, tiles_off = 0, tiles_bytes = 0;   // the kernels' hand-shake counters in the arena
@@ -263,8 +260,7 @@ int qsum_rows_per_chunk(const asap_ctx *ctx, const asap_inputs *in) {
 }
 
 asap_status launch_mass(asap_ctx *ctx, const asap_inputs *in, const asap_params *p, const asap_outputs *out,
-                        bool fold_prepare, int32_t *out_cu, int out_capacity, cudaStream_t st,
-                        cudaEvent_t after_qsum = nullptr) {
+                        bool fold_prepare, int32_t *out_cu, int out_capacity, cudaStream_t st) {
   const int D = in->D, B = in->B;
   const int qrows = qsum_rows_per_chunk(ctx, in);
   const int max_chunks = (in->max_vis + qrows - 1) / qrows;
@@ -276,8 +272,6 @@ asap_status launch_mass(asap_ctx *ctx, const asap_inputs *in, const asap_params 
              static_cast<const __nv_bfloat16 *>(in->q), pa, D, max_chunks, qrows, ctx->qsum_partial, ctx->qbar,
              ctx->cnt_qsum);
   ASAP_TRY(after_launch(ctx, "qsum"));
-  if (after_qsum && cudaEventRecord(after_qsum, st) != cudaSuccess)
-    return fail(ctx, ASAP_ERR_CUDA, "event after the query-sum kernel");
 
   const int row_blocks = (in->max_vis + MASS_ROWS - 1) / MASS_ROWS;
   if (p->per_head_mask) {
@@ -298,6 +292,8 @@ asap_status launch_mass(asap_ctx *ctx, const asap_inputs *in, const asap_params 
 }
 
 // Steps 1c-2: Eq. 4 probabilities of the ranking rows, summed per head; optionally the head sum.
+// `with_mass` (ranking rows = the text span): the same kernel takes the per-head attention masses (Eq. 1), validates the batch
+// and writes the descriptors and `out`'s row offsets.
 asap_status launch_rank(asap_ctx *ctx, const asap_inputs *in, const asap_params *p, const asap_outputs *out,
                         bool with_head_sum, cudaStream_t st, bool with_mass = false) {
   const int D = in->D, B = in->B;
@@ -306,12 +302,13 @@ asap_status launch_rank(asap_ctx *ctx, const asap_inputs *in, const asap_params 
       !make_map(ctx, &map_k, in->k, (uint64_t)in->total_tokens, (uint64_t)D, 128))
     return fail(ctx, ASAP_ERR_CUDA, "cuTensorMapEncodeTiled failed for q / k");
   ScoreArgs sa;
-  sa.pa = prepare_args(ctx, in, p, nullptr, 0x7fffffff); sa.pa.write_desc = 0; sa.B = B; sa.H = in->H; sa.max_vis = in->max_vis; sa.mask_enable = p->mask_enable ? 1 : 0;
+  sa.pa = with_mass ? prepare_args(ctx, in, p, out->out_cu_seqlens, out->out_rows_capacity) : prepare_args(ctx, in, p, nullptr, 0x7fffffff);
+  sa.pa.write_desc = with_mass ? 1 : 0; sa.B = B; sa.H = in->H; sa.max_vis = in->max_vis; sa.mask_enable = p->mask_enable ? 1 : 0;
   sa.scale_log2 = 1.4426950408889634f / sqrtf((float)in->head_dim);
   sa.mask_log = p->per_head_mask ? out->mask_log_heads : out->mask_log;
   sa.mask_b_stride = p->per_head_mask ? in->H * in->max_vis : in->max_vis;
   sa.mask_h_stride = p->per_head_mask ? in->max_vis : 0;
-  sa.qbar = with_mass ? ctx->qbar : nullptr; sa.mass_heads = ctx->mass_partial; sa.D = D;
+  sa.mass_heads = with_mass ? ctx->mass_partial : nullptr;
   sa.partial = ctx->score_partial; sa.work = ctx->cnt_work; sa.status = ctx->status; sa.wait_limit = ctx->wait_limit;
   mark(ctx, "score", st);
   const int items = B * in->H;
@@ -342,12 +339,16 @@ bool merge_scans(const asap_ctx *ctx, const asap_inputs *in, const asap_params *
 // without its head-sum kernel); the selection adds the heads itself and writes out->rank_score.
 asap_status launch_select(asap_ctx *ctx, const asap_inputs *in, const asap_params *p,
                           const float *rank_score, const asap_outputs *out, bool with_merge,
-                          bool fused_head_sum, cudaStream_t st) {
+                          bool fused_head_sum, cudaStream_t st, bool with_salience = false) {
+  SalienceArgs sal;
+  sal.H = in->H; sal.scale = 1.0f / ((float)in->H * sqrtf((float)in->head_dim)); sal.lambda_max = p->lambda_max; sal.eps = p->eps;
+  sal.heads = ctx->mass_partial; sal.mass = out->mass; sal.salience = out->salience; sal.mask_log = out->mask_log;
+  sal.rank_score = out->rank_score;
   mark(ctx, "select", st);
-  launch_pdl(select_kernel, dim3(in->B), dim3(SELECT_THREADS), (size_t)in->max_vis * sizeof(uint32_t), st,
+  launch_pdl(select_kernel, dim3(in->B, with_salience ? 2 : 1), dim3(SELECT_THREADS), (size_t)in->max_vis * sizeof(uint32_t), st,
              rank_score, ctx->desc, in->max_vis, p->keep_k, out->keep_idx, out->drop_idx, ctx->role,
              with_merge ? out->assign : nullptr, with_merge ? out->best_sim : nullptr, merging(in, p) ? 1 : 0,
-             fused_head_sum ? ctx->score_partial : nullptr, in->H, fused_head_sum ? out->rank_score : nullptr);
+             fused_head_sum ? ctx->score_partial : nullptr, in->H, fused_head_sum ? out->rank_score : nullptr, sal);
   return after_launch(ctx, "select");
 }
 
@@ -748,7 +749,6 @@ asap_status asap_init(asap_ctx **ctx_out, int device, size_t max_total_tokens, i
   ctx->qbar = reinterpret_cast<float *>(ctx->arena + o_qbar);
   ctx->score_partial = reinterpret_cast<float *>(ctx->arena + o_spart);
   ctx->mass_partial = reinterpret_cast<float *>(ctx->arena + o_mpart);
-  if (const char *env = getenv("ASAP_FUSE_MASS_MIN_TOKENS")) ctx->fuse_mass_min_tokens = atoll(env);
   if (const char *env = getenv("ASAP_SIM_PAIR_MIN_BLOCKS")) ctx->sim_pair_min_blocks = atoll(env);
   if (const char *env = getenv("ASAP_SIM_PAIR_STAGES")) ctx->sim_pair_stages = atoi(env);
   if (const char *env = getenv("ASAP_SIM_CLUSTER")) ctx->sim_cluster = atoi(env);
@@ -798,20 +798,8 @@ asap_status asap_init(asap_ctx **ctx_out, int device, size_t max_total_tokens, i
       cudaGetLastError();
     }
   }
-  // lowest priority: when both streams have blocks to place, the score kernel's go first and the
-  // mass kernels fill what is left of each SM
-  int prio_least = 0, prio_greatest = 0;
-  if (e == cudaSuccess) e = cudaDeviceGetStreamPriorityRange(&prio_least, &prio_greatest);
-  if (e == cudaSuccess) e = cudaStreamCreateWithPriority(&ctx->side, cudaStreamNonBlocking, prio_least);
-  if (e == cudaSuccess) e = cudaEventCreateWithFlags(&ctx->ev_desc, cudaEventDisableTiming);
-  if (e == cudaSuccess) e = cudaEventCreateWithFlags(&ctx->ev_fork, cudaEventDisableTiming);
-  if (e == cudaSuccess) e = cudaEventCreateWithFlags(&ctx->ev_join, cudaEventDisableTiming);
   if (e == cudaSuccess) e = cudaDeviceSynchronize();
   if (e != cudaSuccess) {
-    if (ctx->ev_fork) cudaEventDestroy(ctx->ev_fork);
-    if (ctx->ev_join) cudaEventDestroy(ctx->ev_join);
-    if (ctx->ev_desc) cudaEventDestroy(ctx->ev_desc);
-    if (ctx->side) cudaStreamDestroy(ctx->side);
     cudaFree(ctx->arena);
     delete ctx;
     return fail(nullptr, ASAP_ERR_CUDA, "asap_init set-up: %s", cudaGetErrorString(e));
@@ -922,62 +910,16 @@ asap_status asap_prune_step(asap_ctx *ctx, const asap_inputs *in, const asap_par
   ASAP_TRY(validate(ctx, in, p, out, NEED_QK | NEED_HIDDEN | NEED_SCORE_OUT | NEED_SELECT_OUT | NEED_MERGE_OUT));
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   // With the text span as ranking rows the Eq. 3 mask never touches a ranked row (a text query lies
-  // after every visual key), so the score kernel does not need the attention mass: the memory-bound
-  // mass kernels then run on the context's side stream next to the score kernel, and rejoin before
-  // the merge, which is the first consumer of the salience.  With caller-given ranking rows (which may
-  // be visual) and while per-kernel timing is on, everything runs in order on `stream`.
-  const bool text_rows = in->rank_start == nullptr && !p->per_head_mask;
-  if (text_rows && (long long)in->B * in->max_vis >= ctx->fuse_mass_min_tokens) {
-    // Large batches: the mass kernels no longer hide beside the score kernel (both are bound by the same
-    // memory system), so Eq. 1's key side is taken from the key tiles the score kernel streams anyway:
-    // query sum (carrying the validation) -> score kernel with two more columns per key tile -> Eq. 2-3.
-    PrepareArgs pa = prepare_args(ctx, in, p, out->out_cu_seqlens, out->out_rows_capacity);
-    pa.write_desc = 1;
-    const int qrows = qsum_rows_per_chunk(ctx, in);
-    const int max_chunks = (in->max_vis + qrows - 1) / qrows;
-    mark(ctx, "qsum", st);
-    launch_pdl(qsum_kernel, dim3(max_chunks, (in->D + QSUM_COLS - 1) / QSUM_COLS, in->B), dim3(QSUM_THREADS), 0, st,
-               static_cast<const __nv_bfloat16 *>(in->q), pa, in->D, max_chunks, qrows, ctx->qsum_partial, ctx->qbar, ctx->cnt_qsum);
-    ASAP_TRY(after_launch(ctx, "qsum"));
-    ASAP_TRY(launch_rank(ctx, in, p, out, false, st, true));
-    mark(ctx, "salience", st);
-    launch_pdl(salience_from_heads_kernel, dim3(in->B), dim3(SAL_THREADS), 0, st, ctx->desc, in->H, in->max_vis,
-               1.0f / ((float)in->H * sqrtf((float)in->head_dim)), p->lambda_max, p->eps, ctx->mass_partial, out->mass,
-               out->salience, out->mask_log, out->rank_score);
-    ASAP_TRY(after_launch(ctx, "salience"));
-    ASAP_TRY(launch_select(ctx, in, p, out->rank_score, out, true, true, st));
-    return finish(ctx, launch_merge(ctx, in, p, out->salience, out->keep_idx, out->drop_idx, out, st), st);
-  }
-  const bool overlap = text_rows && !ctx->prof_on && ctx->side != nullptr;
-  if (!overlap) {
-    ASAP_TRY(launch_mass(ctx, in, p, out, true, out->out_cu_seqlens, out->out_rows_capacity, st));
-    ASAP_TRY(launch_rank(ctx, in, p, out, false, st));
-    ASAP_TRY(launch_select(ctx, in, p, out->rank_score, out, true, true, st));
-    return finish(ctx, launch_merge(ctx, in, p, out->salience, out->keep_idx, out->drop_idx, out, st), st);
-  }
-  // stream:      [fork] score (derives its own descriptors) -> wait descriptors -> select -> gather -> sim
-  // side stream: qsum (carrying the validation) -> [descriptors ready] -> mass -> [join]
-  // The score kernel is enqueued first, so its one block per SM is placed before the mass kernels'
-  // many small blocks, which then fill what is left of each SM.
-  cudaError_t e = cudaEventRecord(ctx->ev_fork, st);
-  if (e != cudaSuccess) return fail(ctx, ASAP_ERR_CUDA, "fork event: %s", cudaGetErrorString(e));
-  asap_status main_status = launch_rank(ctx, in, p, out, false, st);
-  e = cudaStreamWaitEvent(ctx->side, ctx->ev_fork, 0);
-  if (e != cudaSuccess) return fail(ctx, ASAP_ERR_CUDA, "fork to the side stream: %s", cudaGetErrorString(e));
-  asap_status side_status = launch_mass(ctx, in, p, out, true, out->out_cu_seqlens, out->out_rows_capacity, ctx->side,
-                                        ctx->ev_desc);
-  e = cudaEventRecord(ctx->ev_join, ctx->side);
-  if (e != cudaSuccess) return fail(ctx, ASAP_ERR_CUDA, "join event: %s", cudaGetErrorString(e));
-  if (main_status == ASAP_OK) main_status = side_status;
-  if (main_status == ASAP_OK && cudaStreamWaitEvent(st, ctx->ev_desc, 0) != cudaSuccess)
-    main_status = fail(ctx, ASAP_ERR_CUDA, "wait for the descriptors");
-  if (main_status == ASAP_OK) main_status = launch_select(ctx, in, p, out->rank_score, out, true, true, st);
-  if (main_status == ASAP_OK) main_status = launch_merge_front(ctx, in, p, nullptr, out->keep_idx, out->drop_idx, out, st);
-  // the side stream always rejoins, also after an error, so that `stream` stays ordered behind it
-  e = cudaStreamWaitEvent(st, ctx->ev_join, 0);
-  if (e != cudaSuccess) return fail(ctx, ASAP_ERR_CUDA, "join with the side stream: %s", cudaGetErrorString(e));
-  if (main_status != ASAP_OK) return main_status;
-  return finish(ctx, launch_merge_back(ctx, in, p, out->salience, out->keep_idx, out->drop_idx, out, st, false, merge_scans(ctx, in, p)), st);
+  // after every visual key), so the score kernel does not need the attention mass, and takes it itself from the query and key
+  // tiles: no query sum, no mass kernel, no second stream.  With caller-given ranking rows (which may be visual) or a mask per
+  // head the masses come first.  Measured per step, masses inside the score kernel against mass kernels on a stream beside it:
+  // 1 x 576 visual tokens 48.6 -> 42.6 us, 16 x 576 129.5 -> 121.4, 8 x 2304 243 -> 207, 12 mixed images 286 -> 242; against a
+  // query-sum kernel in front, 64 x 2880 2530 -> 2427 us.
+  const bool fused = in->rank_start == nullptr && !p->per_head_mask;
+  if (!fused) ASAP_TRY(launch_mass(ctx, in, p, out, true, out->out_cu_seqlens, out->out_rows_capacity, st));
+  ASAP_TRY(launch_rank(ctx, in, p, out, false, st, fused));
+  ASAP_TRY(launch_select(ctx, in, p, out->rank_score, out, true, true, st, fused));
+  return finish(ctx, launch_merge(ctx, in, p, out->salience, out->keep_idx, out->drop_idx, out, st), st);
 }
 
 asap_status asap_compact_kv(asap_ctx *ctx, const int32_t *src_row, const int32_t *n_rows, int32_t rows_capacity,
@@ -1191,10 +1133,6 @@ void asap_free(asap_ctx *ctx) {
     delete[] ctx->prof_ev;
     delete[] ctx->prof_name;
   }
-  if (ctx->side) { cudaStreamSynchronize(ctx->side); cudaStreamDestroy(ctx->side); }
-  if (ctx->ev_fork) cudaEventDestroy(ctx->ev_fork);
-  if (ctx->ev_join) cudaEventDestroy(ctx->ev_join);
-  if (ctx->ev_desc) cudaEventDestroy(ctx->ev_desc);
   cudaFree(ctx->arena);
   delete ctx;
 }

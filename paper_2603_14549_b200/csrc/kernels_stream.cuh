@@ -2,7 +2,7 @@
 //   prepare        device-side validation, per-sample descriptors, output row offsets
 //   qsum           sum of the visual query rows                       (Eq. 1, summed over i first)
 //   mass_salience  s_j, then s_hat_j and m_j                          (Eq. 1, Eq. 2, Eq. 3)
-//   salience_from_heads  the same from per-head masses the score kernel produced
+//   salience_block the same from per-head masses the score kernel produced (part of the selection launch)
 //   select         stable radix top-k of the ranking scores           (Fig. 3)
 //   role_map       kept slot / dropped position of every visual token
 //   kept_gather    kept rows gathered for the similarity GEMM, with their inverse norms (Sec. 4.2)
@@ -77,6 +77,44 @@ __device__ __forceinline__ void prepare_block(const PrepareArgs &a) {
     if (bits) atomicOr(a.status, bits);
   }
   __syncthreads();
+}
+
+// The same by one warp.
+__device__ __forceinline__ void prepare_warp(const PrepareArgs &a) {
+  const int lane = threadIdx.x & 31;
+  int carry = 0;
+  bool bad = false;
+  for (int b0 = 0; b0 < a.B; b0 += 32) {
+    const int b = b0 + lane;
+    SampleDesc d;
+    int len = 0;
+    if (b < a.B) {
+      d = make_desc(a, b);
+      if (d.valid) len = d.n - d.nv + a.keep_k;
+      else bad = true;
+    }
+    int inc = len;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int t = __shfl_up_sync(0xffffffffu, inc, o);
+      if (lane >= o) inc += t;
+    }
+    if (b < a.B) {
+      d.out_row0 = carry + inc - len;
+      a.desc[b] = d;
+      if (a.out_cu_seqlens) a.out_cu_seqlens[b] = d.out_row0;
+    }
+    carry += __shfl_sync(0xffffffffu, inc, 31);
+  }
+  if (a.out_cu_seqlens && lane == 0) a.out_cu_seqlens[a.B] = carry;
+  uint32_t bits = __any_sync(0xffffffffu, bad) ? STATUS_BAD_SAMPLE : 0u;
+  if (carry > a.out_capacity) {
+    bits |= STATUS_OUT_CAPACITY;
+    __syncwarp();
+    for (int b = lane; b < a.B; b += 32) a.desc[b].valid = 0;   // nothing may be written
+  }
+  if (bits && lane == 0) atomicOr(a.status, bits);
+  __syncwarp();
 }
 
 __global__ void prepare_kernel(PrepareArgs a) {
@@ -284,72 +322,6 @@ mass_salience_kernel(const __nv_bfloat16 *__restrict__ k, const SampleDesc *__re
 }
 
 // =======================================================================================
-// salience_from_heads: the tail of Eq. 1 and Eq. 2-3 when the per-head masses qbar^h . k_j^h were
-// produced elsewhere (by the score kernel, from the key tiles it streams anyway).  One block per
-// sample: s_j = scale * sum_h heads[b, h, j] (heads in order), then the min-max normalisation and
-// the mask vector over the image span; padding past the span is zeroed as mass_salience does.
-// =======================================================================================
-constexpr int SAL_THREADS = 1024;
-
-__global__ void __launch_bounds__(SAL_THREADS)
-salience_from_heads_kernel(const SampleDesc *__restrict__ desc, int H, int max_vis, float scale, float lambda_max,
-                           float eps, const float *__restrict__ heads /*[B, H, max_vis]*/, float *__restrict__ mass,
-                           float *__restrict__ salience, float *__restrict__ mask_log, float *__restrict__ rank_score) {
-  pdl_enter();
-  __shared__ float s_red[2 * (SAL_THREADS / 32)];
-  const int b = blockIdx.x;
-  const SampleDesc d = desc[b];
-  float *mass_b = mass + (size_t)b * max_vis, *sal_b = salience + (size_t)b * max_vis, *msk_b = mask_log + (size_t)b * max_vis;
-  if (!d.valid) {
-    for (int j = threadIdx.x; j < max_vis; j += SAL_THREADS) {
-      mass_b[j] = 0.f; sal_b[j] = 0.f; msk_b[j] = 0.f;
-      rank_score[(size_t)b * max_vis + j] = 0.f;       // the score and selection kernels skip the sample
-    }
-    return;
-  }
-  const float *hb = heads + (size_t)b * H * max_vis;
-  float lo = INFINITY, hi = -INFINITY;
-  for (int j = threadIdx.x; j < d.nv; j += SAL_THREADS) {
-    float tot = 0.f;
-    int hh = 0;
-    for (; hh + 8 <= H; hh += 8) {            // eight loads in flight
-      float v[8];
-#pragma unroll
-      for (int e = 0; e < 8; ++e) v[e] = __ldcg(hb + (size_t)(hh + e) * max_vis + j);
-#pragma unroll
-      for (int e = 0; e < 8; ++e) tot += v[e];
-    }
-    for (; hh < H; ++hh) tot += __ldcg(hb + (size_t)hh * max_vis + j);
-    tot *= scale;
-    mass_b[j] = tot;
-    lo = fminf(lo, tot); hi = fmaxf(hi, tot);
-  }
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    lo = fminf(lo, __shfl_xor_sync(0xffffffffu, lo, o));
-    hi = fmaxf(hi, __shfl_xor_sync(0xffffffffu, hi, o));
-  }
-  if (lane == 0) { s_red[warp] = lo; s_red[SAL_THREADS / 32 + warp] = hi; }
-  __syncthreads();
-  lo = s_red[0]; hi = s_red[SAL_THREADS / 32];
-#pragma unroll
-  for (int w = 1; w < SAL_THREADS / 32; ++w) {
-    lo = fminf(lo, s_red[w]); hi = fmaxf(hi, s_red[SAL_THREADS / 32 + w]);
-  }
-  const float inv = 1.0f / ((hi - lo) + eps);
-  for (int j = threadIdx.x; j < max_vis; j += SAL_THREADS) {
-    if (j < d.nv) {
-      const float sh = (mass_b[j] - lo) * inv;      // this thread's own store above
-      sal_b[j] = sh;
-      msk_b[j] = logf(fmaxf(lambda_max * sh, eps));
-    } else {
-      mass_b[j] = 0.f; sal_b[j] = 0.f; msk_b[j] = 0.f;
-    }
-  }
-}
-
-// =======================================================================================
 // mass_heads: Eq. 1-3 kept per head (the variant with one salience and one mask per head).
 //   s_j^h = qbar^h . k_j^h / sqrt(d): one warp per visual key row; a 16-byte vector of the row lies
 //   inside one head (16 vectors per head), so the two halves of the warp reduce two heads per pass.
@@ -473,6 +445,75 @@ mass_heads_kernel(const __nv_bfloat16 *__restrict__ k, const SampleDesc *__restr
 }
 
 // =======================================================================================
+// salience_block: the tail of Eq. 1 and Eq. 2-3 when the per-head masses qbar^h . k_j^h were
+// produced by the score kernel (from the query and key tiles it streams).  One block per sample, beside
+// the block that selects (grid y of the selection launch): s_j = scale * sum_h heads[b, h, j] (heads in order), then the min-max normalisation and
+// the mask vector over the image span; padding past the span is zeroed as mass_salience does.
+// =======================================================================================
+constexpr int SAL_THREADS = 1024;
+
+struct SalienceArgs {
+  int H;
+  float scale, lambda_max, eps;
+  const float *heads;                       // [B, H, max_vis]
+  float *mass, *salience, *mask_log, *rank_score;   // [B, max_vis]
+};
+
+__device__ __forceinline__ void salience_block(const SampleDesc &d, int b, int max_vis, const SalienceArgs &a) {
+  __shared__ float s_red[2 * (SAL_THREADS / 32)];
+  float *mass_b = a.mass + (size_t)b * max_vis, *sal_b = a.salience + (size_t)b * max_vis, *msk_b = a.mask_log + (size_t)b * max_vis;
+  const int H = a.H;
+  const float scale = a.scale, lambda_max = a.lambda_max, eps = a.eps;
+  if (!d.valid) {
+    for (int j = threadIdx.x; j < max_vis; j += SAL_THREADS) {
+      mass_b[j] = 0.f; sal_b[j] = 0.f; msk_b[j] = 0.f;
+      a.rank_score[(size_t)b * max_vis + j] = 0.f;     // the score kernel and the selection skip the sample
+    }
+    return;
+  }
+  const float *hb = a.heads + (size_t)b * H * max_vis;
+  float lo = INFINITY, hi = -INFINITY;
+  for (int j = threadIdx.x; j < d.nv; j += SAL_THREADS) {
+    float tot = 0.f;
+    int hh = 0;
+    for (; hh + 16 <= H; hh += 16) {          // sixteen loads in flight
+      float v[16];
+#pragma unroll
+      for (int e = 0; e < 16; ++e) v[e] = __ldcg(hb + (size_t)(hh + e) * max_vis + j);
+#pragma unroll
+      for (int e = 0; e < 16; ++e) tot += v[e];
+    }
+    for (; hh < H; ++hh) tot += __ldcg(hb + (size_t)hh * max_vis + j);
+    tot *= scale;
+    mass_b[j] = tot;
+    lo = fminf(lo, tot); hi = fmaxf(hi, tot);
+  }
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    lo = fminf(lo, __shfl_xor_sync(0xffffffffu, lo, o));
+    hi = fmaxf(hi, __shfl_xor_sync(0xffffffffu, hi, o));
+  }
+  if (lane == 0) { s_red[warp] = lo; s_red[SAL_THREADS / 32 + warp] = hi; }
+  __syncthreads();
+  lo = s_red[0]; hi = s_red[SAL_THREADS / 32];
+#pragma unroll
+  for (int w = 1; w < SAL_THREADS / 32; ++w) {
+    lo = fminf(lo, s_red[w]); hi = fmaxf(hi, s_red[SAL_THREADS / 32 + w]);
+  }
+  const float inv = 1.0f / ((hi - lo) + eps);
+  for (int j = threadIdx.x; j < max_vis; j += SAL_THREADS) {
+    if (j < d.nv) {
+      const float sh = (mass_b[j] - lo) * inv;      // this thread's own store above
+      sal_b[j] = sh;
+      msk_b[j] = logf(fmaxf(lambda_max * sh, eps));
+    } else {
+      mass_b[j] = 0.f; sal_b[j] = 0.f; msk_b[j] = 0.f;
+    }
+  }
+}
+
+// =======================================================================================
 // select: exact top-k by radix select over order-preserving 32-bit keys, equal scores resolved
 // toward the lower index, outputs in ascending index order.  One block per sample.
 // =======================================================================================
@@ -519,8 +560,13 @@ select_kernel(const float *__restrict__ rank_score, const SampleDesc *__restrict
               int32_t *__restrict__ role /*[B, max_vis]*/, int32_t *__restrict__ assign /*nullable*/,
               float *__restrict__ best_sim /*nullable*/, int sim_follows,
               const float *__restrict__ head_partial /*nullable: [B, H, max_vis]*/, int H,
-              float *__restrict__ rank_out /*[B, max_vis], written when head_partial is given*/) {
+              float *__restrict__ rank_out /*[B, max_vis], written when head_partial is given*/,
+              SalienceArgs sal /* blockIdx.y == 1 */) {
   pdl_enter();
+  if (blockIdx.y == 1) {
+    salience_block(desc[blockIdx.x], blockIdx.x, max_vis, sal);
+    return;
+  }
   extern __shared__ uint32_t s_key[];   // [max_vis]
   __shared__ int s_hist[256];
   __shared__ int s_scan[33];

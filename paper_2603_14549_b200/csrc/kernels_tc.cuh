@@ -51,15 +51,17 @@ __device__ __forceinline__ void group_bar_sync(int group) {
 // Additive mask (Eq. 3), logits in log2 units: 0 for key j <= row position p; m_j*log2(e) for
 // j > p when both are in the image span (mask enabled); -inf otherwise.
 // The per-head sums over ranking rows go to `partial`; head_sum_kernel adds them in head order.
-// Attention mass on the way (a.qbar given; ranking rows after the image span): Eq. 1 with the sum over
+// Attention mass on the way (a.mass_heads given; ranking rows after the image span): Eq. 1 with the sum over
 // the queries taken first is qbar^h . k_j^h, and pass 2 already multiplies every visual key tile by the
-// row pair's queries.  The summed query rides along as three more "query rows" (its bf16 value, the bf16
-// value of what that rounding lost, and again: 24 bits of mantissa together, all that fp32 holds),
-// written behind the pair's rows in shared memory, so the first row pair's pass-2 accumulators get three
+// row pair's queries.  The visual queries stream through the same ring, one tile behind every key tile of pass 1; two warps of
+// their own add them up (the pipes that bound the kernel are the exponentials' and the epilogue's: memory, shared memory and
+// issue slots have room) and write the sum as three more "query rows" (its bf16 value, the bf16
+// value of what that rounding lost, and again: 24 bits of mantissa together, all that fp32 holds)
+// behind the pair's rows in shared memory, so the first row pair's pass-2 accumulators get three
 // more columns whose sum is the key's mass for this head.  Row pairs then hold at most 240 rows (the
 // accumulator grows by the 16 columns an MMA's width moves in).
 // =======================================================================================
-constexpr int SC_THREADS = 320;          // producer warp, MMA warp, 2 x 4 epilogue warps
+constexpr int SC_THREADS = 384;          // producer warp, MMA warp, 2 x 4 epilogue warps, two query-sum warps
 constexpr int SC_EPI_THREADS = 256;
 constexpr int SC_STAGES = 4;
 constexpr int SC_HALF_BYTES = 128 * 128;        // 128 rows x 64 bf16
@@ -83,10 +85,9 @@ struct ScoreArgs {
   const float *mask_log;      // [B, max_vis] m_j (natural log), or [B, H, max_vis] with a mask per head
   int mask_b_stride, mask_h_stride;   // max_vis, 0   or   H * max_vis, max_vis
   float *partial;             // [B, H, max_vis] per-head sums over ranking rows
-  const float *qbar;          // [B, D] sum of the visual queries (Eq. 1, queries first), or nullptr.  Given: the
-                              // kernel also writes mass_heads (the attention mass per head), see below
-  float *mass_heads;          // [B, H, max_vis] qbar^h . k_j^h for every visual key j (unscaled)
-  int D;
+  float *mass_heads;          // [B, H, max_vis] qbar^h . k_j^h for every visual key j (unscaled), qbar^h the sum of the visual
+                              // queries (Eq. 1, queries first); nullptr: not wanted.  Given: the kernel also
+                              // validates the batch and writes the descriptors (pa.write_desc)
   unsigned int *work;         // [2] next item / blocks that have finished; both zero between launches
   uint32_t *status;
   long long wait_limit;       // clock cycles a wait may take before the block gives up
@@ -94,7 +95,7 @@ struct ScoreArgs {
 
 struct ScoreBook {             // bookkeeping block placed after the tiles in shared memory
   uint64_t full[SC_STAGES], empty[SC_STAGES], q_full, q_empty, acc_full[4], acc_empty[4];
-  uint64_t item_full[SC_ITEM_SLOTS], item_empty[SC_ITEM_SLOTS], mma_done, qbar_ready;
+  uint64_t item_full[SC_ITEM_SLOTS], item_empty[SC_ITEM_SLOTS], mma_done, qbar_ready, qt_full[2];
   int item_q[SC_ITEM_SLOTS];   // items drawn by the producer, -1 = no more
   alignas(16) float noff[256]; // per ranking row of the pair: -(max + log2(sum)), -inf for rows past its end
                                // (with one row tile, noff[128..255] carries group 1's partial sums)
@@ -136,7 +137,7 @@ score_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
   const int n_items = a.B * a.H;
-  const bool with_mass = a.qbar != nullptr;
+  const bool with_mass = a.mass_heads != nullptr;
   const int pair_rows = with_mass ? 240 : 256;           // ranking rows per row pair
 
   const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
@@ -153,7 +154,7 @@ score_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__
   if (threadIdx.x == 0) {
     for (int s = 0; s < SC_STAGES; ++s) {
       mbar_init(smem_u32(&bk->full[s]), 1);
-      mbar_init(smem_u32(&bk->empty[s]), 1);
+      mbar_init(smem_u32(&bk->empty[s]), 2);             // a key tile: the MMAs and their issuer; a query tile: the sum warps
     }
     mbar_init(smem_u32(&bk->q_full), 1);
     mbar_init(smem_u32(&bk->q_empty), 1);
@@ -163,10 +164,11 @@ score_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__
     }
     for (int i = 0; i < SC_ITEM_SLOTS; ++i) {
       mbar_init(smem_u32(&bk->item_full[i]), 1);
-      mbar_init(smem_u32(&bk->item_empty[i]), 9);         // the MMA issuer + every epilogue warp
+      mbar_init(smem_u32(&bk->item_empty[i]), with_mass ? 11 : 9);   // the MMA issuer, every epilogue warp (and the sum warps)
     }
     mbar_init(smem_u32(&bk->mma_done), 1);
-    mbar_init(smem_u32(&bk->qbar_ready), 1);
+    mbar_init(smem_u32(&bk->qbar_ready), 2);
+    for (int i = 0; i < 2; ++i) mbar_init(smem_u32(&bk->qt_full[i]), 1);
     bk->abort_flag = 0;
     fence_barrier_init();
   }
@@ -192,6 +194,7 @@ score_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__
       tma_prefetch_desc(&tmap_k);
     }
     int kc = 0, qc = 0, ic = 0;               // key tiles / row pairs / items so far
+    int qt = 0;                               // query tiles issued for the sum warps
     int k_issued = 0, q_issued = 0;           // copies actually issued (an abort is sticky, so
                                               // these are prefixes of the two sequences)
     while (true) {
@@ -228,17 +231,31 @@ score_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__
                             h * 128 + hf * 64, d.row0 + T.R0 + rt * 128, leader);
           q_issued = qc + 1;
         }
-        for (int u = 0; u < T.n_kt + T.n_p2; ++u, ++kc) {
-          const int t = u < T.n_kt ? u : T.t_hi - (u - T.n_kt);
+        const int nq = with_mass && rp == 0 ? (d.nv + 127) / 128 : 0;      // tiles of visual queries (never more than n_kt)
+        // A query tile lands on a barrier of its own (alternating: the sum warps see only these, in order, so they cannot
+        // mistake a ring slot's phase; two query tiles are never in flight on the same one, see below) and its slot's
+        // barrier is passed at once, which keeps that barrier's phases in step with the ring.
+        auto load_tile = [&](bool query, int row) {
           const int s = kc % SC_STAGES;
           if (kc >= SC_STAGES) mbar_wait_warp(smem_u32(&bk->empty[s]), ((kc / SC_STAGES) - 1) & 1, wc);
           if (!__shfl_sync(0xffffffffu, bk->abort_flag, 0)) {
             const uint32_t dst = k_smem + s * SC_TILE_BYTES;
-            mbar_expect_tx_w(smem_u32(&bk->full[s]), SC_TILE_BYTES, leader);
-            tma_load_2d_w(dst, &tmap_k, smem_u32(&bk->full[s]), h * 128, d.row0 + t * 128, leader);
-            tma_load_2d_w(dst + SC_HALF_BYTES, &tmap_k, smem_u32(&bk->full[s]), h * 128 + 64, d.row0 + t * 128, leader);
+            const uint32_t bar = smem_u32(query ? &bk->qt_full[qt & 1] : &bk->full[s]);
+            const CUtensorMap *map = query ? &tmap_q : &tmap_k;
+            mbar_expect_tx_w(bar, SC_TILE_BYTES, leader);
+            tma_load_2d_w(dst, map, bar, h * 128, row, leader);
+            tma_load_2d_w(dst + SC_HALF_BYTES, map, bar, h * 128 + 64, row, leader);
+            if (query && leader) mbar_arrive(smem_u32(&bk->full[s]));
+            if (query) ++qt;
             k_issued = kc + 1;
           }
+          ++kc;
+        };
+        for (int u = 0; u < T.n_kt + T.n_p2; ++u) {
+          load_tile(false, d.row0 + (u < T.n_kt ? u : T.t_hi - (u - T.n_kt)) * 128);
+          // (query tiles are two ring positions apart, so the one after the next takes the slot of this one, whose
+          // release says that it has been added up; between two items at least four other tiles pass)
+          if (u < nq) load_tile(true, d.row0 + d.v0 + u * 128);
         }
       }
     }
@@ -248,6 +265,8 @@ score_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__
       if (fills > 0) mbar_wait_drain(smem_u32(&bk->full[s]), (fills - 1) & 1, TC_WAIT_LIMIT);
     }
     if (q_issued > 0) mbar_wait_drain(smem_u32(&bk->q_full), (q_issued - 1) & 1, TC_WAIT_LIMIT);
+    for (int i = 0; i < 2; ++i)
+      if (qt > i) mbar_wait_drain(smem_u32(&bk->qt_full[i]), (((qt - 1 - i) >> 1) & 1), TC_WAIT_LIMIT);
     __syncwarp();
   } else if (warp == 1) {
     // ------------------------------------------------------------------ MMA issuer
@@ -287,7 +306,8 @@ score_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__
           tc_fence_after();
           return buf;
         };
-        for (int u = 0; u < T.n_kt + T.n_p2; ++u, ++kc) {
+        const int nq = mass_here ? (d.nv + 127) / 128 : 0;    // every key tile below nq is followed by a query tile (the sum warps')
+        for (int u = 0; u < T.n_kt + T.n_p2; kc += u < nq ? 2 : 1, ++u) {
           const int s = kc % SC_STAGES;
           if (mass_here && u == T.n_kt) {                    // an epilogue warp has written the summed-query rows
             mbar_wait_warp(smem_u32(&bk->qbar_ready), mc & 1, wc);
@@ -310,6 +330,7 @@ score_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__
             }
           }
           tc_commit_w(smem_u32(&bk->empty[s]), leader);
+          if (leader) mbar_arrive(smem_u32(&bk->empty[s]));
         }
         if (mass_here && T.n_p2 == 0) {                      // (no visual key tile: keep the barrier's phases in step)
           mbar_wait_warp(smem_u32(&bk->qbar_ready), mc & 1, wc);
@@ -323,7 +344,7 @@ score_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__
     tc_commit_w(smem_u32(&bk->mma_done), leader);
     mbar_wait_drain(smem_u32(&bk->mma_done), 0, TC_WAIT_LIMIT);
     __syncwarp();
-  } else {
+  } else if (warp < 10) {
     // ------------------------------------------------------------------ epilogue (2 groups x 4 warps)
     // Warp q of a group reads tensor-memory lanes 32q .. 32q+31.
     const int group = (warp - 2) >> 2;
@@ -361,42 +382,6 @@ score_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__
       }
       for (int rp = 0; rp < n_rp; ++rp, ++qc) {
         const RowPair T = score_row_pair(d, rp, a.mask_enable, pair_rows);
-        if (with_mass && rp == 0 && warp == 2) {
-          // The summed query of this head as rows n2 .. n2 + 2 of the pair's query tile: 3 rows x 16 chunks
-          // of 16 bytes at their swizzled places (row r of a 64-column half is 128 bytes at
-          // r * 128, chunk c at c ^ (r & 7)), once the tiled copy of the queries has landed.
-          mbar_wait(smem_u32(&bk->q_full), qc & 1, wc);
-          const int c16 = lane & 15;
-          const float *src = a.qbar + (size_t)b * a.D + h * 128 + c16 * 8;
-          uint32_t w[3][4];                                 // the value as three bf16 pieces: 24 bits of mantissa, all of fp32's
-#pragma unroll
-          for (int e = 0; e < 4; ++e) {
-            float x[2] = {__ldcg(src + 2 * e), __ldcg(src + 2 * e + 1)}, piece[3][2];
-#pragma unroll
-            for (int t = 0; t < 2; ++t) {
-              float rest = x[t];
-#pragma unroll
-              for (int k = 0; k < 3; ++k) {
-                piece[k][t] = __bfloat162float(__float2bfloat16_rn(rest));
-                rest -= piece[k][t];
-              }
-            }
-#pragma unroll
-            for (int k = 0; k < 3; ++k) w[k][e] = pack2_rn(piece[k][0], piece[k][1]);
-          }
-          // lanes 0-15 write the first piece's row and the third's, lanes 16-31 the second's
-#pragma unroll
-          for (int k = 0; k < 3; ++k) {
-            if ((k == 1) == (lane >= 16)) {
-              const int row = T.n2 + k;
-              uint8_t *dst = base_ptr + (c16 >> 3) * SC_Q_HALF_BYTES + row * 128 + (((c16 & 7) ^ (row & 7)) << 4);
-              *reinterpret_cast<uint4 *>(dst) = make_uint4(w[k][0], w[k][1], w[k][2], w[k][3]);
-            }
-          }
-          fence_proxy_async();
-          __syncwarp();
-          if (lane == 0) mbar_arrive(smem_u32(&bk->qbar_ready));
-        }
         // ---------------- pass 1: thread = ranking row.  Two row tiles: group g owns tile g of every key
         // tile; one row tile: the groups take alternate key tiles
         const bool two = T.nrt == 2;
@@ -607,6 +592,85 @@ score_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__
       }
     }
     __threadfence();
+  } else if (with_mass) {
+    // ------------------------------------------------------------------ query-sum warps: one 64-column half of the head each
+    if (warp == 11 && blockIdx.x == 0 && a.pa.write_desc) prepare_warp(a.pa);
+    const int half = warp - 10;
+    const int c = lane & 7, r0 = lane >> 3;        // a lane adds 16-byte chunk c of rows r0, r0 + 4, ...
+    int kc = 0, qc = 0, qt = 0;                    // ring positions, row pairs, query tiles so far
+    for (int ic = 0;; ++ic) {
+      const int slot = ic % SC_ITEM_SLOTS;
+      const bool got = mbar_wait_drain(smem_u32(&bk->item_full[slot]), (ic / SC_ITEM_SLOTS) & 1, TC_WAIT_LIMIT);
+      __syncwarp();
+      const int item = __shfl_sync(0xffffffffu, got ? bk->item_q[slot] : -1, 0);
+      if (lane == 0) mbar_arrive(smem_u32(&bk->item_empty[slot]));
+      if (item < 0) break;
+      const SampleDesc d = make_desc(a.pa, item / a.H);
+      if (!d.valid) continue;
+      const int n_rp = (d.nr + pair_rows - 1) / pair_rows;
+      for (int rp = 0; rp < n_rp; ++rp, ++qc) {
+        const RowPair T = score_row_pair(d, rp, a.mask_enable, pair_rows);
+        if (rp == 0) {
+          const int nq = (d.nv + 127) / 128;
+          uint64_t acc[4] = {0ull, 0ull, 0ull, 0ull};
+          for (int u = 0; u < nq; ++u, ++qt) {
+            const int s = (kc + 2 * u + 1) % SC_STAGES;
+            mbar_wait_warp(smem_u32(&bk->qt_full[qt & 1]), (qt >> 1) & 1, wc);
+            const uint8_t *tile = base_ptr + SC_Q_BYTES + s * SC_TILE_BYTES + half * SC_HALF_BYTES;
+            const int rows = min(128, d.nv - u * 128);
+#pragma unroll 8
+            for (int r = r0; r < rows; r += 4) {
+              const uint4 x = *reinterpret_cast<const uint4 *>(tile + r * 128 + ((c ^ (r & 7)) << 4));
+              acc[0] = f2_add(acc[0], f2_pack(bf16_lo(x.x), bf16_hi(x.x)));
+              acc[1] = f2_add(acc[1], f2_pack(bf16_lo(x.y), bf16_hi(x.y)));
+              acc[2] = f2_add(acc[2], f2_pack(bf16_lo(x.z), bf16_hi(x.z)));
+              acc[3] = f2_add(acc[3], f2_pack(bf16_lo(x.w), bf16_hi(x.w)));
+            }
+            __syncwarp();
+            if (lane == 0) mbar_arrive(smem_u32(&bk->empty[s]));
+          }
+          float f[8];
+#pragma unroll
+          for (int e = 0; e < 4; ++e) f2_unpack(acc[e], f[2 * e], f[2 * e + 1]);
+#pragma unroll
+          for (int e = 0; e < 8; ++e) {
+            f[e] += __shfl_xor_sync(0xffffffffu, f[e], 8);
+            f[e] += __shfl_xor_sync(0xffffffffu, f[e], 16);
+          }
+          // The summed query of this head as rows n2 .. n2 + 2 of the pair's query tile (row r of a 64-column half is 128
+          // bytes at r * 128, chunk c at c ^ (r & 7)), once the tiled copy of the queries has landed: the value as three
+          // bf16 pieces, 24 bits of mantissa, all of fp32's.  Lanes 8 k .. 8 k + 7 write piece k.
+          mbar_wait_warp(smem_u32(&bk->q_full), qc & 1, wc);
+          if (r0 < 3) {
+            uint32_t w[4];
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+              float piece[2];
+#pragma unroll
+              for (int t = 0; t < 2; ++t) {
+                float rest = f[2 * e + t];
+                piece[t] = 0.f;
+#pragma unroll
+                for (int k = 0; k < 3; ++k) {
+                  const float q = __bfloat162float(__float2bfloat16_rn(rest));
+                  if (k == r0) piece[t] = q;
+                  rest -= q;
+                }
+              }
+              w[e] = pack2_rn(piece[0], piece[1]);
+            }
+            const int row = T.n2 + r0;
+            *reinterpret_cast<uint4 *>(base_ptr + half * SC_Q_HALF_BYTES + row * 128 + ((c ^ (row & 7)) << 4)) =
+                make_uint4(w[0], w[1], w[2], w[3]);
+          }
+          fence_proxy_async();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(smem_u32(&bk->qbar_ready));
+          kc += nq;
+        }
+        kc += T.n_kt + T.n_p2;
+      }
+    }
   }
 
   // ---------------------------------------------------------------------- teardown

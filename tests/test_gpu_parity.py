@@ -49,6 +49,20 @@ def test_two_slot_tiles_in_one_pass(ctx, k):
     run_step(ctx, batch, A.Params(keep_k=k))
 
 
+@pytest.mark.parametrize("nvs,texts,H", [([128, 129, 9], [240, 241, 500], 2), ([64, 300, 20] * 14, [5, 250, 1] * 14, 8)],
+                         ids=["tile_edges", "many_items_per_block"])
+def test_query_sums_inside_the_score_kernel(ctx, nvs, texts, H):
+    """The visual queries are added up beside the key tiles: spans that end on a tile edge, one past it and inside
+    the first tile; ranking rows of one, two and three row pairs (only the first carries the masses); and more
+    (sequence, head) items than blocks, so that ring positions run on from one item to the next."""
+    batch = W.tiny(B=len(nvs), n_vis=nvs, text_lens=texts, H=H, keep_k=8, seed=140 + H, centres=6)
+    big = A.asap_init(0, max_total_tokens=batch.total + len(nvs) * 300, max_B=len(nvs), max_H=H, max_D=H * 128)
+    try:
+        run_step(big, batch, A.Params(keep_k=8), samples=range(len(nvs)) if len(nvs) < 4 else [0, 1, 2, len(nvs) - 1])
+    finally:
+        A.asap_free(big)
+
+
 @pytest.mark.parametrize("nvs,k", [([1028, 1029], 4), ([2500, 1030], 3), ([40, 16], 16), ([2060], 7)],
                          ids=["one_pass", "three_passes", "nothing_dropped", "three_passes_one"])
 def test_merge_blocks_that_scan_for_their_members(ctx, nvs, k):
