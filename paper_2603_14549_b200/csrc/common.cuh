@@ -236,6 +236,26 @@ __device__ __forceinline__ void tma_load_2d_w(uint32_t smem_dst, const void *tma
       ::"r"(smem_dst), "l"(tmap), "r"(bar), "r"(x), "r"(y), "r"(leader)
       : "memory");
 }
+// ... with an L2 eviction policy (l2_evict_first / l2_evict_normal)
+__device__ __forceinline__ void tma_load_2d_hint_w(uint32_t smem_dst, const void *tmap, uint32_t bar, int32_t x, int32_t y,
+                                                   uint64_t policy, uint32_t leader) {
+  asm volatile(
+      "{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %5, 0;\n\t"
+      "@q cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint "
+      "[%0], [%1, {%3, %4}], [%2], %6;\n\t}"
+      ::"r"(smem_dst), "l"(tmap), "r"(bar), "r"(x), "r"(y), "r"(leader), "l"(policy)
+      : "memory");
+}
+__device__ __forceinline__ uint64_t l2_evict_first() {
+  uint64_t p;
+  asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(p));
+  return p;
+}
+__device__ __forceinline__ uint64_t l2_evict_normal() {
+  uint64_t p;
+  asm volatile("createpolicy.fractional.L2::evict_normal.b64 %0, 1.0;" : "=l"(p));
+  return p;
+}
 __device__ __forceinline__ void mbar_expect_tx_w(uint32_t bar, uint32_t bytes, uint32_t leader) {
   asm volatile(
       "{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %2, 0;\n\t"
