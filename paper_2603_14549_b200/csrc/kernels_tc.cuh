@@ -532,42 +532,56 @@ score_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__
             mbar_wait(smem_u32(&bk->acc_full[buf]), (ops >> 1) & 1, wc);
             tc_fence_after();
             if (warp_keys && !bk->abort_flag) {
-              const int n_here = min(128, T.n2 - h0);
-#pragma unroll 1
-              for (int c = 0; c < n_here; c += 32) {
-                uint32_t r[32];
-                if (c + 32 <= n_here) tmem_ld32p(tlane + c, r);
-                else {                                // n2 is a multiple of 16: the last chunk may be half
-                  tmem_ld16p(tlane + c, r);
+              const int n_here = min(128, T.n2 - h0);       // (a multiple of 16)
+              // rows past the pair's end have the offset -inf (every entry up to the next multiple of 128 is
+              // written), so their terms vanish; four offsets per shared-memory load
+              auto add32 = [&](const uint32_t (&r)[32], int c) {
 #pragma unroll
-                  for (int e = 16; e < 32; ++e) r[e] = 0u;
+                for (int e = 0; e < 32; e += 4) {
+                  const ulonglong2 o = *reinterpret_cast<const ulonglong2 *>(bk->noff + h0 + c + e);
+                  float x0, x1, x2, x3;
+                  f2_unpack(f2_fma(f2_pack(__uint_as_float(r[e]), __uint_as_float(r[e + 1])), scale2, o.x), x0, x1);
+                  f2_unpack(f2_fma(f2_pack(__uint_as_float(r[e + 2]), __uint_as_float(r[e + 3])), scale2, o.y), x2, x3);
+                  sm2[(e >> 1) & 3] = f2_add(sm2[(e >> 1) & 3], f2_pack(fast_exp2(x0), fast_exp2(x1)));
+                  sm2[((e >> 1) + 1) & 3] = f2_add(sm2[((e >> 1) + 1) & 3], f2_pack(fast_exp2(x2), fast_exp2(x3)));
                 }
+              };
+              int c = 0;
+              if (fast && n_here >= 32) {
+                // the next 32 columns are on their way while these are exponentiated
+                const int last = (n_here & ~31) - 32;
+                uint32_t ra[32], rb[32];
+                tmem_ld32(tlane, ra);
                 tmem_wait_ld();
-                // rows past the pair's end have the offset -inf (every entry up to the next multiple of 128 is
-                // written), so their terms vanish; four offsets per shared-memory load
-                if (fast) {
-#pragma unroll
-                  for (int e = 0; e < 32; e += 4) {
-                    const ulonglong2 o = *reinterpret_cast<const ulonglong2 *>(bk->noff + h0 + c + e);
-                    float x0, x1, x2, x3;
-                    f2_unpack(f2_fma(f2_pack(__uint_as_float(r[e]), __uint_as_float(r[e + 1])), scale2, o.x), x0, x1);
-                    f2_unpack(f2_fma(f2_pack(__uint_as_float(r[e + 2]), __uint_as_float(r[e + 3])), scale2, o.y), x2, x3);
-                    sm2[(e >> 1) & 3] = f2_add(sm2[(e >> 1) & 3], f2_pack(fast_exp2(x0), fast_exp2(x1)));
-                    sm2[((e >> 1) + 1) & 3] = f2_add(sm2[((e >> 1) + 1) & 3], f2_pack(fast_exp2(x2), fast_exp2(x3)));
+#pragma unroll 1
+                for (; c <= last; c += 64) {
+                  if (c < last) tmem_ld32(tlane + c + 32, rb);
+                  add32(ra, c);
+                  tmem_wait_ld();
+                  if (c < last) {
+                    if (c + 32 < last) tmem_ld32(tlane + c + 64, ra);
+                    add32(rb, c + 32);
+                    tmem_wait_ld();
                   }
-                } else {
+                }
+                c = last + 32;
+              }
+#pragma unroll 1
+              for (; c < n_here; c += 16) {
+                uint32_t r[16];
+                tmem_ld16(tlane + c, r);
+                tmem_wait_ld();
 #pragma unroll
-                  for (int e = 0; e < 32; e += 2) {
-                    const float2 o = *reinterpret_cast<const float2 *>(bk->noff + h0 + c + e);
-                    float x[2];
+                for (int e = 0; e < 16; e += 2) {
+                  const float2 o = *reinterpret_cast<const float2 *>(bk->noff + h0 + c + e);
+                  float x[2];
 #pragma unroll
-                    for (int k = 0; k < 2; ++k) {
-                      const int p = T.R0 + h0 + c + e + k;
-                      const float above = (p >= d.v0 && p < v_end) ? soft_j : -INFINITY;
-                      x[k] = fast_exp2(fmaf(__uint_as_float(r[e + k]), scale, (j <= p) ? 0.f : above) + (k ? o.y : o.x));
-                    }
-                    sm2[(e >> 1) & 3] = f2_add(sm2[(e >> 1) & 3], f2_pack(x[0], x[1]));
+                  for (int k = 0; k < 2; ++k) {
+                    const int p = T.R0 + h0 + c + e + k;
+                    const float above = (p >= d.v0 && p < v_end) ? soft_j : -INFINITY;
+                    x[k] = fast_exp2(fmaf(__uint_as_float(r[e + k]), scale, (j <= p) ? 0.f : above) + (k ? o.y : o.x));
                   }
+                  sm2[(e >> 1) & 3] = f2_add(sm2[(e >> 1) & 3], f2_pack(x[0], x[1]));
                 }
               }
               if (with_mass && rp == 0 && T.n2 - h0 >= 0 && T.n2 - h0 < 128) {
