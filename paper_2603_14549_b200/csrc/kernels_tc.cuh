@@ -409,86 +409,76 @@ score_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__
           mbar_wait(smem_u32(&bk->acc_full[buf]), (ops >> 1) & 1, wc);
           tc_fence_after();
           if (warp_rows && !bk->abort_flag) {
-#pragma unroll 1
-            for (int c = 0; c < 128; c += 64) {
-              uint32_t r[64];
-              tmem_ld32p(tlane + c, r);
-              tmem_ld32p(tlane + c + 32, r + 32);
-              tmem_wait_ld();
-              bool summed = false;
-              if (fast && m > -INFINITY) {
-                // every key admitted, no mask, and the row already has a reference maximum: add
-                // exp2(dot * scale - m) without looking for a new maximum (a stale reference only scales
-                // the sum; off_i = m + log2(l) comes out the same).  Should a term outgrow fp32's range
-                // the chunk is done again below, with its true maximum as the new reference.
-                const uint64_t negm2 = f2_pack(-m, -m);
-                uint64_t sm2[4] = {0ull, 0ull, 0ull, 0ull};
+            bool summed = false;
+            if (fast && __all_sync(0xffffffffu, !row_ok || m > -INFINITY)) {
+              // every key admitted, no mask, and the rows already have a reference maximum: add
+              // exp2(dot * scale - m) without looking for a new maximum (a stale reference only scales
+              // the sum; off_i = m + log2(l) comes out the same), the next 32 columns on their way meanwhile.  Should a
+              // row's sum outgrow fp32's range the tile is done again below, with true maxima as new references.
+              const float neg_m = row_ok ? -m : 0.f;
+              const uint64_t negm2 = f2_pack(neg_m, neg_m);
+              uint64_t sm2[4] = {0ull, 0ull, 0ull, 0ull};
+              auto add32 = [&](const uint32_t (&r)[32]) {
 #pragma unroll
-                for (int e = 0; e < 64; e += 2) {
+                for (int e = 0; e < 32; e += 2) {
                   float x0, x1;
                   f2_unpack(f2_fma(f2_pack(__uint_as_float(r[e]), __uint_as_float(r[e + 1])), scale2, negm2), x0, x1);
                   sm2[(e >> 1) & 3] = f2_add(sm2[(e >> 1) & 3], f2_pack(fast_exp2(x0), fast_exp2(x1)));
                 }
-                float cs, c1;
-                f2_unpack(f2_add(f2_add(sm2[0], sm2[1]), f2_add(sm2[2], sm2[3])), cs, c1);
-                cs += c1;
-                if (cs < 1e30f) {
-                  if (row_ok) l += cs;
-                  summed = true;
-                }
+              };
+              uint32_t ra[32], rb[32];
+              tmem_ld32(tlane, ra);
+              tmem_wait_ld();
+#pragma unroll 1
+              for (int c = 0; c < 128; c += 64) {
+                tmem_ld32(tlane + c + 32, rb);
+                add32(ra);
+                tmem_wait_ld();
+                if (c == 0) tmem_ld32(tlane + 64, ra);
+                add32(rb);
+                tmem_wait_ld();
               }
-              if (summed) {
-              } else if (fast) {
-                // every key admitted, no mask: max on the raw dot products (scale > 0), then
-                // exp2(dot * scale - max) into eight independent partial sums
-                float mx[8];
+              float cs, c1;
+              f2_unpack(f2_add(f2_add(sm2[0], sm2[1]), f2_add(sm2[2], sm2[3])), cs, c1);
+              cs += c1;
+              if (!__any_sync(0xffffffffu, row_ok && !(cs < 1e30f))) {
+                if (row_ok) l += cs;
+                summed = true;
+              }
+            }
+#pragma unroll 1
+            for (int c = summed ? 128 : 0; c < 128; c += 32) {
+              // with a new maximum per chunk: the first tile of a row pair, tiles that cross a row's own position (selects only,
+              // no branches), and the rare second try.  `lim` = last column of this chunk the row may attend to without
+              // the soft mask
+              uint32_t r[32];
+              tmem_ld32(tlane + c, r);
+              tmem_wait_ld();
+              const int lim = p_i - (j0 + c);
+              float mx[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
+              if (!stage_soft) {
 #pragma unroll
-                for (int e = 0; e < 8; ++e) mx[e] = __uint_as_float(r[e]);
-#pragma unroll
-                for (int e = 8; e < 64; ++e) mx[e & 7] = fmaxf(mx[e & 7], __uint_as_float(r[e]));
-                const float cmax = fmaxf(fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3])),
-                                         fmaxf(fmaxf(mx[4], mx[5]), fmaxf(mx[6], mx[7])));
-                const float m_new = fmaxf(m, cmax * scale);
-                if (row_ok) {
-                  float sm[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-                  for (int e = 0; e < 64; ++e) sm[e & 7] += fast_exp2(fmaf(__uint_as_float(r[e]), scale, -m_new));
-                  l = l * fast_exp2(m - m_new) +
-                      (((sm[0] + sm[1]) + (sm[2] + sm[3])) + ((sm[4] + sm[5]) + (sm[6] + sm[7])));
-                  m = m_new;
+                for (int e = 0; e < 32; ++e) {
+                  const float x = (e <= lim) ? __uint_as_float(r[e]) * scale : -INFINITY;
+                  r[e] = __float_as_uint(x);
+                  mx[e & 3] = fmaxf(mx[e & 3], x);
                 }
               } else {
-                // tile that crosses a row's own position: selects only, no branches.  `lim` =
-                // last column of this chunk the row may attend to without the soft mask
-                const int lim = p_i - (j0 + c);
-                float mx[8] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY, -INFINITY, -INFINITY, -INFINITY, -INFINITY};
-                if (!stage_soft) {
 #pragma unroll
-                  for (int e = 0; e < 64; ++e) {
-                    const float x = (e <= lim) ? __uint_as_float(r[e]) * scale : -INFINITY;
-                    r[e] = __float_as_uint(x);
-                    mx[e & 7] = fmaxf(mx[e & 7], x);
-                  }
-                } else {
-#pragma unroll
-                  for (int e = 0; e < 64; ++e) {
-                    const float sv = row_vis ? soft[c + e] : -INFINITY;
-                    const float x = fmaf(__uint_as_float(r[e]), scale, (e <= lim) ? 0.f : sv);
-                    r[e] = __float_as_uint(x);
-                    mx[e & 7] = fmaxf(mx[e & 7], x);
-                  }
+                for (int e = 0; e < 32; ++e) {
+                  const float sv = row_vis ? soft[c + e] : -INFINITY;
+                  const float x = fmaf(__uint_as_float(r[e]), scale, (e <= lim) ? 0.f : sv);
+                  r[e] = __float_as_uint(x);
+                  mx[e & 3] = fmaxf(mx[e & 3], x);
                 }
-                const float cmax = fmaxf(fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3])),
-                                         fmaxf(fmaxf(mx[4], mx[5]), fmaxf(mx[6], mx[7])));
-                const float m_new = fmaxf(m, cmax);
-                if (row_ok && m_new > -INFINITY) {
-                  float sm[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+              }
+              const float m_new = fmaxf(m, fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3])));
+              if (row_ok && m_new > -INFINITY) {
+                float sm[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
-                  for (int e = 0; e < 64; ++e) sm[e & 7] += fast_exp2(__uint_as_float(r[e]) - m_new);
-                  l = l * fast_exp2(m - m_new) +
-                      (((sm[0] + sm[1]) + (sm[2] + sm[3])) + ((sm[4] + sm[5]) + (sm[6] + sm[7])));
-                  m = m_new;
-                }
+                for (int e = 0; e < 32; ++e) sm[e & 3] += fast_exp2(__uint_as_float(r[e]) - m_new);
+                l = l * fast_exp2(m - m_new) + ((sm[0] + sm[1]) + (sm[2] + sm[3]));
+                m = m_new;
               }
             }
           }
