@@ -44,7 +44,8 @@ struct asap_ctx {
         *kept_inv = nullptr;
   unsigned int *cnt_qsum = nullptr, *cnt_mass = nullptr, *cnt_score = nullptr, *cnt_sim = nullptr,
                *cnt_tiles = nullptr, *cnt_work = nullptr;
-  float *mass_partial = nullptr;    // [B, H, max_vis] per-head attention masses written by the score kernel
+  float *mass_partial = nullptr;    // [B, H, max_vis] per-head attention masses
+  float *head_norm = nullptr;       // [B, H, 2] minimum and 1 / range of a head's masses (per-head masks)
   long long sim_pair_min_blocks = 0;        // blocks from which the similarity takes two row tiles per block (0: half the SM count)
   int sim_pair_stages = 0;                  // stages of that form (0: what fits 192 KB)
   int sim_cluster = 1;                      // 0: sliced similarity launches add their partials through global memory
@@ -241,7 +242,7 @@ PrepareArgs prepare_args(asap_ctx *ctx, const asap_inputs *in, const asap_params
 asap_status launch_prepare(asap_ctx *ctx, const asap_inputs *in, const asap_params *p,
                            int32_t *out_cu, int out_capacity, cudaStream_t st) {
   mark(ctx, "prepare", st);
-  launch_pdl(prepare_kernel, dim3(1), dim3(256), 0, st, prepare_args(ctx, in, p, out_cu, out_capacity));
+  launch_pdl(prepare_kernel, dim3(1), dim3(32), 0, st, prepare_args(ctx, in, p, out_cu, out_capacity));
   return after_launch(ctx, "prepare");
 }
 
@@ -275,13 +276,16 @@ asap_status launch_mass(asap_ctx *ctx, const asap_inputs *in, const asap_params 
 
   const int row_blocks = (in->max_vis + MASS_ROWS - 1) / MASS_ROWS;
   if (p->per_head_mask) {
-    // the per-head masses go through the scratch the score kernel fills afterwards
+    // (the head means, which nothing before the merge needs, come later: beside the selection, or in asap_score at its end)
     mark(ctx, "mass_heads", st);
-    launch_pdl(mass_heads_kernel, dim3(row_blocks, B), dim3(MASS_THREADS), (size_t)(D + 2 * in->H) * sizeof(float), st,
+    launch_pdl(mass_heads_kernel, dim3(row_blocks, B), dim3(MASS_THREADS), (size_t)D * sizeof(float), st,
                static_cast<const __nv_bfloat16 *>(in->k), ctx->desc, D, in->H, in->max_vis,
-               1.0f / sqrtf((float)in->head_dim), p->lambda_max, p->eps, ctx->qbar, ctx->score_partial, out->mass,
-               out->salience, out->mask_log, out->mask_log_heads, out->rank_score, ctx->cnt_mass);
-    return after_launch(ctx, "mass_heads");
+               1.0f / sqrtf((float)in->head_dim), ctx->qbar, ctx->mass_partial);
+    ASAP_TRY(after_launch(ctx, "mass_heads"));
+    mark(ctx, "mask_heads", st);
+    launch_pdl(mask_heads_kernel, dim3(in->H, B), dim3(MASS_THREADS), 0, st, ctx->desc, in->H, in->max_vis, p->lambda_max, p->eps,
+               ctx->mass_partial, out->mask_log_heads, ctx->head_norm);
+    return after_launch(ctx, "mask_heads");
   }
   const float scale = 1.0f / ((float)in->H * sqrtf((float)in->head_dim));
   mark(ctx, "mass_salience", st);
@@ -335,15 +339,20 @@ bool merge_scans(const asap_ctx *ctx, const asap_inputs *in, const asap_params *
   return merging(in, p) && passes * p->keep_k * in->B <= 8LL * ctx->num_sms;
 }
 
+SalienceArgs salience_args(const asap_ctx *ctx, const asap_inputs *in, const asap_params *p, const asap_outputs *out) {
+  SalienceArgs a;
+  a.H = in->H; a.scale = 1.0f / ((float)in->H * sqrtf((float)in->head_dim)); a.lambda_max = p->lambda_max; a.eps = p->eps;
+  a.heads = ctx->mass_partial; a.norm = p->per_head_mask ? ctx->head_norm : nullptr; a.mass = out->mass; a.salience = out->salience;
+  a.mask_log = out->mask_log; a.rank_score = out->rank_score;
+  return a;
+}
+
 // `fused_head_sum`: the ranking scores are still per-head sums in scratch (the score kernel ran
 // without its head-sum kernel); the selection adds the heads itself and writes out->rank_score.
 asap_status launch_select(asap_ctx *ctx, const asap_inputs *in, const asap_params *p,
                           const float *rank_score, const asap_outputs *out, bool with_merge,
                           bool fused_head_sum, cudaStream_t st, bool with_salience = false) {
-  SalienceArgs sal;
-  sal.H = in->H; sal.scale = 1.0f / ((float)in->H * sqrtf((float)in->head_dim)); sal.lambda_max = p->lambda_max; sal.eps = p->eps;
-  sal.heads = ctx->mass_partial; sal.mass = out->mass; sal.salience = out->salience; sal.mask_log = out->mask_log;
-  sal.rank_score = out->rank_score;
+  const SalienceArgs sal = salience_args(ctx, in, p, out);
   mark(ctx, "select", st);
   launch_pdl(select_kernel, dim3(in->B, with_salience ? 2 : 1), dim3(SELECT_THREADS), (size_t)in->max_vis * sizeof(uint32_t), st,
              rank_score, ctx->desc, in->max_vis, p->keep_k, out->keep_idx, out->drop_idx, ctx->role,
@@ -726,6 +735,7 @@ asap_status asap_init(asap_ctx **ctx_out, int device, size_t max_total_tokens, i
   const size_t o_qbar = carve(Bc * Dc * sizeof(float));
   const size_t o_spart = carve(Hc * T * sizeof(float));
   const size_t o_mpart = carve(Hc * T * sizeof(float));
+  const size_t o_hnorm = carve(Bc * Hc * 2 * sizeof(float));
   const size_t o_inv = carve(T * sizeof(float));
   const size_t o_kinv = carve(max_keep_rows * sizeof(float));
   const size_t o_cnt = carve((Bc * col_blocks + 3 * Bc + 4) * sizeof(unsigned int));
@@ -752,6 +762,7 @@ asap_status asap_init(asap_ctx **ctx_out, int device, size_t max_total_tokens, i
   if (const char *env = getenv("ASAP_SIM_PAIR_MIN_BLOCKS")) ctx->sim_pair_min_blocks = atoll(env);
   if (const char *env = getenv("ASAP_SIM_PAIR_STAGES")) ctx->sim_pair_stages = atoi(env);
   if (const char *env = getenv("ASAP_SIM_CLUSTER")) ctx->sim_cluster = atoi(env);
+  ctx->head_norm = reinterpret_cast<float *>(ctx->arena + o_hnorm);
   ctx->inv_norm = reinterpret_cast<float *>(ctx->arena + o_inv);
   ctx->kept_inv = reinterpret_cast<float *>(ctx->arena + o_kinv);
   ctx->counters_off = o_cnt; ctx->counters_bytes = (Bc * col_blocks + 3 * Bc + 4) * sizeof(unsigned int);
@@ -813,7 +824,11 @@ asap_status asap_score(asap_ctx *ctx, const asap_inputs *in, const asap_params *
   ASAP_TRY(validate(ctx, in, p, out, NEED_QK | NEED_SCORE_OUT));
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   ASAP_TRY(launch_mass(ctx, in, p, out, true, nullptr, 0x7fffffff, st));
-  return finish(ctx, launch_rank(ctx, in, p, out, true, st), st);
+  ASAP_TRY(launch_rank(ctx, in, p, out, true, st));
+  if (!p->per_head_mask) return finish(ctx, ASAP_OK, st);
+  mark(ctx, "salience_heads", st);
+  launch_pdl(salience_heads_kernel, dim3(in->B), dim3(MASS_THREADS), 0, st, ctx->desc, in->max_vis, salience_args(ctx, in, p, out));
+  return finish(ctx, after_launch(ctx, "salience_heads"), st);
 }
 
 asap_status asap_select(asap_ctx *ctx, const asap_inputs *in, const asap_params *p, const float *rank_score,
@@ -918,7 +933,7 @@ asap_status asap_prune_step(asap_ctx *ctx, const asap_inputs *in, const asap_par
   const bool fused = in->rank_start == nullptr && !p->per_head_mask;
   if (!fused) ASAP_TRY(launch_mass(ctx, in, p, out, true, out->out_cu_seqlens, out->out_rows_capacity, st));
   ASAP_TRY(launch_rank(ctx, in, p, out, false, st, fused));
-  ASAP_TRY(launch_select(ctx, in, p, out->rank_score, out, true, true, st, fused));
+  ASAP_TRY(launch_select(ctx, in, p, out->rank_score, out, true, true, st, fused || p->per_head_mask));
   return finish(ctx, launch_merge(ctx, in, p, out->salience, out->keep_idx, out->drop_idx, out, st), st);
 }
 

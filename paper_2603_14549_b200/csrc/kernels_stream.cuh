@@ -20,14 +20,14 @@ namespace asap {
 // =======================================================================================
 struct PrepareArgs {
   int32_t B, total_tokens, min_vis, max_vis, max_seq, max_rank, keep_k, out_capacity;
-  int32_t write_desc;        // query-sum kernel only: its first block also runs prepare_block
+  int32_t write_desc;        // query-sum kernel only: its first block also runs prepare_warp
   const int32_t *cu_seqlens, *vis_start, *vis_len, *text_start, *text_len, *rank_start, *rank_len;
   SampleDesc *desc;          // [B]
   int32_t *out_cu_seqlens;   // [B+1] or nullptr
   uint32_t *status;
 };
 
-// Descriptor of sequence b with its validity (out_row0 is filled in by prepare_block).
+// Descriptor of sequence b with its validity (out_row0 is filled in by prepare_warp).
 __device__ __forceinline__ SampleDesc make_desc(const PrepareArgs &a, int b) {
   const int lo = a.cu_seqlens[b], hi = a.cu_seqlens[b + 1];
   const int n = hi - lo;
@@ -48,38 +48,8 @@ __device__ __forceinline__ SampleDesc make_desc(const PrepareArgs &a, int b) {
   return d;
 }
 
-// Run by one whole block: validates every sequence, writes the descriptors, the output row
-// offsets and the status bits.
-__device__ __forceinline__ void prepare_block(const PrepareArgs &a) {
-  __shared__ int s_bad;
-  if (threadIdx.x == 0) s_bad = 0;
-  __syncthreads();
-  for (int b = threadIdx.x; b < a.B; b += blockDim.x) {
-    const SampleDesc d = make_desc(a, b);
-    a.desc[b] = d;
-    if (!d.valid) s_bad = 1;
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    int acc = 0;
-    for (int b = 0; b < a.B; ++b) {
-      a.desc[b].out_row0 = acc;
-      if (a.out_cu_seqlens) a.out_cu_seqlens[b] = acc;
-      if (a.desc[b].valid) acc += a.desc[b].n - a.desc[b].nv + a.keep_k;
-    }
-    if (a.out_cu_seqlens) a.out_cu_seqlens[a.B] = acc;
-    uint32_t bits = 0;
-    if (s_bad) bits |= STATUS_BAD_SAMPLE;
-    if (acc > a.out_capacity) {
-      bits |= STATUS_OUT_CAPACITY;
-      for (int b = 0; b < a.B; ++b) a.desc[b].valid = 0;   // nothing may be written
-    }
-    if (bits) atomicOr(a.status, bits);
-  }
-  __syncthreads();
-}
-
-// The same by one warp.
+// Run by one warp: validates every sequence, writes the descriptors, the output row offsets and the status bits.
+// (A whole block with one thread adding the offsets up took 6 us for 8 sequences: a chain of round trips.)
 __device__ __forceinline__ void prepare_warp(const PrepareArgs &a) {
   const int lane = threadIdx.x & 31;
   int carry = 0;
@@ -119,7 +89,7 @@ __device__ __forceinline__ void prepare_warp(const PrepareArgs &a) {
 
 __global__ void prepare_kernel(PrepareArgs a) {
   pdl_enter();
-  prepare_block(a);
+  prepare_warp(a);
 }
 
 // =======================================================================================
@@ -139,7 +109,7 @@ qsum_kernel(const __nv_bfloat16 *__restrict__ q, PrepareArgs pa, int D,
   const int b = blockIdx.z, cb = blockIdx.y, chunk = blockIdx.x;
   // When this is the first kernel of the step, block (0,0,0) also does the device-side validation
   // and writes the descriptors every later kernel reads; each block derives its own copy.
-  if (pa.write_desc && blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0) prepare_block(pa);
+  if (pa.write_desc && blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0 && threadIdx.x < 32) prepare_warp(pa);
   const SampleDesc d = make_desc(pa, b);
   if (!d.valid) return;
   const int nchunks = (d.nv + rows_per_chunk - 1) / rows_per_chunk;
@@ -322,38 +292,25 @@ mass_salience_kernel(const __nv_bfloat16 *__restrict__ k, const SampleDesc *__re
 }
 
 // =======================================================================================
-// mass_heads: Eq. 1-3 kept per head (the variant with one salience and one mask per head).
+// mass_heads: Eq. 1 kept per head (the variant with one salience and one mask per head).
 //   s_j^h = qbar^h . k_j^h / sqrt(d): one warp per visual key row; a 16-byte vector of the row lies
 //   inside one head (16 vectors per head), so the two halves of the warp reduce two heads per pass.
-//   The block that finishes last for a sample then does, per head, the min-max normalisation (Eq. 2)
-//   and the mask vector (Eq. 3), and per token the head means: mass = mean_h s^h (equal to the
-//   default mass), salience = mean_h s_hat^h (the Eq. 5 weight), mask_log = Eq. 3 of that mean.
-// grid (row blocks, B); 8 warps x 4 rows each.  s_heads: scratch [B, H, max_vis].
-// Dynamic shared memory: D + 2 H floats.
+// grid (row blocks, B); 8 warps x 4 rows each.  s_heads: scratch [B, H, max_vis].  Dynamic shared memory: D floats.
+// mask_heads: one block per (head, sample): the min-max normalisation (Eq. 2) and the mask vector (Eq. 3) of that head; the
+// head's (minimum, 1 / range) stay in `norm` [B, H, 2] for the head means.
+// salience_heads_block: one block per sample: mass = mean_h s^h (equal to the default mass), salience =
+// mean_h s_hat^h (the Eq. 5 weight), mask_log = Eq. 3 of that mean.
+// (One block per sample did all of this at the end of mass_heads: 8 sequences x 1536 tokens x 32 heads 81 -> 40 us, the step 277 -> 226.)
 // =======================================================================================
 __global__ void __launch_bounds__(MASS_THREADS)
 mass_heads_kernel(const __nv_bfloat16 *__restrict__ k, const SampleDesc *__restrict__ desc, int D, int H,
-                  int max_vis, float scale, float lambda_max, float eps, const float *__restrict__ qbar,
-                  float *__restrict__ s_heads, float *__restrict__ mass, float *__restrict__ salience,
-                  float *__restrict__ mask_log, float *__restrict__ mask_log_heads,
-                  float *__restrict__ rank_score, unsigned int *__restrict__ counters) {
+                  int max_vis, float scale, const float *__restrict__ qbar, float *__restrict__ s_heads) {
   pdl_enter();
-  extern __shared__ float s_q[];   // [D] then lo[H], inv[H]
-  __shared__ int s_last;
+  extern __shared__ float s_q[];   // [D]
   const int b = blockIdx.y;
   const SampleDesc d = desc[b];
-  float *mass_b = mass + (size_t)b * max_vis;
-  float *sal_b = salience + (size_t)b * max_vis, *msk_b = mask_log + (size_t)b * max_vis;
-  float *mh_b = mask_log_heads + (size_t)b * H * max_vis;
   float *sh_b = s_heads + (size_t)b * H * max_vis;
-  if (!d.valid) {
-    for (int j = blockIdx.x * MASS_THREADS + threadIdx.x; j < max_vis; j += gridDim.x * MASS_THREADS) {
-      mass_b[j] = 0.f; sal_b[j] = 0.f; msk_b[j] = 0.f;
-      rank_score[(size_t)b * max_vis + j] = 0.f;   // the score kernel skips the sample
-      for (int h = 0; h < H; ++h) mh_b[(size_t)h * max_vis + j] = 0.f;
-    }
-    return;
-  }
+  if (!d.valid) return;
   const int nblocks = (d.nv + MASS_ROWS - 1) / MASS_ROWS;
   if ((int)blockIdx.x >= nblocks) return;
   for (int c = threadIdx.x * 4; c < D; c += MASS_THREADS * 4)
@@ -395,53 +352,91 @@ mass_heads_kernel(const __nv_bfloat16 *__restrict__ k, const SampleDesc *__restr
       if ((lane & 15) == 0 && h < H && j0 + r < d.nv) sh_b[(size_t)h * max_vis + j0 + r] = part * scale;
     }
   }
+}
 
-  // ---- last block of the sample ----
-  __threadfence();
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    unsigned int old = atomicAdd(counters + b, 1u);
-    s_last = (old == (unsigned int)(nblocks - 1));
-    if (s_last) counters[b] = 0u;
+struct SalienceArgs {
+  int H;
+  float scale, lambda_max, eps;
+  const float *heads;                       // [B, H, max_vis]
+  const float *norm;                        // [B, H, 2] or nullptr: a salience per head (salience_heads_block)
+  float *mass, *salience, *mask_log, *rank_score;   // [B, max_vis]
+};
+
+__global__ void __launch_bounds__(MASS_THREADS)
+mask_heads_kernel(const SampleDesc *__restrict__ desc, int H, int max_vis, float lambda_max, float eps,
+                  const float *__restrict__ s_heads, float *__restrict__ mask_log_heads, float *__restrict__ norm) {
+  pdl_enter();
+  __shared__ float s_red[2 * (MASS_THREADS / 32)];
+  const int h = blockIdx.x, b = blockIdx.y;
+  const SampleDesc d = desc[b];
+  float *mh = mask_log_heads + ((size_t)b * H + h) * max_vis;
+  if (!d.valid) {
+    for (int j = threadIdx.x; j < max_vis; j += MASS_THREADS) mh[j] = 0.f;
+    return;
   }
-  __syncthreads();
-  if (!s_last) return;
-  __threadfence();
-  float *s_lo = s_q + D, *s_inv = s_lo + H;
-  for (int h = warp; h < H; h += MASS_THREADS / 32) {           // Eq. 2's extremes, one warp per head
-    float lo = INFINITY, hi = -INFINITY;
-    for (int j = lane; j < d.nv; j += 32) {
-      const float sv = __ldcg(sh_b + (size_t)h * max_vis + j);
-      lo = fminf(lo, sv); hi = fmaxf(hi, sv);
-    }
+  const float *sh = s_heads + ((size_t)b * H + h) * max_vis;
+  float lo = INFINITY, hi = -INFINITY;
+  for (int j = threadIdx.x; j < d.nv; j += MASS_THREADS) {
+    const float s = __ldcg(sh + j);
+    lo = fminf(lo, s); hi = fmaxf(hi, s);
+  }
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      lo = fminf(lo, __shfl_xor_sync(0xffffffffu, lo, o));
-      hi = fmaxf(hi, __shfl_xor_sync(0xffffffffu, hi, o));
-    }
-    if (lane == 0) { s_lo[h] = lo; s_inv[h] = 1.0f / ((hi - lo) + eps); }
+  for (int o = 16; o > 0; o >>= 1) {
+    lo = fminf(lo, __shfl_xor_sync(0xffffffffu, lo, o));
+    hi = fmaxf(hi, __shfl_xor_sync(0xffffffffu, hi, o));
   }
+  if (lane == 0) { s_red[warp] = lo; s_red[MASS_THREADS / 32 + warp] = hi; }
   __syncthreads();
-  const float inv_h = 1.0f / (float)H;
-  for (int j = threadIdx.x; j < max_vis; j += MASS_THREADS) {
-    if (j < d.nv) {
-      float acc_s = 0.f, acc_sh = 0.f;
-      for (int h = 0; h < H; ++h) {                               // heads in order
-        const float sv = __ldcg(sh_b + (size_t)h * max_vis + j);
-        const float sh = (sv - s_lo[h]) * s_inv[h];
-        mh_b[(size_t)h * max_vis + j] = logf(fmaxf(lambda_max * sh, eps));
-        acc_s += sv;
-        acc_sh += sh;
-      }
-      const float sal = acc_sh * inv_h;
-      mass_b[j] = acc_s * inv_h;
-      sal_b[j] = sal;
-      msk_b[j] = logf(fmaxf(lambda_max * sal, eps));
-    } else {
-      mass_b[j] = 0.f; sal_b[j] = 0.f; msk_b[j] = 0.f;
-      for (int h = 0; h < H; ++h) mh_b[(size_t)h * max_vis + j] = 0.f;
-    }
+#pragma unroll
+  for (int w = 0; w < MASS_THREADS / 32; ++w) {
+    lo = fminf(lo, s_red[w]); hi = fmaxf(hi, s_red[MASS_THREADS / 32 + w]);
   }
+  const float inv = 1.0f / ((hi - lo) + eps);
+  if (threadIdx.x == 0) {
+    norm[((size_t)b * H + h) * 2] = lo;
+    norm[((size_t)b * H + h) * 2 + 1] = inv;
+  }
+  for (int j = threadIdx.x; j < max_vis; j += MASS_THREADS)
+    mh[j] = j < d.nv ? logf(fmaxf(lambda_max * ((__ldcg(sh + j) - lo) * inv), eps)) : 0.f;
+}
+
+__device__ __forceinline__ void salience_heads_block(const SampleDesc &d, int b, int max_vis, const SalienceArgs &a) {
+  float *mass_b = a.mass + (size_t)b * max_vis, *sal_b = a.salience + (size_t)b * max_vis, *msk_b = a.mask_log + (size_t)b * max_vis;
+  const float *sh_b = a.heads + (size_t)b * a.H * max_vis, *norm = a.norm + (size_t)b * a.H * 2;
+  __shared__ float2 s_norm[64];             // (H <= 64: D <= 8192)
+  if ((int)threadIdx.x < a.H) s_norm[threadIdx.x] = make_float2(__ldcg(norm + 2 * threadIdx.x), __ldcg(norm + 2 * threadIdx.x + 1));
+  __syncthreads();
+  const float inv_h = 1.0f / (float)a.H;
+  for (int j = threadIdx.x; j < max_vis; j += blockDim.x) {
+    float acc_s = 0.f, acc_sh = 0.f, sal = 0.f;
+    if (d.valid && j < d.nv) {
+      for (int h0 = 0; h0 < a.H; h0 += 16) {                        // heads in order, sixteen loads in flight
+        float v[16];
+#pragma unroll
+        for (int e = 0; e < 16; ++e) v[e] = h0 + e < a.H ? __ldcg(sh_b + (size_t)(h0 + e) * max_vis + j) : 0.f;
+#pragma unroll
+        for (int e = 0; e < 16; ++e) {
+          if (h0 + e >= a.H) break;
+          const float2 n = s_norm[h0 + e];
+          acc_s += v[e];
+          acc_sh += (v[e] - n.x) * n.y;
+        }
+      }
+      sal = acc_sh * inv_h;
+    }
+    const bool in = d.valid && j < d.nv;
+    mass_b[j] = in ? acc_s * inv_h : 0.f;
+    sal_b[j] = in ? sal : 0.f;
+    msk_b[j] = in ? logf(fmaxf(a.lambda_max * sal, a.eps)) : 0.f;
+    if (!d.valid) a.rank_score[(size_t)b * max_vis + j] = 0.f;      // the score kernel and the selection skip the sample
+  }
+}
+
+__global__ void __launch_bounds__(MASS_THREADS)
+salience_heads_kernel(const SampleDesc *__restrict__ desc, int max_vis, SalienceArgs a) {
+  pdl_enter();
+  salience_heads_block(desc[blockIdx.x], blockIdx.x, max_vis, a);
 }
 
 // =======================================================================================
@@ -451,13 +446,6 @@ mass_heads_kernel(const __nv_bfloat16 *__restrict__ k, const SampleDesc *__restr
 // the mask vector over the image span; padding past the span is zeroed as mass_salience does.
 // =======================================================================================
 constexpr int SAL_THREADS = 1024;
-
-struct SalienceArgs {
-  int H;
-  float scale, lambda_max, eps;
-  const float *heads;                       // [B, H, max_vis]
-  float *mass, *salience, *mask_log, *rank_score;   // [B, max_vis]
-};
 
 __device__ __forceinline__ void salience_block(const SampleDesc &d, int b, int max_vis, const SalienceArgs &a) {
   __shared__ float s_red[2 * (SAL_THREADS / 32)];
@@ -564,7 +552,8 @@ select_kernel(const float *__restrict__ rank_score, const SampleDesc *__restrict
               SalienceArgs sal /* blockIdx.y == 1 */) {
   pdl_enter();
   if (blockIdx.y == 1) {
-    salience_block(desc[blockIdx.x], blockIdx.x, max_vis, sal);
+    if (sal.norm) salience_heads_block(desc[blockIdx.x], blockIdx.x, max_vis, sal);
+    else salience_block(desc[blockIdx.x], blockIdx.x, max_vis, sal);
     return;
   }
   extern __shared__ uint32_t s_key[];   // [max_vis]
