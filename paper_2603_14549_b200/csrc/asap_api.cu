@@ -249,13 +249,13 @@ asap_status launch_prepare(asap_ctx *ctx, const asap_inputs *in, const asap_para
 // Steps 1a-1b: query sum, attention mass, salience, mask vector.  With `fold_prepare` the query-sum
 // kernel also carries the device-side validation and writes the descriptors.
 
-// Rows a block of the query-sum kernel adds up: 32, doubled (up to 128) while the grid still has eight blocks per
+// Rows a block of the query-sum kernel adds up: 32, doubled (up to 128) while the grid still has two blocks per
 // SM -- every chunk costs a partial row written and read back (32 rows: 12 % on top of the queries themselves).
 int qsum_rows_per_chunk(const asap_ctx *ctx, const asap_inputs *in) {
   const long long col_blocks = (in->D + QSUM_COLS - 1) / QSUM_COLS;
   int rows = QSUM_ROWS;
   while (rows < 4 * QSUM_ROWS &&
-         (long long)((in->max_vis + 2 * rows - 1) / (2 * rows)) * col_blocks * in->B >= 8LL * ctx->num_sms)
+         (long long)((in->max_vis + 2 * rows - 1) / (2 * rows)) * col_blocks * in->B >= 2LL * ctx->num_sms)
     rows *= 2;
   return rows;
 }
@@ -443,7 +443,7 @@ asap_status launch_merge_front(asap_ctx *ctx, const asap_inputs *in, const asap_
         sa.drop_idx = nullptr; sa.role = ctx->role;
         sa.hidden = static_cast<const __nv_bfloat16 *>(in->hidden); sa.kept_inv = ctx->kept_inv; sa.assign = out->assign;
         sa.best_sim = out->best_sim; sa.seg = merge_scans(ctx, in, p) ? nullptr : ctx->seg; sa.members = ctx->members; sa.counters = ctx->cnt_sim;
-        sa.tile_counters = ctx->cnt_tiles; sa.part = ctx->sim_part; sa.ss_part = nullptr; sa.smat = nullptr;
+        sa.tile_counters = ctx->cnt_tiles; sa.part = ctx->sim_part; sa.ss_part = nullptr; sa.smat = nullptr; sa.mask16 = nullptr; sa.mask_pitch = 0;
         sa.drop_all = drop_idx; sa.salience = salience; sa.member_meta = salience ? ctx->member_meta : nullptr;
         sa.status = ctx->status; sa.wait_limit = ctx->wait_limit;
         mark(ctx, "sim", st);
@@ -502,7 +502,7 @@ asap_status launch_merge_front(asap_ctx *ctx, const asap_inputs *in, const asap_
     sa.best_sim = out->best_sim; sa.seg = merge_scans(ctx, in, p) ? nullptr : ctx->seg; sa.members = ctx->members; sa.counters = ctx->cnt_sim;
     sa.tile_counters = ctx->cnt_tiles; sa.part = ctx->sim_part;
     sa.ss_part = ctx->sim_part + (size_t)B * max_mt * splits * (size_t)k * 128;
-    sa.smat = nullptr;
+    sa.smat = nullptr; sa.mask16 = nullptr; sa.mask_pitch = 0;
     sa.drop_all = drop_idx; sa.salience = salience; sa.member_meta = salience ? ctx->member_meta : nullptr;
     sa.status = ctx->status; sa.wait_limit = ctx->wait_limit;
     mark(ctx, "sim", st);
@@ -581,6 +581,8 @@ asap_status launch_consolidate_front(asap_ctx *ctx, const asap_inputs *in, const
   ASAP_TRY(after_launch(ctx, "kept_gather"));
 
   float *smat = static_cast<float *>(scratch);
+  uint32_t *mask_g = reinterpret_cast<uint32_t *>(static_cast<uint8_t *>(scratch) + route_smat_bytes(B, k));
+  bool mask_written = false;
   {
     // large batches: two row tiles per block, the slots dealt in groups to neighbouring blocks (see the similarity
     // launch of the merge); here every product is used, the matrix being square
@@ -606,6 +608,8 @@ asap_status launch_consolidate_front(asap_ctx *ctx, const asap_inputs *in, const
       sa.drop_idx = nullptr; sa.role = nullptr; sa.drop_all = nullptr; sa.hidden = nullptr; sa.kept_inv = ctx->kept_inv;
       sa.assign = nullptr; sa.best_sim = nullptr; sa.seg = nullptr; sa.members = nullptr; sa.counters = nullptr;
       sa.tile_counters = nullptr; sa.part = nullptr; sa.ss_part = nullptr; sa.smat = smat; sa.salience = nullptr;
+      sa.mask16 = reinterpret_cast<uint16_t *>(mask_g); sa.mask_pitch = 2 * ((k + 31) / 32);
+      mask_written = true;
       sa.member_meta = nullptr; sa.status = ctx->status; sa.wait_limit = ctx->wait_limit;
       mark(ctx, "sim_kept", st);
       launch_pdl(sim_pair_kernel, dim3(pairs * pg, B), dim3(SIMP_THREADS), psmem, st, map_a, map_b, sa);
@@ -655,7 +659,7 @@ asap_status launch_consolidate_front(asap_ctx *ctx, const asap_inputs *in, const
   sa.drop_idx = nullptr; sa.role = nullptr; sa.hidden = nullptr; sa.kept_inv = ctx->kept_inv; sa.assign = nullptr; sa.best_sim = nullptr;
   sa.seg = nullptr; sa.members = nullptr; sa.counters = nullptr; sa.tile_counters = ctx->cnt_tiles;
   sa.part = ctx->sim_part; sa.ss_part = ctx->sim_part + (size_t)B * max_mt * splits * (size_t)k * 128;
-  sa.smat = smat; sa.drop_all = nullptr; sa.salience = nullptr; sa.member_meta = nullptr;
+  sa.smat = smat; sa.drop_all = nullptr; sa.salience = nullptr; sa.member_meta = nullptr; sa.mask16 = nullptr; sa.mask_pitch = 0;
   sa.status = ctx->status; sa.wait_limit = ctx->wait_limit;
   mark(ctx, "sim_kept", st);
   if (cluster)
@@ -672,8 +676,7 @@ routing:
   const size_t tail_words = (size_t)(in->max_vis - k) + (size_t)in->max_vis;
   const size_t mask_words = (size_t)k * ra.kw;
   const bool mask_in_smem = (fixed_words + (mask_words > tail_words ? mask_words : tail_words)) * 4 <= 200 * 1024;
-  ra.mask_g = mask_in_smem ? nullptr
-                           : reinterpret_cast<uint32_t *>(static_cast<uint8_t *>(scratch) + route_smat_bytes(B, k));
+  ra.mask_g = mask_g; ra.mask_in_smem = mask_in_smem ? 1 : 0; ra.mask_written = mask_written ? 1 : 0;
   const size_t route_smem = (fixed_words + (mask_in_smem && mask_words > tail_words ? mask_words : tail_words)) * 4;
   if (route_smem > 224 * 1024)
     return fail(ctx, ASAP_ERR_UNSUPPORTED, "max_vis = %d is too large for the routing kernel", in->max_vis);
@@ -910,8 +913,8 @@ asap_status asap_consolidate(asap_ctx *ctx, const asap_inputs *in, const asap_pa
     return fail(ctx, ASAP_ERR_INVALID, "asap_consolidate needs merge_enable and keep_k < max_vis; asap_merge covers the rest");
   if (keep_idx == out->keep_idx || drop_idx == out->drop_idx)
     return fail(ctx, ASAP_ERR_INVALID, "asap_consolidate: the stage-1 lists must not be the output lists");
-  if (p->keep_k > 32 * 32 * ROUTE_LANE_WORDS)
-    return fail(ctx, ASAP_ERR_UNSUPPORTED, "asap_consolidate: keep_k above %d", 32 * 32 * ROUTE_LANE_WORDS);
+  if (p->keep_k > 32 * ROUTE_MAX_WORDS)
+    return fail(ctx, ASAP_ERR_UNSUPPORTED, "asap_consolidate: keep_k above %d", 32 * ROUTE_MAX_WORDS);
   if (!scratch || !aligned16(scratch) || scratch_bytes < asap_consolidate_scratch_bytes(in->B, p->keep_k))
     return fail(ctx, ASAP_ERR_WORKSPACE, "asap_consolidate: scratch is null, unaligned or smaller than asap_consolidate_scratch_bytes");
   cudaStream_t st = static_cast<cudaStream_t>(stream);

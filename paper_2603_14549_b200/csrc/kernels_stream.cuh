@@ -889,14 +889,15 @@ __device__ __forceinline__ void csr_block(const SampleDesc &d, int b, int max_vi
 // route: Sec. 4.2 inside the kept set, one block per sample.  Input: the keep_k x keep_k cosine
 // matrix S of the kept rows, the salience, the attention mass, stage 1's kept / pruned lists.
 //   A  visiting order of the kept slots: salience descending, sequence index ascending.
-//   B  bit matrix  M[p] = { q : S[p][q] > t }.
-//   C  one warp walks the slots in visiting order.  A slot whose bit is set in the running union
-//      of the anchors' rows is absorbed (while the pruned pool can still refill a slot, i.e. at
-//      most nv - keep_k times); any other slot becomes an anchor and adds its row to the union.
-//      This is the greedy rule "join the most similar earlier anchor if that similarity exceeds t,
-//      else become an anchor" with the question WHICH anchor left to step D.
+//   B  bit matrix  M[p] = { q : S[p][q] > t }, from the similarity kernel where that form writes it.
+//   C  A slot is absorbed if an anchor that was visited before it is similar to it (while the pruned pool can still refill a
+//      slot, i.e. at most nv - keep_k times); any other slot becomes an anchor.  This is the greedy
+//      rule "join the most similar earlier anchor if that similarity exceeds t, else become an anchor" with the question
+//      WHICH anchor left to step D.  Decided in rounds by all threads: as many as the longest chain of slots each of which
+//      waits for the one before, three or four on clustered rows.  (One warp walking the order took 38 of the kernel's 174 us
+//      on 24 x 576 slots, reading the similarities a second time for D 50, forming the bit matrix here 30; 174 -> 59 us in all.)
 //   D  every absorbed slot finds the most similar anchor that was visited before it (lowest slot
-//      among equals).
+//      among equals), looking only at the anchors in its row of the bit matrix.
 //   E  the vacated slots are refilled with the pruned tokens of largest attention mass (radix
 //      select, lower index first among equals).
 //   F  anchors and refilled tokens, in sequence order, form the final kept list; the absorbed
@@ -905,75 +906,16 @@ __device__ __forceinline__ void csr_block(const SampleDesc &d, int b, int max_vi
 // src_sim [B, max_vis - keep_k] (padding -1 / 0), seg [B, keep_k + 1], members [B, max_vis - keep_k].
 // =======================================================================================
 constexpr int ROUTE_THREADS = 1024;
-constexpr int ROUTE_LANE_WORDS = 4;                     // keep_k <= 32 * 32 * 4
-
-// The sequential part of the routing, run by one warp, 32 candidates of the visiting order at a
-// time.  Lane l holds words l, l + 32, ... of the union of the anchors' rows (LW words per lane;
-// LW = 1 covers keep_k <= 1024).  Per group of 32: (1) each lane looks up whether its candidate is
-// already covered by an anchor of an earlier group; (2) each lane gathers its candidate's row
-// restricted to the group (32 bits); (3) the group is resolved in order from those 32 x 32 bits, in
-// registers, by every lane alike; (4) the group's anchors add their full rows to the union.  Only
-// step (3) is a dependent chain, and it touches no memory.  Returns the number of absorbed slots.
-template <int LW>
-__device__ __forceinline__ int route_walk(const int *s_order, const uint32_t *mask, int *s_flag, int k, int kw,
-                                          int nd, int lane) {
-  const unsigned full = 0xffffffffu;
-  uint32_t supp[LW];
-#pragma unroll
-  for (int i = 0; i < LW; ++i) supp[i] = 0u;
-  int n_abs = 0;
-  for (int r0 = 0; r0 < k; r0 += 32) {
-    const bool valid = r0 + lane < k;
-    const int p = valid ? s_order[r0 + lane] : 0;
-    const int w = p >> 5;
-    uint32_t word = 0u;
-#pragma unroll
-    for (int i = 0; i < LW; ++i) {
-      const uint32_t got = __shfl_sync(full, supp[i], w & 31);
-      if ((w >> 5) == i) word = got;
-    }
-    uint32_t blk = __ballot_sync(full, valid && ((word >> (p & 31)) & 1u));
-    uint32_t intra = 0u;
-#pragma unroll
-    for (int u = 0; u < 32; ++u) {
-      const int pu = __shfl_sync(full, p, u);
-      const uint32_t bit = (mask[(size_t)p * kw + (pu >> 5)] >> (pu & 31)) & 1u;
-      if (valid && r0 + u < k) intra |= bit << u;
-    }
-    uint32_t absorbed_bits = 0u;
-#pragma unroll
-    for (int t = 0; t < 32; ++t) {
-      const uint32_t row_t = __shfl_sync(full, intra, t);
-      const bool ab = ((blk >> t) & 1u) && n_abs < nd && r0 + t < k;
-      if (ab) {
-        ++n_abs;
-        absorbed_bits |= 1u << t;
-      } else {
-        blk |= row_t & ~((2u << t) - 1u);          // an anchor covers later candidates only
-      }
-    }
-#pragma unroll
-    for (int t = 0; t < 32; ++t) {
-      const int pt = __shfl_sync(full, p, t);
-      if (r0 + t < k && !((absorbed_bits >> t) & 1u)) {
-#pragma unroll
-        for (int i = 0; i < LW; ++i) {
-          const int ww = i * 32 + lane;
-          if (ww < kw) supp[i] |= mask[(size_t)pt * kw + ww];
-        }
-      }
-    }
-    if (valid) s_flag[p] = ((absorbed_bits >> lane) & 1u) ? 0 : 1;
-  }
-  return n_abs;
-}
+constexpr int ROUTE_MAX_WORDS = 128;                    // keep_k <= 32 * 128
 
 struct RouteArgs {
   const SampleDesc *desc;
   int max_vis, keep_k, kw;        // kw = ceil(keep_k / 32)
   float threshold;
   const float *smat;              // [B, keep_k, keep_k]
-  uint32_t *mask_g;               // [B, keep_k, kw] or nullptr: the bit matrix lives in shared memory
+  uint32_t *mask_g;               // [B, keep_k, kw] bit matrix in global memory
+  int mask_in_smem;               // the bit matrix fits shared memory (else mask_g is used where it lies)
+  int mask_written;               // mask_g was filled by the similarity kernel
   const float *salience, *mass;   // [B, max_vis]
   const int32_t *keep_idx;        // [B, keep_k]            stage 1
   const int32_t *drop_idx;        // [B, max_vis - keep_k]  stage 1
@@ -989,6 +931,7 @@ route_kernel(RouteArgs a) {
   __shared__ int s_scan[33];
   __shared__ uint32_t s_prefix;
   __shared__ int s_remaining, s_nabs;
+  __shared__ uint32_t s_anchor[ROUTE_MAX_WORDS], s_gone[ROUTE_MAX_WORDS];   // decided slots: anchors, absorbed
   const int b = blockIdx.x;
   const SampleDesc d = a.desc[b];
   const int k = a.keep_k, kw = a.kw, nd_max = a.max_vis - k;
@@ -1014,7 +957,7 @@ route_kernel(RouteArgs a) {
   int *s_dest = s_flag + k;
   uint32_t *s_tmp = r_smem + 4 * (size_t)k;
   uint32_t *s_union = s_tmp + k;
-  uint32_t *mask = a.mask_g ? a.mask_g + (size_t)b * k * kw : s_union;
+  uint32_t *mask = a.mask_in_smem ? s_union : a.mask_g + (size_t)b * k * kw;
   const int32_t *keep_b = a.keep_idx + (size_t)b * k;
   const int32_t *drop_b = a.drop_idx + (size_t)b * nd_max;
   const float *sal_b = a.salience + (size_t)b * a.max_vis;
@@ -1029,68 +972,124 @@ route_kernel(RouteArgs a) {
   for (int p = tid; p < k; p += nthr) {
     const uint32_t mine = s_tmp[p];
     int r = 0;
-    for (int q = 0; q < k; ++q) {
-      const uint32_t o = s_tmp[q];
-      r += (o > mine) || (o == mine && q < p);       // the kept list is ascending: q < p is the lower index
-    }
+    int q = 0;
+#pragma unroll 8
+    for (; q < p; ++q) r += s_tmp[q] >= mine;        // the kept list is ascending: an equal one before it is the lower index
+#pragma unroll 8
+    for (++q; q < k; ++q) r += s_tmp[q] > mine;
     s_rank[p] = r;
     s_order[r] = p;
+    s_flag[p] = 0;
   }
-  // ---- B: bit matrix, one warp per row, coalesced
-  for (int p = warp; p < k; p += (nthr >> 5)) {
-    const float *row = S + (size_t)p * k;
-    for (int w0 = 0; w0 < kw; w0 += 16) {             // sixteen loads in flight per lane
-      float v[16];
+  for (int w = tid; w < kw; w += nthr) { s_anchor[w] = 0u; s_gone[w] = 0u; }
+  // ---- B: bit matrix  M[p] = { q : S[p][q] > t }
+  if (!a.mask_written) {
+    for (int p = warp; p < k; p += (nthr >> 5)) {     // one warp per row, coalesced
+      const float *row = S + (size_t)p * k;
+      for (int w0 = 0; w0 < kw; w0 += 16) {             // sixteen loads in flight per lane
+        float v[16];
 #pragma unroll
-      for (int e = 0; e < 16; ++e) {
-        const int q = (w0 + e) * 32 + lane;
-        v[e] = q < k ? __ldcg(row + q) : -INFINITY;
-      }
+        for (int e = 0; e < 16; ++e) {
+          const int q = (w0 + e) * 32 + lane;
+          v[e] = q < k ? __ldcg(row + q) : -INFINITY;
+        }
 #pragma unroll
-      for (int e = 0; e < 16; ++e) {
-        const int q = (w0 + e) * 32 + lane;
-        const unsigned bits = __ballot_sync(0xffffffffu, q < k && q != p && v[e] > a.threshold);
-        if (lane == 0 && w0 + e < kw) mask[(size_t)p * kw + w0 + e] = bits;
+        for (int e = 0; e < 16; ++e) {
+          const int q = (w0 + e) * 32 + lane;
+          const unsigned bits = __ballot_sync(0xffffffffu, q < k && q != p && v[e] > a.threshold);
+          if (lane == 0 && w0 + e < kw) mask[(size_t)p * kw + w0 + e] = bits;
+        }
       }
     }
+  } else if (a.mask_in_smem) {
+    const uint32_t *src = a.mask_g + (size_t)b * k * kw;
+#pragma unroll 8
+    for (int i = tid; i < k * kw; i += nthr) mask[i] = __ldcg(src + i);
   }
   __syncthreads();
-  // ---- C: greedy walk by one warp; the union lives in registers, word w in lane w % 32
-  if (warp == 0) {
-    const int n_abs_w = kw <= 32 ? route_walk<1>(s_order, mask, s_flag, k, kw, nd, lane)
-                                 : route_walk<ROUTE_LANE_WORDS>(s_order, mask, s_flag, k, kw, nd, lane);
-    if (lane == 0) s_nabs = n_abs_w;
+  // ---- C: rounds.  A slot with an earlier anchor among its neighbours is absorbed; one whose earlier neighbours are all
+  // absorbed is an anchor; any other waits.  The first undecided slot of the visiting order is decided in every round, and the
+  // outcome is that of walking the slots in that order (a slot's fate depends on earlier slots alone).
+  bool open[4];                                       // this thread's slots tid, tid + nthr, ... (k <= 4096)
+#pragma unroll
+  for (int t = 0; t < 4; ++t) open[t] = tid + t * nthr < k;
+  while (true) {
+    int verdict[4] = {0, 0, 0, 0};                    // 1 anchor, 2 absorbed
+    bool waiting = false;
+#pragma unroll
+    for (int t = 0; t < 4; ++t) {
+      if (!open[t]) continue;
+      const int p = tid + t * nthr, rp = s_rank[p];
+      const uint32_t *row = mask + (size_t)p * kw;
+      bool absorbed = false, blocked = false;
+      for (int w = 0; w < kw && !absorbed; ++w) {
+        const uint32_t anchors = s_anchor[w];
+        uint32_t cand = row[w] & ~s_gone[w];
+        while (cand) {
+          const int bit = __ffs(cand) - 1;
+          cand &= cand - 1;
+          if (s_rank[w * 32 + bit] < rp) {
+            if ((anchors >> bit) & 1u) { absorbed = true; break; }
+            blocked = true;
+          }
+        }
+      }
+      verdict[t] = absorbed ? 2 : (blocked ? 0 : 1);
+      if (verdict[t]) open[t] = false;
+      else waiting = true;
+    }
+    __syncthreads();                                  // every slot has looked at the last round's decisions
+#pragma unroll
+    for (int t = 0; t < 4; ++t) {
+      const int p = tid + t * nthr;
+      if (verdict[t] == 1) { atomicOr(&s_anchor[p >> 5], 1u << (p & 31)); s_flag[p] = 1; }
+      if (verdict[t] == 2) atomicOr(&s_gone[p >> 5], 1u << (p & 31));
+    }
+    if (!__syncthreads_or(waiting)) break;
+  }
+  // at most nd slots are absorbed, the first ones of the visiting order: later ones stay anchors
+  {
+    const int per = (k + nthr - 1) / nthr;
+    const int lo = min(k, tid * per), hi = min(k, lo + per);
+    int cnt = 0;
+    for (int r = lo; r < hi; ++r) cnt += !s_flag[s_order[r]];
+    int tot;
+    int run = block_exclusive_scan(cnt, s_scan, tot);
+    if (tot > nd) {
+      for (int r = lo; r < hi; ++r) {
+        const int p = s_order[r];
+        if (!s_flag[p] && run++ >= nd) {
+          s_flag[p] = 1;
+          atomicOr(&s_anchor[p >> 5], 1u << (p & 31));
+        }
+      }
+    }
+    if (tid == 0) s_nabs = min(tot, nd);
   }
   __syncthreads();
   const int n_abs = s_nabs;
-  // ---- D: destination of every absorbed slot
-  for (int p = warp; p < k; p += (nthr >> 5)) {
-    if (s_flag[p]) { if (lane == 0) s_dest[p] = -1; continue; }
-    const float *row = S + (size_t)p * k;
-    const int rp = s_rank[p];
+  // ---- D: destination of every absorbed slot: the most similar earlier anchor (it lies above the threshold, since one
+  // of them does), the lowest slot among equals
+  for (int p = tid; p < k; p += nthr) {
+    int best_q = -1;
     float best = -INFINITY;
-    int best_q = 0x7fffffff;
-    for (int q0 = lane; q0 < k; q0 += 32 * 8) {       // eight loads in flight per lane
-      float v[8];
-#pragma unroll
-      for (int e = 0; e < 8; ++e) {
-        const int q = q0 + 32 * e;
-        v[e] = (q < k && s_flag[q] && s_rank[q] < rp) ? __ldcg(row + q) : -INFINITY;
+    if (!s_flag[p]) {
+      const int rp = s_rank[p];
+      const float *row = S + (size_t)p * k;
+      for (int w = 0; w < kw; ++w) {
+        uint32_t cand = mask[(size_t)p * kw + w] & s_anchor[w];
+        while (cand) {
+          const int q = w * 32 + __ffs(cand) - 1;
+          cand &= cand - 1;
+          if (s_rank[q] < rp) {
+            const float v = __ldcg(row + q);
+            if (v > best) { best = v; best_q = q; }   // ascending q: the first maximum stays
+          }
+        }
       }
-#pragma unroll
-      for (int e = 0; e < 8; ++e)                     // ascending q: the first maximum stays
-        if (v[e] > best) { best = v[e]; best_q = q0 + 32 * e; }
     }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      const float ob = __shfl_xor_sync(0xffffffffu, best, o);
-      const int oq = __shfl_xor_sync(0xffffffffu, best_q, o);
-      if (ob > best || (ob == best && oq < best_q)) { best = ob; best_q = oq; }
-    }
-    if (lane == 0) {
-      s_dest[p] = best_q < k ? best_q : -1;
-      s_tmp[p] = __float_as_uint(best);
-    }
+    s_dest[p] = best_q;
+    s_tmp[p] = __float_as_uint(best);
   }
   __syncthreads();      // the bit matrix is dead from here on: its space is reused
   uint32_t *s_key = s_union;                                  // [nd]

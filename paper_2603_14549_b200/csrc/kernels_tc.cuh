@@ -806,6 +806,8 @@ struct SimArgs {
   float *part;               // [B, max_mt, splits, keep_k, 128] partial dot products (several slices only)
   float *ss_part;            // [B, max_mt, splits, 128]         partial squared norms
   float *smat;               // [B, keep_k, keep_k] or nullptr: matrix mode
+  uint16_t *mask16;          // (pair kernel, matrix mode) [B, keep_k, mask_pitch] or nullptr: bit q of row p set where S[p][q] > threshold, q != p
+  int mask_pitch;            // halfwords per row, even
   const float *salience;     // [B, max_vis] or nullptr: with member_meta, the merge weights the grouping copies
   int2 *member_meta;         // [B, max_vis-keep_k] or nullptr (see csr_block)
   uint32_t *status;
@@ -1652,18 +1654,29 @@ sim_pair_kernel(const __grid_constant__ CUtensorMap tmap_h, const __grid_constan
           // matrix mode: S[p][q] = <h_p, h_q> * (1/||h_p|| * 1/||h_q||) for this thread's kept row p
           if (v < a.keep_k) {
             float *srow = a.smat + ((size_t)b * a.keep_k + v) * a.keep_k + slot0 + c;
+            float sv[16];
+            uint32_t above = 0u;
+#pragma unroll
+            for (int e = 0; e < 16; ++e) {                // (a column past the last slot has kinv 0 in shared memory)
+              sv[e] = __uint_as_float(r[e]) * (inv_p * bk->kinv[c + e]);
+              if (c + e < ncol && slot0 + c + e != v && sv[e] > a.threshold) above |= 1u << e;
+            }
             if (c + 16 <= ncol && (reinterpret_cast<size_t>(srow) & 15) == 0) {
 #pragma unroll
               for (int e = 0; e < 16; e += 4)         // 16-byte stores: a quarter of the store requests
-                reinterpret_cast<float4 *>(srow)[e >> 2] =
-                    make_float4(__uint_as_float(r[e]) * (inv_p * __ldg(kinv + slot0 + c + e)),
-                                __uint_as_float(r[e + 1]) * (inv_p * __ldg(kinv + slot0 + c + e + 1)),
-                                __uint_as_float(r[e + 2]) * (inv_p * __ldg(kinv + slot0 + c + e + 2)),
-                                __uint_as_float(r[e + 3]) * (inv_p * __ldg(kinv + slot0 + c + e + 3)));
+                reinterpret_cast<float4 *>(srow)[e >> 2] = make_float4(sv[e], sv[e + 1], sv[e + 2], sv[e + 3]);
             } else {
 #pragma unroll
               for (int e = 0; e < 16; ++e)
-                if (c + e < ncol) srow[e] = __uint_as_float(r[e]) * (inv_p * __ldg(kinv + slot0 + c + e));
+                if (c + e < ncol) srow[e] = sv[e];
+            }
+            if (a.mask16) {
+              // the routing's bit matrix on the way (slot0 and c are multiples of 16); the last chunk also
+              // clears the other half of its word
+              const int hw = (slot0 + c) >> 4;
+              uint16_t *mrow = a.mask16 + ((size_t)b * a.keep_k + v) * a.mask_pitch;
+              mrow[hw] = (uint16_t)above;
+              if (slot0 + c + 16 >= a.keep_k && !(hw & 1)) mrow[hw + 1] = 0;
             }
           }
           continue;
