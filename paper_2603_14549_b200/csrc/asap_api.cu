@@ -672,12 +672,14 @@ routing:
   RouteArgs ra;
   ra.desc = ctx->desc; ra.max_vis = in->max_vis; ra.keep_k = k; ra.kw = (k + 31) / 32;
   ra.threshold = p->sim_threshold; ra.smat = smat;
-  const size_t fixed_words = 5 * (size_t)k;
+  const size_t fixed_words = 5 * (size_t)k + 3;
   const size_t tail_words = (size_t)(in->max_vis - k) + (size_t)in->max_vis;
   const size_t mask_words = (size_t)k * ra.kw;
   const bool mask_in_smem = (fixed_words + (mask_words > tail_words ? mask_words : tail_words)) * 4 <= 200 * 1024;
   ra.mask_g = mask_g; ra.mask_in_smem = mask_in_smem ? 1 : 0; ra.mask_written = mask_written ? 1 : 0;
-  const size_t route_smem = (fixed_words + (mask_in_smem && mask_words > tail_words ? mask_words : tail_words)) * 4;
+  const size_t union_words = mask_in_smem && mask_words > tail_words ? mask_words : tail_words;
+  ra.union_words = (int)union_words;
+  const size_t route_smem = (fixed_words + union_words) * 4;
   if (route_smem > 224 * 1024)
     return fail(ctx, ASAP_ERR_UNSUPPORTED, "max_vis = %d is too large for the routing kernel", in->max_vis);
   ra.salience = salience; ra.mass = mass; ra.keep_idx = keep_idx; ra.drop_idx = drop_idx;

@@ -916,6 +916,7 @@ struct RouteArgs {
   uint32_t *mask_g;               // [B, keep_k, kw] bit matrix in global memory
   int mask_in_smem;               // the bit matrix fits shared memory (else mask_g is used where it lies)
   int mask_written;               // mask_g was filled by the similarity kernel
+  int union_words;                // 32-bit words of the last region of shared memory
   const float *salience, *mass;   // [B, max_vis]
   const int32_t *keep_idx;        // [B, keep_k]            stage 1
   const int32_t *drop_idx;        // [B, max_vis - keep_k]  stage 1
@@ -950,13 +951,15 @@ route_kernel(RouteArgs a) {
     return;
   }
   const int nv = d.nv, nd = nv - k;
-  // shared memory: [order k][rank k][flag k][dest k][tmp k] [union: bit matrix k*kw | key nd_max + pos max_vis]
-  int *s_order = reinterpret_cast<int *>(r_smem);
+  // shared memory: [tmp k4][order k][rank k][flag k][dest k] [union: bit matrix k*kw | key nd_max + pos max_vis], k4 = k rounded up
+  // to a multiple of four
+  const int k4 = (k + 3) & ~3;
+  uint32_t *s_tmp = r_smem;
+  int *s_order = reinterpret_cast<int *>(r_smem + k4);
   int *s_rank = s_order + k;
   int *s_flag = s_rank + k;
   int *s_dest = s_flag + k;
-  uint32_t *s_tmp = r_smem + 4 * (size_t)k;
-  uint32_t *s_union = s_tmp + k;
+  uint32_t *s_union = r_smem + k4 + 4 * (size_t)k;
   uint32_t *mask = a.mask_in_smem ? s_union : a.mask_g + (size_t)b * k * kw;
   const int32_t *keep_b = a.keep_idx + (size_t)b * k;
   const int32_t *drop_b = a.drop_idx + (size_t)b * nd_max;
@@ -968,15 +971,38 @@ route_kernel(RouteArgs a) {
     const int j = min(max(keep_b[p], 0), nv - 1);
     s_tmp[p] = score_key(sal_b[j]);
   }
+  if (tid < k4 - k) s_tmp[k + tid] = 0u;
+  // the attention mass of this thread's first pruned tokens, for E: two dependent loads that end long before they are needed
+  uint32_t mass_key[4];
+#pragma unroll
+  for (int t = 0; t < 4; ++t) {
+    const int i = tid + t * nthr;
+    mass_key[t] = i < nd ? score_key(__ldg(a.mass + (size_t)b * a.max_vis + min(max(__ldg(drop_b + i), 0), nv - 1))) : 0u;
+  }
   __syncthreads();
   for (int p = tid; p < k; p += nthr) {
     const uint32_t mine = s_tmp[p];
+    // the kept list is ascending: an equal key before p is the lower index.  Four keys per (broadcast) load; the keys are
+    // padded to a multiple of four with zeros, which no key after p is below
     int r = 0;
-    int q = 0;
-#pragma unroll 8
-    for (; q < p; ++q) r += s_tmp[q] >= mine;        // the kept list is ascending: an equal one before it is the lower index
-#pragma unroll 8
-    for (++q; q < k; ++q) r += s_tmp[q] > mine;
+    const uint4 *t4 = reinterpret_cast<const uint4 *>(s_tmp);
+    const int pc = p >> 2, nc = k4 >> 2;
+#pragma unroll 4
+    for (int c = 0; c < pc; ++c) {
+      const uint4 o = t4[c];
+      r += (o.x >= mine) + (o.y >= mine) + (o.z >= mine) + (o.w >= mine);
+    }
+    {
+      const uint4 o = t4[pc];
+      const uint32_t ov[4] = {o.x, o.y, o.z, o.w};
+#pragma unroll
+      for (int e = 0; e < 4; ++e) r += ov[e] > mine || (ov[e] == mine && pc * 4 + e < p);
+    }
+#pragma unroll 4
+    for (int c = pc + 1; c < nc; ++c) {
+      const uint4 o = t4[c];
+      r += (o.x > mine) + (o.y > mine) + (o.z > mine) + (o.w > mine);
+    }
     s_rank[p] = r;
     s_order[r] = p;
     s_flag[p] = 0;
@@ -1010,31 +1036,42 @@ route_kernel(RouteArgs a) {
   // ---- C: rounds.  A slot with an earlier anchor among its neighbours is absorbed; one whose earlier neighbours are all
   // absorbed is an anchor; any other waits.  The first undecided slot of the visiting order is decided in every round, and the
   // outcome is that of walking the slots in that order (a slot's fate depends on earlier slots alone).
+  // First every row of the matrix loses the slots that come after its own (a thread works on its own rows only): from then on
+  // a round is a few words of bit operations per slot.
   bool open[4];                                       // this thread's slots tid, tid + nthr, ... (k <= 4096)
 #pragma unroll
-  for (int t = 0; t < 4; ++t) open[t] = tid + t * nthr < k;
+  for (int t = 0; t < 4; ++t) {
+    const int p = tid + t * nthr;
+    open[t] = p < k;
+    if (!open[t]) continue;
+    const int rp = s_rank[p];
+    uint32_t *row = mask + (size_t)p * kw;
+#pragma unroll 4
+    for (int w = 0; w < kw; ++w) {
+      uint32_t word = row[w], rest = word;
+      while (rest) {
+        const int bit = __ffs(rest) - 1;
+        rest &= rest - 1;
+        if (s_rank[w * 32 + bit] > rp) word &= ~(1u << bit);
+      }
+      row[w] = word;
+    }
+  }
   while (true) {
     int verdict[4] = {0, 0, 0, 0};                    // 1 anchor, 2 absorbed
     bool waiting = false;
 #pragma unroll
     for (int t = 0; t < 4; ++t) {
       if (!open[t]) continue;
-      const int p = tid + t * nthr, rp = s_rank[p];
-      const uint32_t *row = mask + (size_t)p * kw;
-      bool absorbed = false, blocked = false;
-      for (int w = 0; w < kw && !absorbed; ++w) {
-        const uint32_t anchors = s_anchor[w];
-        uint32_t cand = row[w] & ~s_gone[w];
-        while (cand) {
-          const int bit = __ffs(cand) - 1;
-          cand &= cand - 1;
-          if (s_rank[w * 32 + bit] < rp) {
-            if ((anchors >> bit) & 1u) { absorbed = true; break; }
-            blocked = true;
-          }
-        }
+      const uint32_t *row = mask + (size_t)(tid + t * nthr) * kw;
+      uint32_t by_anchor = 0u, left = 0u;
+#pragma unroll 4
+      for (int w = 0; w < kw; ++w) {
+        const uint32_t word = row[w];
+        by_anchor |= word & s_anchor[w];
+        left |= word & ~s_gone[w];
       }
-      verdict[t] = absorbed ? 2 : (blocked ? 0 : 1);
+      verdict[t] = by_anchor ? 2 : (left ? 0 : 1);
       if (verdict[t]) open[t] = false;
       else waiting = true;
     }
@@ -1074,17 +1111,15 @@ route_kernel(RouteArgs a) {
     int best_q = -1;
     float best = -INFINITY;
     if (!s_flag[p]) {
-      const int rp = s_rank[p];
       const float *row = S + (size_t)p * k;
+#pragma unroll 4
       for (int w = 0; w < kw; ++w) {
         uint32_t cand = mask[(size_t)p * kw + w] & s_anchor[w];
         while (cand) {
           const int q = w * 32 + __ffs(cand) - 1;
           cand &= cand - 1;
-          if (s_rank[q] < rp) {
-            const float v = __ldcg(row + q);
-            if (v > best) { best = v; best_q = q; }   // ascending q: the first maximum stays
-          }
+          const float v = __ldcg(row + q);
+          if (v > best) { best = v; best_q = q; }     // ascending q: the first maximum stays
         }
       }
     }
@@ -1097,7 +1132,10 @@ route_kernel(RouteArgs a) {
   // ---- E: the n_abs pruned tokens of largest attention mass
   const float *mass_b = a.mass + (size_t)b * a.max_vis;
   for (int v = tid; v < nv; v += nthr) s_pos[v] = 0;
-  for (int i = tid; i < nd; i += nthr) {
+#pragma unroll
+  for (int t = 0; t < 4; ++t)
+    if (tid + t * nthr < nd) s_key[tid + t * nthr] = mass_key[t];
+  for (int i = tid + 4 * nthr; i < nd; i += nthr) {
     const int j = min(max(drop_b[i], 0), nv - 1);
     s_key[i] = score_key(mass_b[j]);
   }
@@ -1202,20 +1240,36 @@ route_kernel(RouteArgs a) {
   }
   if (tid == 0 && a.n_absorbed) a.n_absorbed[b] = n_abs;
   __syncthreads();
-  // grouping by destination (counting sort, stable in source order)
+  // grouping by destination (counting sort, stable in source order): as many warps as there is room for a histogram each, up to
+  // eight, take a contiguous chunk of the sources
   {
     int *s_cnt = s_order;                     // reuse: the visiting order is no longer needed
-    for (int sl = tid; sl < k; sl += nthr) s_cnt[sl] = 0;
+    int *hist = reinterpret_cast<int *>(s_union) + n_abs;      // [W][k] behind the sources' slots
+    const int W = min(8, (a.union_words - n_abs) / k);
+    const int nw = max(W, 1);
+    if (W < 1) hist = s_cnt;                  // (one warp: its histogram becomes the offsets in place)
+    const int chunk = (((n_abs + nw - 1) / nw) + 31) & ~31;
+    const int p_lo = min(n_abs, warp * chunk), p_hi = warp < nw ? min(n_abs, p_lo + chunk) : p_lo;
+    for (int i = tid; i < nw * k; i += nthr) hist[i] = 0;
     __syncthreads();
-    for (int i = tid; i < n_abs; i += nthr) {
+    for (int i = p_lo + lane; i < p_hi; i += 32) {
       const int sl = (int)s_key[i];
-      if (sl >= 0 && sl < k) atomicAdd(&s_cnt[sl], 1);
+      if (sl >= 0 && sl < k) atomicAdd(&hist[warp * k + sl], 1);
     }
     __syncthreads();
     const int per = (k + nthr - 1) / nthr;
     const int lo = min(k, tid * per), hi = min(k, lo + per);
     int mine = 0;
-    for (int sl = lo; sl < hi; ++sl) mine += s_cnt[sl];
+    for (int sl = lo; sl < hi; ++sl) {
+      int run = 0;
+      for (int w = 0; w < nw; ++w) {
+        const int c = hist[w * k + sl];
+        if (W >= 1) hist[w * k + sl] = run;   // this warp's offset inside the slot
+        run += c;
+      }
+      s_cnt[sl] = run;
+      mine += run;
+    }
     int tot;
     int run = block_exclusive_scan(mine, s_scan, tot);
     for (int sl = lo; sl < hi; ++sl) {
@@ -1226,23 +1280,21 @@ route_kernel(RouteArgs a) {
     }
     if (tid == 0) seg_b[k] = tot;
     __syncthreads();
-    // one warp walks the sources 32 at a time in ascending order, so members stay ascending inside a slot
-    if (warp == 0) {
-      for (int base = 0; base < n_abs; base += 32) {
-        const int i = base + lane;
-        int sl = i < n_abs ? (int)s_key[i] : -1;
-        if (sl >= k) sl = -1;
-        const unsigned peers = __match_any_sync(0xffffffffu, sl);
-        const int rank = __popc(peers & ((1u << lane) - 1u));
-        int at = 0;
-        if (sl >= 0) at = s_cnt[sl];
-        __syncwarp();
-        if (sl >= 0) {
-          mem_b[at + rank] = i;
-          if (rank == 0) s_cnt[sl] = at + __popc(peers);
-        }
-        __syncwarp();
+    // every warp walks its chunk 32 sources at a time in ascending order, so members stay ascending inside a slot
+    for (int base = p_lo; base < p_hi; base += 32) {
+      const int i = base + lane;
+      int sl = i < p_hi ? (int)s_key[i] : -1;
+      if (sl >= k) sl = -1;
+      const unsigned peers = __match_any_sync(0xffffffffu, sl);
+      const int rank = __popc(peers & ((1u << lane) - 1u));
+      int at = 0;
+      if (sl >= 0) at = W >= 1 ? hist[warp * k + sl] : s_cnt[sl];
+      __syncwarp();
+      if (sl >= 0) {
+        mem_b[(W >= 1 ? s_cnt[sl] : 0) + at + rank] = i;
+        if (rank == 0) (W >= 1 ? hist[warp * k + sl] : s_cnt[sl]) = at + __popc(peers);
       }
+      __syncwarp();
     }
   }
 }
