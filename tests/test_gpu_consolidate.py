@@ -274,3 +274,21 @@ def test_threshold_minus_infinity_absorbs_until_the_pool_is_empty(ctx):
     out, n_abs, st1 = _run(ctx, batch, 60, -math.inf)
     assert n_abs.tolist() == [30, 50]
     _check(batch, 60, -math.inf, out, n_abs, st1)
+
+
+@pytest.mark.parametrize("nv,k,t", [(700, 273, 0.8), (700, 305, 0.8), (600, 288, 0.8), (320, 300, -2.0), (700, 290, 0.02)],
+                         ids=["half_word", "ragged_word", "whole_words", "all_similar_capped", "long_chains"])
+def test_routing_from_the_written_bit_matrix(nv, k, t):
+    """Batches large enough for the two-row-tile similarity form, which writes the bit matrix of the routing:
+    a last word filled by one half only, a ragged one, none; every pair similar with a refill pool of 20 (the
+    cap); and a threshold in the noise, so that many rounds are needed until every slot is decided.  The oracle
+    checks the first, a middle and the last sequence."""
+    B = 20
+    c = A.asap_init(0, max_total_tokens=B * (nv + 40), max_B=B, max_H=2, max_D=256, max_keep_rows=B * k)
+    try:
+        batch = W.tiny(B=B, n_vis=[nv] * B, text_lens=[5] * B, H=2, keep_k=k, seed=900 + k, centres=k // 5)
+        out, n_abs, st1 = _run(c, batch, k, t, stage1=lambda bt, b, kk: W.random_stage1(bt, b, kk, 31))
+        _check(batch, k, t, out, n_abs, st1, samples=[0, 9, B - 1])
+        assert n_abs.min() > 0
+    finally:
+        A.asap_free(c)
