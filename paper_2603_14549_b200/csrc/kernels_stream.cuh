@@ -1355,6 +1355,7 @@ merge_compact_kernel(MergeArgs a) {
   const int nvec = a.D / 8;
   const int k = a.keep_k;
   if ((int)blockIdx.x >= k) {
+    if (blockIdx.z) return;
     // ---------------------------------------------------------------- copy rows, one per warp
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int c = ((int)blockIdx.x - k) * MERGE_COPY_ROWS + warp;     // index among prefix + suffix rows
@@ -1384,7 +1385,8 @@ merge_compact_kernel(MergeArgs a) {
   const int vi = min(max(a.keep_idx[(size_t)b * k + slot], 0), d.nv - 1);   // visual index
   const size_t grow = (size_t)(d.row0 + d.v0 + vi);
   const int orow = d.out_row0 + d.v0 + slot;
-  if (threadIdx.x == 0) {
+  const int v0 = blockIdx.z * (NV * MERGE_THREADS) + threadIdx.x;       // grid z: pieces of NV * 256 vectors of the row
+  if (threadIdx.x == 0 && blockIdx.z == 0) {
     a.out_pos[orow] = a.pos_ids[grow];
     a.src_row[orow] = (int32_t)grow;
   }
@@ -1401,13 +1403,13 @@ merge_compact_kernel(MergeArgs a) {
   uint4 self[NV];
 #pragma unroll
   for (int u = 0; u < NV; ++u) {
-    const int v = threadIdx.x + u * MERGE_THREADS;
+    const int v = v0 + u * MERGE_THREADS;
     if (v < nvec) self[u] = __ldg(src + v);
   }
   if (m_hi <= m_lo) {
 #pragma unroll
     for (int u = 0; u < NV; ++u) {
-      const int v = threadIdx.x + u * MERGE_THREADS;
+      const int v = v0 + u * MERGE_THREADS;
       if (v < nvec) dst[v] = self[u];
     }
     return;
@@ -1490,7 +1492,7 @@ merge_compact_kernel(MergeArgs a) {
           const uint4 *msrc = reinterpret_cast<const uint4 *>(vis0 + (size_t)s_j[m0 + t] * a.D);
 #pragma unroll
           for (int u = 0; u < NV; ++u) {
-            const int v = threadIdx.x + u * MERGE_THREADS;
+            const int v = v0 + u * MERGE_THREADS;
             if (v < nvec) x[t][u] = __ldg(msrc + v);
           }
         }
@@ -1514,14 +1516,14 @@ merge_compact_kernel(MergeArgs a) {
   if (den <= a.eps || !merged) {
 #pragma unroll
     for (int u = 0; u < NV; ++u) {
-      const int v = threadIdx.x + u * MERGE_THREADS;
+      const int v = v0 + u * MERGE_THREADS;
       if (v < nvec) dst[v] = self[u];
     }
   } else {
     const float inv = 1.0f / den;
 #pragma unroll
     for (int u = 0; u < NV; ++u) {
-      const int v = threadIdx.x + u * MERGE_THREADS;
+      const int v = v0 + u * MERGE_THREADS;
       if (v < nvec) {
         uint4 o;
         o.x = pack2_rn(acc[u][0] * inv, acc[u][1] * inv);
