@@ -447,6 +447,26 @@ salience_heads_kernel(const SampleDesc *__restrict__ desc, int max_vis, Salience
 // =======================================================================================
 constexpr int SAL_THREADS = 1024;
 
+// Sums over the heads, in head order, of four neighbouring columns (max_vis a multiple of four): 16-byte loads, sixteen in
+// flight.  With 4-byte loads the request rate of one SM bound this (2880 columns x 32 heads: 18 thousand clocks).
+__device__ __forceinline__ bool wide_columns(int max_vis, int nv) { return (max_vis & 3) == 0 && nv > SAL_THREADS; }
+__device__ __forceinline__ float4 head_sum4(const float *p, int H, int max_vis) {
+  float4 t = make_float4(0.f, 0.f, 0.f, 0.f);
+  int hh = 0;
+  for (; hh + 8 <= H; hh += 8) {
+    float4 v[8];
+#pragma unroll
+    for (int e = 0; e < 8; ++e) v[e] = __ldcg(reinterpret_cast<const float4 *>(p + (size_t)(hh + e) * max_vis));
+#pragma unroll
+    for (int e = 0; e < 8; ++e) { t.x += v[e].x; t.y += v[e].y; t.z += v[e].z; t.w += v[e].w; }
+  }
+  for (; hh < H; ++hh) {
+    const float4 v = __ldcg(reinterpret_cast<const float4 *>(p + (size_t)hh * max_vis));
+    t.x += v.x; t.y += v.y; t.z += v.z; t.w += v.w;
+  }
+  return t;
+}
+
 __device__ __forceinline__ void salience_block(const SampleDesc &d, int b, int max_vis, const SalienceArgs &a) {
   __shared__ float s_red[2 * (SAL_THREADS / 32)];
   float *mass_b = a.mass + (size_t)b * max_vis, *sal_b = a.salience + (size_t)b * max_vis, *msk_b = a.mask_log + (size_t)b * max_vis;
@@ -461,7 +481,20 @@ __device__ __forceinline__ void salience_block(const SampleDesc &d, int b, int m
   }
   const float *hb = a.heads + (size_t)b * H * max_vis;
   float lo = INFINITY, hi = -INFINITY;
-  for (int j = threadIdx.x; j < d.nv; j += SAL_THREADS) {
+  const bool vec = wide_columns(max_vis, d.nv);
+  if (vec) {
+    for (int j = threadIdx.x * 4; j < d.nv; j += SAL_THREADS * 4) {
+      const float4 t4 = head_sum4(hb + j, H, max_vis);
+      const float tv[4] = {t4.x * scale, t4.y * scale, t4.z * scale, t4.w * scale};
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        if (j + e >= d.nv) break;
+        mass_b[j + e] = tv[e];
+        lo = fminf(lo, tv[e]); hi = fmaxf(hi, tv[e]);
+      }
+    }
+  }
+  for (int j = vec ? d.nv : (int)threadIdx.x; j < d.nv; j += SAL_THREADS) {
     float tot = 0.f;
     int hh = 0;
     for (; hh + 16 <= H; hh += 16) {          // sixteen loads in flight
@@ -492,7 +525,7 @@ __device__ __forceinline__ void salience_block(const SampleDesc &d, int b, int m
   const float inv = 1.0f / ((hi - lo) + eps);
   for (int j = threadIdx.x; j < max_vis; j += SAL_THREADS) {
     if (j < d.nv) {
-      const float sh = (mass_b[j] - lo) * inv;      // this thread's own store above
+      const float sh = (mass_b[j] - lo) * inv;      // (stored above, before the block's barrier)
       sal_b[j] = sh;
       msk_b[j] = logf(fmaxf(lambda_max * sh, eps));
     } else {
@@ -559,8 +592,8 @@ select_kernel(const float *__restrict__ rank_score, const SampleDesc *__restrict
   extern __shared__ uint32_t s_key[];   // [max_vis]
   __shared__ int s_hist[256];
   __shared__ int s_scan[33];
-  __shared__ uint32_t s_prefix;
-  __shared__ int s_remaining;
+  __shared__ uint32_t s_prefix, s_lo[32], s_hi[32];
+  __shared__ int s_remaining, s_bucket;
   const int b = blockIdx.x;
   const SampleDesc d = desc[b];
   const int nd_max = max_vis - keep_k;
@@ -587,7 +620,20 @@ select_kernel(const float *__restrict__ rank_score, const SampleDesc *__restrict
     // r_j = mean over heads and ranking rows of the Eq. 4 probabilities: the per-head sums
     // over ranking rows are added here in head order, and r is also written out
     const float inv = 1.0f / ((float)H * (float)d.nr);
-    for (int j = threadIdx.x; j < max_vis; j += blockDim.x) {
+    const bool vec = wide_columns(max_vis, nv);
+    if (vec) {
+      for (int j = threadIdx.x * 4; j < max_vis; j += SELECT_THREADS * 4) {
+        const float4 t4 = j < nv ? head_sum4(head_partial + (size_t)b * H * max_vis + j, H, max_vis) : make_float4(0.f, 0.f, 0.f, 0.f);
+        const float tv[4] = {t4.x, t4.y, t4.z, t4.w};
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          const float tot = j + e < nv ? tv[e] * inv : 0.f;
+          if (j + e < nv) s_key[j + e] = score_key(tot);
+          rank_out[(size_t)b * max_vis + j + e] = tot;
+        }
+      }
+    }
+    for (int j = vec ? max_vis : (int)threadIdx.x; j < max_vis; j += blockDim.x) {
       float tot = 0.f;
       if (j < nv) {
         const float *p = head_partial + (size_t)b * H * max_vis + j;
@@ -616,54 +662,73 @@ select_kernel(const float *__restrict__ rank_score, const SampleDesc *__restrict
     for (int j = threadIdx.x; j < nv; j += blockDim.x)
       s_key[j] = score_key(rank_score[(size_t)b * max_vis + j]);
   }
-  if (threadIdx.x == 0) { s_prefix = 0u; s_remaining = keep_k; }
   __syncthreads();
+  // The bits in which the keys differ at all: scores of one sequence share their sign and most of their exponent, and a digit
+  // that all keys have in common costs a pass of atomics on one counter.
+  uint32_t k_lo = 0xffffffffu, k_hi = 0u;
+  for (int j = threadIdx.x; j < nv; j += blockDim.x) { k_lo = min(k_lo, s_key[j]); k_hi = max(k_hi, s_key[j]); }
+  k_lo = __reduce_min_sync(0xffffffffu, k_lo);
+  k_hi = __reduce_max_sync(0xffffffffu, k_hi);
+  if ((threadIdx.x & 31) == 0) { s_lo[threadIdx.x >> 5] = k_lo; s_hi[threadIdx.x >> 5] = k_hi; }
+  for (int i = threadIdx.x; i < 256; i += blockDim.x) s_hist[i] = 0;
+  __syncthreads();
+  k_lo = __reduce_min_sync(0xffffffffu, s_lo[threadIdx.x & 31]);
+  k_hi = __reduce_max_sync(0xffffffffu, s_hi[threadIdx.x & 31]);
+  const int top = k_lo == k_hi ? 0 : 32 - __clz(k_lo ^ k_hi);        // the keys agree in all bits from `top` up
 
-  // four 8-bit digits, most significant first: find the key of the keep_k-th largest score
-  uint32_t known = 0u;   // mask of the digits fixed so far
-  for (int shift = 24; shift >= 0; shift -= 8) {
-    for (int i = threadIdx.x; i < 256; i += blockDim.x) s_hist[i] = 0;
-    __syncthreads();
-    const uint32_t prefix = s_prefix;
+  // 8-bit digits, most significant first, until the bucket of the keep_k-th largest score is kept whole: that score's key
+  // (or, when the pass ends early, the key just below the bucket)
+  uint32_t known = top >= 32 ? 0u : ~((1u << top) - 1u);   // mask of the digits fixed so far
+  uint32_t prefix = k_lo & known;
+  int remaining = keep_k;
+  for (int hi_bit = top; hi_bit > 0;) {
+    const int shift = max(hi_bit - 8, 0);
     for (int j = threadIdx.x; j < nv; j += blockDim.x) {
       const uint32_t key = s_key[j];
-      if ((key & known) == prefix) atomicAdd(&s_hist[(key >> shift) & 255u], 1);
+      if ((key & known) == prefix) atomicAdd(&s_hist[(key >> shift) & ((1u << (hi_bit - shift)) - 1u)], 1);
     }
     __syncthreads();
     if (threadIdx.x < 32) {
       const int lane = threadIdx.x;
       // lane L owns digits 255-8L .. 248-8L (descending); find where the running count reaches `remaining`
-      int mine = 0;
+      int c[8], mine = 0;
 #pragma unroll
-      for (int e = 0; e < 8; ++e) mine += s_hist[255 - 8 * lane - e];
+      for (int e = 0; e < 8; ++e) { c[e] = s_hist[255 - 8 * lane - e]; mine += c[e]; }
       int inc = mine;
 #pragma unroll
       for (int o = 1; o < 32; o <<= 1) {
         int t = __shfl_up_sync(0xffffffffu, inc, o);
         if (lane >= o) inc += t;
       }
-      const int remaining = s_remaining;
-      __syncwarp();   // every lane has read s_remaining before one of them rewrites it
       const int before = inc - mine;
       if (before < remaining && remaining <= inc) {
         int run = before;
+#pragma unroll
         for (int e = 0; e < 8; ++e) {
-          const int digit = 255 - 8 * lane - e;
-          const int c = s_hist[digit];
-          if (run + c >= remaining) {
-            s_prefix = prefix | ((uint32_t)digit << shift);
+          if (run < remaining && run + c[e] >= remaining) {
+            s_prefix = prefix | ((uint32_t)(255 - 8 * lane - e) << shift);
             s_remaining = remaining - run;
-            break;
+            s_bucket = c[e];
           }
-          run += c;
+          run += c[e];
         }
       }
+      // the counters of the next pass
+      __syncwarp();
+#pragma unroll
+      for (int e = 0; e < 8; ++e) s_hist[255 - 8 * lane - e] = 0;
     }
-    known |= 255u << shift;
+    known |= ((1u << (hi_bit - shift)) - 1u) << shift;
+    hi_bit = shift;
     __syncthreads();
+    prefix = s_prefix;
+    remaining = s_remaining;
+    if (remaining == s_bucket) {            // the whole bucket is kept: everything above the key just below it
+      if (prefix != 0u) { prefix -= 1u; remaining = 0; break; }
+    }
   }
-  const uint32_t kth = s_prefix;      // key of the keep_k-th largest score
-  const int take_equal = s_remaining; // how many tokens with exactly that key are kept (lowest indices)
+  const uint32_t kth = prefix;        // key of the keep_k-th largest score
+  const int take_equal = remaining;   // how many tokens with exactly that key are kept (lowest indices)
 
   // ordered emission: thread t owns the contiguous indices [t*per, (t+1)*per)
   const int per = (nv + blockDim.x - 1) / blockDim.x;
