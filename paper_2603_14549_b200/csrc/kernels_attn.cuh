@@ -172,12 +172,23 @@ attn_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__ 
     reg_dec<72>();
     if (warp == 0) {
       // ---------------------------------------------------------------- items, query / key / value tiles
-      if (lane == 0) {
-        int ic = 0;                               // items published
-        bool first = true;                        // every block's first item is its own number, the others are drawn
-        // Draws the next item that has rows and publishes it.  The item queue keeps working after an abort (its waits
-        // ignore the flag and are bounded on their own): every consumer must see the same sequence, ending with -1.
-        auto draw = [&](AttnItem &it) {
+      // (the whole warp walks the loop and stays converged, see tma_load_2d_w; lane 0 draws the items)
+      const uint32_t leader = warp_leader();
+      int ic = 0;                                 // items published
+      bool first = true;                          // every block's first item is its own number, the others are drawn
+      // Draws the next item that has rows and publishes it.  The item queue keeps working after an abort (its waits
+      // ignore the flag and are bounded on their own): every consumer must see the same sequence, ending with -1.
+      auto draw = [&](AttnItem &it) {
+        const int slot = ic % AT_ITEM_SLOTS;
+        bool room = true;
+        if (ic >= AT_ITEM_SLOTS)
+          room = mbar_wait_drain(smem_u32(&bk->item_empty[slot]), ((ic / AT_ITEM_SLOTS) - 1) & 1, AT_WAIT_LIMIT);
+        __syncwarp();
+        if (!__shfl_sync(0xffffffffu, room ? 1 : 0, 0)) {
+          it.b = -1;
+          return;
+        }
+        if (lane == 0) {
           while (true) {
             const int item = bk->abort_flag ? a.n_items : (first ? (int)blockIdx.x : (int)(gridDim.x + atomicAdd(a.work, 1u)));
             first = false;
@@ -195,67 +206,65 @@ attn_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__ 
             if (it.q_base + 128 < d.n) it.n_kt[1] = (attn_key_end(d, it.q_base + 128, a.mask_enable, it.sees[1]) + 127) / 128;
             break;
           }
-          const int slot = ic % AT_ITEM_SLOTS;
-          if (ic >= AT_ITEM_SLOTS &&
-              !mbar_wait_drain(smem_u32(&bk->item_empty[slot]), ((ic / AT_ITEM_SLOTS) - 1) & 1, AT_WAIT_LIMIT)) {
-            it.b = -1;
-            return;
-          }
           bk->item[slot] = it;
           mbar_arrive(smem_u32(&bk->item_full[slot]));      // release: the slot's content is visible to the waiters
-          ++ic;
-        };
-        AttnItem cur, nxt;
-        int tc = 0, qc[2] = {0, 0};               // key / value tiles and query tiles so far
-        int t_issued = 0, q_issued[2] = {0, 0};   // copies actually issued
-        draw(cur);
-        while (cur.b >= 0) {
-          auto load_q = [&](int g) {
-            if (cur.n_kt[g] == 0) return;
-            if (qc[g] >= 1) mbar_wait(smem_u32(&bk->q_empty[g]), (qc[g] - 1) & 1, wc);
-            if (!bk->abort_flag) {
-              const uint32_t bar = smem_u32(&bk->q_full[g]);
-              const int row = cur.row0 + cur.q_base + g * 128;
-              mbar_expect_tx(bar, AT_TILE_BYTES);
-              tma_load_2d(q_smem + g * AT_TILE_BYTES, &tmap_q, bar, cur.h * 128, row);
-              tma_load_2d(q_smem + g * AT_TILE_BYTES + AT_BLOCK_BYTES, &tmap_q, bar, cur.h * 128 + 64, row);
-              q_issued[g] = qc[g] + 1;
-            }
-            ++qc[g];
-          };
-          auto load_tile = [&](const CUtensorMap *map, int kt) {
-            const int s = tc % AT_SLOTS;
-            if (tc >= AT_SLOTS) mbar_wait(smem_u32(&bk->empty[s]), ((tc / AT_SLOTS) - 1) & 1, wc);
-            if (!bk->abort_flag) {
-              const uint32_t bar = smem_u32(&bk->full[s]), dst = ring + s * AT_TILE_BYTES;
-              const int row = cur.row0 + kt * 128;
-              mbar_expect_tx(bar, AT_TILE_BYTES);
-              tma_load_2d(dst, map, bar, cur.h * 128, row);
-              tma_load_2d(dst + AT_BLOCK_BYTES, map, bar, cur.h * 128 + 64, row);
-              t_issued = tc + 1;
-            }
-            ++tc;
-          };
-          const int n_max = max(cur.n_kt[0], cur.n_kt[1]);
-          load_q(0);
-          load_tile(&tmap_k, 0);
-          load_q(1);
-          load_tile(&tmap_v, 0);
-          draw(nxt);                              // its look-ups overlap this item's work
-          for (int kt = 1; kt < n_max; ++kt) {
-            load_tile(&tmap_k, kt);
-            load_tile(&tmap_v, kt);
+        }
+        __syncwarp();
+        it = bk->item[slot];                      // (the slot is not reused before this warp draws four more)
+        ++ic;
+      };
+      AttnItem cur, nxt;
+      int tc = 0, qc[2] = {0, 0};                 // key / value tiles and query tiles so far
+      int t_issued = 0, q_issued[2] = {0, 0};     // copies actually issued
+      auto stopped = [&]() { return __shfl_sync(0xffffffffu, bk->abort_flag, 0) != 0; };
+      draw(cur);
+      while (cur.b >= 0) {
+        auto load_q = [&](int g) {
+          if (cur.n_kt[g] == 0) return;
+          if (qc[g] >= 1) mbar_wait_warp(smem_u32(&bk->q_empty[g]), (qc[g] - 1) & 1, wc);
+          if (!stopped()) {
+            const uint32_t bar = smem_u32(&bk->q_full[g]);
+            const int row = cur.row0 + cur.q_base + g * 128;
+            mbar_expect_tx_w(bar, AT_TILE_BYTES, leader);
+            tma_load_2d_w(q_smem + g * AT_TILE_BYTES, &tmap_q, bar, cur.h * 128, row, leader);
+            tma_load_2d_w(q_smem + g * AT_TILE_BYTES + AT_BLOCK_BYTES, &tmap_q, bar, cur.h * 128 + 64, row, leader);
+            q_issued[g] = qc[g] + 1;
           }
-          cur = nxt;
+          ++qc[g];
+        };
+        auto load_tile = [&](const CUtensorMap *map, int kt) {
+          const int s = tc % AT_SLOTS;
+          if (tc >= AT_SLOTS) mbar_wait_warp(smem_u32(&bk->empty[s]), ((tc / AT_SLOTS) - 1) & 1, wc);
+          if (!stopped()) {
+            const uint32_t bar = smem_u32(&bk->full[s]), dst = ring + s * AT_TILE_BYTES;
+            const int row = cur.row0 + kt * 128;
+            mbar_expect_tx_w(bar, AT_TILE_BYTES, leader);
+            tma_load_2d_w(dst, map, bar, cur.h * 128, row, leader);
+            tma_load_2d_w(dst + AT_BLOCK_BYTES, map, bar, cur.h * 128 + 64, row, leader);
+            t_issued = tc + 1;
+          }
+          ++tc;
+        };
+        const int n_max = max(cur.n_kt[0], cur.n_kt[1]);
+        load_q(0);
+        load_tile(&tmap_k, 0);
+        load_q(1);
+        load_tile(&tmap_v, 0);
+        draw(nxt);                                // its look-ups overlap this item's work
+        for (int kt = 1; kt < n_max; ++kt) {
+          load_tile(&tmap_k, kt);
+          load_tile(&tmap_v, kt);
         }
-        // drain: every copy issued must have landed before the block leaves
-        for (int g = 0; g < 2; ++g)
-          if (q_issued[g] > 0) mbar_wait_drain(smem_u32(&bk->q_full[g]), (q_issued[g] - 1) & 1, AT_WAIT_LIMIT);
-        for (int s = 0; s < AT_SLOTS; ++s) {
-          const int fills = t_issued > s ? (t_issued - s + AT_SLOTS - 1) / AT_SLOTS : 0;
-          if (fills > 0) mbar_wait_drain(smem_u32(&bk->full[s]), (fills - 1) & 1, AT_WAIT_LIMIT);
-        }
+        cur = nxt;
       }
+      // drain: every copy issued must have landed before the block leaves
+      for (int g = 0; g < 2; ++g)
+        if (q_issued[g] > 0) mbar_wait_drain(smem_u32(&bk->q_full[g]), (q_issued[g] - 1) & 1, AT_WAIT_LIMIT);
+      for (int s = 0; s < AT_SLOTS; ++s) {
+        const int fills = t_issued > s ? (t_issued - s + AT_SLOTS - 1) / AT_SLOTS : 0;
+        if (fills > 0) mbar_wait_drain(smem_u32(&bk->full[s]), (fills - 1) & 1, AT_WAIT_LIMIT);
+      }
+      __syncwarp();
     } else if (warp == 1) {
       // ---------------------------------------------------------------- MMA issuer
       // Per key tile and row tile: S of this key tile, then P V of the PREVIOUS one.  In that order an S never waits in the
