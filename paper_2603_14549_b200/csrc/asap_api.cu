@@ -410,8 +410,23 @@ asap_status launch_merge_front(asap_ctx *ctx, const asap_inputs *in, const asap_
     // SM).  Gathering is taken for batches large enough not to be sliced, from two fifths of the rows kept
     // (measured at a fifth, 576 of 2880: 1.11 ms gathered against 1.04 ms tiled; at a half, 1152 of 2304:
     // 0.56 ms against 0.92 ms).
-    const bool gather_rows = splits == 1 && (long long)k * 5 >= 2LL * in->max_vis &&
-                             (long long)max_mt * B > ctx->num_sms;
+    bool gather_rows = splits == 1 && (long long)k * 5 >= 2LL * in->max_vis && (long long)max_mt * B > ctx->num_sms;
+    // The gathered form makes a single pass over the hidden dimension with all of a block's accumulators live: more than 384
+    // kept slots are dealt in groups (of one or two tiles) to neighbouring blocks, and the last block of a row tile combines
+    // the groups' best slots.  Several passes inside one block would read the dropped rows from memory once per pass: the rows
+    // that all resident blocks hold between two passes do not fit L2.
+    int groups = 1;
+    if (gather_rows) {
+      const int mt_g = (in->max_vis - k + 127) / 128;
+      int g = (k + 383) / 384;
+      const int per_group = (k + g - 1) / g;
+      const int tiles_g = per_group > 256 ? 2 : 1;
+      const int tile_g = (((per_group + tiles_g - 1) / tiles_g) + 15) & ~15;
+      g = (k + tiles_g * tile_g - 1) / (tiles_g * tile_g);
+      gather_rows = (size_t)B * mt_g <= ctx->cap_tiles &&
+                    (g == 1 || (size_t)B * mt_g * g * 256 * sizeof(float) <= ctx->sim_part_bytes);
+      if (gather_rows) { groups = g; n_nt = tiles_g; n_tile = tile_g; max_mt = mt_g; }
+    }
     // Every visual row, two row tiles per block, the kept slots dealt in groups of at most 256 to the
     // blocks of a pair, one pass each: fewer bytes out of L2 per product, which is what bounds the
     // similarity of a large batch.  Taken when that grid fills at least half of the SMs (measured: 96 blocks
@@ -438,7 +453,7 @@ asap_status launch_merge_front(asap_ctx *ctx, const asap_inputs *in, const asap_
           return fail(ctx, ASAP_ERR_CUDA, "cuTensorMapEncodeTiled failed for hidden / kept rows");
         SimArgs sa;
         sa.desc = ctx->desc; sa.D = D; sa.max_vis = in->max_vis; sa.keep_k = k; sa.n_tile = ptile;
-        sa.n_nt = 1; sa.stages = pstages; sa.splits = 1; sa.max_mt = pairs; sa.tmem_cols = pcols;
+        sa.n_nt = 1; sa.stages = pstages; sa.a_stages = 0; sa.splits = 1; sa.max_mt = pairs; sa.tmem_cols = pcols;
         sa.wide = 1; sa.groups = pg; sa.cluster = 0; sa.threshold = p->sim_threshold;
         sa.drop_idx = nullptr; sa.role = ctx->role;
         sa.hidden = static_cast<const __nv_bfloat16 *>(in->hidden); sa.kept_inv = ctx->kept_inv; sa.assign = out->assign;
@@ -451,24 +466,7 @@ asap_status launch_merge_front(asap_ctx *ctx, const asap_inputs *in, const asap_
         return after_launch(ctx, "sim");
       }
     }
-    if (gather_rows) max_mt = (in->max_vis - k + 127) / 128;
-    bool wide = n_nt >= 2 && n_nt * n_tile <= 512 && 3 * (SIM_A_BYTES + n_nt * n_tile * 128) <= 192 * 1024;
-    // More slots than that, and enough row tiles that the hidden dimension is not sliced: the slot tiles are
-    // dealt to several blocks per row tile (groups of at most 384 slots = one or two tiles), each a single
-    // pass in the layout above; the last block of a row tile combines the groups' best slots.  Several
-    // passes inside one block would read the dropped rows from memory once per pass: the rows that all
-    // resident blocks hold between two passes do not fit L2.
-    int groups = 1;
-    if (gather_rows && !wide && n_nt >= 2 && D % 64 == 0 && (size_t)B * max_mt <= ctx->cap_tiles) {
-      int g = (k + 383) / 384;
-      const int per_group = (k + g - 1) / g;
-      const int tiles_g = per_group > 256 ? 2 : 1;
-      const int tile_g = (((per_group + tiles_g - 1) / tiles_g) + 15) & ~15;
-      g = (k + tiles_g * tile_g - 1) / (tiles_g * tile_g);
-      if ((size_t)B * max_mt * g * 256 * sizeof(float) <= ctx->sim_part_bytes) {
-        groups = g; n_nt = tiles_g; n_tile = tile_g; wide = true;
-      }
-    }
+    const bool wide = gather_rows || (n_nt >= 2 && n_nt * n_tile <= 512 && 3 * (SIM_A_BYTES + n_nt * n_tile * 128) <= 192 * 1024);
     const int stage_bytes = 2 * (SIM_A_BYTES + n_tile * 128);   // two adjacent 64-column blocks per stage
     uint32_t tmem_cols = 32;
     while ((int)tmem_cols < (wide ? n_nt * n_tile : 2 * n_tile)) tmem_cols <<= 1;
@@ -480,9 +478,20 @@ asap_status launch_merge_front(asap_ctx *ctx, const asap_inputs *in, const asap_
     // the SM its 32 KB of L1
     int stages = ((two_per_sm ? 96 : 192) * 1024) / stage_bytes_used;
     if (stages > SIM_MAX_STAGES) stages = SIM_MAX_STAGES;
-    const size_t smem = (size_t)stages * stage_bytes_used + SIM_BOOK_BYTES + 1024;
+    // gathered form: the rows arrive slowly (16 KB in about 1000 clocks, the load unit's requests in flight) and the kept rows
+    // fast, so the rows have a ring of their own with as many slots as the kept rows leave (one ring of three stages with both:
+    // three steps of 32 x 2304, 5120 wide, 887 -> 773 us)
+    const int b_tile = n_nt * n_tile * 128;
+    int a_stages = 0;
+    if (gather_rows) {
+      stages = b_tile > 32 * 1024 ? 2 : 3;
+      a_stages = (192 * 1024 - stages * b_tile) / SIM_A_BYTES;
+      if (a_stages > SIM_MAX_STAGES) a_stages = SIM_MAX_STAGES;
+    }
+    const size_t ring = gather_rows ? (size_t)a_stages * SIM_A_BYTES + (size_t)stages * b_tile : (size_t)stages * stage_bytes_used;
+    const size_t smem = ring + SIM_BOOK_BYTES + 1024;
     const int sim_threads = gather_rows ? SIM_THREADS : SIM_THREADS_TILED;
-    if ((size_t)(sim_threads / 32 + 1) * k * sizeof(int) > (size_t)stages * stage_bytes_used)
+    if ((size_t)(sim_threads / 32 + 1) * k * sizeof(int) > ring)
       return fail(ctx, ASAP_ERR_UNSUPPORTED, "keep_k = %d is too large for the merge path", k);
     CUtensorMap map_h, map_kept;
     if (!make_map(ctx, &map_h, in->hidden, (uint64_t)in->total_tokens, (uint64_t)D, 128) ||
@@ -490,7 +499,7 @@ asap_status launch_merge_front(asap_ctx *ctx, const asap_inputs *in, const asap_
       return fail(ctx, ASAP_ERR_CUDA, "cuTensorMapEncodeTiled failed for hidden / kept rows");
     SimArgs sa;
     sa.desc = ctx->desc; sa.D = D; sa.max_vis = in->max_vis; sa.keep_k = k; sa.n_tile = n_tile;
-    sa.n_nt = n_nt; sa.stages = stages; sa.splits = splits; sa.max_mt = max_mt; sa.tmem_cols = tmem_cols;
+    sa.n_nt = n_nt; sa.stages = stages; sa.a_stages = a_stages; sa.splits = splits; sa.max_mt = max_mt; sa.tmem_cols = tmem_cols;
     sa.wide = wide ? 1 : 0;
     sa.groups = groups;
     const bool cluster = cluster_ok && splits > 1 && !wide && !gather_rows &&
@@ -606,7 +615,7 @@ asap_status launch_consolidate_front(asap_ctx *ctx, const asap_inputs *in, const
         return fail(ctx, ASAP_ERR_CUDA, "cuTensorMapEncodeTiled failed for the kept rows");
       SimArgs sa;
       sa.desc = ctx->desc; sa.D = D; sa.max_vis = in->max_vis; sa.keep_k = k; sa.n_tile = ptile;
-      sa.n_nt = 1; sa.stages = pstages; sa.splits = 1; sa.max_mt = pairs; sa.tmem_cols = pcols;
+      sa.n_nt = 1; sa.stages = pstages; sa.a_stages = 0; sa.splits = 1; sa.max_mt = pairs; sa.tmem_cols = pcols;
       sa.wide = 1; sa.groups = pg; sa.cluster = 0; sa.threshold = p->sim_threshold;
       sa.drop_idx = nullptr; sa.role = nullptr; sa.drop_all = nullptr; sa.hidden = nullptr; sa.kept_inv = ctx->kept_inv;
       sa.assign = nullptr; sa.best_sim = nullptr; sa.seg = nullptr; sa.members = nullptr; sa.counters = nullptr;
@@ -652,7 +661,7 @@ asap_status launch_consolidate_front(asap_ctx *ctx, const asap_inputs *in, const
     return fail(ctx, ASAP_ERR_CUDA, "cuTensorMapEncodeTiled failed for the kept rows");
   SimArgs sa;
   sa.desc = ctx->desc; sa.D = D; sa.max_vis = in->max_vis; sa.keep_k = k; sa.n_tile = n_tile;
-  sa.n_nt = n_nt; sa.stages = stages; sa.splits = splits; sa.max_mt = max_mt; sa.tmem_cols = tmem_cols;
+  sa.n_nt = n_nt; sa.stages = stages; sa.a_stages = 0; sa.splits = splits; sa.max_mt = max_mt; sa.tmem_cols = tmem_cols;
   sa.wide = 0;
   sa.groups = 1;
   const bool cluster = cluster_ok && splits > 1 &&

@@ -781,10 +781,12 @@ constexpr int SIM_A_BYTES = 128 * 128;           // 128 rows x 64 bf16
 constexpr int SIM_BOOK_BYTES = 2048;
 constexpr uint32_t SIM_TMEM_COLS = 512;
 constexpr int SIM_MAX_STAGES = 8;
+constexpr int SIM_B_STAGES = 4;
 
 struct SimArgs {
   const SampleDesc *desc;
   int D, max_vis, keep_k, n_tile, n_nt, stages, splits, max_mt;
+  int a_stages;              // gathered form: slots of the row ring (`stages` counts those of the kept-row ring)
   int wide;                  // 1: one pass, all slot tiles' accumulators live at once
   int groups;                // > 1: slot tiles dealt to `groups` blocks per row tile (n_nt counts one group's tiles)
   int cluster;               // 1: the `splits` slices of a row tile form a thread-block cluster (grid z) and add their
@@ -816,6 +818,7 @@ struct SimArgs {
 
 struct SimBook {
   uint64_t full[SIM_MAX_STAGES], empty[SIM_MAX_STAGES], acc_full[2], acc_empty[2], mma_done;
+  uint64_t full_b[SIM_B_STAGES], empty_b[SIM_B_STAGES];   // gathered form: the kept rows' own ring
   uint32_t tmem_base;
   int abort_flag;
   int is_last;
@@ -899,7 +902,9 @@ sim_kernel(const __grid_constant__ CUtensorMap tmap_h, const __grid_constant__ C
   // [ rows, block 0 | rows, block 1 | kept, block 0 | kept, block 1 ]
   const int b_bytes = a.n_tile * 128;
   const int stage_bytes = a.wide ? SIM_A_BYTES + a.n_nt * b_bytes : 2 * (SIM_A_BYTES + b_bytes);
-  SimBook *bk = reinterpret_cast<SimBook *>(base_ptr + (size_t)a.stages * stage_bytes);
+  // (gathered form: a ring of a_stages row tiles, then one of `stages` kept-row tiles, one 64-column block each)
+  const int ring_bytes = GATHER ? a.a_stages * SIM_A_BYTES + a.stages * a.n_nt * b_bytes : a.stages * stage_bytes;
+  SimBook *bk = reinterpret_cast<SimBook *>(base_ptr + (size_t)ring_bytes);
   if (n_rows <= 0) {
     // nothing was dropped in this sample: only the (empty) grouping has to be written
     pdl_enter();
@@ -908,8 +913,14 @@ sim_kernel(const __grid_constant__ CUtensorMap tmap_h, const __grid_constant__ C
   }
 
   if (threadIdx.x == 0) {
-    for (int s = 0; s < a.stages; ++s) {
-      mbar_init(smem_u32(&bk->full[s]), GATHER ? 1 + 32 * SIM_GWARPS : 1);  // the copy warp's announcement (+ every gather thread)
+    if (GATHER) {
+      for (int s = 0; s < a.stages; ++s) {
+        mbar_init(smem_u32(&bk->full_b[s]), 1);
+        mbar_init(smem_u32(&bk->empty_b[s]), 1);
+      }
+    }
+    for (int s = 0; s < (GATHER ? a.a_stages : a.stages); ++s) {
+      mbar_init(smem_u32(&bk->full[s]), GATHER ? 32 * SIM_GWARPS : 1);      // every gather thread, or the copy warp's announcement
       mbar_init(smem_u32(&bk->empty[s]), 5);      // the MMAs that read the stage + four epilogue warps
     }
     for (int i = 0; i < 2; ++i) {
@@ -965,27 +976,25 @@ sim_kernel(const __grid_constant__ CUtensorMap tmap_h, const __grid_constant__ C
     const int row_b = b * a.keep_k;
     // tiled row operand: rows of the dense kept array (matrix mode) or of the image span
     const int row_a = a.smat ? row_b + mt * 128 : d.row0 + d.v0 + mt * 128;
-    const int tx_bytes = gather ? stage_bytes - (a.wide ? 1 : 2) * SIM_A_BYTES : stage_bytes;
+    const int tx_bytes = gather ? a.n_nt * b_bytes : stage_bytes;
     // every block walks its k-blocks from a different starting point, so that at any moment
     // the blocks read different 128-byte columns of the rows and spread over the memory channels
     const int rot = (mt * 5 + b * 3) % n_kb;
     int issued = 0, nt = 0, kr = 0, kb = kb0 + rot;           // slot tile, step of its pass, column step
     RingPos r;
     for (int it = 0; it < total_it; ++it) {
-      const uint32_t full = smem_u32(&bk->full[r.slot]);
-      if (it >= a.stages) mbar_wait_warp(smem_u32(&bk->empty[r.slot]), r.phase ^ 1u, wc);
+      const uint32_t full = smem_u32(GATHER ? &bk->full_b[r.slot] : &bk->full[r.slot]);
+      if (it >= a.stages) mbar_wait_warp(smem_u32(GATHER ? &bk->empty_b[r.slot] : &bk->empty[r.slot]), r.phase ^ 1u, wc);
       if (__shfl_sync(0xffffffffu, bk->abort_flag, 0)) break;
-      const uint32_t dst = base + r.slot * stage_bytes;
+      const uint32_t dst = GATHER ? base + a.a_stages * SIM_A_BYTES + r.slot * a.n_nt * b_bytes - SIM_A_BYTES : base + r.slot * stage_bytes;
       mbar_expect_tx_w(full, tx_bytes, leader);
-      if (a.wide) {
+      if (GATHER || a.wide) {
         if (!gather) tma_load_2d_w(dst, &tmap_h, full, kb * 64, row_a, leader);
         for (int t = 0; t < a.n_nt; ++t)
           tma_load_2d_w(dst + SIM_A_BYTES + t * b_bytes, &tmap_kept, full, kb * 64, row_b + (tile0 + t) * a.n_tile, leader);
       } else {
-        if (!gather) {
-          tma_load_2d_w(dst, &tmap_h, full, kb * 128, row_a, leader);
-          tma_load_2d_w(dst + SIM_A_BYTES, &tmap_h, full, kb * 128 + 64, row_a, leader);
-        }
+        tma_load_2d_w(dst, &tmap_h, full, kb * 128, row_a, leader);
+        tma_load_2d_w(dst + SIM_A_BYTES, &tmap_h, full, kb * 128 + 64, row_a, leader);
         tma_load_2d_w(dst + 2 * SIM_A_BYTES, &tmap_kept, full, kb * 128, row_b + nt * a.n_tile, leader);
         tma_load_2d_w(dst + 2 * SIM_A_BYTES + b_bytes, &tmap_kept, full, kb * 128 + 64, row_b + nt * a.n_tile, leader);
       }
@@ -998,9 +1007,7 @@ sim_kernel(const __grid_constant__ CUtensorMap tmap_h, const __grid_constant__ C
     for (int s = 0; s < a.stages; ++s) {
       if (issued > s) {
         const int last = ((issued - 1 - s) / a.stages) * a.stages + s;
-        // after an abort the gather warps may not have handed their part of the stage over, so the
-        // barrier may never complete: the tiled copies themselves land within microseconds
-        mbar_wait_drain(smem_u32(&bk->full[s]), (last / a.stages) & 1, bk->abort_flag ? 400000LL : TC_WAIT_LIMIT);
+        mbar_wait_drain(smem_u32(GATHER ? &bk->full_b[s] : &bk->full[s]), (last / a.stages) & 1, TC_WAIT_LIMIT);
       }
     }
     __syncwarp();
@@ -1017,36 +1024,35 @@ sim_kernel(const __grid_constant__ CUtensorMap tmap_h, const __grid_constant__ C
     if (gather) {
       const int g = warp - 6;
       constexpr int RW = 128 / SIM_GWARPS;                // rows of the tile per gather warp
-      const int cpr = a.wide ? 8 : 16;                   // 16-byte chunks per row and stage
-      const int c = lane & (cpr - 1), rsub = lane / cpr, rpi = 32 / cpr, n_i = RW / rpi;
+      const int c = lane & 7, rsub = lane >> 3;           // 16-byte chunk of the 128-byte piece, row of the group of four
       const int32_t *drop_b = a.drop_idx + (size_t)b * (a.max_vis - a.keep_k);
       for (int r = g * RW + lane; r < (g + 1) * RW; r += 32) {
         const int dp = min(mt * 128 + r, nd - 1);        // the ragged tail repeats the last dropped token
         bk->rows[r] = d.row0 + d.v0 + min(max(__ldg(drop_b + dp), 0), d.nv - 1);
       }
       __syncwarp();
-      const uint8_t *hid = reinterpret_cast<const uint8_t *>(a.hidden) + (size_t)c * 16;
-      const size_t pitch = (size_t)a.D * 2;
-      const uint32_t dst_c = (uint32_t)((c >> 3) * SIM_A_BYTES);
-      const int stage_cols_bytes = a.wide ? 128 : 256;
-      const int rot = (mt * 5 + b * 3) % n_kb;
+      const uint8_t *src[RW / 4];
+#pragma unroll
+      for (int i = 0; i < RW / 4; ++i)
+        src[i] = reinterpret_cast<const uint8_t *>(a.hidden) + (size_t)bk->rows[g * RW + i * 4 + rsub] * ((size_t)a.D * 2) + c * 16;
+      const uint32_t dst0 = base + (g * RW + rsub) * 128;
+      int kb = kb0 + (mt * 5 + b * 3) % n_kb;
+      RingPos r;
       for (int it = 0; it < total_it; ++it) {
-        const int s = it % a.stages, nt = it / n_kb, kb = kb0 + (it - nt * n_kb + rot) % n_kb;
         int go = 1;
         if (lane == 0) {
-          if (it >= a.stages) mbar_wait(smem_u32(&bk->empty[s]), ((it / a.stages) - 1) & 1, wc);
+          if (it >= a.a_stages) mbar_wait(smem_u32(&bk->empty[r.slot]), r.phase ^ 1u, wc);
           go = bk->abort_flag ? 0 : 1;
         }
         go = __shfl_sync(0xffffffffu, go, 0);
         if (!go) break;
-        const uint32_t dst = base + s * stage_bytes + dst_c;
-        const uint8_t *src = hid + (size_t)kb * stage_cols_bytes;
-#pragma unroll 8
-        for (int i = 0; i < n_i; ++i) {
-          const int r = g * RW + i * rpi + rsub;
-          cp_async16(dst + r * 128 + (((c & 7) ^ (r & 7)) << 4), src + (size_t)bk->rows[r] * pitch);
-        }
-        cp_async_arrive_on(smem_u32(&bk->full[s]));       // this lane's share of the stage, once it has landed
+        const uint32_t dst = dst0 + r.slot * SIM_A_BYTES;
+#pragma unroll
+        for (int i = 0; i < RW / 4; ++i)                   // (row r of a block: its chunk c at position c ^ (r & 7))
+          cp_async16(dst + i * 512 + (((c ^ ((i * 4 + rsub) & 7))) << 4), src[i] + (size_t)kb * 128);
+        cp_async_arrive_on(smem_u32(&bk->full[r.slot]));  // this lane's share of the tile, once it has landed
+        r.step(a.a_stages);
+        if (++kb == kb0 + n_kb) kb = kb0;
       }
       cp_async_commit();
       cp_async_wait<0>();                                 // nothing of this thread's is in flight when the block leaves
@@ -1054,23 +1060,35 @@ sim_kernel(const __grid_constant__ CUtensorMap tmap_h, const __grid_constant__ C
   } else if (warp == 1) {
     // ---- MMA issuer: the whole warp walks the loop and stays converged (see warp_leader).  After an abort its waits return
     // at once and it goes on multiplying whatever lies in the block's own memory: nothing of it is used.
-    // With gathered rows one lane issues alone: there the shared-memory writes of the gather warps pace the kernel, and the
-    // converged warp, which issues a stage's MMAs in one burst, was slower (1152 of 2304 slots, 32 sequences: 880 -> 1000 us).
-    const uint32_t leader = GATHER ? (lane == 0 ? 1u : 0u) : warp_leader();
+    const uint32_t leader = warp_leader();
     const uint32_t tm = __shfl_sync(0xffffffffu, tmem_base, 0);
     const uint32_t idesc = umma_idesc_bf16(128, a.n_tile);
     const uint64_t desc0 = umma_desc_sw128(base);
-    auto wait = [&](uint32_t bar, uint32_t parity) {
-      mbar_wait(bar, parity, wc);
-      if (!GATHER) __syncwarp();
-    };
     int it = 0;
-    if (!GATHER || lane == 0) {
+    if (GATHER) {
+      const uint64_t bdesc0 = umma_desc_sw128(base + a.a_stages * SIM_A_BYTES);
+      RingPos ra, rb;
+      for (int kb = 0; kb < n_kb; ++kb) {
+        mbar_wait_warp(smem_u32(&bk->full[ra.slot]), ra.phase, wc);
+        mbar_wait_warp(smem_u32(&bk->full_b[rb.slot]), rb.phase, wc);
+        fence_proxy_async();                   // the gathered rows were written by ordinary asynchronous copies
+        tc_fence_after();
+        const uint64_t da = desc0 + (uint32_t)(ra.slot * SIM_A_BYTES) / 16, db = bdesc0 + (uint32_t)(rb.slot * a.n_nt * b_bytes) / 16;
+        for (int t = 0; t < a.n_nt; ++t)
+#pragma unroll
+          for (int kk = 0; kk < 4; ++kk)
+            tc_mma_bf16_w(tm + t * a.n_tile, da + kk * 2, db + t * (b_bytes / 16) + kk * 2, idesc, (kb > 0 || kk > 0) ? 1u : 0u, leader);
+        tc_commit_w(smem_u32(&bk->empty_b[rb.slot]), leader);
+        tc_commit_w(smem_u32(&bk->empty[ra.slot]), leader);
+        ra.step(a.a_stages);
+        rb.step(a.stages);
+      }
+      tc_commit_w(smem_u32(&bk->acc_full[0]), leader);
+    } else {
       if (a.wide) {
         for (int kb = 0; kb < n_kb; ++kb) {
           const int s = kb % a.stages;
-          wait(smem_u32(&bk->full[s]), (kb / a.stages) & 1);
-          if (gather) fence_proxy_async();       // the gathered rows were written by ordinary asynchronous copies
+          mbar_wait_warp(smem_u32(&bk->full[s]), (kb / a.stages) & 1, wc);
           tc_fence_after();
           const uint64_t da = desc0 + (uint32_t)(s * stage_bytes) / 16, db = da + SIM_A_BYTES / 16;
           for (int t = 0; t < a.n_nt; ++t)
@@ -1084,12 +1102,11 @@ sim_kernel(const __grid_constant__ CUtensorMap tmap_h, const __grid_constant__ C
       }
       for (int nt = 0; nt < (a.wide ? 0 : a.n_nt); ++nt) {
         const int buf = nt & 1;
-        if (nt >= 2) wait(smem_u32(&bk->acc_empty[buf]), ((nt >> 1) - 1) & 1);
+        if (nt >= 2) mbar_wait_warp(smem_u32(&bk->acc_empty[buf]), ((nt >> 1) - 1) & 1, wc);
         const uint32_t dcol = tm + buf * (a.tmem_cols >> 1);
         for (int kb = 0; kb < n_kb; ++kb, ++it) {
           const int s = it % a.stages;
-          wait(smem_u32(&bk->full[s]), (it / a.stages) & 1);
-          if (gather) fence_proxy_async();
+          mbar_wait_warp(smem_u32(&bk->full[s]), (it / a.stages) & 1, wc);
           tc_fence_after();
           const uint64_t da = desc0 + (uint32_t)(s * stage_bytes) / 16, db = da + 2 * SIM_A_BYTES / 16;
   #pragma unroll
@@ -1102,11 +1119,11 @@ sim_kernel(const __grid_constant__ CUtensorMap tmap_h, const __grid_constant__ C
         }
         tc_commit_w(smem_u32(&bk->acc_full[buf]), leader);
       }
-      // every MMA this warp issued has completed before tensor memory is given back: after an abort the
-      // epilogue warps no longer wait for the accumulators, so nothing else would hold the block until then
-      tc_commit_w(smem_u32(&bk->mma_done), leader);
-      mbar_wait_drain(smem_u32(&bk->mma_done), 0, TC_WAIT_LIMIT);
     }
+    // every MMA this warp issued has completed before tensor memory is given back: after an abort the
+    // epilogue warps no longer wait for the accumulators, so nothing else would hold the block until then
+    tc_commit_w(smem_u32(&bk->mma_done), leader);
+    mbar_wait_drain(smem_u32(&bk->mma_done), 0, TC_WAIT_LIMIT);
     __syncwarp();
     if (a.cluster) { cluster_sync_all(); cluster_sync_all(); }
   } else {
@@ -1118,13 +1135,13 @@ sim_kernel(const __grid_constant__ CUtensorMap tmap_h, const __grid_constant__ C
     // Row r of a tile is 128 bytes; its 16-byte chunk c sits at chunk position c ^ (r & 7).
     float ssq[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
     for (int it = 0; it < (a.smat ? 0 : n_kb); ++it) {
-      const int s = it % a.stages;
-      mbar_wait(smem_u32(&bk->full[s]), (it / a.stages) & 1, wc);
+      const int ring = GATHER ? a.a_stages : a.stages, s = it % ring;
+      mbar_wait(smem_u32(&bk->full[s]), (it / ring) & 1, wc);
       if (!bk->abort_flag) {
 #pragma unroll
         for (int hb = 0; hb < 2; ++hb) {
-          if (hb == 1 && a.wide) break;                  // one 64-column block of the rows per stage
-          const uint4 *row = reinterpret_cast<const uint4 *>(base_ptr + (size_t)s * stage_bytes +
+          if (hb == 1 && (GATHER || a.wide)) break;      // one 64-column block of the rows per stage
+          const uint4 *row = reinterpret_cast<const uint4 *>(base_ptr + (size_t)s * (GATHER ? SIM_A_BYTES : stage_bytes) +
                                                              hb * SIM_A_BYTES + lrow * 128);
 #pragma unroll
           for (int c = 0; c < 8; ++c) {
