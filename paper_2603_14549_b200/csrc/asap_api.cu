@@ -405,12 +405,12 @@ asap_status launch_merge_front(asap_ctx *ctx, const asap_inputs *in, const asap_
     // block of the rows and of every slot tile).
     // Taken only while three such stages still fit (up to 384 slots): with two, the shorter copies
     // cost more than the second read of the rows (measured: 320 slots 87 -> 77 us, 510 slots 91 -> 96 us).
-    // The row operand: every visual row by tiled copies (a fifth to a half of the products are then thrown
-    // away), or the dropped rows alone, gathered (half the bytes per clock, four more warps, one block per
-    // SM).  Gathering is taken for batches large enough not to be sliced, from two fifths of the rows kept
-    // (measured at a fifth, 576 of 2880: 1.11 ms gathered against 1.04 ms tiled; at a half, 1152 of 2304:
-    // 0.56 ms against 0.92 ms).
-    bool gather_rows = splits == 1 && (long long)k * 5 >= 2LL * in->max_vis && (long long)max_mt * B > ctx->num_sms;
+    // The row operand: every visual row by tiled copies (the kept rows' products are then thrown
+    // away), or the dropped rows alone, gathered (four more warps, one block per
+    // SM).  Gathering is taken for batches large enough not to be sliced, from a quarter of the rows kept
+    // (measured on 32 x 2880 rows, tiled against gathered: 576 kept 412 / 403 us with the step the same, 860 565 / 533,
+    // 1000 613 / 553, 1290 859 / 663).
+    bool gather_rows = splits == 1 && (long long)k * 4 >= (long long)in->max_vis && (long long)max_mt * B > ctx->num_sms;
     // The gathered form makes a single pass over the hidden dimension with all of a block's accumulators live: more than 384
     // kept slots are dealt in groups (of one or two tiles) to neighbouring blocks, and the last block of a row tile combines
     // the groups' best slots.  Several passes inside one block would read the dropped rows from memory once per pass: the rows
