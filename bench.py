@@ -111,6 +111,9 @@ def algorithmic(batch, keep_k, rank_visual=False):
             v0 = int(batch.vis_start[b])
             out["score"]["bytes"] += nv * row
             out["score"]["flops"] += 2 * nv * (v0 + nv) * D
+        else:               # text rows alone: the kernel also sums the visual queries and takes the masses (Eq. 1)
+            out["score"]["bytes"] += nv * row
+            out["score"]["flops"] += 3 * nv * D
         out["select"]["bytes"] += nv * 4 + nv * 4
         out["head_sum"]["bytes"] += batch.H * nv * 4 + nv * 4
         out["kept_gather"]["bytes"] += 2 * keep_k * row

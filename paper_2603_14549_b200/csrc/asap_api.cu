@@ -40,9 +40,9 @@ struct asap_ctx {
   size_t cap_chunks = 0;      // rows of the query-sum partial buffer
   uint8_t *arena = nullptr;   // one allocation, carved below
   SampleDesc *desc = nullptr;
-  float *qsum_partial = nullptr, *qbar = nullptr, *score_partial = nullptr, *inv_norm = nullptr,
+  float *qsum_partial = nullptr, *qbar = nullptr, *score_partial = nullptr,
         *kept_inv = nullptr;
-  unsigned int *cnt_qsum = nullptr, *cnt_mass = nullptr, *cnt_score = nullptr, *cnt_sim = nullptr,
+  unsigned int *cnt_qsum = nullptr, *cnt_mass = nullptr, *cnt_sim = nullptr,
                *cnt_tiles = nullptr, *cnt_work = nullptr;
   float *mass_partial = nullptr;    // [B, H, max_vis] per-head attention masses
   float *head_norm = nullptr;       // [B, H, 2] minimum and 1 / range of a head's masses (per-head masks)
@@ -753,9 +753,8 @@ asap_status asap_init(asap_ctx **ctx_out, int device, size_t max_total_tokens, i
   const size_t o_spart = carve(Hc * T * sizeof(float));
   const size_t o_mpart = carve(Hc * T * sizeof(float));
   const size_t o_hnorm = carve(Bc * Hc * 2 * sizeof(float));
-  const size_t o_inv = carve(T * sizeof(float));
   const size_t o_kinv = carve(max_keep_rows * sizeof(float));
-  const size_t o_cnt = carve((Bc * col_blocks + 3 * Bc + 4) * sizeof(unsigned int));
+  const size_t o_cnt = carve((Bc * col_blocks + 2 * Bc + 4) * sizeof(unsigned int));
   const size_t o_role = carve(T * sizeof(int32_t));
   const size_t o_seg = carve((max_keep_rows + Bc) * sizeof(int32_t));
   const size_t o_mem = carve(T * sizeof(int32_t));
@@ -780,14 +779,12 @@ asap_status asap_init(asap_ctx **ctx_out, int device, size_t max_total_tokens, i
   if (const char *env = getenv("ASAP_SIM_PAIR_STAGES")) ctx->sim_pair_stages = atoi(env);
   if (const char *env = getenv("ASAP_SIM_CLUSTER")) ctx->sim_cluster = atoi(env);
   ctx->head_norm = reinterpret_cast<float *>(ctx->arena + o_hnorm);
-  ctx->inv_norm = reinterpret_cast<float *>(ctx->arena + o_inv);
   ctx->kept_inv = reinterpret_cast<float *>(ctx->arena + o_kinv);
-  ctx->counters_off = o_cnt; ctx->counters_bytes = (Bc * col_blocks + 3 * Bc + 4) * sizeof(unsigned int);
+  ctx->counters_off = o_cnt; ctx->counters_bytes = (Bc * col_blocks + 2 * Bc + 4) * sizeof(unsigned int);
   ctx->tiles_off = o_tiles; ctx->tiles_bytes = ctx->cap_tiles * sizeof(unsigned int);
   ctx->cnt_qsum = reinterpret_cast<unsigned int *>(ctx->arena + o_cnt);
   ctx->cnt_mass = ctx->cnt_qsum + Bc * col_blocks;
-  ctx->cnt_score = ctx->cnt_mass + Bc;
-  ctx->cnt_sim = ctx->cnt_score + Bc;
+  ctx->cnt_sim = ctx->cnt_mass + Bc;
   ctx->cnt_work = ctx->cnt_sim + Bc;
   ctx->role = reinterpret_cast<int32_t *>(ctx->arena + o_role);
   ctx->seg = reinterpret_cast<int32_t *>(ctx->arena + o_seg);
@@ -797,7 +794,7 @@ asap_status asap_init(asap_ctx **ctx_out, int device, size_t max_total_tokens, i
   ctx->cnt_tiles = reinterpret_cast<unsigned int *>(ctx->arena + o_tiles);
   ctx->sim_part = reinterpret_cast<float *>(ctx->arena + o_simpart);
   ctx->status = reinterpret_cast<uint32_t *>(ctx->arena + o_status);
-  e = cudaMemset(ctx->arena + o_cnt, 0, (Bc * col_blocks + 3 * Bc + 4) * sizeof(unsigned int));
+  e = cudaMemset(ctx->arena + o_cnt, 0, (Bc * col_blocks + 2 * Bc + 4) * sizeof(unsigned int));
   if (e == cudaSuccess) e = cudaMemset(ctx->arena + o_tiles, 0, ctx->cap_tiles * sizeof(unsigned int));
   if (e == cudaSuccess) e = cudaMemset(ctx->status, 0, sizeof(uint32_t));
   // kernels whose dynamic shared memory exceeds the 48 KB default
@@ -943,8 +940,8 @@ asap_status asap_prune_step(asap_ctx *ctx, const asap_inputs *in, const asap_par
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   // With the text span as ranking rows the Eq. 3 mask never touches a ranked row (a text query lies
   // after every visual key), so the score kernel does not need the attention mass, and takes it itself from the query and key
-  // tiles: no query sum, no mass kernel, no second stream.  With caller-given ranking rows (which may be visual) or a mask per
-  // head the masses come first.  Measured per step, masses inside the score kernel against mass kernels on a stream beside it:
+  // tiles: no query sum, no mass kernel.  With caller-given ranking rows (which may be visual) or a mask per
+  // head the masses come first.  Measured per step, masses inside the score kernel against mass kernels on a second stream:
   // 1 x 576 visual tokens 48.6 -> 42.6 us, 16 x 576 129.5 -> 121.4, 8 x 2304 243 -> 207, 12 mixed images 286 -> 242; against a
   // query-sum kernel in front, 64 x 2880 2530 -> 2427 us.
   const bool fused = in->rank_start == nullptr && !p->per_head_mask;

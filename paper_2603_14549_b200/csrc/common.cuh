@@ -117,10 +117,6 @@ __device__ __forceinline__ uint32_t smem_u32(const void *p) {
 __device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
   asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count) : "memory");
 }
-__device__ __forceinline__ void mbar_expect_tx(uint32_t bar, uint32_t bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes)
-               : "memory");
-}
 __device__ __forceinline__ void mbar_arrive(uint32_t bar) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
 }
@@ -217,14 +213,6 @@ struct RingPos {
 // ---------------------------------------------------------------------------------------
 // TMA (tiled 2-D load, completion on an mbarrier)
 // ---------------------------------------------------------------------------------------
-__device__ __forceinline__ void tma_load_2d(uint32_t smem_dst, const void *tmap, uint32_t bar,
-                                            int32_t x, int32_t y) {
-  asm volatile(
-      "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes "
-      "[%0], [%1, {%3, %4}], [%2];"
-      ::"r"(smem_dst), "l"(tmap), "r"(bar), "r"(x), "r"(y)
-      : "memory");
-}
 // The copying warp's form: the whole warp executes the statement and stays converged, `leader` (see warp_leader) issues.
 // One lane under a branch needs about 770 clocks per ring slot (wait, expectation, copy) whatever the copy's size; the
 // converged warp 360 (measured, 128 x 64 boxes out of L2 on all SMs, three per slot: 57 against 92 bytes per clock and SM).

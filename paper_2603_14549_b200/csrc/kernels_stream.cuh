@@ -1,12 +1,14 @@
 // The memory-bound and latency-bound kernels of the ASAP prune step:
-//   prepare        device-side validation, per-sample descriptors, output row offsets
+//   prepare        device-side validation, per-sample descriptors, output row offsets (one warp of a kernel that runs anyway)
 //   qsum           sum of the visual query rows                       (Eq. 1, summed over i first)
 //   mass_salience  s_j, then s_hat_j and m_j                          (Eq. 1, Eq. 2, Eq. 3)
-//   salience_block the same from per-head masses the score kernel produced (part of the selection launch)
+//   mass_heads, mask_heads, salience_heads   the same with a mask per head
+//   salience_block s_hat_j from per-head masses the score kernel produced (part of the selection launch)
 //   select         stable radix top-k of the ranking scores           (Fig. 3)
 //   role_map       kept slot / dropped position of every visual token
 //   kept_gather    kept rows gathered for the similarity GEMM, with their inverse norms (Sec. 4.2)
 //   csr_block      dropped tokens grouped by destination slot (tail of the similarity kernel)
+//   route          Sec. 4.2 inside the kept set, from the bit matrix of similar pairs
 //   merge_compact  Eq. 5 and the hand-off of Fig. 3
 //   gather_rows    KV-cache compaction with the row map of the hand-off
 #pragma once

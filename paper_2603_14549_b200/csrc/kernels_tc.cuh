@@ -7,8 +7,9 @@
 //   sim_kernel    Sec. 4.2: cosine similarity of every visual row against the kept rows with
 //                 the arg-max over kept slots taken in the epilogue.
 //
-// Both use one TMA-producer warp, one MMA-issuer warp (a single elected lane) and four
-// epilogue warps that read tensor memory (warp w may touch lanes 32*(w%4) .. 32*(w%4)+31).
+// All use one TMA-producer warp and one MMA-issuer warp, both walking their loops converged with one elected lane issuing
+// (see warp_leader), and one or two groups of four epilogue warps that read tensor memory (warp w may touch lanes
+// 32*(w%4) .. 32*(w%4)+31).
 // Every mbarrier wait is bounded (see WaitCtx); after an abort the block keeps walking its
 // uniform control flow so that every named barrier and the final teardown are still reached.
 #pragma once
@@ -41,13 +42,12 @@ __device__ __forceinline__ void group_bar_sync(int group) {
 //   pass 2  D = K_tile Q_rows^T   (M = 128 keys, N = all rows of the pair, up to 256): thread-per-key
 //           sum over rows of exp2(logit + mask - off_i), i.e. of the Eq. 4 probabilities A[i, j]
 // Key tiles stream through a shared-memory ring in one linear order (pass 1 ascending, pass 2
-// over the tiles that hold visual keys, coming back from L2); tensor memory holds two halves of 256
-// columns that alternate between consecutive operations, so the MMA issuer runs one operation ahead
-// of the epilogue warps.
+// over the tiles that hold visual keys, coming back from L2).  Tensor memory holds four accumulators of 128 columns, two per
+// epilogue group: an operation is one such accumulator (a pass-2 accumulator wider than 128 columns is two operations), a group
+// alternates between its two, and the MMA issuer runs one operation ahead of each group.
 // Epilogue: two groups of four warps.  Pass 1 with two row tiles: group g owns row tile g of every
-// key tile.  Pass 1 with one row tile, and pass 2: the groups take alternate operations.  Every
-// epilogue warp passes every operation's barriers (waits for the accumulator, releases it), whether
-// it has work on it or not, so the barrier counts never depend on the shape of the item.
+// key tile.  Pass 1 with one row tile, and pass 2: the groups take alternate key tiles.  A group waits for and gives back only
+// its own operations; issuer and groups derive the same deal from the item's shape.
 // Additive mask (Eq. 3), logits in log2 units: 0 for key j <= row position p; m_j*log2(e) for
 // j > p when both are in the image span (mask enabled); -inf otherwise.
 // The per-head sums over ranking rows go to `partial`; head_sum_kernel adds them in head order.
@@ -70,11 +70,11 @@ constexpr int SC_Q_HALF_BYTES = 256 * 128;      // 256 rows x 64 bf16: one 64-co
 constexpr int SC_Q_BYTES = 2 * SC_Q_HALF_BYTES;
 constexpr int SC_SMEM_MAIN = SC_Q_BYTES + SC_STAGES * SC_TILE_BYTES;
 // Total dynamic shared memory stays at 195 KB: with the 1 KB the system reserves per block that
-// is the 196 KB carve-out, which leaves the SM 32 KB of L1 for the memory-bound kernels that run
-// beside this one; one byte more selects the 228 KB carve-out and costs them about 10 us.
+// is the 196 KB carve-out; one byte more selects the 228 KB carve-out, and an SM that changes its carve-out between this
+// kernel and its neighbours delays the next launch by about 10 us.
 constexpr int SC_BOOK_BYTES = 3072;
 constexpr int SC_SMEM_BYTES = SC_SMEM_MAIN + SC_BOOK_BYTES;
-constexpr uint32_t SC_TMEM_COLS = 512;     // two halves of 256 columns
+constexpr uint32_t SC_TMEM_COLS = 512;     // four accumulators of 128 columns
 constexpr int SC_ITEM_SLOTS = 4;
 
 struct ScoreArgs {
@@ -737,10 +737,9 @@ head_sum_kernel(const SampleDesc *__restrict__ desc, int H, int max_vis,
 //                   warps (16-byte asynchronous copies, written in the 128-byte-swizzled layout the
 //                   tiled copies produce), so that only rows whose result is used are multiplied; or
 //                   every visual row by plain tiled copies, the kept rows' results being thrown away.
-//                   The gather path moves at most ~23 bytes per clock and SM (the load/store unit's
-//                   requests in flight; a gather copy of four rows per instruction through the
-//                   tensor-map unit managed a third of that), the tiled path twice as much, so the host
-//                   gathers only when the kept rows are a large share of the span (two fifths or more).
+//                   A gathered row costs the gather warps' 16-byte copies (their requests in flight bound them) what
+//                   several rows cost the tiled path, so the host gathers only from a quarter of the span kept on, where the
+//                   products saved outweigh it (the line and both sides' times stand at the rule in asap_api.cu).
 // While the first
 // accumulator is being built the epilogue warps also read every row tile from shared memory and
 // add up the squares (the row norms of Sec. 4.2's cosine similarity).
@@ -1471,15 +1470,12 @@ sim_kernel(const __grid_constant__ CUtensorMap tmap_h, const __grid_constant__ C
 // sim_pair_kernel
 //
 // The all-rows form of sim_kernel for batches large enough to fill the machine without slicing the
-// hidden dimension.  There the similarity kernel is bound by the bytes an SM can take in, not by the
-// tensor pipe: measured, the tiled copies of a block deliver about 34 bytes per clock whatever the
-// stage size or count (9.6 TB/s over 148 SMs), and a block of sim_kernel streams 128 rows and
-// n_tile kept rows per 64 columns, (128 + n_tile) * 128 bytes for 128 * n_tile * 64 products.  This
-// kernel multiplies TWO row tiles against each stage's kept rows -- (256 + n_tile) * 128 bytes for
-// twice the products, 30 % fewer bytes per product at n_tile = 192; tensor memory (512 columns =
-// 2 tiles x n_tile <= 256) allows no larger block.  (MMAs spanning a pair of CTAs, each CTA loading half
-// of the kept rows, were built and measured: the half an SM reads from its partner's shared memory
-// arrives through the same 34 bytes per clock, once per row tile, and the kernel ran 30 % slower.)
+// hidden dimension.  A block of sim_kernel streams 128 rows and n_tile kept rows per 64 columns, (128 + n_tile) * 128 bytes
+// for 128 * n_tile * 64 products, more than an SM takes in (about 92 bytes per clock with converged issue) while the tensor
+// pipe works on them at small n_tile.  This kernel multiplies TWO row tiles against each stage's kept rows -- (256 + n_tile) *
+// 128 bytes for twice the products, 30 % fewer bytes per product at n_tile = 192; tensor memory (512 columns = 2 tiles x
+// n_tile <= 256) allows no larger block.  (MMAs spanning a pair of CTAs, each loading half of the kept rows, ran 30 % slower
+// than this form when both issued from one lane under a branch.)
 // It makes a single pass over the hidden dimension: the kept slots are dealt in groups of n_tile <= 256 to `groups` blocks per
 // pair of row tiles (blockIdx.x = pair * groups + group).  The blocks of a pair are neighbours in
 // launch order and stream the same rows at the same pace, so the rows come from memory once and
