@@ -596,12 +596,16 @@ asap_status launch_consolidate_front(asap_ctx *ctx, const asap_inputs *in, const
   uint32_t *mask_g = reinterpret_cast<uint32_t *>(static_cast<uint8_t *>(scratch) + route_smat_bytes(B, k));
   bool mask_written = false;
   {
-    // large batches: two row tiles per block, the slots dealt in groups to neighbouring blocks (see the similarity
-    // launch of the merge); here every product is used, the matrix being square
+    // Two row tiles per block, the slots dealt in groups to neighbouring blocks (see the similarity launch of the merge); here
+    // every product is used, the matrix being square, no block waits for another and the routing's bits come with it.  With more
+    // than 256 slots always: the sliced form then adds its partial products up through global memory (width 4096, sliced -> this
+    // form, whole call: 1 sequence with 576 slots 223 -> 94 us, 4 with 288 126 -> 81, 7 with 576 269 -> 134).  With one slot
+    // tile, where the slices add up inside a cluster, from an eighth of the SMs on (192 slots: 8 blocks 85 against 90 us, 24
+    // blocks 131 against 123).
     const int pairs = (k + 255) / 256;
     const int pg = (k + 255) / 256;
     const int ptile = (((k + pg - 1) / pg) + 15) & ~15;
-    const long long min_blocks = ctx->sim_pair_min_blocks > 0 ? ctx->sim_pair_min_blocks : (ctx->num_sms + 1) / 2;
+    const long long min_blocks = ctx->sim_pair_min_blocks > 0 ? ctx->sim_pair_min_blocks : k > 256 ? 1 : ctx->num_sms / 8;
     const int pstage = 2 * SIM_A_BYTES + ptile * 128;
     int pstages = ctx->sim_pair_stages > 0 ? ctx->sim_pair_stages : (192 * 1024) / pstage;
     if (pstages > SIM_MAX_STAGES) pstages = SIM_MAX_STAGES;
