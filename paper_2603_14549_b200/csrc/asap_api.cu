@@ -428,15 +428,16 @@ asap_status launch_merge_front(asap_ctx *ctx, const asap_inputs *in, const asap_
       if (gather_rows) { groups = g; n_nt = tiles_g; n_tile = tile_g; max_mt = mt_g; }
     }
     // Every visual row, two row tiles per block, the kept slots dealt in groups of at most 256 to the
-    // blocks of a pair, one pass each: fewer bytes out of L2 per product, which is what bounds the
-    // similarity of a large batch.  Taken when that grid fills at least half of the SMs (measured: 96 blocks
-    // 91 -> 75 us, 144 blocks 78 -> 72 us, 2304 blocks 1038 -> 845 us; 48 blocks 39 -> 57 us, where slicing
-    // the hidden dimension over more blocks is worth more).
+    // blocks of a pair, one pass each: fewer bytes out of L2 per product.  With more than 256 slots always: the sliced form
+    // then adds its partial products up through global memory (step, sliced -> this form: 1 x 2304 with 320 kept 116 -> 97 us,
+    // 4 x 2304 160 -> 131, 1 x 2880 with 576 246 -> 180).  With one slot tile, where the slices add up inside a cluster, from a
+    // grid of half the SMs on (step: 96 blocks of 12 mixed images 252 -> 229 us; 48 blocks of 16 x 576 114 against 123, of 4 mixed images
+    // 151 against 163, though 36 blocks of 4 x 2304 with 160 kept 138 -> 128).
     {
       const int pairs = (in->max_vis + 255) / 256;
       const int pg = (k + 255) / 256;
       const int ptile = (((k + pg - 1) / pg) + 15) & ~15;
-      const long long min_blocks = ctx->sim_pair_min_blocks > 0 ? ctx->sim_pair_min_blocks : (ctx->num_sms + 1) / 2;
+      const long long min_blocks = ctx->sim_pair_min_blocks > 0 ? ctx->sim_pair_min_blocks : k > 256 ? 1 : (ctx->num_sms + 1) / 2;
       const int pstage = 2 * SIM_A_BYTES + ptile * 128;
       int pstages = ctx->sim_pair_stages > 0 ? ctx->sim_pair_stages : (192 * 1024) / pstage;
       if (pstages > SIM_MAX_STAGES) pstages = SIM_MAX_STAGES;
