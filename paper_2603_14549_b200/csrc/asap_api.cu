@@ -701,7 +701,7 @@ routing:
     return fail(ctx, ASAP_ERR_UNSUPPORTED, "max_vis = %d is too large for the routing kernel", in->max_vis);
   ra.salience = salience; ra.mass = mass; ra.keep_idx = keep_idx; ra.drop_idx = drop_idx;
   ra.final_keep = out->keep_idx; ra.src_idx = out->drop_idx; ra.src_assign = out->assign;
-  ra.seg = ctx->seg; ra.members = ctx->members; ra.n_absorbed = n_absorbed; ra.src_sim = out->best_sim;
+  ra.seg = ctx->seg; ra.members = ctx->members; ra.n_absorbed = n_absorbed; ra.src_sim = out->best_sim; ra.status = ctx->status;
   mark(ctx, "route", st);
   launch_pdl(route_kernel, dim3(B), dim3(ROUTE_THREADS), route_smem, st, ra);
   return after_launch(ctx, "route");

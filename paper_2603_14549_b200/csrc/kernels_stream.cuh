@@ -999,6 +999,7 @@ struct RouteArgs {
   const int32_t *drop_idx;        // [B, max_vis - keep_k]  stage 1
   int32_t *final_keep, *src_idx, *src_assign, *seg, *members, *n_absorbed;
   float *src_sim;                 // nullable
+  const uint32_t *status;
 };
 
 __global__ void __launch_bounds__(ROUTE_THREADS)
@@ -1020,7 +1021,9 @@ route_kernel(RouteArgs a) {
   float *ss_b = a.src_sim ? a.src_sim + (size_t)b * nd_max : nullptr;
   int32_t *seg_b = a.seg + (size_t)b * (k + 1);
   int32_t *mem_b = a.members + (size_t)b * nd_max;
-  if (!d.valid) {
+  // A similarity kernel that gave up has left the matrices unwritten: they hold whatever the caller's scratch held.
+  const bool gave_up = __syncthreads_or((__ldcg(a.status) & STATUS_SIM_TIMEOUT) != 0u);
+  if (!d.valid || gave_up) {
     for (int j = tid; j < k; j += nthr) fk_b[j] = -1;
     for (int j = tid; j < nd_max; j += nthr) { si_b[j] = -1; sa_b[j] = -1; if (ss_b) ss_b[j] = 0.f; }
     for (int j = tid; j <= k; j += nthr) seg_b[j] = 0;
@@ -1134,7 +1137,8 @@ route_kernel(RouteArgs a) {
       row[w] = word;
     }
   }
-  while (true) {
+  // (every round decides a slot, so k rounds are enough whatever the matrix holds)
+  for (int round = 0; round < k; ++round) {
     int verdict[4] = {0, 0, 0, 0};                    // 1 anchor, 2 absorbed
     bool waiting = false;
 #pragma unroll

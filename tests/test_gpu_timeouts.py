@@ -100,3 +100,38 @@ def test_attention_kernel_gives_up_and_the_context_recovers(ctx):
     A.asap_attention(ctx, inp, p, out.mask_log, v, scratch, again)
     torch.cuda.synchronize(); A.asap_check(ctx)
     assert torch.equal(good, again)
+
+
+@pytest.mark.parametrize("k", [150, 290], ids=["one_slot_tile", "written_bit_matrix"])
+def test_consolidation_gives_up_and_the_context_recovers(ctx, k):
+    """The similarity kernel gives up and leaves the matrices that the routing reads unwritten (the scratch is filled with
+    ones, no valid bit matrix): the routing leaves with its padding, and so does a call made while the bit is still set."""
+    batch = W.tiny(B=2, n_vis=[400, 330], text_lens=[9, 12], H=2, keep_k=k, seed=604, centres=20)
+    inp = A.make_inputs(batch, DEV)
+    p = A.Params(keep_k=k, sim_threshold=0.8)
+    out = A.alloc_outputs(inp, k, fill=True)
+    A.asap_prune_step(ctx, inp, A.Params(keep_k=k), out)
+    torch.cuda.synchronize(); A.asap_check(ctx)
+    lists = (out.mass.clone(), out.salience.clone(), out.keep_idx.clone(), out.drop_idx.clone())
+
+    def call():
+        scratch = torch.full((A.asap_consolidate_scratch_bytes(2, k),), 255, dtype=torch.uint8, device=DEV)
+        o = A.alloc_outputs(inp, k, fill=True)
+        n = torch.full((2,), -7, dtype=torch.int32, device=DEV)
+        A.asap_consolidate(ctx, inp, p, *lists, scratch, o, n)
+        torch.cuda.synchronize()
+        return o, n
+
+    good, n_good = call()
+    A.asap_check(ctx)
+    A.asap_debug_wait_limit(ctx, 1)
+    for _ in range(2):                                # the call that gives up, and one that finds the bit set
+        bad, n_bad = call()
+        assert torch.all(bad.keep_idx == -1) and torch.all(bad.assign == -1) and torch.all(n_bad == 0)
+    with pytest.raises(A.AsapError) as e:
+        A.asap_check(ctx)
+    assert e.value.status == -6 and "timed out in the similarity kernel" in str(e.value)
+    again, n_again = call()
+    A.asap_check(ctx)
+    assert torch.equal(n_good, n_again) and int(n_good.min()) > 0
+    _same(good, again, ("keep_idx", "drop_idx", "assign", "best_sim", "out_hidden", "out_pos", "src_row", "out_cu_seqlens"))
