@@ -971,8 +971,10 @@ __device__ __forceinline__ void csr_block(const SampleDesc &d, int b, int max_vi
 //      slot, i.e. at most nv - keep_k times); any other slot becomes an anchor.  This is the greedy
 //      rule "join the most similar earlier anchor if that similarity exceeds t, else become an anchor" with the question
 //      WHICH anchor left to step D.  Decided in rounds by all threads: as many as the longest chain of slots each of which
-//      waits for the one before, three or four on clustered rows.  (One warp walking the order took 38 of the kernel's 174 us
-//      on 24 x 576 slots, reading the similarities a second time for D 50, forming the bit matrix here 30; 174 -> 59 us in all.)
+//      waits for the one before, two to four on clustered rows; after some rounds that decide few slots the rest is taken in order
+//      (route_walk).  (One warp walking the order took 38 of the kernel's 174 us on 24 x 576 slots, reading the similarities a
+//      second time for D 50, forming the bit matrix here 30; 174 -> 48 us in all, 45 with D's loads after its scan.
+//      Rounds alone: 0.57 ms on a chain through 576 slots and 9.5 ms through 1024; with the walk 64 and 271 us.)
 //   D  every absorbed slot finds the most similar anchor that was visited before it (lowest slot
 //      among equals), looking only at the anchors in its row of the bit matrix.
 //   E  the vacated slots are refilled with the pruned tokens of largest attention mass (radix
@@ -984,6 +986,8 @@ __device__ __forceinline__ void csr_block(const SampleDesc &d, int b, int max_vi
 // =======================================================================================
 constexpr int ROUTE_THREADS = 1024;
 constexpr int ROUTE_MAX_WORDS = 128;                    // keep_k <= 32 * 128
+constexpr int ROUTE_WALK_BELOW = 32;                    // threads that decide something in a round, below which it is a slow one
+constexpr int ROUTE_SLOW_ROUNDS = 8;
 
 struct RouteArgs {
   const SampleDesc *desc;
@@ -1001,6 +1005,41 @@ struct RouteArgs {
   float *src_sim;                 // nullable
   const uint32_t *status;
 };
+
+// The undecided slots in visiting order, 32 at a time, by the whole block.  Rows hold earlier slots only, and those before the group
+// are all decided: warp w looks whether the group's w-th slot has an anchor among them and which of the group come before
+// it; one warp then decides the 32 one after the other out of registers.
+__device__ __forceinline__ void route_walk(const int *s_order, const uint32_t *mask, uint32_t *s_anchor, const uint32_t *s_gone,
+                                           int *s_flag, uint32_t *s_before, int k, int kw) {
+  static_assert(ROUTE_THREADS == 1024, "a warp per slot of a group");
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  for (int r0 = 0; r0 < k; r0 += 32) {
+    const int q = r0 + lane < k ? s_order[r0 + lane] : -1;
+    const uint32_t todo = __ballot_sync(0xffffffffu, q >= 0 && !(((s_anchor[q >> 5] | s_gone[q >> 5]) >> (q & 31)) & 1u));
+    if (todo == 0u) continue;                             // (the same in every warp)
+    if ((todo >> warp) & 1u) {
+      const uint32_t *row = mask + (size_t)__shfl_sync(0xffffffffu, q, warp) * kw;
+      uint32_t hit = 0u;
+      for (int w = lane; w < kw; w += 32) hit |= row[w] & s_anchor[w];
+      const uint32_t before = __ballot_sync(0xffffffffu, q >= 0 && ((row[q >> 5] >> (q & 31)) & 1u));
+      const bool by_anchor = __any_sync(0xffffffffu, hit != 0u);
+      if (lane == 0) s_before[warp] = by_anchor ? before | (1u << warp) : before & ~(1u << warp);
+    }
+    __syncthreads();
+    if (warp == 0) {
+      const uint32_t before = s_before[lane];
+      uint32_t anchors = 0u;
+#pragma unroll 4
+      for (int t = 0; t < 32; ++t)
+        if (!(__shfl_sync(0xffffffffu, before, t) & (anchors | (1u << t)))) anchors |= (1u << t) & todo;
+      if ((anchors >> lane) & 1u) {
+        atomicOr(&s_anchor[q >> 5], 1u << (q & 31));
+        s_flag[q] = 1;
+      }
+    }
+    __syncthreads();
+  }
+}
 
 __global__ void __launch_bounds__(ROUTE_THREADS)
 route_kernel(RouteArgs a) {
@@ -1021,9 +1060,9 @@ route_kernel(RouteArgs a) {
   float *ss_b = a.src_sim ? a.src_sim + (size_t)b * nd_max : nullptr;
   int32_t *seg_b = a.seg + (size_t)b * (k + 1);
   int32_t *mem_b = a.members + (size_t)b * nd_max;
-  // A similarity kernel that gave up has left the matrices unwritten: they hold whatever the caller's scratch held.
-  const bool gave_up = __syncthreads_or((__ldcg(a.status) & STATUS_SIM_TIMEOUT) != 0u);
-  if (!d.valid || gave_up) {
+  // (a similarity kernel that gave up has left the matrices unwritten: they hold whatever the caller's scratch held.  Nothing
+  // writes the status word while this kernel runs)
+  if (!d.valid || (__ldcg(a.status) & STATUS_SIM_TIMEOUT)) {
     for (int j = tid; j < k; j += nthr) fk_b[j] = -1;
     for (int j = tid; j < nd_max; j += nthr) { si_b[j] = -1; sa_b[j] = -1; if (ss_b) ss_b[j] = 0.f; }
     for (int j = tid; j <= k; j += nthr) seg_b[j] = 0;
@@ -1137,10 +1176,12 @@ route_kernel(RouteArgs a) {
       row[w] = word;
     }
   }
-  // (every round decides a slot, so k rounds are enough whatever the matrix holds)
-  for (int round = 0; round < k; ++round) {
+  // A round costs the same whether it decides one slot or all.  After ROUTE_SLOW_ROUNDS in a row that decide fewer slots than the
+  // walk does in their time (one such round says nothing: the next may absorb all others) the rest is taken in order, so the
+  // rounds are bounded whatever the matrix holds.
+  for (int slow = 0;;) {
     int verdict[4] = {0, 0, 0, 0};                    // 1 anchor, 2 absorbed
-    bool waiting = false;
+    bool waiting = false, decided = false;
 #pragma unroll
     for (int t = 0; t < 4; ++t) {
       if (!open[t]) continue;
@@ -1153,10 +1194,10 @@ route_kernel(RouteArgs a) {
         left |= word & ~s_gone[w];
       }
       verdict[t] = by_anchor ? 2 : (left ? 0 : 1);
-      if (verdict[t]) open[t] = false;
+      if (verdict[t]) { open[t] = false; decided = true; }
       else waiting = true;
     }
-    __syncthreads();                                  // every slot has looked at the last round's decisions
+    const int progress = __syncthreads_count(decided);    // (and every slot has looked at the last round's decisions)
 #pragma unroll
     for (int t = 0; t < 4; ++t) {
       const int p = tid + t * nthr;
@@ -1164,6 +1205,11 @@ route_kernel(RouteArgs a) {
       if (verdict[t] == 2) atomicOr(&s_gone[p >> 5], 1u << (p & 31));
     }
     if (!__syncthreads_or(waiting)) break;
+    slow = progress < ROUTE_WALK_BELOW ? slow + 1 : 0;
+    if (slow == ROUTE_SLOW_ROUNDS) {
+      route_walk(s_order, mask, s_anchor, s_gone, s_flag, reinterpret_cast<uint32_t *>(s_hist), k, kw);
+      break;
+    }
   }
   // at most nd slots are absorbed, the first ones of the visiting order: later ones stay anchors
   {
@@ -1193,14 +1239,40 @@ route_kernel(RouteArgs a) {
     float best = -INFINITY;
     if (!s_flag[p]) {
       const float *row = S + (size_t)p * k;
+      // (a few such anchors are the rule: their similarities are loaded after the scan, by all lanes together.  Inside the scan
+      // the lanes come upon theirs in different words, a trip to memory each)
+      constexpr int FEW = 6;
+      int c[FEW], n_words = 0, n_cand = 0;              // the latest words' lowest candidates, c[0] the last
+#pragma unroll
+      for (int e = 0; e < FEW; ++e) c[e] = 0;
 #pragma unroll 4
       for (int w = 0; w < kw; ++w) {
-        uint32_t cand = mask[(size_t)p * kw + w] & s_anchor[w];
-        while (cand) {
-          const int q = w * 32 + __ffs(cand) - 1;
-          cand &= cand - 1;
-          const float v = __ldcg(row + q);
-          if (v > best) { best = v; best_q = q; }     // ascending q: the first maximum stays
+        const uint32_t cand = mask[(size_t)p * kw + w] & s_anchor[w];
+        if (cand) {
+#pragma unroll
+          for (int e = FEW - 1; e > 0; --e) c[e] = c[e - 1];
+          c[0] = w * 32 + __ffs(cand) - 1;
+          ++n_words;
+        }
+        n_cand += __popc(cand);
+      }
+      if (n_words == n_cand && n_cand <= FEW) {
+        float v[FEW];
+#pragma unroll
+        for (int e = 0; e < FEW; ++e) v[e] = e < n_cand ? __ldcg(row + c[e]) : -INFINITY;
+#pragma unroll
+        for (int e = FEW - 1; e >= 0; --e)              // ascending slots: the first maximum stays
+          if (v[e] > best) { best = v[e]; best_q = c[e]; }
+      } else {
+#pragma unroll 4
+        for (int w = 0; w < kw; ++w) {
+          uint32_t cand = mask[(size_t)p * kw + w] & s_anchor[w];
+          while (cand) {
+            const int q = w * 32 + __ffs(cand) - 1;
+            cand &= cand - 1;
+            const float v = __ldcg(row + q);
+            if (v > best) { best = v; best_q = q; }
+          }
         }
       }
     }

@@ -292,3 +292,75 @@ def test_routing_from_the_written_bit_matrix(nv, k, t):
         assert n_abs.min() > 0
     finally:
         A.asap_free(c)
+
+
+def _chain(B, nv, k, H, seed):
+    """Every kept token is similar to the one before it and the one after it in visiting order, and to no other: tokens become
+    anchors and are absorbed in turn, and none can be decided before the one in front of it."""
+    batch = W.tiny(B=B, n_vis=[nv] * B, text_lens=[5] * B, H=H, keep_k=k, seed=seed, centres=9)
+    D = H * 128
+    i = torch.arange(k)
+    rows = torch.zeros(k, D)
+    rows[i, i % D] = 1.0
+    rows[i, (i + 1) % D] = 1.0
+
+    def stage1(bt, b, kk):
+        m, s, kp, dp = W.random_stage1(bt, b, kk, 77)
+        s = s.copy()
+        order = np.random.default_rng(78).permutation(kk)          # visiting order -> kept slot
+        s[kp[order]] = np.linspace(1.0, 0.5, kk, dtype=np.float32)
+        lo = int(bt.cu_seqlens[b]) + int(bt.vis_start[b])
+        bt.hidden[torch.from_numpy(lo + kp[order].astype(np.int64))] = rows.to(torch.bfloat16)
+        return m, s, kp, dp
+
+    return batch, stage1
+
+
+@pytest.mark.parametrize("nv,k,H", [(150, 70, 2), (1000, 500, 8), (2600, 1300, 8)], ids=["two_words", "shared", "global"])
+def test_routing_walks_a_chain(nv, k, H):
+    """One slot per round is decided: a warp takes the rest of the visiting order.  At 500 slots every second token is
+    absorbed; beyond the hidden size the chain meets itself again (equal rows)."""
+    c = A.asap_init(0, max_total_tokens=2 * (nv + 40), max_B=2, max_H=H, max_D=128 * H, max_keep_rows=2 * k)
+    try:
+        batch, stage1 = _chain(2, nv, k, H, 930)
+        # (the visual rows are overwritten by stage1, which _run calls before the inputs go to the device)
+        for b in range(2):
+            stage1(batch, b, k)
+        out, n_abs, st1 = _run(c, batch, k, 0.4, stage1=stage1)
+        _check(batch, k, 0.4, out, n_abs, st1)
+        if k <= 128 * H:
+            assert n_abs.tolist() == [k // 2] * 2
+    finally:
+        A.asap_free(c)
+
+
+def test_a_chain_costs_little_more_than_clusters():
+    """1024 slots: 0.20 ms on clusters; on a chain 9.6 ms when every slot took a round of its own, 0.34 with the walk."""
+    k, nv = 1024, 2048
+    c = A.asap_init(0, max_total_tokens=nv + 40, max_B=1, max_H=16, max_D=2048, max_keep_rows=k)
+    try:
+        ms = []
+        for chain in (False, True):
+            batch, stage1 = _chain(1, nv, k, 16, 931)
+            if not chain:
+                batch = W.tiny(B=1, n_vis=[nv], text_lens=[5], H=16, keep_k=k, seed=932, centres=60)
+                stage1 = lambda bt, b, kk: W.random_stage1(bt, b, kk, 77)
+            m, s, kp, dp = (torch.from_numpy(x)[None].to(DEV) for x in stage1(batch, 0, k))
+            inp = A.make_inputs(batch, DEV)
+            out = A.alloc_outputs(inp, k, fill=True)
+            scratch = torch.empty(A.asap_consolidate_scratch_bytes(1, k), dtype=torch.uint8, device=DEV)
+            p = A.Params(keep_k=k, sim_threshold=0.4)
+            a, e = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            best = math.inf
+            for _ in range(5):
+                a.record()
+                A.asap_consolidate(c, inp, p, m.float(), s.float(), kp.int(), dp.int(), scratch, out)
+                e.record()
+                torch.cuda.synchronize()
+                best = min(best, a.elapsed_time(e))
+            A.asap_check(c)
+            ms.append(best)
+        print("clusters, chain (ms):", ms)
+        assert ms[1] < 6.0 * ms[0]
+    finally:
+        A.asap_free(c)
