@@ -189,7 +189,7 @@ asap_status asap_consolidate(asap_ctx *ctx, const asap_inputs *in, const asap_pa
  *     out[i, h, :] = sum_j Softmax_j( q_i^h . k_j^h / sqrt(head_dim) + M_ij ) v_j^h
  * for every row i of every sequence, with M_ij = 0 for j <= i, M_ij = mask_log[b][j - vis_start]
  * for i < j when both i and j lie in the image span, and -infinity otherwise (other sequences of
- * the packed batch are never attended).  With p->mask_enable == 0 this is causal attention and
+ * the packed batch are never attended, and whatever they hold, NaN included, changes nothing here).  With p->mask_enable == 0 this is causal attention and
  * `mask_log` may be NULL; otherwise `mask_log` is the device array [B, max_vis] that asap_score
  * writes (asap_outputs::mask_log), or with p->per_head_mask the array [B, H, max_vis] of
  * asap_outputs::mask_log_heads (head h then uses its own vector).  Only B, H, head_dim, D, total_tokens, the bounds, cu_seqlens,

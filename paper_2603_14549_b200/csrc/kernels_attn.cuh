@@ -25,7 +25,7 @@ namespace asap {
 
 enum : uint32_t { STATUS_ATTN_TIMEOUT = 16u };   // a bounded wait ran out in the attention kernel
 
-constexpr int AT_THREADS = 384;                 // warp 0: items and copies, warp 1: MMA issue, warp 2: Eq. 3's addends, warps 4-11: two softmax warpgroups
+constexpr int AT_THREADS = 384;                 // warp 0: items and copies, warp 1: MMA issue, warp 2: Eq. 3's addends, rows past the sequence, warps 4-11: two softmax warpgroups
 constexpr int AT_TILE_BYTES = 128 * 128 * 2;    // 128 rows x 128 bf16 as two 64-column blocks of 16 KB
 constexpr int AT_BLOCK_BYTES = AT_TILE_BYTES / 2;
 constexpr int AT_SLOTS = 4;                     // ring of key and value tiles in the order K0 V0 K1 V1 ...
@@ -72,6 +72,7 @@ struct AttnBook {
   uint64_t full[AT_SLOTS], empty[AT_SLOTS], q_full[2], q_empty[2], s_full[2], s_empty, p_ready[2], pv_done[2];
   uint64_t m_full[2], m_empty[2], ext_full[AT_EXT_BUFS], ext_empty[AT_EXT_BUFS], rows_full[2], rows_empty[2];
   uint64_t item_full[AT_ITEM_SLOTS], item_empty[AT_ITEM_SLOTS], mma_done;
+  uint64_t raw[AT_SLOTS];      // a tile that reaches past its sequence lands here; warp 2 passes it on
   AttnItem item[AT_ITEM_SLOTS];
   uint32_t tmem_base;
   int abort_flag;
@@ -102,6 +103,12 @@ __device__ __forceinline__ AttnTileKind attn_tile_kind(int sees, int q_lo, int k
   return k;
 }
 
+// The item's last key tile lies above the diagonal of one of its row tiles (see attn_tile_kind).
+__device__ __forceinline__ bool attn_last_above(const int (&n_kt)[2], const int (&sees)[2], int q_base) {
+  const int kt = max(n_kt[0], n_kt[1]) - 1;
+  return (kt < n_kt[0] && attn_tile_kind(sees[0], q_base, kt).above) || (kt < n_kt[1] && attn_tile_kind(sees[1], q_base + 128, kt).above);
+}
+
 // What bounds it: at the largest size the power cap (1.04 PFLOP/s algorithmic, 75 % of what a library GEMM sustains under
 // the same cap); below that the hand-overs between the tensor pipe and the softmax warps: a key tile of both row tiles takes
 // about 3000 clocks where either alone needs 2048.  Measured per call (before: a block per pair of row tiles, a kernel that
@@ -125,6 +132,7 @@ attn_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__ 
     for (int s = 0; s < AT_SLOTS; ++s) {
       mbar_init(smem_u32(&bk->full[s]), 1);
       mbar_init(smem_u32(&bk->empty[s]), 1);
+      mbar_init(smem_u32(&bk->raw[s]), 1);
     }
     for (int g = 0; g < 2; ++g) {
       mbar_init(smem_u32(&bk->q_full[g]), 1);
@@ -216,6 +224,7 @@ attn_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__ 
       AttnItem cur, nxt;
       int tc = 0, qc[2] = {0, 0};                 // key / value tiles and query tiles so far
       int t_issued = 0, q_issued[2] = {0, 0};     // copies actually issued
+      uint32_t raw_any = 0u, raw_odd = 0u, raw_last = 0u;     // per ring slot: copies through `raw`: any, an odd number, the latest one
       auto stopped = [&]() { return __shfl_sync(0xffffffffu, bk->abort_flag, 0) != 0; };
       draw(cur);
       while (cur.b >= 0) {
@@ -232,12 +241,14 @@ attn_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__ 
           }
           ++qc[g];
         };
-        auto load_tile = [&](const CUtensorMap *map, int kt) {
+        auto load_tile = [&](const CUtensorMap *map, int kt, bool past) {
           const int s = tc % AT_SLOTS;
           if (tc >= AT_SLOTS) mbar_wait_warp(smem_u32(&bk->empty[s]), ((tc / AT_SLOTS) - 1) & 1, wc);
           if (!stopped()) {
-            const uint32_t bar = smem_u32(&bk->full[s]), dst = ring + s * AT_TILE_BYTES;
+            const uint32_t bar = smem_u32(past ? &bk->raw[s] : &bk->full[s]), dst = ring + s * AT_TILE_BYTES, bit = 1u << s;
             const int row = cur.row0 + kt * 128;
+            raw_last = past ? raw_last | bit : raw_last & ~bit;
+            if (past) { raw_any |= bit; raw_odd ^= bit; }
             mbar_expect_tx_w(bar, AT_TILE_BYTES, leader);
             tma_load_2d_w(dst, map, bar, cur.h * 128, row, leader);
             tma_load_2d_w(dst + AT_BLOCK_BYTES, map, bar, cur.h * 128 + 64, row, leader);
@@ -246,14 +257,14 @@ attn_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__ 
           ++tc;
         };
         const int n_max = max(cur.n_kt[0], cur.n_kt[1]);
+        const bool ragged = n_max * 128 > cur.n, clear_k = ragged && attn_last_above(cur.n_kt, cur.sees, cur.q_base);
         load_q(0);
-        load_tile(&tmap_k, 0);
-        load_q(1);
-        load_tile(&tmap_v, 0);
-        draw(nxt);                                // its look-ups overlap this item's work
-        for (int kt = 1; kt < n_max; ++kt) {
-          load_tile(&tmap_k, kt);
-          load_tile(&tmap_v, kt);
+#pragma unroll 1
+        for (int kt = 0; kt < n_max; ++kt) {
+          load_tile(&tmap_k, kt, clear_k && kt == n_max - 1);
+          if (kt == 0) load_q(1);
+          load_tile(&tmap_v, kt, ragged && kt == n_max - 1);
+          if (kt == 0) draw(nxt);                 // its look-ups overlap this item's work
         }
         cur = nxt;
       }
@@ -262,7 +273,8 @@ attn_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__ 
         if (q_issued[g] > 0) mbar_wait_drain(smem_u32(&bk->q_full[g]), (q_issued[g] - 1) & 1, AT_WAIT_LIMIT);
       for (int s = 0; s < AT_SLOTS; ++s) {
         const int fills = t_issued > s ? (t_issued - s + AT_SLOTS - 1) / AT_SLOTS : 0;
-        if (fills > 0) mbar_wait_drain(smem_u32(&bk->full[s]), (fills - 1) & 1, AT_WAIT_LIMIT);
+        if ((raw_any >> s) & 1u) mbar_wait_drain(smem_u32(&bk->raw[s]), ((raw_odd >> s) & 1u) ^ 1u, AT_WAIT_LIMIT);
+        if (fills > 0 && !((raw_last >> s) & 1u)) mbar_wait_drain(smem_u32(&bk->full[s]), (fills - 1) & 1, AT_WAIT_LIMIT);
       }
       __syncwarp();
     } else if (warp == 1) {
@@ -365,6 +377,30 @@ attn_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__ 
       for (int t = lane; t < (2 + AT_EXT_BUFS) * AT_EXT_BYTES / 16; t += 32)
         reinterpret_cast<uint4 *>(at_smem + AT_EXT_OFF)[t] = make_uint4(0u, 0u, 0u, 0u);
       __syncwarp();
+      // The last key and value tile of a sequence reaches into the next one (or past the tensors).  Its probabilities there are
+      // exactly zero, but 0 * NaN and an addend on a NaN are NaN: value rows there, and key rows where the mask is an addend, are
+      // cleared before the tiles are multiplied.  Such tiles land on `raw` and are handed on here.  (A warp of its own for this
+      // cost 2 % on short sequences: it polls beside the softmax warps of its scheduler.)
+      int t0 = 0;                                 // first tile of the item in the ring
+      uint32_t raw_phase = 0u;                    // per ring slot
+      auto clear_past = [&](const AttnItem &it) {
+        const int n_max = max(it.n_kt[0], it.n_kt[1]), rows = it.n - (n_max - 1) * 128;     // rows inside the sequence
+        for (int v = rows >= 128 ? 2 : (attn_last_above(it.n_kt, it.sees, it.q_base) ? 0 : 1); v < 2; ++v) {
+          const int s = (t0 + 2 * n_max - 2 + v) & (AT_SLOTS - 1);
+          const bool landed = mbar_wait(smem_u32(&bk->raw[s]), (raw_phase >> s) & 1u, wc);
+          raw_phase ^= 1u << s;
+          if (!__all_sync(0xffffffffu, landed)) continue;     // (gave up: the copy may not have been issued)
+          uint8_t *tile = at_smem + (2 + s) * AT_TILE_BYTES;
+          for (int i = rows * 8 + lane; i < 128 * 8; i += 32) {
+            reinterpret_cast<uint4 *>(tile)[i] = make_uint4(0u, 0u, 0u, 0u);
+            reinterpret_cast<uint4 *>(tile + AT_BLOCK_BYTES)[i] = make_uint4(0u, 0u, 0u, 0u);
+          }
+          fence_proxy_async();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(smem_u32(&bk->full[s]));
+        }
+        t0 += 2 * n_max;
+      };
       int rc[2] = {0, 0}, mc[2] = {0, 0}, ec = 0;             // row-side, diagonal and key-side addend tiles so far
       for (int ic = 0;; ++ic) {
         const int slot = ic % AT_ITEM_SLOTS;
@@ -375,66 +411,68 @@ attn_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__ 
         __syncwarp();
         if (lane == 0) mbar_arrive(smem_u32(&bk->item_empty[slot]));
         if (it.b < 0) break;
-        if (!it.sees[0] && !it.sees[1]) continue;
-        const float *mlog = a.mask_log + (size_t)it.b * a.mask_b_stride + (size_t)it.h * a.mask_h_stride - it.v0;
-        // row side: columns 0-2 are 1 for a row of the span (they meet the three pieces of m_j), column 3 for any other row
-        // (it meets AT_NEVER)
-#pragma unroll
-        for (int g = 0; g < 2; ++g) {
-          if (!it.sees[g]) continue;
-          if (rc[g] >= 1) mbar_wait_warp(smem_u32(&bk->rows_empty[g]), (rc[g] - 1) & 1, wc);
-          for (int r = lane; r < 128; r += 32) {
-            const int i = it.q_base + g * 128 + r;
-            const bool vis = i >= it.v0 && i < it.v_end;
-            *ext_row(g, r) = vis ? make_uint4(0x3f803f80u, 0x00003f80u, 0u, 0u) : make_uint4(0u, 0x3f800000u, 0u, 0u);
-          }
-          fence_proxy_async();
-          __syncwarp();
-          if (lane == 0) mbar_arrive(smem_u32(&bk->rows_full[g]));
-          ++rc[g];
-        }
-        const int n_max = max(it.n_kt[0], it.n_kt[1]);
-        for (int kt = 0; kt < n_max; ++kt) {
-          AttnTileKind kind[2];
-#pragma unroll
-          for (int g = 0; g < 2; ++g) kind[g] = attn_tile_kind(kt < it.n_kt[g] ? it.sees[g] : 0, it.q_base + g * 128, kt);
-          if (!kind[0].above && !kind[1].above && !kind[0].crossed && !kind[1].crossed) continue;
-          float m[4];                                         // keys kt * 128 + lane + 32 e
-#pragma unroll
-          for (int e = 0; e < 4; ++e) {
-            const int j = kt * 128 + lane + 32 * e;
-            m[e] = j >= it.v0 && j < it.v_end ? fmaxf(__ldg(mlog + j) * m_to_raw, AT_NEVER) : AT_NEVER;
-          }
+        if (it.sees[0] || it.sees[1]) {
+          const float *mlog = a.mask_log + (size_t)it.b * a.mask_b_stride + (size_t)it.h * a.mask_h_stride - it.v0;
+          // row side: columns 0-2 are 1 for a row of the span (they meet the three pieces of m_j), column 3 for any other row
+          // (it meets AT_NEVER)
 #pragma unroll
           for (int g = 0; g < 2; ++g) {
-            if (!kind[g].crossed) continue;
-            if (mc[g] >= 1) mbar_wait_warp(smem_u32(&bk->m_empty[g]), (mc[g] - 1) & 1, wc);
-#pragma unroll
-            for (int e = 0; e < 4; ++e) bk->m_tile[g][lane + 32 * e] = m[e];
-            __syncwarp();
-            if (lane == 0) mbar_arrive(smem_u32(&bk->m_full[g]));
-            ++mc[g];
-          }
-          if (kind[0].above || kind[1].above) {
-            const int eb = ec % AT_EXT_BUFS;
-            if (ec >= AT_EXT_BUFS) mbar_wait_warp(smem_u32(&bk->ext_empty[eb]), ((ec / AT_EXT_BUFS) - 1) & 1, wc);
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-              // the addend as three bf16 pieces: 24 bits of mantissa, all of fp32's
-              float piece[3], rest = m[e];
-#pragma unroll
-              for (int k = 0; k < 3; ++k) {
-                piece[k] = __bfloat162float(__float2bfloat16_rn(rest));
-                rest -= piece[k];
-              }
-              *ext_row(2 + eb, lane + 32 * e) = make_uint4(pack2_rn(piece[0], piece[1]), pack2_rn(piece[2], AT_NEVER), 0u, 0u);
+            if (!it.sees[g]) continue;
+            if (rc[g] >= 1) mbar_wait_warp(smem_u32(&bk->rows_empty[g]), (rc[g] - 1) & 1, wc);
+            for (int r = lane; r < 128; r += 32) {
+              const int i = it.q_base + g * 128 + r;
+              const bool vis = i >= it.v0 && i < it.v_end;
+              *ext_row(g, r) = vis ? make_uint4(0x3f803f80u, 0x00003f80u, 0u, 0u) : make_uint4(0u, 0x3f800000u, 0u, 0u);
             }
             fence_proxy_async();
             __syncwarp();
-            if (lane == 0) mbar_arrive(smem_u32(&bk->ext_full[eb]));
-            ++ec;
+            if (lane == 0) mbar_arrive(smem_u32(&bk->rows_full[g]));
+            ++rc[g];
+          }
+          const int n_max = max(it.n_kt[0], it.n_kt[1]);
+          for (int kt = 0; kt < n_max; ++kt) {
+            AttnTileKind kind[2];
+#pragma unroll
+            for (int g = 0; g < 2; ++g) kind[g] = attn_tile_kind(kt < it.n_kt[g] ? it.sees[g] : 0, it.q_base + g * 128, kt);
+            if (!kind[0].above && !kind[1].above && !kind[0].crossed && !kind[1].crossed) continue;
+            float m[4];                                         // keys kt * 128 + lane + 32 e
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+              const int j = kt * 128 + lane + 32 * e;
+              m[e] = j >= it.v0 && j < it.v_end ? fmaxf(__ldg(mlog + j) * m_to_raw, AT_NEVER) : AT_NEVER;
+            }
+#pragma unroll
+            for (int g = 0; g < 2; ++g) {
+              if (!kind[g].crossed) continue;
+              if (mc[g] >= 1) mbar_wait_warp(smem_u32(&bk->m_empty[g]), (mc[g] - 1) & 1, wc);
+#pragma unroll
+              for (int e = 0; e < 4; ++e) bk->m_tile[g][lane + 32 * e] = m[e];
+              __syncwarp();
+              if (lane == 0) mbar_arrive(smem_u32(&bk->m_full[g]));
+              ++mc[g];
+            }
+            if (kind[0].above || kind[1].above) {
+              const int eb = ec % AT_EXT_BUFS;
+              if (ec >= AT_EXT_BUFS) mbar_wait_warp(smem_u32(&bk->ext_empty[eb]), ((ec / AT_EXT_BUFS) - 1) & 1, wc);
+#pragma unroll
+              for (int e = 0; e < 4; ++e) {
+                // the addend as three bf16 pieces: 24 bits of mantissa, all of fp32's
+                float piece[3], rest = m[e];
+#pragma unroll
+                for (int k = 0; k < 3; ++k) {
+                  piece[k] = __bfloat162float(__float2bfloat16_rn(rest));
+                  rest -= piece[k];
+                }
+                *ext_row(2 + eb, lane + 32 * e) = make_uint4(pack2_rn(piece[0], piece[1]), pack2_rn(piece[2], AT_NEVER), 0u, 0u);
+              }
+              fence_proxy_async();
+              __syncwarp();
+              if (lane == 0) mbar_arrive(smem_u32(&bk->ext_full[eb]));
+              ++ec;
+            }
           }
         }
+        clear_past(it);
       }
     }
   } else {

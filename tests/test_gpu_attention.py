@@ -89,6 +89,37 @@ def test_a_late_dominant_key_moves_the_softmax_reference(ctx, where, scale):
     _compare(batch, v, _run(ctx, batch, v, m), ms)
 
 
+@pytest.mark.parametrize("skipped", [False, True], ids=["valid", "skipped"])
+@pytest.mark.parametrize("nv,text", [(300, 30), (300, 100), (40, 5), (380, 1), (250, 3), (600, 31)])
+def test_a_sequence_does_not_see_its_neighbours(ctx, nv, text, skipped):
+    """NaN and infinities in the keys and values of the next sequence, which the last key tile of a sequence reaches into
+    unless its length is a multiple of 128 (250 + 3 + 3): not one bit of the sequence's own rows changes.  The same when the
+    next sequence fails the validation."""
+    batch = W.tiny(B=2, n_vis=[nv, 200], text_lens=[text, 9], H=2, keep_k=8, seed=617)
+    v = W.draw_values(batch, 87)
+    m, _ = _mask_vectors(batch, 1.0)
+    n0 = int(batch.cu_seqlens[1])
+    good = _run(ctx, batch, v, m)[:n0].clone()
+    bad = torch.tensor([float("nan"), float("inf"), -float("inf")], dtype=torch.bfloat16)
+    rows = torch.arange(n0, n0 + 200)
+    batch.k[rows] = bad[rows % 3][:, None, None]
+    v[rows] = bad[(rows + 1) % 3][:, None, None]
+    inp = A.make_inputs(batch, DEV)
+    if skipped:
+        inp.text_len[1] = 9999
+    out = torch.zeros_like(v, device=DEV)
+    scratch = torch.empty(A.asap_attention_scratch_bytes(batch.total, batch.D), dtype=torch.uint8, device=DEV)
+    A.asap_attention(ctx, inp, A.Params(keep_k=1), m.to(DEV), v.to(DEV), scratch, out)
+    torch.cuda.synchronize()
+    if skipped:
+        with pytest.raises(A.AsapError):
+            A.asap_check(ctx)
+    else:
+        A.asap_check(ctx)
+    assert torch.isfinite(good.float()).all()
+    assert torch.equal(out[:n0].cpu(), good.cpu())
+
+
 def test_mask_off_is_causal_attention_and_only_visual_rows_differ(ctx):
     batch = W.tiny(B=2, n_vis=[200, 333], text_lens=[17, 5], H=2, keep_k=8, seed=610)
     v = W.draw_values(batch, 78)
