@@ -157,14 +157,14 @@ score_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__
       mbar_init(smem_u32(&bk->empty[s]), 2);             // a key tile: the MMAs and their issuer; a query tile: the sum warps
     }
     mbar_init(smem_u32(&bk->q_full), 1);
-    mbar_init(smem_u32(&bk->q_empty), 1);
+    mbar_init(smem_u32(&bk->q_empty), 3);                    // the MMAs and both sum warps
     for (int i = 0; i < 4; ++i) {
       mbar_init(smem_u32(&bk->acc_full[i]), 1);
       mbar_init(smem_u32(&bk->acc_empty[i]), 4);          // the epilogue warps of the group that owns the buffer
     }
     for (int i = 0; i < SC_ITEM_SLOTS; ++i) {
       mbar_init(smem_u32(&bk->item_full[i]), 1);
-      mbar_init(smem_u32(&bk->item_empty[i]), with_mass ? 11 : 9);   // the MMA issuer, every epilogue warp (and the sum warps)
+      mbar_init(smem_u32(&bk->item_empty[i]), 11);   // the MMA issuer, every epilogue warp, the sum warps
     }
     mbar_init(smem_u32(&bk->mma_done), 1);
     mbar_init(smem_u32(&bk->qbar_ready), 2);
@@ -279,7 +279,7 @@ score_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__
     // goes on multiplying whatever lies in the block's own memory: nothing of it is used)
     const uint32_t leader = warp_leader();
     const uint32_t tm = __shfl_sync(0xffffffffu, tmem_base, 0);
-    int kc = 0, qc = 0, ic = 0, mc = 0;               // mc: items whose summed-query rows were waited for
+    int kc = 0, qc = 0, ic = 0, mc = 0;               // mc: row pairs whose query tile the sum warps complete
     int ops0 = 0, ops1 = 0;                           // operations given to either epilogue group
     const uint32_t idesc1 = umma_idesc_bf16(128, 128);
     const uint64_t qdesc = umma_desc_sw128(q_smem), kdesc0 = umma_desc_sw128(k_smem);   // (every tile lies below 256 KB: offsets never carry out of the address field)
@@ -300,6 +300,7 @@ score_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__
         const RowPair T = score_row_pair(d, rp, a.mask_enable, pair_rows);
         const bool mass_here = with_mass && rp == 0;         // three more columns (16 with padding): the summed query
         const int n2 = T.n2 + (mass_here ? 16 : 0);          // columns of a pass-2 accumulator
+        const bool fixed = mass_here || T.nrows < T.n2;
         mbar_wait_warp(smem_u32(&bk->q_full), qc & 1, wc);
         // the accumulator of group gr's next operation, once the group has given it back
         auto acc = [&](int gr) -> int {
@@ -313,7 +314,7 @@ score_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__
         const int nq = mass_here ? (d.nv + 127) / 128 : 0;    // every key tile below nq is followed by a query tile (the sum warps')
         for (int u = 0; u < T.n_kt + T.n_p2; kc += u < nq ? 2 : 1, ++u) {
           const int s = kc % SC_STAGES;
-          if (mass_here && u == T.n_kt) {                    // an epilogue warp has written the summed-query rows
+          if (fixed && u == T.n_kt) {                        // the sum warps have written their rows
             mbar_wait_warp(smem_u32(&bk->qbar_ready), mc & 1, wc);
             ++mc;
           }
@@ -336,7 +337,7 @@ score_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__
           tc_commit_w(smem_u32(&bk->empty[s]), leader);
           if (leader) mbar_arrive(smem_u32(&bk->empty[s]));
         }
-        if (mass_here && T.n_p2 == 0) {                      // (no visual key tile: keep the barrier's phases in step)
+        if (fixed && T.n_p2 == 0) {                          // (no visual key tile: keep the barrier's phases in step)
           mbar_wait_warp(smem_u32(&bk->qbar_ready), mc & 1, wc);
           ++mc;
         }
@@ -467,7 +468,9 @@ score_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__
 #pragma unroll
                 for (int e = 0; e < 32; ++e) {
                   const float sv = row_vis ? soft[c + e] : -INFINITY;
-                  const float x = fmaf(__uint_as_float(r[e]), scale, (e <= lim) ? 0.f : sv);
+                  // (a select, not the sum with -inf: the key may belong to the next sequence and its logit be a NaN)
+                  const float v = fmaf(__uint_as_float(r[e]), scale, (e <= lim) ? 0.f : sv);
+                  const float x = (e > lim && sv == -INFINITY) ? -INFINITY : v;
                   r[e] = __float_as_uint(x);
                   mx[e & 3] = fmaxf(mx[e & 3], x);
                 }
@@ -600,8 +603,10 @@ score_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__
       }
     }
     __threadfence();
-  } else if (with_mass) {
+  } else {
     // ------------------------------------------------------------------ query-sum warps: one 64-column half of the head each
+    // They also clear the query rows between a pair's last row and the next multiple of 16: those belong to whatever lies behind
+    // the ranking rows, the next sequence perhaps, and a NaN there would pass through the offset of -inf into every key's sum.
     if (warp == 11 && blockIdx.x == 0 && a.pa.write_desc) prepare_warp(a.pa);
     const int half = warp - 10;
     const int c = lane & 7, r0 = lane >> 3;        // a lane adds 16-byte chunk c of rows r0, r0 + 4, ...
@@ -618,7 +623,9 @@ score_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__
       const int n_rp = (d.nr + pair_rows - 1) / pair_rows;
       for (int rp = 0; rp < n_rp; ++rp, ++qc) {
         const RowPair T = score_row_pair(d, rp, a.mask_enable, pair_rows);
-        if (rp == 0) {
+        const bool mass_here = with_mass && rp == 0, fixed = mass_here || T.nrows < T.n2;
+        float f[8];
+        if (mass_here) {
           const int nq = (d.nv + 127) / 128;
           uint64_t acc[4] = {0ull, 0ull, 0ull, 0ull};
           for (int u = 0; u < nq; ++u, ++qt) {
@@ -637,7 +644,6 @@ score_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__
             __syncwarp();
             if (lane == 0) mbar_arrive(smem_u32(&bk->empty[s]));
           }
-          float f[8];
 #pragma unroll
           for (int e = 0; e < 4; ++e) f2_unpack(acc[e], f[2 * e], f[2 * e + 1]);
 #pragma unroll
@@ -645,11 +651,16 @@ score_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__
             f[e] += __shfl_xor_sync(0xffffffffu, f[e], 8);
             f[e] += __shfl_xor_sync(0xffffffffu, f[e], 16);
           }
+          kc += nq;
+        }
+        mbar_wait_warp(smem_u32(&bk->q_full), qc & 1, wc);    // (of every row pair, in order: its phases cannot be mistaken)
+        if (fixed) {
           // The summed query of this head as rows n2 .. n2 + 2 of the pair's query tile (row r of a 64-column half is 128
           // bytes at r * 128, chunk c at c ^ (r & 7)), once the tiled copy of the queries has landed: the value as three
           // bf16 pieces, 24 bits of mantissa, all of fp32's.  Lanes 8 k .. 8 k + 7 write piece k.
-          mbar_wait_warp(smem_u32(&bk->q_full), qc & 1, wc);
-          if (r0 < 3) {
+          uint8_t *qrows = base_ptr + half * SC_Q_HALF_BYTES;
+          for (int i = T.nrows * 8 + lane; i < T.n2 * 8; i += 32) reinterpret_cast<uint4 *>(qrows)[i] = make_uint4(0u, 0u, 0u, 0u);
+          if (mass_here && r0 < 3) {
             uint32_t w[4];
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
@@ -668,14 +679,13 @@ score_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__
               w[e] = pack2_rn(piece[0], piece[1]);
             }
             const int row = T.n2 + r0;
-            *reinterpret_cast<uint4 *>(base_ptr + half * SC_Q_HALF_BYTES + row * 128 + ((c ^ (row & 7)) << 4)) =
-                make_uint4(w[0], w[1], w[2], w[3]);
+            *reinterpret_cast<uint4 *>(qrows + row * 128 + ((c ^ (row & 7)) << 4)) = make_uint4(w[0], w[1], w[2], w[3]);
           }
           fence_proxy_async();
           __syncwarp();
           if (lane == 0) mbar_arrive(smem_u32(&bk->qbar_ready));
-          kc += nq;
         }
+        if (lane == 0) mbar_arrive(smem_u32(&bk->q_empty));
         kc += T.n_kt + T.n_p2;
       }
     }

@@ -63,6 +63,38 @@ def test_query_sums_inside_the_score_kernel(ctx, nvs, texts, H):
         A.asap_free(big)
 
 
+@pytest.mark.parametrize("per_head,visual", [(False, 0), (False, 5), (True, 0), (True, 5)], ids=["text", "rows", "heads", "heads_rows"])
+@pytest.mark.parametrize("text", [3, 37, 127, 128, 245, 491])
+def test_a_sequence_does_not_see_its_neighbours(ctx, text, per_head, visual):
+    """Everything of the next sequence is NaN or infinite (query rows up to the next multiple of 16 are multiplied with a
+    sequence's last ranking rows, key and hidden rows lie in its last tiles): not one bit of the sequence's results changes."""
+    batch = W.tiny(B=2, n_vis=[150, 140], text_lens=[text, 9], H=2, keep_k=30, seed=619, centres=6)
+    rank = (batch.text_start - visual, batch.text_len + visual) if visual else (None, None)
+    p = A.Params(keep_k=30, per_head_mask=per_head)
+    outs = []
+    for spoil in (False, True):
+        if spoil:
+            bad = torch.tensor([float("nan"), float("inf"), -float("inf")], dtype=torch.bfloat16)
+            rows = torch.arange(int(batch.cu_seqlens[1]), batch.total)
+            for i, t in enumerate((batch.q, batch.k, batch.hidden)):
+                t[rows] = bad[(rows + i) % 3].reshape(-1, *([1] * (t.dim() - 1)))
+        inp = A.make_inputs(batch, DEV, *rank)
+        out = A.alloc_outputs(inp, 30, fill=True, per_head=per_head)
+        A.asap_prune_step(ctx, inp, p, out)
+        score = A.alloc_outputs(inp, 30, fill=True, per_head=per_head)
+        A.asap_score(ctx, inp, p, score)
+        torch.cuda.synchronize()
+        A.asap_check(ctx)
+        outs.append((out, score))
+    n = int(outs[0][0].out_cu_seqlens[1])
+    for good, bad in zip(*outs):
+        for f in ("mass", "salience", "mask_log", "rank_score", "keep_idx", "drop_idx", "assign", "best_sim", "mask_log_heads"):
+            if getattr(good, f) is not None and (good is outs[0][0] or f in ("mass", "salience", "rank_score")):
+                assert torch.equal(getattr(good, f)[0], getattr(bad, f)[0]), f
+    for f in ("out_hidden", "out_pos", "src_row"):
+        assert torch.equal(getattr(outs[0][0], f)[:n], getattr(outs[1][0], f)[:n]), f
+
+
 @pytest.mark.parametrize("nvs,k", [([1028, 1029], 4), ([2500, 1030], 3), ([40, 16], 16), ([2060], 7)],
                          ids=["one_pass", "three_passes", "nothing_dropped", "three_passes_one"])
 def test_merge_blocks_that_scan_for_their_members(ctx, nvs, k):
