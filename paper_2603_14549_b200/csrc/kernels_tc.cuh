@@ -1048,13 +1048,9 @@ sim_kernel(const __grid_constant__ CUtensorMap tmap_h, const __grid_constant__ C
       int kb = kb0 + (mt * 5 + b * 3) % n_kb;
       RingPos r;
       for (int it = 0; it < total_it; ++it) {
-        int go = 1;
-        if (lane == 0) {
-          if (it >= a.a_stages) mbar_wait(smem_u32(&bk->empty[r.slot]), r.phase ^ 1u, wc);
-          go = bk->abort_flag ? 0 : 1;
-        }
-        go = __shfl_sync(0xffffffffu, go, 0);
-        if (!go) break;
+        // (every lane waits: each overwrites rows that the epilogue warps have read and the MMAs multiplied)
+        if (it >= a.a_stages) mbar_wait_warp(smem_u32(&bk->empty[r.slot]), r.phase ^ 1u, wc);
+        if (__shfl_sync(0xffffffffu, bk->abort_flag, 0)) break;
         const uint32_t dst = dst0 + r.slot * SIM_A_BYTES;
 #pragma unroll
         for (int i = 0; i < RW / 4; ++i)                   // (row r of a block: its chunk c at position c ^ (r & 7))

@@ -76,6 +76,37 @@ def test_similarity_kernel_gives_up_and_the_context_recovers(ctx):
     _same(ref, again, ("assign", "best_sim", "out_hidden", "out_pos", "src_row", "out_cu_seqlens"))
 
 
+def test_gathered_similarity_gives_up_and_the_context_recovers():
+    """Enough sequences with two fifths of their rows kept: the row operand is gathered by warps of its own, whose waits for a
+    free ring slot (16 rounds through rings of a few slots) are bounded like the others.  Calls before and after agree bit for bit."""
+    B, k = 40, 200
+    batch = W.tiny(B=B, n_vis=[500] * (B - 1) + [431], text_lens=[5] * B, H=8, keep_k=k, seed=605, centres=30)
+    c = A.asap_init(0, max_total_tokens=batch.total + B * 500, max_B=B, max_H=8, max_D=1024, max_keep_rows=B * k)
+    try:
+        inp = A.make_inputs(batch, DEV)
+        p = A.Params(keep_k=k)
+        names = ("assign", "best_sim", "out_hidden", "out_pos", "src_row", "out_cu_seqlens")
+        good = A.alloc_outputs(inp, k, fill=True)
+        A.asap_prune_step(c, inp, p, good)
+        torch.cuda.synchronize(); A.asap_check(c)
+        args = (good.salience.clone(), good.keep_idx.clone(), good.drop_idx.clone())
+        for limit in (0, 0, 1, 0, 0):
+            out = A.alloc_outputs(inp, k, fill=True)
+            if limit:
+                A.asap_debug_wait_limit(c, limit)
+            A.asap_merge(c, inp, p, *args, out)
+            torch.cuda.synchronize()
+            if limit:
+                with pytest.raises(A.AsapError) as e:
+                    A.asap_check(c)
+                assert e.value.status == -6 and "timed out in the similarity kernel" in str(e.value)
+            else:
+                A.asap_check(c)
+                _same(good, out, names)
+    finally:
+        A.asap_free(c)
+
+
 def test_attention_kernel_gives_up_and_the_context_recovers(ctx):
     batch = W.tiny(B=2, n_vis=[300, 200], text_lens=[30, 11], H=2, keep_k=40, seed=603, centres=6)
     inp = A.make_inputs(batch, DEV)
