@@ -416,6 +416,8 @@ asap_status launch_merge_front(asap_ctx *ctx, const asap_inputs *in, const asap_
     // the groups' best slots.  Several passes inside one block would read the dropped rows from memory once per pass: the rows
     // that all resident blocks hold between two passes do not fit L2.
     int groups = 1;
+    int a_stages = 0, b_stages = 0;                      // gathered form: slots of the rows' ring and of the kept rows'
+    size_t gather_ring = 0;
     if (gather_rows) {
       const int mt_g = (in->max_vis - k + 127) / 128;
       int g = (k + 383) / 384;
@@ -423,7 +425,16 @@ asap_status launch_merge_front(asap_ctx *ctx, const asap_inputs *in, const asap_
       const int tiles_g = per_group > 256 ? 2 : 1;
       const int tile_g = (((per_group + tiles_g - 1) / tiles_g) + 15) & ~15;
       g = (k + tiles_g * tile_g - 1) / (tiles_g * tile_g);
-      gather_rows = (size_t)B * mt_g <= ctx->cap_tiles &&
+      // the rows arrive slowly (16 KB in about 1000 clocks, the load unit's requests in flight) and the kept rows fast, so the
+      // rows have a ring of their own with as many slots as the kept rows leave (one ring of three stages with both: three steps
+      // of 32 x 2304, 5120 wide, 887 -> 773 us)
+      const int b_tile = tiles_g * tile_g * 128;
+      b_stages = b_tile > 32 * 1024 ? 2 : 3;
+      a_stages = (192 * 1024 - b_stages * b_tile) / SIM_A_BYTES;
+      if (a_stages > SIM_MAX_STAGES) a_stages = SIM_MAX_STAGES;
+      gather_ring = (size_t)a_stages * SIM_A_BYTES + (size_t)b_stages * b_tile;
+      // (the grouping's counters lie in the rings, one set per warp: above some 4400 slots the tiled form, with fewer warps)
+      gather_rows = (size_t)B * mt_g <= ctx->cap_tiles && (size_t)(SIM_THREADS / 32 + 1) * k * sizeof(int) <= gather_ring &&
                     (g == 1 || (size_t)B * mt_g * g * 256 * sizeof(float) <= ctx->sim_part_bytes);
       if (gather_rows) { groups = g; n_nt = tiles_g; n_tile = tile_g; max_mt = mt_g; }
     }
@@ -479,17 +490,8 @@ asap_status launch_merge_front(asap_ctx *ctx, const asap_inputs *in, const asap_
     // the SM its 32 KB of L1
     int stages = ((two_per_sm ? 96 : 192) * 1024) / stage_bytes_used;
     if (stages > SIM_MAX_STAGES) stages = SIM_MAX_STAGES;
-    // gathered form: the rows arrive slowly (16 KB in about 1000 clocks, the load unit's requests in flight) and the kept rows
-    // fast, so the rows have a ring of their own with as many slots as the kept rows leave (one ring of three stages with both:
-    // three steps of 32 x 2304, 5120 wide, 887 -> 773 us)
-    const int b_tile = n_nt * n_tile * 128;
-    int a_stages = 0;
-    if (gather_rows) {
-      stages = b_tile > 32 * 1024 ? 2 : 3;
-      a_stages = (192 * 1024 - stages * b_tile) / SIM_A_BYTES;
-      if (a_stages > SIM_MAX_STAGES) a_stages = SIM_MAX_STAGES;
-    }
-    const size_t ring = gather_rows ? (size_t)a_stages * SIM_A_BYTES + (size_t)stages * b_tile : (size_t)stages * stage_bytes_used;
+    if (gather_rows) stages = b_stages;
+    const size_t ring = gather_rows ? gather_ring : (size_t)stages * stage_bytes_used;
     const size_t smem = ring + SIM_BOOK_BYTES + 1024;
     const int sim_threads = gather_rows ? SIM_THREADS : SIM_THREADS_TILED;
     if ((size_t)(sim_threads / 32 + 1) * k * sizeof(int) > ring)

@@ -106,6 +106,16 @@ def test_pair_form_matches_the_oracle(ctx_pair_form, n_vis, k):
     _merge_matches_oracle(ctx_pair_form, n_vis, k, H=2, seed=911)
 
 
+def test_many_kept_slots_of_a_long_sequence():
+    """A third of 15000 rows kept: enough for the gathered form, but the grouping's counters do not fit its shared memory; the
+    tiled form with its fewer warps takes the call (20 slot tiles that share two accumulators)."""
+    c = A.asap_init(0, max_total_tokens=31000, max_B=2, max_H=2, max_D=256, max_keep_rows=10000)
+    try:
+        _merge_matches_oracle(c, [15000, 5100], 5000, H=2, seed=934)
+    finally:
+        A.asap_free(c)
+
+
 def test_pair_form_gives_up_and_the_context_recovers(ctx_pair_form):
     """The bounded waits of this form, in the harmless way: the wait limit of one call is a single clock
     cycle, the call returns, the status names the kernel, and the next call is a fresh one bit for bit."""
