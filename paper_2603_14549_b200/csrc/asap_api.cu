@@ -691,7 +691,7 @@ routing:
   RouteArgs ra;
   ra.desc = ctx->desc; ra.max_vis = in->max_vis; ra.keep_k = k; ra.kw = (k + 31) / 32;
   ra.threshold = p->sim_threshold; ra.smat = smat;
-  const size_t fixed_words = 5 * (size_t)k + 3;
+  const size_t fixed_words = 5 * (size_t)k;
   const size_t tail_words = (size_t)(in->max_vis - k) + (size_t)in->max_vis;
   const size_t mask_words = (size_t)k * ra.kw;
   const bool mask_in_smem = (fixed_words + (mask_words > tail_words ? mask_words : tail_words)) * 4 <= 200 * 1024;

@@ -1070,15 +1070,13 @@ route_kernel(RouteArgs a) {
     return;
   }
   const int nv = d.nv, nd = nv - k;
-  // shared memory: [tmp k4][order k][rank k][flag k][dest k] [union: bit matrix k*kw | key nd_max + pos max_vis], k4 = k rounded up
-  // to a multiple of four
-  const int k4 = (k + 3) & ~3;
+  // shared memory: [tmp k][order k][rank k][flag k][dest k] [union: bit matrix k*kw | key nd_max + pos max_vis]
   uint32_t *s_tmp = r_smem;
-  int *s_order = reinterpret_cast<int *>(r_smem + k4);
+  int *s_order = reinterpret_cast<int *>(r_smem + k);
   int *s_rank = s_order + k;
   int *s_flag = s_rank + k;
   int *s_dest = s_flag + k;
-  uint32_t *s_union = r_smem + k4 + 4 * (size_t)k;
+  uint32_t *s_union = r_smem + 5 * (size_t)k;
   uint32_t *mask = a.mask_in_smem ? s_union : a.mask_g + (size_t)b * k * kw;
   const int32_t *keep_b = a.keep_idx + (size_t)b * k;
   const int32_t *drop_b = a.drop_idx + (size_t)b * nd_max;
@@ -1090,7 +1088,6 @@ route_kernel(RouteArgs a) {
     const int j = min(max(keep_b[p], 0), nv - 1);
     s_tmp[p] = score_key(sal_b[j]);
   }
-  if (tid < k4 - k) s_tmp[k + tid] = 0u;
   // the attention mass of this thread's first pruned tokens, for E: two dependent loads that end long before they are needed
   uint32_t mass_key[4];
 #pragma unroll
@@ -1101,22 +1098,23 @@ route_kernel(RouteArgs a) {
   __syncthreads();
   for (int p = tid; p < k; p += nthr) {
     const uint32_t mine = s_tmp[p];
-    // the kept list is ascending: an equal key before p is the lower index.  Four keys per (broadcast) load; the keys are
-    // padded to a multiple of four with zeros, which no key after p is below
+    // the kept list is ascending: an equal key before p is the lower index.  Four keys per (broadcast) load
     int r = 0;
     const uint4 *t4 = reinterpret_cast<const uint4 *>(s_tmp);
-    const int pc = p >> 2, nc = k4 >> 2;
+    const int pc = p >> 2, nc = k >> 2;
 #pragma unroll 4
     for (int c = 0; c < pc; ++c) {
       const uint4 o = t4[c];
       r += (o.x >= mine) + (o.y >= mine) + (o.z >= mine) + (o.w >= mine);
     }
-    {
-      const uint4 o = t4[pc];
-      const uint32_t ov[4] = {o.x, o.y, o.z, o.w};
+    uint32_t own[4], last[4];                           // p's own four, and the up to three past the last whole four
 #pragma unroll
-      for (int e = 0; e < 4; ++e) r += ov[e] > mine || (ov[e] == mine && pc * 4 + e < p);
+    for (int e = 0; e < 4; ++e) {
+      own[e] = pc * 4 + e < k ? s_tmp[pc * 4 + e] : 0u;
+      last[e] = pc < nc && nc * 4 + e < k ? s_tmp[nc * 4 + e] : 0u;
     }
+#pragma unroll
+    for (int e = 0; e < 4; ++e) r += (own[e] > mine || (own[e] == mine && pc * 4 + e < p)) + (last[e] > mine);
 #pragma unroll 4
     for (int c = pc + 1; c < nc; ++c) {
       const uint4 o = t4[c];

@@ -219,6 +219,21 @@ def test_bit_matrix_in_global_memory_for_large_keep(ctx):
     assert _check(batch, 1400, 0.85, out, n_abs, st1) > 0
 
 
+def test_the_longest_span_the_routing_has_room_for():
+    """4096 of 20480 tokens kept: the routing's lists fill its 224 KB of shared memory to the last word, and one token more is refused."""
+    c = A.asap_init(0, max_total_tokens=20600, max_B=1, max_H=1, max_D=128, max_keep_rows=4096)
+    try:
+        batch = W.tiny(B=1, n_vis=[20480], text_lens=[8], H=1, keep_k=4096, seed=517, centres=90)
+        stage1 = lambda bt, b, kk: W.random_stage1(bt, b, kk, 79)
+        out, n_abs, st1 = _run(c, batch, 4096, 0.85, stage1=stage1)
+        assert _check(batch, 4096, 0.85, out, n_abs, st1) > 0
+        with pytest.raises(A.AsapError) as e:
+            _run(c, W.tiny(B=1, n_vis=[20481], text_lens=[8], H=1, keep_k=4096, seed=518, centres=90), 4096, 0.85, stage1=stage1)
+        assert e.value.status == -5
+    finally:
+        A.asap_free(c)
+
+
 @pytest.fixture(scope="module")
 def big_ctx():
     c = A.asap_init(0, max_total_tokens=32 * (35 + 2304 + 128) + 2304, max_B=32, max_H=40, max_D=5120,
