@@ -281,16 +281,7 @@ asap_status asap_select_static(const asap_inputs *in, const asap_params *p, cons
 typedef struct {
   char name[32];     /* kernel name: "qsum", "mass_salience", "score", "select", "sim", ... */
   uint64_t launches; /* launches timed since profiling was enabled */
-  double total_ms;   /* Diagnostics for the bounded waits of the tensor-core kernels (conventions above; the paper has no
- * counterpart).  The next call of an entry point on this context -- and only that call -- runs with
- * `cycles` clock cycles as the limit of every wait, instead of about a second.  With a limit of a few
- * cycles a healthy run gives up at its first wait that is not satisfied at once: the call returns
- * normally, its results are invalid, and asap_check reports ASAP_ERR_DEVICE with the kernel's
- * time-out bit.  This is how the give-up path is exercised without making anything hang.  cycles must
- * be positive. */
-asap_status asap_debug_wait_limit(asap_ctx *ctx, long long cycles);
-
-/* sum over those launches of (next event - this kernel's event) */
+  double total_ms;   /* sum over those launches of (next event - this kernel's event) */
 } asap_kernel_time;
 asap_status asap_profile(asap_ctx *ctx, int enable);
 
@@ -299,6 +290,15 @@ asap_status asap_profile(asap_ctx *ctx, int enable);
  * many kernels have a total.  A kernel's time runs to the start of the next kernel of the same
  * call, so it includes the launch gap behind it. */
 int asap_profile_read(asap_ctx *ctx, asap_kernel_time *out, int capacity);
+
+/* Diagnostics for the bounded waits of the tensor-core kernels (conventions above; the paper has no
+ * counterpart).  The next call of an entry point on this context -- and only that call -- runs with
+ * `cycles` clock cycles as the limit of every wait, instead of about a second.  With a limit of a few
+ * cycles a healthy run gives up at its first wait that is not satisfied at once: the call returns
+ * normally, its results are invalid, and asap_check reports ASAP_ERR_DEVICE with the kernel's
+ * time-out bit.  This is how the give-up path is exercised without making anything hang.  cycles must
+ * be positive. */
+asap_status asap_debug_wait_limit(asap_ctx *ctx, long long cycles);
 
 /* Number of kernel launches the library has enqueued through this context so far. */
 uint64_t asap_launch_count(const asap_ctx *ctx);

@@ -3,6 +3,7 @@ header declares; the binding's structs match the header's field order."""
 import ctypes
 import os
 import re
+import subprocess
 
 import pytest
 
@@ -26,6 +27,17 @@ def test_every_declared_symbol_is_exported(lib):
         assert hasattr(lib, name), name
 
 
+@pytest.mark.parametrize("lang,std", [("c", "c99"), ("c++", "c++17")])
+def test_the_header_is_c_and_declares_every_function(tmp_path, lang, std):
+    """A C program that takes the address of every exported function compiles against the header alone."""
+    src = tmp_path / "use.c"
+    src.write_text('#include "asap.h"\nvoid *use[] = {' + ", ".join(f"(void *)&{n}" for n in A.EXPORTS) + "};\n"
+                   "unsigned long size(void) { return (unsigned long)sizeof(asap_kernel_time); }\n")
+    res = subprocess.run(["gcc", "-x", lang, f"-std={std}", "-Wall", "-Wextra", "-Werror", "-fsyntax-only",
+                          "-I", os.path.join(ROOT, "include"), str(src)], capture_output=True, text=True)
+    assert res.returncode == 0, res.stderr
+
+
 def _struct_fields(name):
     body = re.search(r"typedef struct \{([^}]*)\}\s*" + name + ";", HEADER, re.S).group(1)
     body = re.sub(r"/\*.*?\*/", "", body, flags=re.S)
@@ -35,12 +47,12 @@ def _struct_fields(name):
         if not decl:
             continue
         for part in decl.split(","):
-            fields.append(re.findall(r"\*?\s*([A-Za-z_0-9]+)\s*$", part.strip())[0])
+            fields.append(re.findall(r"\*?\s*([A-Za-z_0-9]+)\s*(?:\[\d+\])?$", part.strip())[0])
     return fields
 
 
 @pytest.mark.parametrize("cname,cls", [("asap_inputs", A.CInputs), ("asap_params", A.CParams),
-                                       ("asap_outputs", A.COutputs)])
+                                       ("asap_outputs", A.COutputs), ("asap_kernel_time", A.CKernelTime)])
 def test_binding_struct_matches_header(cname, cls):
     assert _struct_fields(cname) == [f[0] for f in cls._fields_]
 
