@@ -341,7 +341,7 @@ bool merge_scans(const asap_ctx *ctx, const asap_inputs *in, const asap_params *
 
 SalienceArgs salience_args(const asap_ctx *ctx, const asap_inputs *in, const asap_params *p, const asap_outputs *out) {
   SalienceArgs a;
-  a.H = in->H; a.scale = 1.0f / ((float)in->H * sqrtf((float)in->head_dim)); a.lambda_max = p->lambda_max; a.eps = p->eps;
+  a.H = in->H; a.scale = 1.0 / ((double)in->H * sqrt((double)in->head_dim)); a.lambda_max = p->lambda_max; a.eps = p->eps;
   a.heads = ctx->mass_partial; a.norm = p->per_head_mask ? ctx->head_norm : nullptr; a.mass = out->mass; a.salience = out->salience;
   a.mask_log = out->mask_log; a.rank_score = out->rank_score;
   return a;

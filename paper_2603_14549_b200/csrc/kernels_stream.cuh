@@ -368,7 +368,8 @@ mass_heads_kernel(const __nv_bfloat16 *__restrict__ k, const SampleDesc *__restr
 
 struct SalienceArgs {
   int H;
-  float scale, lambda_max, eps;
+  double scale;                             // 1 / (H sqrt(head_dim))
+  float lambda_max, eps;
   const float *heads;                       // [B, H, max_vis]
   const float *norm;                        // [B, H, 2] or nullptr: a salience per head (salience_heads_block)
   float *mass, *salience, *mask_log, *rank_score;   // [B, max_vis]
@@ -454,7 +455,7 @@ salience_heads_kernel(const SampleDesc *__restrict__ desc, int max_vis, Salience
 // =======================================================================================
 // salience_block: the tail of Eq. 1 and Eq. 2-3 when the per-head masses qbar^h . k_j^h were
 // produced by the score kernel (from the query and key tiles it streams).  One block per sample, beside
-// the block that selects (grid y of the selection launch): s_j = scale * sum_h heads[b, h, j] (heads in order), then the min-max normalisation and
+// the block that selects (grid y of the selection launch): s_j = scale * sum_h heads[b, h, j], then the min-max normalisation and
 // the mask vector over the image span; padding past the span is zeroed as mass_salience does.
 // =======================================================================================
 constexpr int SAL_THREADS = 1024;
@@ -479,11 +480,22 @@ __device__ __forceinline__ float4 head_sum4(const float *p, int H, int max_vis) 
   return t;
 }
 
+// The masses' own sums over the heads: sixteen in pairs, the sixteens and the scale in 64 bits.  One after the other in 32 bits, 32
+// heads lose more than the masses themselves do (error against 64 bits 9.3e-8 instead of 5.0e-8 with their exact sum).
+template <int N>
+__device__ __forceinline__ float pair_sum(float (&v)[N]) {
+#pragma unroll
+  for (int o = 1; o < N; o <<= 1)
+#pragma unroll
+    for (int e = 0; e < N; e += 2 * o) v[e] += v[e + o];
+  return v[0];
+}
+
 __device__ __forceinline__ void salience_block(const SampleDesc &d, int b, int max_vis, const SalienceArgs &a) {
   __shared__ float s_red[2 * (SAL_THREADS / 32)];
   float *mass_b = a.mass + (size_t)b * max_vis, *sal_b = a.salience + (size_t)b * max_vis, *msk_b = a.mask_log + (size_t)b * max_vis;
   const int H = a.H;
-  const float scale = a.scale, lambda_max = a.lambda_max, eps = a.eps;
+  const float lambda_max = a.lambda_max, eps = a.eps;
   if (!d.valid) {
     for (int j = threadIdx.x; j < max_vis; j += SAL_THREADS) {
       mass_b[j] = 0.f; sal_b[j] = 0.f; msk_b[j] = 0.f;
@@ -496,28 +508,42 @@ __device__ __forceinline__ void salience_block(const SampleDesc &d, int b, int m
   const bool vec = wide_columns(max_vis, d.nv);
   if (vec) {
     for (int j = threadIdx.x * 4; j < d.nv; j += SAL_THREADS * 4) {
-      const float4 t4 = head_sum4(hb + j, H, max_vis);
-      const float tv[4] = {t4.x * scale, t4.y * scale, t4.z * scale, t4.w * scale};
+      double tot[4] = {0.0, 0.0, 0.0, 0.0};
+      for (int h0 = 0; h0 < H; h0 += 8) {
+        float v[4][8];
+#pragma unroll
+        for (int e = 0; e < 8; ++e) {
+          const float4 x = h0 + e < H ? __ldcg(reinterpret_cast<const float4 *>(hb + (size_t)(h0 + e) * max_vis + j)) : make_float4(0.f, 0.f, 0.f, 0.f);
+          v[0][e] = x.x; v[1][e] = x.y; v[2][e] = x.z; v[3][e] = x.w;
+        }
+#pragma unroll
+        for (int c = 0; c < 4; ++c) tot[c] += (double)pair_sum(v[c]);
+      }
 #pragma unroll
       for (int e = 0; e < 4; ++e) {
         if (j + e >= d.nv) break;
-        mass_b[j + e] = tv[e];
-        lo = fminf(lo, tv[e]); hi = fmaxf(hi, tv[e]);
+        const float m = (float)(tot[e] * a.scale);
+        mass_b[j + e] = m;
+        lo = fminf(lo, m); hi = fmaxf(hi, m);
       }
     }
   }
   for (int j = vec ? d.nv : (int)threadIdx.x; j < d.nv; j += SAL_THREADS) {
-    float tot = 0.f;
+    double sum = 0.0;
     int hh = 0;
     for (; hh + 16 <= H; hh += 16) {          // sixteen loads in flight
       float v[16];
 #pragma unroll
       for (int e = 0; e < 16; ++e) v[e] = __ldcg(hb + (size_t)(hh + e) * max_vis + j);
-#pragma unroll
-      for (int e = 0; e < 16; ++e) tot += v[e];
+      sum += (double)pair_sum(v);
     }
-    for (; hh < H; ++hh) tot += __ldcg(hb + (size_t)hh * max_vis + j);
-    tot *= scale;
+    if (hh < H) {
+      float v[16];
+#pragma unroll
+      for (int e = 0; e < 16; ++e) v[e] = hh + e < H ? __ldcg(hb + (size_t)(hh + e) * max_vis + j) : 0.f;
+      sum += (double)pair_sum(v);
+    }
+    const float tot = (float)(sum * a.scale);
     mass_b[j] = tot;
     lo = fminf(lo, tot); hi = fmaxf(hi, tot);
   }

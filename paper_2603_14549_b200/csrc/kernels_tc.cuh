@@ -55,9 +55,9 @@ __device__ __forceinline__ void group_bar_sync(int group) {
 // the queries taken first is qbar^h . k_j^h, and pass 2 already multiplies every visual key tile by the
 // row pair's queries.  The visual queries stream through the same ring, one tile behind every key tile of pass 1; two warps of
 // their own add them up (the pipes that bound the kernel are the exponentials' and the epilogue's: memory, shared memory and
-// issue slots have room) and write the sum as three more "query rows" (its bf16 value, the bf16
-// value of what that rounding lost, and again: 24 bits of mantissa together, all that fp32 holds)
-// behind the pair's rows in shared memory, so the first row pair's pass-2 accumulators get three
+// issue slots have room) and write the sum as ten more "query rows" (its bf16 value, dealt to eight rows by k-step, the
+// bf16 value of what that rounding lost, and again: 24 bits of mantissa together, all that fp32 holds)
+// behind the pair's rows in shared memory, so the first row pair's pass-2 accumulators get ten
 // more columns whose sum is the key's mass for this head.  Row pairs then hold at most 240 rows (the
 // accumulator grows by the 16 columns an MMA's width moves in).
 // =======================================================================================
@@ -298,7 +298,7 @@ score_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__
       const int n_rp = (d.nr + pair_rows - 1) / pair_rows;
       for (int rp = 0; rp < n_rp; ++rp, ++qc) {
         const RowPair T = score_row_pair(d, rp, a.mask_enable, pair_rows);
-        const bool mass_here = with_mass && rp == 0;         // three more columns (16 with padding): the summed query
+        const bool mass_here = with_mass && rp == 0;         // ten more columns (16 with padding): the summed query
         const int n2 = T.n2 + (mass_here ? 16 : 0);          // columns of a pass-2 accumulator
         const bool fixed = mass_here || T.nrows < T.n2;
         mbar_wait_warp(smem_u32(&bk->q_full), qc & 1, wc);
@@ -578,13 +578,14 @@ score_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__
                 }
               }
               if (with_mass && rp == 0 && T.n2 - h0 >= 0 && T.n2 - h0 < 128) {
-                // columns n2 .. n2 + 2: the three pieces of the summed query against this key
+                // columns n2 .. n2 + 9: the pieces of the summed query against this key
                 uint32_t r[16];
                 tmem_ld16(tlane + (T.n2 - h0), r);
                 tmem_wait_ld();
+                auto g = [&](int e) { return __uint_as_float(r[e]); };
                 if (key_ok)
                   a.mass_heads[((size_t)b * a.H + h) * a.max_vis + (j - d.v0)] =
-                      (__uint_as_float(r[0]) + __uint_as_float(r[1])) + __uint_as_float(r[2]);
+                      (((g(0) + g(1)) + (g(2) + g(3))) + ((g(4) + g(5)) + (g(6) + g(7)))) + (g(8) + g(9));
               }
             }
             tc_fence_before();
@@ -655,31 +656,35 @@ score_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__
         }
         mbar_wait_warp(smem_u32(&bk->q_full), qc & 1, wc);    // (of every row pair, in order: its phases cannot be mistaken)
         if (fixed) {
-          // The summed query of this head as rows n2 .. n2 + 2 of the pair's query tile (row r of a 64-column half is 128
-          // bytes at r * 128, chunk c at c ^ (r & 7)), once the tiled copy of the queries has landed: the value as three
-          // bf16 pieces, 24 bits of mantissa, all of fp32's.  Lanes 8 k .. 8 k + 7 write piece k.
+          // The summed query of this head as rows n2 .. n2 + 9 of the pair's query tile (row r of a 64-column half is 128
+          // bytes at r * 128, chunk c at c ^ (r & 7)), once the tiled copy of the queries has landed: the value as three bf16
+          // pieces, 24 bits of mantissa, all of fp32's.  The first piece is dealt to eight rows, one per k-step, zero elsewhere: the
+          // accumulator drops bits at every k-step that adds to it, so each step gets an accumulator of its own and
+          // the epilogue adds them up with rounding.  The other two pieces are small enough for a row each.
           uint8_t *qrows = base_ptr + half * SC_Q_HALF_BYTES;
           for (int i = T.nrows * 8 + lane; i < T.n2 * 8; i += 32) reinterpret_cast<uint4 *>(qrows)[i] = make_uint4(0u, 0u, 0u, 0u);
-          if (mass_here && r0 < 3) {
-            uint32_t w[4];
+          if (mass_here) {
+            uint32_t w[3][4];                               // [piece][two elements of this lane's chunk]
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
-              float piece[2];
+              float rest[2] = {f[2 * e], f[2 * e + 1]};
 #pragma unroll
-              for (int t = 0; t < 2; ++t) {
-                float rest = f[2 * e + t];
-                piece[t] = 0.f;
-#pragma unroll
-                for (int k = 0; k < 3; ++k) {
-                  const float q = __bfloat162float(__float2bfloat16_rn(rest));
-                  if (k == r0) piece[t] = q;
-                  rest -= q;
-                }
+              for (int k = 0; k < 3; ++k) {
+                w[k][e] = pack2_rn(rest[0], rest[1]);
+                rest[0] -= bf16_lo(w[k][e]);
+                rest[1] -= bf16_hi(w[k][e]);
               }
-              w[e] = pack2_rn(piece[0], piece[1]);
             }
-            const int row = T.n2 + r0;
-            *reinterpret_cast<uint4 *>(qrows + row * 128 + ((c ^ (row & 7)) << 4)) = make_uint4(w[0], w[1], w[2], w[3]);
+#pragma unroll
+            for (int i = 0; i < 3; ++i) {
+              const int j = r0 + 4 * i;                     // lanes 8 r0 .. 8 r0 + 7 write rows r0, r0 + 4 and r0 + 8 of the ten
+              const bool step = i < 2 && (j >> 2) == half && (j & 3) == c >> 1;
+              uint4 x = make_uint4(0u, 0u, 0u, 0u);
+              if (i < 2 && step) x = make_uint4(w[0][0], w[0][1], w[0][2], w[0][3]);
+              if (i == 2) x = r0 == 0 ? make_uint4(w[1][0], w[1][1], w[1][2], w[1][3]) : make_uint4(w[2][0], w[2][1], w[2][2], w[2][3]);
+              const int row = T.n2 + j;
+              if (j < 10) *reinterpret_cast<uint4 *>(qrows + row * 128 + ((c ^ (row & 7)) << 4)) = x;
+            }
           }
           fence_proxy_async();
           __syncwarp();

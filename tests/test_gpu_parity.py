@@ -95,6 +95,29 @@ def test_a_sequence_does_not_see_its_neighbours(ctx, text, per_head, visual):
         assert torch.equal(getattr(outs[0][0], f)[:n], getattr(outs[1][0], f)[:n]), f
 
 
+@pytest.mark.parametrize("H", [16, 20, 32, 40])
+@pytest.mark.parametrize("nvs", [[576], [1201, 1204, 300]], ids=["one", "ragged"])
+def test_masses_in_the_score_kernel_lose_no_precision(ctx, nvs, H):
+    """Eq. 1 from the tensor cores against 64 bits, heads of either sign.  The rounding of the result alone is 2^-24 / sqrt(3) =
+    3.4e-8 (2-norm); separate fp32 kernels for query sum and masses are off by 1.04e-7 to 1.33e-7 on these batches, and one
+    accumulator that all k-steps of a head add to by 1.26e-7 to 1.75e-7."""
+    batch = W.tiny(B=len(nvs), n_vis=nvs, text_lens=[9 + b for b in range(len(nvs))], H=H, keep_k=40, seed=160 + H, centres=9)
+    inp = A.make_inputs(batch, DEV)
+    out = A.alloc_outputs(inp, 40, fill=True)
+    A.asap_prune_step(ctx, inp, A.Params(keep_k=40), out)
+    torch.cuda.synchronize()
+    A.asap_check(ctx)
+    err = tot = 0.0
+    for b, nv in enumerate(nvs):
+        lo = int(batch.cu_seqlens[b]) + int(batch.vis_start[b])
+        q, k = inp.q[lo:lo + nv].double(), inp.k[lo:lo + nv].double()
+        s = (k * q.sum(0)).sum((1, 2)) / (H * math.sqrt(128))
+        err += float(((out.mass[b, :nv].double() - s) ** 2).sum())
+        tot += float((s ** 2).sum())
+    print("mass error, 2-norm:", math.sqrt(err / tot))
+    assert math.sqrt(err / tot) < 1.04e-7
+
+
 @pytest.mark.parametrize("nvs,k", [([1028, 1029], 4), ([2500, 1030], 3), ([40, 16], 16), ([2060], 7)],
                          ids=["one_pass", "three_passes", "nothing_dropped", "three_passes_one"])
 def test_merge_blocks_that_scan_for_their_members(ctx, nvs, k):
