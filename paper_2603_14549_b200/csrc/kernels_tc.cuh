@@ -7,6 +7,9 @@
 //   sim_kernel    Sec. 4.2: cosine similarity of every visual row against the kept rows with
 //                 the arg-max over kept slots taken in the epilogue.
 //
+// Nothing that the directly preceding kernel of the stream writes (mask vectors, inverse norms) is read by __ldg: these kernels
+// start while that one runs, and such a load promises that its data never change.
+//
 // All use one TMA-producer warp and one MMA-issuer warp, both walking their loops converged with one elected lane issuing
 // (see warp_leader), and one or two groups of four epilogue warps that read tensor memory (warp w may touch lanes
 // 32*(w%4) .. 32*(w%4)+31).
@@ -403,7 +406,7 @@ score_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__
           const bool stage_soft = T.use_soft && !fast;
           if (stage_soft) {
             const int j = j0 + lrow;
-            soft[lrow] = (j >= d.v0 && j < v_end) ? __ldg(mlog + (j - d.v0)) * LOG2E_F : -INFINITY;
+            soft[lrow] = (j >= d.v0 && j < v_end) ? mlog[j - d.v0] * LOG2E_F : -INFINITY;
             group_bar_sync(group);
           }
           const uint32_t tlane = tlane0 + buf * 128;
@@ -516,7 +519,7 @@ score_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__
           const bool key_ok = j >= d.v0 && j < v_end;
           const bool fast = (j0 + 127 <= T.R0);
           const bool warp_keys = (j0 + quarter * 32 + 31 >= d.v0) && (j0 + quarter * 32 < v_end);
-          const float soft_j = (T.use_soft && key_ok) ? __ldg(mlog + (j - d.v0)) * LOG2E_F : -INFINITY;
+          const float soft_j = (T.use_soft && key_ok) ? mlog[j - d.v0] * LOG2E_F : -INFINITY;
           uint64_t sm2[4] = {0ull, 0ull, 0ull, 0ull};
 #pragma unroll 1
           for (int h0 = 0; h0 < n2; h0 += 128, ++ops) {
@@ -1190,7 +1193,7 @@ sim_kernel(const __grid_constant__ CUtensorMap tmap_h, const __grid_constant__ C
 #pragma unroll
       for (int e = 0; e < 4; ++e) {
         const int c = e * 128 + lrow, slot = tile0 * a.n_tile + c;
-        if (c < a.n_nt * a.n_tile && slot < a.keep_k) kreg[e] = __ldg(kinv + slot);
+        if (c < a.n_nt * a.n_tile && slot < a.keep_k) kreg[e] = kinv[slot];
       }
     }
     for (int nt = 0; nt < a.n_nt; ++nt) {
@@ -1226,7 +1229,7 @@ sim_kernel(const __grid_constant__ CUtensorMap tmap_h, const __grid_constant__ C
 #pragma unroll
             for (int e = 0; e < 32; ++e) {
               const int slot = slot0 + c0 + e;
-              const float val = __uint_as_float(r[e]) * __ldg(kinv + slot);
+              const float val = __uint_as_float(r[e]) * kinv[slot];
               if (val > best) { best = val; best_slot = slot; }
             }
           }
@@ -1239,11 +1242,11 @@ sim_kernel(const __grid_constant__ CUtensorMap tmap_h, const __grid_constant__ C
         tmem_wait_ld();
         if (a.smat && !part) {
           if (v < a.keep_k && !bk->abort_flag) {
-            const float inv_p = __ldg(kinv + v);
+            const float inv_p = kinv[v];
             float *srow = a.smat + ((size_t)b * a.keep_k + v) * a.keep_k + slot0 + c;
 #pragma unroll
             for (int e = 0; e < 16; ++e)
-              if (c + e < ncol) srow[e] = __uint_as_float(r[e]) * (inv_p * __ldg(kinv + slot0 + c + e));
+              if (c + e < ncol) srow[e] = __uint_as_float(r[e]) * (inv_p * kinv[slot0 + c + e]);
           }
         } else if (part) {
 #pragma unroll
@@ -1254,7 +1257,7 @@ sim_kernel(const __grid_constant__ CUtensorMap tmap_h, const __grid_constant__ C
           for (int e = 0; e < 16; ++e) {
             const int slot = slot0 + c + e;
             if (c + e < ncol) {
-              const float val = __uint_as_float(r[e]) * __ldg(kinv + slot);
+              const float val = __uint_as_float(r[e]) * kinv[slot];
               if (val > best) { best = val; best_slot = slot; }
             }
           }
@@ -1296,7 +1299,7 @@ sim_kernel(const __grid_constant__ CUtensorMap tmap_h, const __grid_constant__ C
 #pragma unroll
         for (int u = 0; u < U; ++u) {
           const int slot = min(s_lo + i0 + 4 * u, a.keep_k - 1);
-          ks[u] = __ldg(kinv + slot);
+          ks[u] = kinv[slot];
 #pragma unroll
           for (int zz = 0; zz < Z; ++zz)
             if (zz < S) x[u][zz] = ld_cluster_v4f32(pz[zz] + (uint32_t)slot * 512u);
@@ -1314,7 +1317,7 @@ sim_kernel(const __grid_constant__ CUtensorMap tmap_h, const __grid_constant__ C
             if (a.smat) {
               const int vr = mt * 128 + lane * 4 + j;
               if (vr < a.keep_k && !bk->abort_flag)
-                a.smat[((size_t)b * a.keep_k + vr) * a.keep_k + slot] = acc[j] * (__ldg(kinv + vr) * ks[u]);
+                a.smat[((size_t)b * a.keep_k + vr) * a.keep_k + slot] = acc[j] * (kinv[vr] * ks[u]);
             } else {
               const float val = acc[j] * ks[u];
               if (val > wb[j]) { wb[j] = val; wsl[j] = slot; }
@@ -1389,11 +1392,11 @@ sim_kernel(const __grid_constant__ CUtensorMap tmap_h, const __grid_constant__ C
           }
           if (a.smat) {
             if (v < a.keep_k && !bk->abort_flag) {
-              const float inv_p = __ldg(kinv + v);
+              const float inv_p = kinv[v];
               float *srow = a.smat + ((size_t)b * a.keep_k + v) * a.keep_k + s0;
 #pragma unroll
               for (int e = 0; e < 16; ++e)
-                if (s0 + e < a.keep_k) srow[e] = acc[e] * (inv_p * __ldg(kinv + s0 + e));
+                if (s0 + e < a.keep_k) srow[e] = acc[e] * (inv_p * kinv[s0 + e]);
             }
             continue;
           }
@@ -1401,7 +1404,7 @@ sim_kernel(const __grid_constant__ CUtensorMap tmap_h, const __grid_constant__ C
           for (int e = 0; e < 16; ++e) {
             const int slot = s0 + e;
             if (slot < a.keep_k) {
-              const float val = acc[e] * __ldg(kinv + slot);
+              const float val = acc[e] * kinv[slot];
               if (val > best) { best = val; best_slot = slot; }
             }
           }
@@ -1655,13 +1658,13 @@ sim_pair_kernel(const __grid_constant__ CUtensorMap tmap_h, const __grid_constan
     int best_slot = 0;
     const int slot0 = gz * a.n_tile;
     const int ncol = max(0, min(a.n_tile, a.keep_k - slot0));
-    bk->kinv[prow] = prow < ncol ? __ldg(kinv + slot0 + prow) : 0.f;
+    bk->kinv[prow] = prow < ncol ? kinv[slot0 + prow] : 0.f;
     asm volatile("bar.sync 1, 256;" ::: "memory");
     mbar_wait(smem_u32(&bk->acc_full), 0, wc);
     tc_fence_after();
     if (active && !bk->abort_flag) {
       const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + grp * a.n_tile;
-      const float inv_p = (a.smat && v < a.keep_k) ? __ldg(kinv + v) : 0.f;
+      const float inv_p = (a.smat && v < a.keep_k) ? kinv[v] : 0.f;
       int c0 = 0;
       if (!a.smat) {
         // 32 columns per tensor-memory wait while they last: half as many waits on the path every block goes
@@ -1709,7 +1712,7 @@ sim_pair_kernel(const __grid_constant__ CUtensorMap tmap_h, const __grid_constan
         for (int e = 0; e < 16; ++e) {
           const int slot = slot0 + c + e;
           if (c + e < ncol) {
-            const float val = __uint_as_float(r[e]) * __ldg(kinv + slot);
+            const float val = __uint_as_float(r[e]) * kinv[slot];
             if (val > best) { best = val; best_slot = slot; }
           }
         }
