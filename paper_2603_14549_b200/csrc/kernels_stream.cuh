@@ -1614,7 +1614,7 @@ merge_compact_kernel(MergeArgs a) {
       const int32_t *as = a.assign + (size_t)b * nd_max;
       int dst[4];
 #pragma unroll
-      for (int e = 0; e < 4; ++e) dst[e] = p0 + e < m_hi ? __ldcg(as + p0 + e) : -1;      // (no __ldg: the preceding kernel wrote it)
+      for (int e = 0; e < 4; ++e) dst[e] = p0 + e < m_hi ? ld_prev(as + p0 + e) : -1;
       int mine = 0;
 #pragma unroll
       for (int e = 0; e < 4; ++e) mine += dst[e] == slot;
@@ -1650,7 +1650,7 @@ merge_compact_kernel(MergeArgs a) {
       __syncthreads();                    // the previous list has been consumed
       if ((int)threadIdx.x < cnt) {
         if (a.member_meta) {
-          const int2 mm = __ldcg(a.member_meta + (size_t)b * nd_max + base + threadIdx.x);
+          const int2 mm = ld_prev(a.member_meta + (size_t)b * nd_max + base + threadIdx.x);
           s_j[threadIdx.x] = min(max(mm.x, 0), d.nv - 1);
           s_w[threadIdx.x] = __int_as_float(mm.y);
         } else {

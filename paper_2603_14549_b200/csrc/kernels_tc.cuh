@@ -113,6 +113,7 @@ static_assert(sizeof(ScoreBook) <= SC_BOOK_BYTES, "score kernel bookkeeping exce
 struct RowPair {
   int R0, nrows, nrt, n2, n_kt, t_lo, t_hi, n_p2;
   bool use_soft;
+  bool past;                   // -inf is added to logits of the last key tile, which reaches past the sequence
 };
 
 // Row pair rp of a sample's ranking rows: rows R0 .. R0 + nrows - 1 (sequence-relative positions).
@@ -127,6 +128,7 @@ __device__ __forceinline__ RowPair score_row_pair(const SampleDesc &d, int rp, i
   int jmax = p_max;
   if (r.use_soft) jmax = max(jmax, d.v0 + d.nv - 1);
   r.n_kt = jmax / 128 + 1;
+  r.past = r.use_soft && r.n_kt * 128 > d.n;
   r.t_lo = d.v0 / 128;
   r.t_hi = min((d.v0 + d.nv - 1) / 128, r.n_kt - 1);
   r.n_p2 = r.t_hi >= r.t_lo ? r.t_hi - r.t_lo + 1 : 0;
@@ -201,7 +203,8 @@ score_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__
     // work (and to the hidden rows the next kernels read) is worth 1 to 2 % of the step (16 x 576 121.5 -> 119.1 us, 64 x 2880
     // 2378 -> 2350 us)
     const uint64_t keep = l2_evict_normal(), drop = l2_evict_first();
-    int qt = 0;                               // query tiles issued for the sum warps
+    int qt = 0;                               // tiles issued for the sum warps
+    uint32_t last_past = 0u;                  // ring slots whose latest tile is to be cleared
     int k_issued = 0, q_issued = 0;           // copies actually issued (an abort is sticky, so
                                               // these are prefixes of the two sequences)
     while (true) {
@@ -242,34 +245,37 @@ score_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__
         // A query tile lands on a barrier of its own (alternating: the sum warps see only these, in order, so they cannot
         // mistake a ring slot's phase; two query tiles are never in flight on the same one, see below) and its slot's
         // barrier is passed at once, which keeps that barrier's phases in step with the ring.
-        auto load_tile = [&](bool query, int row, uint64_t policy) {
+        // A key tile that needs rows cleared first (`past`; never in a kernel with query tiles) uses the same barriers, and the
+        // clearing warp passes its slot's barrier.
+        auto load_tile = [&](bool query, bool past, int row, uint64_t policy) {
           const int s = kc % SC_STAGES;
           if (kc >= SC_STAGES) mbar_wait_warp(smem_u32(&bk->empty[s]), ((kc / SC_STAGES) - 1) & 1, wc);
           if (!__shfl_sync(0xffffffffu, bk->abort_flag, 0)) {
             const uint32_t dst = k_smem + s * SC_TILE_BYTES;
-            const uint32_t bar = smem_u32(query ? &bk->qt_full[qt & 1] : &bk->full[s]);
+            const uint32_t bar = smem_u32(query || past ? &bk->qt_full[qt & 1] : &bk->full[s]);
             const CUtensorMap *map = query ? &tmap_q : &tmap_k;
             mbar_expect_tx_w(bar, SC_TILE_BYTES, leader);
             tma_load_2d_hint_w(dst, map, bar, h * 128, row, policy, leader);
             tma_load_2d_hint_w(dst + SC_HALF_BYTES, map, bar, h * 128 + 64, row, policy, leader);
             if (query && leader) mbar_arrive(smem_u32(&bk->full[s]));
-            if (query) ++qt;
+            if (query || past) ++qt;
+            last_past = past ? last_past | (1u << s) : last_past & ~(1u << s);
             k_issued = kc + 1;
           }
           ++kc;
         };
         for (int u = 0; u < T.n_kt + T.n_p2; ++u) {
-          load_tile(false, d.row0 + (u < T.n_kt ? u : T.t_hi - (u - T.n_kt)) * 128, u < T.n_kt ? keep : drop);
+          load_tile(false, T.past && u == T.n_kt - 1, d.row0 + (u < T.n_kt ? u : T.t_hi - (u - T.n_kt)) * 128, u < T.n_kt ? keep : drop);
           // (query tiles are two ring positions apart, so the one after the next takes the slot of this one, whose
           // release says that it has been added up; between two items at least four other tiles pass)
-          if (u < nq) load_tile(true, d.row0 + d.v0 + u * 128, drop);
+          if (u < nq) load_tile(true, false, d.row0 + d.v0 + u * 128, drop);
         }
       }
     }
     // every copy this warp issued must have landed before the block may leave
     for (int s = 0; s < SC_STAGES; ++s) {
       const int fills = k_issued > s ? (k_issued - s + SC_STAGES - 1) / SC_STAGES : 0;
-      if (fills > 0) mbar_wait_drain(smem_u32(&bk->full[s]), (fills - 1) & 1, TC_WAIT_LIMIT);
+      if (fills > 0 && !((last_past >> s) & 1u)) mbar_wait_drain(smem_u32(&bk->full[s]), (fills - 1) & 1, TC_WAIT_LIMIT);
     }
     if (q_issued > 0) mbar_wait_drain(smem_u32(&bk->q_full), (q_issued - 1) & 1, TC_WAIT_LIMIT);
     for (int i = 0; i < 2; ++i)
@@ -471,9 +477,7 @@ score_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__
 #pragma unroll
                 for (int e = 0; e < 32; ++e) {
                   const float sv = row_vis ? soft[c + e] : -INFINITY;
-                  // (a select, not the sum with -inf: the key may belong to the next sequence and its logit be a NaN)
-                  const float v = fmaf(__uint_as_float(r[e]), scale, (e <= lim) ? 0.f : sv);
-                  const float x = (e > lim && sv == -INFINITY) ? -INFINITY : v;
+                  const float x = fmaf(__uint_as_float(r[e]), scale, (e <= lim) ? 0.f : sv);
                   r[e] = __float_as_uint(x);
                   mx[e & 3] = fmaxf(mx[e & 3], x);
                 }
@@ -694,6 +698,21 @@ score_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__
           if (lane == 0) mbar_arrive(smem_u32(&bk->qbar_ready));
         }
         if (lane == 0) mbar_arrive(smem_u32(&bk->q_empty));
+        if (T.past) {
+          // key rows of the next sequence (see RowPair), by one of the two warps
+          const int s = (kc + T.n_kt - 1) % SC_STAGES, end = d.n - (T.n_kt - 1) * 128;
+          if (half == 0 && __all_sync(0xffffffffu, mbar_wait(smem_u32(&bk->qt_full[qt & 1]), (qt >> 1) & 1, wc))) {
+            uint8_t *tile = base_ptr + SC_Q_BYTES + s * SC_TILE_BYTES;
+            for (int i = end * 8 + lane; i < 128 * 8; i += 32) {
+              reinterpret_cast<uint4 *>(tile)[i] = make_uint4(0u, 0u, 0u, 0u);
+              reinterpret_cast<uint4 *>(tile + SC_HALF_BYTES)[i] = make_uint4(0u, 0u, 0u, 0u);
+            }
+            fence_proxy_async();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(smem_u32(&bk->full[s]));
+          }
+          ++qt;
+        }
         kc += T.n_kt + T.n_p2;
       }
     }
