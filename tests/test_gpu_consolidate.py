@@ -56,7 +56,7 @@ def _run(ctx, batch, k, t, salience_override=None, stage1=None):
         keep[b] = torch.from_numpy(kp); drop[b, :nv - k] = torch.from_numpy(dp)
         st1.append((m.astype(np.float64), s.astype(np.float64), kp, dp))
     out = A.alloc_outputs(inp, k, fill=True)
-    scratch = torch.empty(A.asap_consolidate_scratch_bytes(B, k), dtype=torch.uint8, device=DEV)
+    scratch = torch.full((A.asap_consolidate_scratch_bytes(B, k),), 255, dtype=torch.uint8, device=DEV)
     n_abs = torch.full((B,), -7, dtype=torch.int32, device=DEV)
     A.asap_consolidate(ctx, inp, p, mass.to(DEV), sal.to(DEV), keep.to(DEV), drop.to(DEV), scratch, out, n_abs)
     torch.cuda.synchronize(); A.asap_check(ctx)
@@ -291,11 +291,12 @@ def test_threshold_minus_infinity_absorbs_until_the_pool_is_empty(ctx):
     _check(batch, 60, -math.inf, out, n_abs, st1)
 
 
-@pytest.mark.parametrize("nv,k,t", [(700, 273, 0.8), (700, 305, 0.8), (600, 288, 0.8), (320, 300, -2.0), (700, 290, 0.02)],
-                         ids=["half_word", "ragged_word", "whole_words", "all_similar_capped", "long_chains"])
+@pytest.mark.parametrize("nv,k,t", [(700, 272, 0.8), (700, 268, 0.8), (700, 273, 0.8), (700, 305, 0.8), (600, 288, 0.8), (320, 300, -2.0), (700, 290, 0.02)],
+                         ids=["half_word", "ragged_half", "one_past_half", "ragged_word", "whole_words", "all_similar_capped", "long_chains"])
 def test_routing_from_the_written_bit_matrix(nv, k, t):
     """Batches large enough for the two-row-tile similarity form, which writes the bit matrix of the routing:
-    a last word filled by one half only, a ragged one, none; every pair similar with a refill pool of 20 (the
+    a last word filled by one half only, a ragged first half (the other half has to be cleared: the scratch starts full of
+    ones), a ragged second half, none; every pair similar with a refill pool of 20 (the
     cap); and a threshold in the noise, so that many rounds are needed until every slot is decided.  The oracle
     checks the first, a middle and the last sequence."""
     B = 20

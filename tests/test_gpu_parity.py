@@ -43,8 +43,8 @@ def test_ragged_multi_tile(ctx):
 
 @pytest.mark.parametrize("k", [300, 512, 257])
 def test_two_slot_tiles_in_one_pass(ctx, k):
-    """257 .. 512 kept slots: two slot tiles whose accumulators share tensor memory, one pass over the
-    hidden dimension (300 and 257 leave a ragged second slot tile, 512 fills every column)."""
+    """257 .. 512 kept slots: two groups of slots, dealt to neighbouring blocks of two row tiles each, one pass over the hidden
+    dimension (300 and 257 leave a ragged second group, 512 fills every column)."""
     batch = W.tiny(B=2, n_vis=[700, 650], text_lens=[12, 40], H=2, keep_k=k, seed=107, centres=30)
     run_step(ctx, batch, A.Params(keep_k=k))
 

@@ -20,17 +20,28 @@ pytestmark = pytest.mark.gpu
 DEV = "cuda:0"
 
 
-@pytest.fixture(scope="module")
-def ctx_pair_form():
+def _context(min_blocks, **capacities):
     old = os.environ.get("ASAP_SIM_PAIR_MIN_BLOCKS")
-    os.environ["ASAP_SIM_PAIR_MIN_BLOCKS"] = "1"          # read once, when the context is made
+    os.environ["ASAP_SIM_PAIR_MIN_BLOCKS"] = str(min_blocks)          # read once, when the context is made
     try:
-        c = A.asap_init(0, max_total_tokens=40000, max_B=8, max_H=8, max_D=1024, max_keep_rows=8000)
+        return A.asap_init(0, **capacities)
     finally:
         if old is None:
             del os.environ["ASAP_SIM_PAIR_MIN_BLOCKS"]
         else:
             os.environ["ASAP_SIM_PAIR_MIN_BLOCKS"] = old
+
+
+@pytest.fixture(scope="module")
+def ctx_pair_form():
+    c = _context(1, max_total_tokens=40000, max_B=8, max_H=8, max_D=1024, max_keep_rows=8000)
+    yield c
+    A.asap_free(c)
+
+
+@pytest.fixture(scope="module")
+def ctx_no_pair_form():
+    c = _context(1 << 40, max_total_tokens=40000, max_B=20, max_H=16, max_D=2048, max_keep_rows=8000)
     yield c
     A.asap_free(c)
 
@@ -104,6 +115,31 @@ def test_cluster_form_matches_the_oracle(ctx_default, n_vis, k, H):
 ])
 def test_pair_form_matches_the_oracle(ctx_pair_form, n_vis, k):
     _merge_matches_oracle(ctx_pair_form, n_vis, k, H=2, seed=911)
+
+
+@pytest.mark.parametrize("n_vis,k,H", [
+    ([700, 650], 257, 2),        # two accumulators in one pass, the second ragged
+    ([700, 650], 384, 2),        # ... and full
+    ([700, 650], 512, 2),        # two accumulators in turn, two passes
+    ([700, 650], 600, 2),        # three
+    ([700], 300, 16),            # slices of the hidden dimension that add up through global memory
+    ([900], 600, 16),
+    ([1300] * 19 + [1041], 260, 2),   # more row tiles than SMs: not sliced, and too few slots kept to be gathered
+], ids=["wide_ragged", "wide_full", "two_passes", "three_passes", "sliced_wide", "sliced", "large"])
+def test_several_slot_tiles_without_the_pair_form(ctx_no_pair_form, n_vis, k, H):
+    """More than 256 kept slots take two row tiles per block, unless that form's partial results outgrow their buffer (above a
+    million visual rows): the forms that serve such a batch, on small ones."""
+    _merge_matches_oracle(ctx_no_pair_form, n_vis, k, H, seed=935)
+
+
+@pytest.mark.parametrize("nv,k,H", [(700, 300, 2), (1300, 600, 2), (700, 300, 16), (500, 150, 16)],
+                         ids=["two_tiles", "three_tiles", "sliced", "cluster"])
+def test_kept_rows_matrix_without_the_pair_form(ctx_no_pair_form, nv, k, H):
+    """The same for the matrix of the kept rows' similarities; the routing then forms its bit matrix itself."""
+    from tests.test_gpu_consolidate import _check, _run
+    batch = W.tiny(B=2, n_vis=[nv, nv - 40], text_lens=[4, 9], H=H, keep_k=k, seed=936, centres=k // 8)
+    out, n_abs, st1 = _run(ctx_no_pair_form, batch, k, 0.8, stage1=lambda bt, b, kk: W.random_stage1(bt, b, kk, 33))
+    assert _check(batch, k, 0.8, out, n_abs, st1) > 0
 
 
 def test_many_kept_slots_of_a_long_sequence():
