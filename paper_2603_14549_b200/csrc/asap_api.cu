@@ -246,8 +246,8 @@ asap_status launch_prepare(asap_ctx *ctx, const asap_inputs *in, const asap_para
   return after_launch(ctx, "prepare");
 }
 
-// Steps 1a-1b: query sum, attention mass, salience, mask vector.  With `fold_prepare` the query-sum
-// kernel also carries the device-side validation and writes the descriptors.
+// Steps 1a-1b: query sum, attention mass, salience, mask vector.  The query-sum kernel also carries the device-side validation and
+// writes the descriptors.
 
 // Rows a block of the query-sum kernel adds up: 32, doubled (up to 128) while the grid still has two blocks per
 // SM -- every chunk costs a partial row written and read back (32 rows: 12 % on top of the queries themselves).
@@ -261,13 +261,13 @@ int qsum_rows_per_chunk(const asap_ctx *ctx, const asap_inputs *in) {
 }
 
 asap_status launch_mass(asap_ctx *ctx, const asap_inputs *in, const asap_params *p, const asap_outputs *out,
-                        bool fold_prepare, int32_t *out_cu, int out_capacity, cudaStream_t st) {
+                        int32_t *out_cu, int out_capacity, cudaStream_t st) {
   const int D = in->D, B = in->B;
   const int qrows = qsum_rows_per_chunk(ctx, in);
   const int max_chunks = (in->max_vis + qrows - 1) / qrows;
   const int col_blocks = (D + QSUM_COLS - 1) / QSUM_COLS;
   PrepareArgs pa = prepare_args(ctx, in, p, out_cu, out_capacity);
-  pa.write_desc = fold_prepare ? 1 : 0;
+  pa.write_desc = 1;
   mark(ctx, "qsum", st);
   launch_pdl(qsum_kernel, dim3(max_chunks, col_blocks, B), dim3(QSUM_THREADS), 0, st,
              static_cast<const __nv_bfloat16 *>(in->q), pa, D, max_chunks, qrows, ctx->qsum_partial, ctx->qbar,
@@ -844,7 +844,7 @@ asap_status asap_score(asap_ctx *ctx, const asap_inputs *in, const asap_params *
                        void *stream) {
   ASAP_TRY(validate(ctx, in, p, out, NEED_QK | NEED_SCORE_OUT));
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  ASAP_TRY(launch_mass(ctx, in, p, out, true, nullptr, 0x7fffffff, st));
+  ASAP_TRY(launch_mass(ctx, in, p, out, nullptr, 0x7fffffff, st));
   ASAP_TRY(launch_rank(ctx, in, p, out, true, st));
   if (!p->per_head_mask) return finish(ctx, ASAP_OK, st);
   mark(ctx, "salience_heads", st);
@@ -952,7 +952,7 @@ asap_status asap_prune_step(asap_ctx *ctx, const asap_inputs *in, const asap_par
   // 1 x 576 visual tokens 48.6 -> 42.6 us, 16 x 576 129.5 -> 121.4, 8 x 2304 243 -> 207, 12 mixed images 286 -> 242; against a
   // query-sum kernel in front, 64 x 2880 2530 -> 2427 us.
   const bool fused = in->rank_start == nullptr && !p->per_head_mask;
-  if (!fused) ASAP_TRY(launch_mass(ctx, in, p, out, true, out->out_cu_seqlens, out->out_rows_capacity, st));
+  if (!fused) ASAP_TRY(launch_mass(ctx, in, p, out, out->out_cu_seqlens, out->out_rows_capacity, st));
   ASAP_TRY(launch_rank(ctx, in, p, out, false, st, fused));
   ASAP_TRY(launch_select(ctx, in, p, out->rank_score, out, true, true, st, fused || p->per_head_mask));
   return finish(ctx, launch_merge(ctx, in, p, out->salience, out->keep_idx, out->drop_idx, out, st), st);

@@ -22,7 +22,7 @@ namespace asap {
 // =======================================================================================
 struct PrepareArgs {
   int32_t B, total_tokens, min_vis, max_vis, max_seq, max_rank, keep_k, out_capacity;
-  int32_t write_desc;        // query-sum kernel only: its first block also runs prepare_warp
+  int32_t write_desc;        // query-sum and score kernel: the first block also runs prepare_warp
   const int32_t *cu_seqlens, *vis_start, *vis_len, *text_start, *text_len, *rank_start, *rank_len;
   SampleDesc *desc;          // [B]
   int32_t *out_cu_seqlens;   // [B+1] or nullptr
@@ -881,10 +881,10 @@ kept_gather_kernel(const __nv_bfloat16 *__restrict__ hidden, const SampleDesc *_
 
 // =======================================================================================
 // csr_block: group the dropped tokens of one sample by destination slot (counting sort, stable
-// in dropped order so the merge adds its members in a fixed order).  Run by one whole block of
-// W <= 8 warps: warp w owns the w-th contiguous chunk of dropped positions, counts its chunk
-// into its own histogram, and after a scan over (slot, warp) writes its chunk's positions behind
-// those of the warps before it.  s_cnt needs (W + 1) * keep_k ints, s_scan 33 ints.
+// in dropped order so the merge adds its members in a fixed order).  Run by one whole block of W
+// warps (six, or ten in the gathered and the two-row-tile forms): warp w owns the w-th contiguous
+// chunk of dropped positions, counts its chunk into its own histogram, and after a scan over (slot,
+// warp) writes its chunk's positions behind those of the warps before it.  s_cnt needs (W + 1) * keep_k ints, s_scan 33 ints.
 // seg [B, keep_k+1], members [B, max_vis-keep_k] (dropped POSITIONS, ascending inside a slot).
 // With drop_idx, salience and member_meta given, member_meta [B, max_vis-keep_k] receives, beside every
 // entry of `members`, the member's visual index and its merge weight (the salience, as bits): the
@@ -1418,16 +1418,14 @@ route_kernel(RouteArgs a) {
   if (tid == 0 && a.n_absorbed) a.n_absorbed[b] = n_abs;
   __syncthreads();
   // grouping by destination (counting sort, stable in source order): as many warps as there is room for a histogram each, up to
-  // eight, take a contiguous chunk of the sources
+  // eight, take a contiguous chunk of the sources (the region holds max_vis - k sources and max_vis words more: one at least)
   {
     int *s_cnt = s_order;                     // reuse: the visiting order is no longer needed
     int *hist = reinterpret_cast<int *>(s_union) + n_abs;      // [W][k] behind the sources' slots
     const int W = min(8, (a.union_words - n_abs) / k);
-    const int nw = max(W, 1);
-    if (W < 1) hist = s_cnt;                  // (one warp: its histogram becomes the offsets in place)
-    const int chunk = (((n_abs + nw - 1) / nw) + 31) & ~31;
-    const int p_lo = min(n_abs, warp * chunk), p_hi = warp < nw ? min(n_abs, p_lo + chunk) : p_lo;
-    for (int i = tid; i < nw * k; i += nthr) hist[i] = 0;
+    const int chunk = (((n_abs + W - 1) / W) + 31) & ~31;
+    const int p_lo = min(n_abs, warp * chunk), p_hi = warp < W ? min(n_abs, p_lo + chunk) : p_lo;
+    for (int i = tid; i < W * k; i += nthr) hist[i] = 0;
     __syncthreads();
     for (int i = p_lo + lane; i < p_hi; i += 32) {
       const int sl = (int)s_key[i];
@@ -1439,9 +1437,9 @@ route_kernel(RouteArgs a) {
     int mine = 0;
     for (int sl = lo; sl < hi; ++sl) {
       int run = 0;
-      for (int w = 0; w < nw; ++w) {
+      for (int w = 0; w < W; ++w) {
         const int c = hist[w * k + sl];
-        if (W >= 1) hist[w * k + sl] = run;   // this warp's offset inside the slot
+        hist[w * k + sl] = run;               // this warp's offset inside the slot
         run += c;
       }
       s_cnt[sl] = run;
@@ -1465,11 +1463,11 @@ route_kernel(RouteArgs a) {
       const unsigned peers = __match_any_sync(0xffffffffu, sl);
       const int rank = __popc(peers & ((1u << lane) - 1u));
       int at = 0;
-      if (sl >= 0) at = W >= 1 ? hist[warp * k + sl] : s_cnt[sl];
+      if (sl >= 0) at = hist[warp * k + sl];
       __syncwarp();
       if (sl >= 0) {
-        mem_b[(W >= 1 ? s_cnt[sl] : 0) + at + rank] = i;
-        if (rank == 0) (W >= 1 ? hist[warp * k + sl] : s_cnt[sl]) = at + __popc(peers);
+        mem_b[s_cnt[sl] + at + rank] = i;
+        if (rank == 0) hist[warp * k + sl] = at + __popc(peers);
       }
       __syncwarp();
     }

@@ -815,7 +815,6 @@ constexpr int SIM_GWARPS = SIM_GWARPS_N;                // gather warps
 constexpr int SIM_THREADS = 192 + 32 * SIM_GWARPS;      // copy warp, MMA warp, four epilogue warps, the gather warps
 constexpr int SIM_A_BYTES = 128 * 128;           // 128 rows x 64 bf16
 constexpr int SIM_BOOK_BYTES = 2048;
-constexpr uint32_t SIM_TMEM_COLS = 512;
 constexpr int SIM_MAX_STAGES = 8;
 constexpr int SIM_B_STAGES = 4;
 
