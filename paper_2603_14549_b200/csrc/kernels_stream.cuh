@@ -999,8 +999,8 @@ __device__ __forceinline__ void csr_block(const SampleDesc &d, int b, int max_vi
 //      WHICH anchor left to step D.  Decided in rounds by all threads: as many as the longest chain of slots each of which
 //      waits for the one before, two to four on clustered rows; after some rounds that decide few slots the rest is taken in order
 //      (route_walk).  (One warp walking the order took 38 of the kernel's 174 us on 24 x 576 slots, reading the similarities a
-//      second time for D 50, forming the bit matrix here 30; 174 -> 48 us in all, 45 with D's loads after its scan.
-//      Rounds alone: 0.57 ms on a chain through 576 slots and 9.5 ms through 1024; with the walk 64 and 271 us.)
+//      second time for D 50, forming the bit matrix here 30; 174 -> 48 us in all, 43 with D's loads after its scan.
+//      Rounds alone: 0.57 ms on a chain through 576 slots and 9.5 ms through 1024; with the walk 62 and 270 us.)
 //   D  every absorbed slot finds the most similar anchor that was visited before it (lowest slot
 //      among equals), looking only at the anchors in its row of the bit matrix.
 //   E  the vacated slots are refilled with the pruned tokens of largest attention mass (radix
@@ -1181,12 +1181,13 @@ route_kernel(RouteArgs a) {
   // outcome is that of walking the slots in that order (a slot's fate depends on earlier slots alone).
   // First every row of the matrix loses the slots that come after its own (a thread works on its own rows only): from then on
   // a round is a few words of bit operations per slot.
-  bool open[4];                                       // this thread's slots tid, tid + nthr, ... (k <= 4096)
-#pragma unroll
-  for (int t = 0; t < 4; ++t) {
+  // (the loops over a thread's slots tid, tid + nthr, ... are not unrolled: up to 1024 slots make one trip, and the kernel is short
+  // enough for the fetching of its code to count)
+  uint32_t open = 0u;                                 // bit t: slot tid + t * nthr is undecided (k <= 4096)
+#pragma unroll 1
+  for (int t = 0; tid + t * nthr < k; ++t) {
     const int p = tid + t * nthr;
-    open[t] = p < k;
-    if (!open[t]) continue;
+    open |= 1u << t;
     const int rp = s_rank[p];
     uint32_t *row = mask + (size_t)p * kw;
 #pragma unroll 4
@@ -1204,11 +1205,10 @@ route_kernel(RouteArgs a) {
   // walk does in their time (one such round says nothing: the next may absorb all others) the rest is taken in order, so the
   // rounds are bounded whatever the matrix holds.
   for (int slow = 0;;) {
-    int verdict[4] = {0, 0, 0, 0};                    // 1 anchor, 2 absorbed
-    bool waiting = false, decided = false;
-#pragma unroll
-    for (int t = 0; t < 4; ++t) {
-      if (!open[t]) continue;
+    uint32_t anchors = 0u, absorbed = 0u;             // this round's verdicts, like `open`
+#pragma unroll 1
+    for (int t = 0; tid + t * nthr < k; ++t) {
+      if (!((open >> t) & 1u)) continue;
       const uint32_t *row = mask + (size_t)(tid + t * nthr) * kw;
       uint32_t by_anchor = 0u, left = 0u;
 #pragma unroll 4
@@ -1217,18 +1217,19 @@ route_kernel(RouteArgs a) {
         by_anchor |= word & s_anchor[w];
         left |= word & ~s_gone[w];
       }
-      verdict[t] = by_anchor ? 2 : (left ? 0 : 1);
-      if (verdict[t]) { open[t] = false; decided = true; }
-      else waiting = true;
+      if (by_anchor) absorbed |= 1u << t;
+      else if (!left) anchors |= 1u << t;
     }
-    const int progress = __syncthreads_count(decided);    // (and every slot has looked at the last round's decisions)
-#pragma unroll
-    for (int t = 0; t < 4; ++t) {
-      const int p = tid + t * nthr;
-      if (verdict[t] == 1) { atomicOr(&s_anchor[p >> 5], 1u << (p & 31)); s_flag[p] = 1; }
-      if (verdict[t] == 2) atomicOr(&s_gone[p >> 5], 1u << (p & 31));
+    open &= ~(anchors | absorbed);
+    const int progress = __syncthreads_count((anchors | absorbed) != 0u);   // (and every slot has looked at the last round's decisions)
+#pragma unroll 1
+    for (uint32_t rest = anchors | absorbed; rest; rest &= rest - 1) {
+      const int t = __ffs(rest) - 1, p = tid + t * nthr;
+      const bool anchor = (anchors >> t) & 1u;
+      atomicOr(anchor ? &s_anchor[p >> 5] : &s_gone[p >> 5], 1u << (p & 31));
+      if (anchor) s_flag[p] = 1;
     }
-    if (!__syncthreads_or(waiting)) break;
+    if (!__syncthreads_or(open != 0u)) break;
     slow = progress < ROUTE_WALK_BELOW ? slow + 1 : 0;
     if (slow == ROUTE_SLOW_ROUNDS) {
       route_walk(s_order, mask, s_anchor, s_gone, s_flag, reinterpret_cast<uint32_t *>(s_hist), k, kw);
