@@ -332,11 +332,13 @@ bool merging(const asap_inputs *in, const asap_params *p) { return p->merge_enab
 
 // true when the merge blocks find their members themselves instead of reading a grouping that the similarity kernel leaves
 // behind.  The grouping is a tail of about 5 us; the scan costs every wave of merge blocks about 1 us per 1024 dropped tokens.
-// Measured per step (grouped -> scanned): 1 x 192 slots of 576 50.5 -> 47.7 us, 16 x 64 of 576 133.0 -> 129.2 us; on the other
-// side of the line, 12 x 145 of 577-2881 286.9 -> 288.2 us, 32 x 576 of 1152 and 288 of 576 (5120 wide) merge 460 -> 500 us.
+// Measured per step (grouped -> scanned) by kept rows x passes: 1024 (16 x 64 of 576) 113.1 -> 110.2 us, 1280 (2 x 320 of 2304)
+// 105.5 -> 102.9, 1536 (24 x 64 of 576) 149.9 -> 148.2, 1920 (4 x 160 of 2304) 129.3 -> 127.9, 2048 (32 x 64 of 576) 181.0 -> 180.4,
+// 2304 (12 x 192 and 8 x 288 of 576) 114.0 -> 113.7 and 102.3 -> 102.1: the line lies where they meet, at two waves of eight blocks
+// per SM.  Beyond it 5220 (12 x 145 of 577-2881) 286.9 -> 288.2 us, 32 x 576 of 1152 and 288 of 576 (5120 wide) merge 460 -> 500 us.
 bool merge_scans(const asap_ctx *ctx, const asap_inputs *in, const asap_params *p) {
   const long long passes = (in->max_vis - p->keep_k + MERGE_SCAN - 1) / MERGE_SCAN;
-  return merging(in, p) && passes * p->keep_k * in->B <= 8LL * ctx->num_sms;
+  return merging(in, p) && passes * p->keep_k * in->B <= 16LL * ctx->num_sms;
 }
 
 SalienceArgs salience_args(const asap_ctx *ctx, const asap_inputs *in, const asap_params *p, const asap_outputs *out) {
@@ -442,8 +444,13 @@ asap_status launch_merge_front(asap_ctx *ctx, const asap_inputs *in, const asap_
     // blocks of a pair, one pass each: fewer bytes out of L2 per product.  With more than 256 slots always: the sliced form
     // then adds its partial products up through global memory (step, sliced -> this form: 1 x 2304 with 320 kept 116 -> 97 us,
     // 4 x 2304 160 -> 131, 1 x 2880 with 576 246 -> 180).  With one slot tile, where the slices add up inside a cluster, from a
-    // grid of half the SMs on (step: 96 blocks of 12 mixed images 252 -> 229 us; 48 blocks of 16 x 576 114 against 123, of 4 mixed images
-    // 151 against 163, though 36 blocks of 4 x 2304 with 160 kept 138 -> 128).
+    // grid of half the SMs on, which is a compromise: where the two meet depends on the slots and the width too.  Measured as
+    // asap_merge, sliced -> this form, by blocks of this form:
+    //   width 4096   64 slots    48 blocks 57 -> 66 us, 72 75 -> 79, 96 109 -> 109, 108 118 -> 113, 120 115 -> 108
+    //              160 slots     28 56 -> 67, 36 64 to 78 -> 75 to 78, 48 88 to 90 -> 86 to 89, 72 107 to 110 -> 100 to 105, 96 133 -> 112
+    //              256 slots     28 65 -> 76, 36 64 to 78 -> 84 to 85, 48 99 to 104 -> 93 to 98, 72 97 to 131 -> 105 to 123, 96 139 -> 118
+    //   width 2048   64 slots    48 32 to 37 -> 36 to 40, 96 62 -> 62; 160 slots 18 36 -> 37, 24 40 -> 38, 36 43 to 54 -> 41 to 43,
+    //              72 67 to 74 -> 60 to 67; 256 slots 24 46 -> 43, 36 38 to 55 -> 44 to 50, 72 60 to 92 -> 65 to 81
     {
       const int pairs = (in->max_vis + 255) / 256;
       const int pg = (k + 255) / 256;
