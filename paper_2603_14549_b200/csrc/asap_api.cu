@@ -405,7 +405,8 @@ asap_status launch_merge_front(asap_ctx *ctx, const asap_inputs *in, const asap_
     // Several slot tiles whose accumulators fit tensor memory together: one pass over the hidden
     // dimension with all of them live, so the visual rows are read once (a stage is then one 64-column
     // block of the rows and of every slot tile).
-    // Taken only while three such stages still fit (up to 384 slots): with two, the shorter copies
+    // (With more than 256 slots the two-row-tile form below comes first; this one is left with the batches whose partial results do
+    // not fit that form's buffer.)  Taken only while three such stages still fit (up to 384 slots): with two, the shorter copies
     // cost more than the second read of the rows (measured: 320 slots 87 -> 77 us, 510 slots 91 -> 96 us).
     // The row operand: every visual row by tiled copies (the kept rows' products are then thrown
     // away), or the dropped rows alone, gathered (four more warps, one block per

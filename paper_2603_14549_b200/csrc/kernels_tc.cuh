@@ -790,7 +790,7 @@ head_sum_kernel(const SampleDesc *__restrict__ desc, int H, int max_vis,
 // Rows past the last dropped token (the ragged tail of the last tile) repeat that token and are
 // not written.  The block that finishes a sample's last row tile groups the dropped tokens by
 // destination.
-//   one pass:       (a.wide, when all kept slots fit the 512 tensor-memory columns) the accumulators of
+//   one pass:       (a.wide, gathered rows, or up to 384 slots of a batch too large for sim_pair_kernel) the accumulators of
 //                   all slot tiles are live at once and a stage is one 64-column block of the rows
 //                   plus the matching block of EVERY slot tile, so the visual rows are read from
 //                   memory once instead of once per slot tile.
