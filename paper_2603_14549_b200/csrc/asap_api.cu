@@ -330,6 +330,23 @@ asap_status launch_rank(asap_ctx *ctx, const asap_inputs *in, const asap_params 
 // dropped token itself)
 bool merging(const asap_inputs *in, const asap_params *p) { return p->merge_enable && in->max_vis > p->keep_k; }
 
+// Limits that depend on shared memory, looked at before anything is launched.  The grouping keeps a counter per slot and warp (and the
+// slots' totals) in the tile ring; of all forms of the similarity launch the tiled one has the most room for them.
+asap_status check_merge_room(asap_ctx *ctx, const asap_inputs *in, const asap_params *p) {
+  if (!merging(in, p)) return ASAP_OK;
+  const int k = p->keep_k, n_nt = (k + 255) / 256, n_tile = (((k + n_nt - 1) / n_nt) + 15) & ~15;
+  const int stage_bytes = 2 * (SIM_A_BYTES + n_tile * 128);
+  int stages = (192 * 1024) / stage_bytes;
+  if (stages > SIM_MAX_STAGES) stages = SIM_MAX_STAGES;
+  if (k > 256 && (size_t)(SIM_THREADS_TILED / 32 + 1) * k * sizeof(int) > (size_t)stages * stage_bytes)
+    return fail(ctx, ASAP_ERR_UNSUPPORTED, "keep_k = %d is too large for the merge path", k);
+  return ASAP_OK;
+}
+
+// Words of shared memory that the routing needs (5 keep_k) plus its last region without the bit matrix.
+size_t route_fixed_words(const asap_params *p) { return 5 * (size_t)p->keep_k; }
+size_t route_tail_words(const asap_inputs *in, const asap_params *p) { return (size_t)(in->max_vis - p->keep_k) + (size_t)in->max_vis; }
+
 // true when the merge blocks find their members themselves instead of reading a grouping that the similarity kernel leaves
 // behind.  The grouping is a tail of about 5 us; the scan costs every wave of merge blocks about 1 us per 1024 dropped tokens.
 // Measured per step (grouped -> scanned) by kept rows x passes: 1024 (16 x 64 of 576) 113.1 -> 110.2 us, 1280 (2 x 320 of 2304)
@@ -699,16 +716,13 @@ routing:
   RouteArgs ra;
   ra.desc = ctx->desc; ra.max_vis = in->max_vis; ra.keep_k = k; ra.kw = (k + 31) / 32;
   ra.threshold = p->sim_threshold; ra.smat = smat;
-  const size_t fixed_words = 5 * (size_t)k;
-  const size_t tail_words = (size_t)(in->max_vis - k) + (size_t)in->max_vis;
+  const size_t fixed_words = route_fixed_words(p), tail_words = route_tail_words(in, p);
   const size_t mask_words = (size_t)k * ra.kw;
   const bool mask_in_smem = (fixed_words + (mask_words > tail_words ? mask_words : tail_words)) * 4 <= 200 * 1024;
   ra.mask_g = mask_g; ra.mask_in_smem = mask_in_smem ? 1 : 0; ra.mask_written = mask_written ? 1 : 0;
   const size_t union_words = mask_in_smem && mask_words > tail_words ? mask_words : tail_words;
   ra.union_words = (int)union_words;
   const size_t route_smem = (fixed_words + union_words) * 4;
-  if (route_smem > 224 * 1024)
-    return fail(ctx, ASAP_ERR_UNSUPPORTED, "max_vis = %d is too large for the routing kernel", in->max_vis);
   ra.salience = salience; ra.mass = mass; ra.keep_idx = keep_idx; ra.drop_idx = drop_idx;
   ra.final_keep = out->keep_idx; ra.src_idx = out->drop_idx; ra.src_assign = out->assign;
   ra.seg = ctx->seg; ra.members = ctx->members; ra.n_absorbed = n_absorbed; ra.src_sim = out->best_sim; ra.status = ctx->status;
@@ -875,6 +889,7 @@ asap_status asap_merge(asap_ctx *ctx, const asap_inputs *in, const asap_params *
   ASAP_TRY(validate(ctx, in, p, out, NEED_HIDDEN | NEED_MERGE_OUT));
   if (!salience || !keep_idx || (!drop_idx && in->max_vis > p->keep_k))
     return fail(ctx, ASAP_ERR_INVALID, "null salience / keep_idx / drop_idx");
+  ASAP_TRY(check_merge_room(ctx, in, p));
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   ASAP_TRY(launch_prepare(ctx, in, p, out->out_cu_seqlens, out->out_rows_capacity, st));
   mark(ctx, "role_map", st);
@@ -941,6 +956,8 @@ asap_status asap_consolidate(asap_ctx *ctx, const asap_inputs *in, const asap_pa
     return fail(ctx, ASAP_ERR_INVALID, "asap_consolidate: the stage-1 lists must not be the output lists");
   if (p->keep_k > 32 * ROUTE_MAX_WORDS)
     return fail(ctx, ASAP_ERR_UNSUPPORTED, "asap_consolidate: keep_k above %d", 32 * ROUTE_MAX_WORDS);
+  if ((route_fixed_words(p) + route_tail_words(in, p)) * 4 > 224 * 1024)
+    return fail(ctx, ASAP_ERR_UNSUPPORTED, "max_vis = %d is too large for the routing kernel", in->max_vis);
   if (!scratch || !aligned16(scratch) || scratch_bytes < asap_consolidate_scratch_bytes(in->B, p->keep_k))
     return fail(ctx, ASAP_ERR_WORKSPACE, "asap_consolidate: scratch is null, unaligned or smaller than asap_consolidate_scratch_bytes");
   cudaStream_t st = static_cast<cudaStream_t>(stream);
@@ -952,6 +969,7 @@ asap_status asap_consolidate(asap_ctx *ctx, const asap_inputs *in, const asap_pa
 asap_status asap_prune_step(asap_ctx *ctx, const asap_inputs *in, const asap_params *p, const asap_outputs *out,
                             void *stream) {
   ASAP_TRY(validate(ctx, in, p, out, NEED_QK | NEED_HIDDEN | NEED_SCORE_OUT | NEED_SELECT_OUT | NEED_MERGE_OUT));
+  ASAP_TRY(check_merge_room(ctx, in, p));
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   // With the text span as ranking rows the Eq. 3 mask never touches a ranked row (a text query lies
   // after every visual key), so the score kernel does not need the attention mass, and takes it itself from the query and key

@@ -293,3 +293,30 @@ def test_per_head_mask_needs_an_even_number_of_heads(ctx):
     with pytest.raises(A.AsapError) as e:
         A.asap_prune_step(ctx, inp, A.Params(keep_k=8, per_head_mask=True), out)
     assert e.value.status == -5 and A.asap_launch_count(ctx) == n0
+
+
+def test_a_call_that_is_refused_for_its_size_launches_nothing():
+    """Limits of shared memory (the grouping's counters in the merge, the routing's lists in the consolidation) are looked at before
+    the first kernel: the outputs stay as they were."""
+    nv, k = 20500, 7100
+    c = A.asap_init(0, max_total_tokens=nv + 40, max_B=1, max_H=1, max_D=128, max_keep_rows=k)
+    try:
+        batch = W.tiny(B=1, n_vis=[nv], text_lens=[4], H=1, keep_k=k, seed=640)
+        inp = A.make_inputs(batch, DEV)
+        lists = (torch.rand(1, nv, device=DEV), torch.arange(k, dtype=torch.int32, device=DEV)[None],
+                 torch.arange(k, nv, dtype=torch.int32, device=DEV)[None])
+        few = (lists[1][:, :4096], torch.arange(4096, nv, dtype=torch.int32, device=DEV)[None])
+        scratch = torch.empty(A.asap_consolidate_scratch_bytes(1, 4096), dtype=torch.uint8, device=DEV)
+        out, out4 = A.alloc_outputs(inp, k, fill=True), A.alloc_outputs(inp, 4096, fill=True)
+        n0 = A.asap_launch_count(c)
+        for call in (lambda: A.asap_prune_step(c, inp, A.Params(keep_k=k), out),
+                     lambda: A.asap_merge(c, inp, A.Params(keep_k=k), *lists, out),
+                     lambda: A.asap_consolidate(c, inp, A.Params(keep_k=4096), lists[0], lists[0], *few, scratch, out4)):
+            with pytest.raises(A.AsapError) as e:
+                call()
+            assert e.value.status == -5
+        torch.cuda.synchronize()
+        assert A.asap_launch_count(c) == n0
+        assert torch.all(out.keep_idx == -7) and torch.all(out4.out_cu_seqlens == -7)
+    finally:
+        A.asap_free(c)
