@@ -922,13 +922,19 @@ sim_kernel(const __grid_constant__ CUtensorMap tmap_h, const __grid_constant__ C
   const int gz = blockIdx.x - mt * a.groups;             // group of slot tiles
   const int tile0 = gz * a.n_nt;                         // first slot tile of this block
   const SampleDesc d = a.desc[b];
-  if (!d.valid) return;
+  if (!d.valid) {
+    pdl_wait();         // (should all blocks leave here, the grid must not complete before the preceding one)
+    return;
+  }
   const int nd = d.nv - a.keep_k;                        // dropped tokens of this sample
   constexpr bool gather = GATHER;                        // a.drop_idx given, not matrix mode
   const int n_rows = a.smat ? a.keep_k : (gather ? nd : d.nv);   // rows of the row operand
   if (mt * 128 >= max(n_rows, 1)) return;
   // (in the cluster form the blocks of a cluster must leave together: decided below, by the cluster's first block)
-  if (!a.cluster && (*reinterpret_cast<volatile uint32_t *>(a.status) & STATUS_SIM_TIMEOUT)) return;
+  if (!a.cluster && (*reinterpret_cast<volatile uint32_t *>(a.status) & STATUS_SIM_TIMEOUT)) {
+    pdl_wait();
+    return;
+  }
   const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
 
   const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
@@ -972,6 +978,7 @@ sim_kernel(const __grid_constant__ CUtensorMap tmap_h, const __grid_constant__ C
     cluster_sync_all();
     if (ld_cluster_s32(cluster_map(smem_u32(&bk->skip), 0))) {
       cluster_sync_all();                                // the first block's shared memory has been read by all
+      pdl_wait();
       return;
     }
   }
@@ -1540,11 +1547,17 @@ sim_pair_kernel(const __grid_constant__ CUtensorMap tmap_h, const __grid_constan
   const int pr = blockIdx.x / a.groups, b = blockIdx.y;
   const int gz = blockIdx.x - pr * a.groups;             // group of kept slots
   const SampleDesc d = a.desc[b];
-  if (!d.valid) return;
+  if (!d.valid) {
+    pdl_wait();         // (as in sim_kernel)
+    return;
+  }
   const int nd = d.nv - a.keep_k;
   const int n_rows = a.smat ? a.keep_k : d.nv;           // matrix mode: the row operand is the dense kept-row array
   if (pr * 256 >= n_rows) return;
-  if (*reinterpret_cast<volatile uint32_t *>(a.status) & STATUS_SIM_TIMEOUT) return;
+  if (*reinterpret_cast<volatile uint32_t *>(a.status) & STATUS_SIM_TIMEOUT) {
+    pdl_wait();
+    return;
+  }
   const bool two = pr * 256 + 128 < n_rows;              // the pair's second row tile holds visual rows
   const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
 
