@@ -347,15 +347,16 @@ asap_status check_merge_room(asap_ctx *ctx, const asap_inputs *in, const asap_pa
 size_t route_fixed_words(const asap_params *p) { return 5 * (size_t)p->keep_k; }
 size_t route_tail_words(const asap_inputs *in, const asap_params *p) { return (size_t)(in->max_vis - p->keep_k) + (size_t)in->max_vis; }
 
-// true when the merge blocks find their members themselves instead of reading a grouping that the similarity kernel leaves
-// behind.  The grouping is a tail of about 5 us; the scan costs every wave of merge blocks about 1 us per 1024 dropped tokens.
-// Measured per step (grouped -> scanned) by kept rows x passes: 1024 (16 x 64 of 576) 113.1 -> 110.2 us, 1280 (2 x 320 of 2304)
-// 105.5 -> 102.9, 1536 (24 x 64 of 576) 149.9 -> 148.2, 1920 (4 x 160 of 2304) 129.3 -> 127.9, 2048 (32 x 64 of 576) 181.0 -> 180.4,
-// 2304 (12 x 192 and 8 x 288 of 576) 114.0 -> 113.7 and 102.3 -> 102.1: the line lies where they meet, at two waves of eight blocks
-// per SM.  Beyond it 5220 (12 x 145 of 577-2881) 286.9 -> 288.2 us, 32 x 576 of 1152 and 288 of 576 (5120 wide) merge 460 -> 500 us.
-bool merge_scans(const asap_ctx *ctx, const asap_inputs *in, const asap_params *p) {
-  const long long passes = (in->max_vis - p->keep_k + MERGE_SCAN - 1) / MERGE_SCAN;
-  return merging(in, p) && passes * p->keep_k * in->B <= 16LL * ctx->num_sms;
+// Words of a slot's row of member bits (bit j: visual token j merges into the slot), and whether a batch's rows fit the query
+// sum's partials, which nothing reads any more by then (they do while keep_k <= max_D: B * ceil(max_vis / 32) is at most the rows
+// of that buffer).  If not, the similarity kernel's last block per sequence groups the dropped tokens by destination: a chain of
+// eight barriers, 10 to 17 us behind the last product of a sequence.  The bits cost an atomic per dropped token and a scan of one
+// row per merge block.  Measured per step, grouped -> bits: 8 x 2304 with 320 kept 193 -> 185 us, 12 x 577-2881 with 145 kept 230 ->
+// 221.5, 8 x 1536 with 340 kept 219 -> 213.5; against blocks that looked for their members among all dropped tokens' destinations,
+// 16 x 576 with 64 kept 113 -> 110, 1 x 576 with 192 kept 39.7 -> 39.6.
+int member_words(const asap_inputs *in) { return (in->max_vis + 31) / 32; }
+bool merge_bits(const asap_ctx *ctx, const asap_inputs *in, const asap_params *p) {
+  return merging(in, p) && (size_t)in->B * p->keep_k * member_words(in) <= ctx->cap_chunks * (size_t)ctx->cap_D;
 }
 
 SalienceArgs salience_args(const asap_ctx *ctx, const asap_inputs *in, const asap_params *p, const asap_outputs *out) {
@@ -388,9 +389,11 @@ asap_status launch_merge_front(asap_ctx *ctx, const asap_inputs *in, const asap_
                                cudaStream_t st) {
   const int B = in->B, D = in->D, k = p->keep_k;
   if (merging(in, p)) {
+    uint32_t *bits = merge_bits(ctx, in, p) ? reinterpret_cast<uint32_t *>(ctx->qsum_partial) : nullptr;
     mark(ctx, "kept_gather", st);
     launch_pdl(kept_gather_kernel, dim3(dim3((k + GATHER_THREADS / 32 - 1) / (GATHER_THREADS / 32), B)), dim3(GATHER_THREADS), 0, st, 
-        static_cast<const __nv_bfloat16 *>(in->hidden), ctx->desc, D, k, keep_idx, ctx->kept_rows, ctx->kept_inv);
+        static_cast<const __nv_bfloat16 *>(in->hidden), ctx->desc, D, k, keep_idx, ctx->kept_rows, ctx->kept_inv, bits,
+        member_words(in));
     ASAP_TRY(after_launch(ctx, "kept_gather"));
 
     int n_nt = (k + 255) / 256;
@@ -494,9 +497,10 @@ asap_status launch_merge_front(asap_ctx *ctx, const asap_inputs *in, const asap_
         sa.wide = 1; sa.groups = pg; sa.cluster = 0; sa.threshold = p->sim_threshold;
         sa.drop_idx = nullptr; sa.role = ctx->role;
         sa.hidden = static_cast<const __nv_bfloat16 *>(in->hidden); sa.kept_inv = ctx->kept_inv; sa.assign = out->assign;
-        sa.best_sim = out->best_sim; sa.seg = merge_scans(ctx, in, p) ? nullptr : ctx->seg; sa.members = ctx->members; sa.counters = ctx->cnt_sim;
+        sa.best_sim = out->best_sim; sa.seg = bits ? nullptr : ctx->seg; sa.members = ctx->members; sa.counters = ctx->cnt_sim;
         sa.tile_counters = ctx->cnt_tiles; sa.part = ctx->sim_part; sa.ss_part = nullptr; sa.smat = nullptr; sa.mask16 = nullptr; sa.mask_pitch = 0;
         sa.drop_all = drop_idx; sa.salience = salience; sa.member_meta = salience ? ctx->member_meta : nullptr;
+    sa.member_bits = bits; sa.bit_words = member_words(in);
         sa.status = ctx->status; sa.wait_limit = ctx->wait_limit;
         mark(ctx, "sim", st);
         launch_pdl(sim_pair_kernel, dim3(pairs * pg, B), dim3(SIMP_THREADS), psmem, st, map_h, map_kept, sa);
@@ -536,11 +540,12 @@ asap_status launch_merge_front(asap_ctx *ctx, const asap_inputs *in, const asap_
     sa.threshold = p->sim_threshold;
     sa.drop_idx = gather_rows ? drop_idx : nullptr; sa.role = ctx->role;
     sa.hidden = static_cast<const __nv_bfloat16 *>(in->hidden); sa.kept_inv = ctx->kept_inv; sa.assign = out->assign;
-    sa.best_sim = out->best_sim; sa.seg = merge_scans(ctx, in, p) ? nullptr : ctx->seg; sa.members = ctx->members; sa.counters = ctx->cnt_sim;
+    sa.best_sim = out->best_sim; sa.seg = bits ? nullptr : ctx->seg; sa.members = ctx->members; sa.counters = ctx->cnt_sim;
     sa.tile_counters = ctx->cnt_tiles; sa.part = ctx->sim_part;
     sa.ss_part = ctx->sim_part + (size_t)B * max_mt * splits * (size_t)k * 128;
     sa.smat = nullptr; sa.mask16 = nullptr; sa.mask_pitch = 0;
     sa.drop_all = drop_idx; sa.salience = salience; sa.member_meta = salience ? ctx->member_meta : nullptr;
+    sa.member_bits = bits; sa.bit_words = member_words(in);
     sa.status = ctx->status; sa.wait_limit = ctx->wait_limit;
     mark(ctx, "sim", st);
     if (gather_rows)
@@ -558,7 +563,7 @@ asap_status launch_merge_front(asap_ctx *ctx, const asap_inputs *in, const asap_
 // Steps 4b-5: weighted merge and compaction (the first consumer of the salience).
 asap_status launch_merge_back(asap_ctx *ctx, const asap_inputs *in, const asap_params *p,
                               const float *salience, const int32_t *keep_idx, const int32_t *drop_idx,
-                              const asap_outputs *out, cudaStream_t st, bool grouped_with_weights = false, bool scan = false) {
+                              const asap_outputs *out, cudaStream_t st, bool grouped_with_weights = false, bool bits = false) {
   const int B = in->B, D = in->D, k = p->keep_k;
   const bool do_merge = merging(in, p);
   MergeArgs ma;
@@ -566,7 +571,7 @@ asap_status launch_merge_back(asap_ctx *ctx, const asap_inputs *in, const asap_p
   ma.D = D; ma.max_vis = in->max_vis; ma.keep_k = k; ma.merge_enable = do_merge ? 1 : 0; ma.eps = p->eps;
   ma.salience = salience; ma.keep_idx = keep_idx; ma.drop_idx = drop_idx; ma.seg = ctx->seg;
   ma.members = ctx->members; ma.member_meta = (do_merge && grouped_with_weights) ? ctx->member_meta : nullptr;
-  ma.assign = out->assign;
+  ma.member_bits = bits ? reinterpret_cast<const uint32_t *>(ctx->qsum_partial) : nullptr; ma.bit_words = member_words(in);
   ma.out_hidden = static_cast<__nv_bfloat16 *>(out->out_hidden);
   ma.out_pos = out->out_pos; ma.src_row = out->src_row;
   const int copy_rows = in->max_seq - in->min_vis;   // prefix + suffix rows of the longest sequence, at most
@@ -576,26 +581,22 @@ asap_status launch_merge_back(asap_ctx *ctx, const asap_inputs *in, const asap_p
   // step 41.6 -> 40.5); beyond that the shorter pieces cost more than they balance (16 x 64 slots 28.8 -> 31.8 us).
   if (nv > 1 && (long long)grid.x * grid.y * nv <= 3LL * ctx->num_sms) { grid.z = nv; nv = 1; }
   mark(ctx, "merge_compact", st);
-  if (scan) {
+  auto launch = [&](auto bits_c) {
+    constexpr bool BITS = decltype(bits_c)::value != 0;
     switch (nv) {
-      case 1: launch_pdl(merge_compact_kernel<1, false, true>, dim3(grid), dim3(MERGE_THREADS), 0, st, ma); break;
-      case 2: launch_pdl(merge_compact_kernel<2, false, true>, dim3(grid), dim3(MERGE_THREADS), 0, st, ma); break;
-      case 3: launch_pdl(merge_compact_kernel<3, false, true>, dim3(grid), dim3(MERGE_THREADS), 0, st, ma); break;
-      default: launch_pdl(merge_compact_kernel<4, false, true>, dim3(grid), dim3(MERGE_THREADS), 0, st, ma); break;
+      case 1: launch_pdl(merge_compact_kernel<1, false, BITS>, grid, dim3(MERGE_THREADS), 0, st, ma); break;
+      case 2:
+        if ((long long)grid.x * grid.y >= 32LL * 3 * ctx->num_sms)       // more than 32 waves of three blocks per SM
+          launch_pdl(merge_compact_kernel<2, true, BITS>, grid, dim3(MERGE_THREADS), 0, st, ma);
+        else
+          launch_pdl(merge_compact_kernel<2, false, BITS>, grid, dim3(MERGE_THREADS), 0, st, ma);
+        break;
+      case 3: launch_pdl(merge_compact_kernel<3, false, BITS>, grid, dim3(MERGE_THREADS), 0, st, ma); break;
+      default: launch_pdl(merge_compact_kernel<4, false, BITS>, grid, dim3(MERGE_THREADS), 0, st, ma); break;
     }
-    return after_launch(ctx, "merge_compact");
-  }
-  switch (nv) {
-    case 1: launch_pdl(merge_compact_kernel<1>, dim3(grid), dim3(MERGE_THREADS), 0, st, ma); break;
-    case 2:
-      if ((long long)grid.x * grid.y >= 32LL * 3 * ctx->num_sms)       // more than 32 waves of three blocks per SM
-        launch_pdl(merge_compact_kernel<2, true>, dim3(grid), dim3(MERGE_THREADS), 0, st, ma);
-      else
-        launch_pdl(merge_compact_kernel<2>, dim3(grid), dim3(MERGE_THREADS), 0, st, ma);
-      break;
-    case 3: launch_pdl(merge_compact_kernel<3>, dim3(grid), dim3(MERGE_THREADS), 0, st, ma); break;
-    default: launch_pdl(merge_compact_kernel<4>, dim3(grid), dim3(MERGE_THREADS), 0, st, ma); break;
-  }
+  };
+  if (bits) launch(IntC<1>());
+  else launch(IntC<0>());
   return after_launch(ctx, "merge_compact");
 }
 
@@ -603,7 +604,7 @@ asap_status launch_merge(asap_ctx *ctx, const asap_inputs *in, const asap_params
                          const float *salience, const int32_t *keep_idx, const int32_t *drop_idx,
                          const asap_outputs *out, cudaStream_t st) {
   ASAP_TRY(launch_merge_front(ctx, in, p, salience, keep_idx, drop_idx, out, st));
-  return launch_merge_back(ctx, in, p, salience, keep_idx, drop_idx, out, st, true, merge_scans(ctx, in, p));
+  return launch_merge_back(ctx, in, p, salience, keep_idx, drop_idx, out, st, true, merge_bits(ctx, in, p));
 }
 
 // Sec. 4.2 inside the kept set: kept rows gathered, their keep_k x keep_k cosine matrix, routing.
@@ -617,7 +618,8 @@ asap_status launch_consolidate_front(asap_ctx *ctx, const asap_inputs *in, const
   const int B = in->B, D = in->D, k = p->keep_k;
   mark(ctx, "kept_gather", st);
   launch_pdl(kept_gather_kernel, dim3((k + GATHER_THREADS / 32 - 1) / (GATHER_THREADS / 32), B), dim3(GATHER_THREADS), 0, st,
-             static_cast<const __nv_bfloat16 *>(in->hidden), ctx->desc, D, k, keep_idx, ctx->kept_rows, ctx->kept_inv);
+             static_cast<const __nv_bfloat16 *>(in->hidden), ctx->desc, D, k, keep_idx, ctx->kept_rows, ctx->kept_inv,
+             static_cast<uint32_t *>(nullptr), 0);
   ASAP_TRY(after_launch(ctx, "kept_gather"));
 
   float *smat = static_cast<float *>(scratch);
@@ -654,7 +656,7 @@ asap_status launch_consolidate_front(asap_ctx *ctx, const asap_inputs *in, const
       sa.tile_counters = nullptr; sa.part = nullptr; sa.ss_part = nullptr; sa.smat = smat; sa.salience = nullptr;
       sa.mask16 = reinterpret_cast<uint16_t *>(mask_g); sa.mask_pitch = 2 * ((k + 31) / 32);
       mask_written = true;
-      sa.member_meta = nullptr; sa.status = ctx->status; sa.wait_limit = ctx->wait_limit;
+      sa.member_meta = nullptr; sa.member_bits = nullptr; sa.bit_words = 0; sa.status = ctx->status; sa.wait_limit = ctx->wait_limit;
       mark(ctx, "sim_kept", st);
       launch_pdl(sim_pair_kernel, dim3(pairs * pg, B), dim3(SIMP_THREADS), psmem, st, map_a, map_b, sa);
       ASAP_TRY(after_launch(ctx, "sim_kept"));
@@ -703,7 +705,7 @@ asap_status launch_consolidate_front(asap_ctx *ctx, const asap_inputs *in, const
   sa.drop_idx = nullptr; sa.role = nullptr; sa.hidden = nullptr; sa.kept_inv = ctx->kept_inv; sa.assign = nullptr; sa.best_sim = nullptr;
   sa.seg = nullptr; sa.members = nullptr; sa.counters = nullptr; sa.tile_counters = ctx->cnt_tiles;
   sa.part = ctx->sim_part; sa.ss_part = ctx->sim_part + (size_t)B * max_mt * splits * (size_t)k * 128;
-  sa.smat = smat; sa.drop_all = nullptr; sa.salience = nullptr; sa.member_meta = nullptr; sa.mask16 = nullptr; sa.mask_pitch = 0;
+  sa.smat = smat; sa.drop_all = nullptr; sa.salience = nullptr; sa.member_meta = nullptr; sa.member_bits = nullptr; sa.bit_words = 0; sa.mask16 = nullptr; sa.mask_pitch = 0;
   sa.status = ctx->status; sa.wait_limit = ctx->wait_limit;
   mark(ctx, "sim_kept", st);
   if (cluster)

@@ -836,7 +836,8 @@ __global__ void role_map_kernel(const SampleDesc *__restrict__ desc, int max_vis
 // =======================================================================================
 // kept_gather: one warp per kept slot.  The kept row is copied to its slot of the dense
 // [B*keep_k, D] operand of the similarity GEMM and its inverse norm 1/||h|| is stored (0 if
-// ||h|| < 1e-12, which makes every similarity to that slot 0)   (Sec. 4.2).
+// ||h|| < 1e-12, which makes every similarity to that slot 0)   (Sec. 4.2).  With member_bits the slot's row of
+// member bits is cleared for the similarity kernel.
 // =======================================================================================
 constexpr int GATHER_THREADS = 256;
 
@@ -844,7 +845,8 @@ __global__ void __launch_bounds__(GATHER_THREADS)
 kept_gather_kernel(const __nv_bfloat16 *__restrict__ hidden, const SampleDesc *__restrict__ desc,
                    int D, int keep_k, const int32_t *__restrict__ keep_idx,
                    __nv_bfloat16 *__restrict__ kept_rows /*[B*keep_k, D]*/,
-                   float *__restrict__ kept_inv /*[B*keep_k]*/) {
+                   float *__restrict__ kept_inv /*[B*keep_k]*/, uint32_t *__restrict__ member_bits /*[B*keep_k, bit_words], nullable*/,
+                   int bit_words) {
   pdl_enter();
   const int b = blockIdx.y;
   const SampleDesc d = desc[b];
@@ -856,6 +858,8 @@ kept_gather_kernel(const __nv_bfloat16 *__restrict__ hidden, const SampleDesc *_
   const uint4 *src = reinterpret_cast<const uint4 *>(hidden + (size_t)(d.row0 + d.v0 + j) * D);
   uint4 *dst = reinterpret_cast<uint4 *>(kept_rows + ((size_t)b * keep_k + slot) * D);
   const int nvec = D / 8;
+  if (member_bits)
+    for (int w = lane; w < bit_words; w += 32) member_bits[((size_t)b * keep_k + slot) * bit_words + w] = 0u;
   float ss = 0.f;
   for (int v = lane; v < nvec; v += 256) {
     uint4 x[8];
@@ -1490,7 +1494,8 @@ constexpr int MERGE_THREADS = 256;
 constexpr int MERGE_COPY_ROWS = MERGE_THREADS / 32;   // copy rows per block
 constexpr int MERGE_LIST = 256;                        // members listed per pass
 constexpr int MERGE_BATCH = 4;                         // member rows in flight per thread
-constexpr int MERGE_SCAN = 4 * MERGE_THREADS;          // destinations looked at per pass of a scan
+constexpr int MERGE_WARP_LIST = 64;                    // BITS: members listed per warp and pass
+constexpr int MERGE_BIT_WORDS = 4;                     // BITS: words of a slot's bits per lane and pass (4096 visual tokens)
 
 struct MergeArgs {
   const __nv_bfloat16 *hidden;
@@ -1501,7 +1506,8 @@ struct MergeArgs {
   const float *salience;
   const int32_t *keep_idx, *drop_idx, *seg, *members;
   const int2 *member_meta;   // [B, max_vis-keep_k] (visual index, weight bits) beside `members`, or nullptr
-  const int32_t *assign;     // [B, max_vis-keep_k] (SCAN only) destination slot of every dropped token
+  const uint32_t *member_bits;   // (BITS only) [B, keep_k, bit_words]: bit j of a slot's row set where visual token j merges into it
+  int bit_words;
   __nv_bfloat16 *out_hidden;
   int32_t *out_pos, *src_row;
 };
@@ -1513,18 +1519,15 @@ struct MergeArgs {
 // few waves the shorter batches cost more than the occupancy gives (c2 24.8 -> 26.6 us), so those keep four rows.
 // Rows of 4097-6144 elements (NV = 3): one member row in flight, 64 registers, four blocks per SM as well
 // (D = 5120, 1152 of 2304 kept: 280 -> 241 us; 576 of 1152: 151 -> 133 us; 288 of 576: 85 -> 75 us).
-// SCAN: no grouping of the dropped tokens exists; the block finds its members itself, reading the destinations of all dropped
-// tokens of the sequence (MERGE_SCAN at a time, ascending, so the members come in the order the grouping would give).
-// Grouping is a chain of eight barriers at the end of the similarity kernel (10-12 thousand clocks with its hand-shake,
-// nothing beside it on a small batch); scanning costs every block 4 (n_v - k) bytes out of L2.
-template <int NV, bool LEAN = false, bool SCAN = false>
-__global__ void __launch_bounds__(MERGE_THREADS, NV >= 4 ? 2 : ((LEAN || (NV == 3 && !SCAN)) ? 4 : 3))
+// BITS: the similarity kernel left a row of bits per slot instead of a grouping.  Every warp lists the slot's members for itself,
+// in ascending order, so the block needs no barrier at all.
+template <int NV, bool LEAN = false, bool BITS = false>
+__global__ void __launch_bounds__(MERGE_THREADS, NV >= 4 ? 2 : ((LEAN || NV == 3) ? 4 : 3))
 merge_compact_kernel(MergeArgs a) {
   constexpr int BATCH = NV == 3 ? 1 : ((NV >= 4 || LEAN) ? 2 : MERGE_BATCH);
   pdl_enter();
-  __shared__ int s_j[SCAN ? MERGE_SCAN : MERGE_LIST];
-  __shared__ float s_w[SCAN ? MERGE_SCAN : MERGE_LIST];
-  __shared__ int s_tot[MERGE_THREADS / 32];
+  __shared__ int s_j[BITS ? (MERGE_THREADS / 32) * MERGE_WARP_LIST : MERGE_LIST];
+  __shared__ float s_w[BITS ? 1 : MERGE_LIST];
   const int b = blockIdx.y;
   const SampleDesc d = a.desc[b];
   if (!d.valid) return;
@@ -1570,19 +1573,31 @@ merge_compact_kernel(MergeArgs a) {
   uint4 *dst = reinterpret_cast<uint4 *>(a.out_hidden + (size_t)orow * a.D);
   const int nd_max = a.max_vis - k;
   int m_lo = 0, m_hi = 0;
-  if (SCAN) {
-    m_hi = d.nv - k;                      // every dropped token is looked at
-  } else if (a.merge_enable) {
+  if (!BITS && a.merge_enable) {
     m_lo = min(max(a.seg[(size_t)b * (k + 1) + slot], 0), nd_max);
     m_hi = min(max(a.seg[(size_t)b * (k + 1) + slot + 1], m_lo), nd_max);
   }
+  // BITS: the lanes of a warp own neighbouring words, so that one scan over the lanes gives every member's place
+  const int lane = threadIdx.x & 31, words = (d.nv + 31) >> 5;
+  const uint32_t *bit_row = BITS ? a.member_bits + ((size_t)b * k + slot) * a.bit_words : nullptr;
+  uint32_t mw[MERGE_BIT_WORDS];
+  int per = 0;
+  auto load_words = [&](int w0) {
+    per = (min(words - w0, 32 * MERGE_BIT_WORDS) + 31) >> 5;
+#pragma unroll
+    for (int g = 0; g < MERGE_BIT_WORDS; ++g) {
+      const int w = w0 + lane * per + g;
+      mw[g] = g < per && w < words ? (uint32_t)ld_prev(reinterpret_cast<const int *>(bit_row + w)) : 0u;
+    }
+  };
+  if (BITS) load_words(0);
   uint4 self[NV];
 #pragma unroll
   for (int u = 0; u < NV; ++u) {
     const int v = v0 + u * MERGE_THREADS;
     if (v < nvec) self[u] = __ldg(src + v);
   }
-  if (m_hi <= m_lo) {
+  if (!BITS && m_hi <= m_lo) {
 #pragma unroll
     for (int u = 0; u < NV; ++u) {
       const int v = v0 + u * MERGE_THREADS;
@@ -1603,50 +1618,77 @@ merge_compact_kernel(MergeArgs a) {
     for (int e = 0; e < 8; ++e) acc[u][e] = w_self * f[e];
   }
   float den = w_self;
-  bool merged = !SCAN;
+  bool merged = !BITS;
   const __nv_bfloat16 *vis0 = a.hidden + (size_t)(d.row0 + d.v0) * a.D;
-  for (int base = m_lo; base < m_hi; base += SCAN ? MERGE_SCAN : MERGE_LIST) {
-    int cnt;
-    if (SCAN) {
-      const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-      const int p0 = base + threadIdx.x * 4;
-      const int32_t *as = a.assign + (size_t)b * nd_max;
-      int dst[4];
+  // adds the members listed in s_j (and s_w, unless BITS) at `at`
+  auto add_members = [&](int at, int cnt) {
+    for (int m0 = 0; m0 < cnt; m0 += BATCH) {
+      uint4 x[BATCH][NV];
+      float wt[BATCH];
 #pragma unroll
-      for (int e = 0; e < 4; ++e) dst[e] = p0 + e < m_hi ? ld_prev(as + p0 + e) : -1;
+      for (int t = 0; t < BATCH; ++t) {
+        if (m0 + t < cnt) {
+          const int j = s_j[at + m0 + t];
+          wt[t] = BITS ? __ldg(sal_b + j) : s_w[at + m0 + t];
+          const uint4 *msrc = reinterpret_cast<const uint4 *>(vis0 + (size_t)j * a.D);
+#pragma unroll
+          for (int u = 0; u < NV; ++u) {
+            const int v = v0 + u * MERGE_THREADS;
+            if (v < nvec) x[t][u] = __ldg(msrc + v);
+          }
+        }
+      }
+#pragma unroll
+      for (int t = 0; t < BATCH; ++t) {
+        if (m0 + t < cnt) {
+          const float w = wt[t];
+          den += w;
+#pragma unroll
+          for (int u = 0; u < NV; ++u) {
+            float f[8];
+            unpack8(x[t][u], f);
+#pragma unroll
+            for (int e = 0; e < 8; ++e) acc[u][e] += w * f[e];
+          }
+        }
+      }
+    }
+  };
+  if (BITS) {
+    const int list0 = (threadIdx.x >> 5) * MERGE_WARP_LIST;
+    // (a pass over more members than the list holds reads the words again: kept, they cost the pass its registers)
+    for (int w0 = 0, c0 = 0; w0 < words;) {
+      if (w0 | c0) load_words(w0);
       int mine = 0;
 #pragma unroll
-      for (int e = 0; e < 4; ++e) mine += dst[e] == slot;
-      int inc = mine;
+      for (int g = 0; g < MERGE_BIT_WORDS; ++g) mine += __popc(mw[g]);
+      int at = mine;                          // inclusive, then exclusive sum over the lanes
       if (__any_sync(0xffffffffu, mine)) {
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
-          const int t = __shfl_up_sync(0xffffffffu, inc, o);
-          if (lane >= o) inc += t;
+          const int t = __shfl_up_sync(0xffffffffu, at, o);
+          if (lane >= o) at += t;
         }
       }
-      __syncthreads();                    // the previous list has been consumed
-      if (lane == 31) s_tot[warp] = inc;
-      __syncthreads();
-      int at = inc - mine;
-      cnt = 0;
+      const int left = __shfl_sync(0xffffffffu, at, 31) - c0;      // members of these words not yet added
+      if (left > 0) {
+        merged = true;
+        int r = at - mine - c0;
 #pragma unroll
-      for (int w = 0; w < MERGE_THREADS / 32; ++w) {
-        if (w < warp) at += s_tot[w];
-        cnt += s_tot[w];
+        for (int g = 0; g < MERGE_BIT_WORDS; ++g)
+          for (uint32_t m = mw[g]; m; m &= m - 1, ++r)
+            if (r >= 0 && r < MERGE_WARP_LIST) s_j[list0 + r] = (w0 + lane * per + g) * 32 + __ffs(m) - 1;
+        __syncwarp();
+        add_members(list0, min(MERGE_WARP_LIST, left));
+        __syncwarp();                         // the list has been read
       }
-#pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        if (dst[e] != slot) continue;
-        const int j = min(max(__ldg(drop_b + p0 + e), 0), d.nv - 1);
-        s_j[at] = j;
-        s_w[at] = __ldg(sal_b + j);
-        ++at;
-      }
-      merged = merged || cnt > 0;
-    } else {
-      cnt = min(MERGE_LIST, m_hi - base);
-      __syncthreads();                    // the previous list has been consumed
+      if (left > MERGE_WARP_LIST) c0 += MERGE_WARP_LIST;
+      else { c0 = 0; w0 += 32 * MERGE_BIT_WORDS; }
+    }
+  } else {
+    for (int base = m_lo; base < m_hi; base += MERGE_LIST) {
+      const int cnt = min(MERGE_LIST, m_hi - base);
+      __syncthreads();                      // the previous list has been consumed
       if ((int)threadIdx.x < cnt) {
         if (a.member_meta) {
           const int2 mm = ld_prev(a.member_meta + (size_t)b * nd_max + base + threadIdx.x);
@@ -1658,35 +1700,8 @@ merge_compact_kernel(MergeArgs a) {
           s_w[threadIdx.x] = sal_b[j];
         }
       }
-    }
-    __syncthreads();
-    for (int m0 = 0; m0 < cnt; m0 += BATCH) {
-      uint4 x[BATCH][NV];
-#pragma unroll
-      for (int t = 0; t < BATCH; ++t) {
-        if (m0 + t < cnt) {
-          const uint4 *msrc = reinterpret_cast<const uint4 *>(vis0 + (size_t)s_j[m0 + t] * a.D);
-#pragma unroll
-          for (int u = 0; u < NV; ++u) {
-            const int v = v0 + u * MERGE_THREADS;
-            if (v < nvec) x[t][u] = __ldg(msrc + v);
-          }
-        }
-      }
-#pragma unroll
-      for (int t = 0; t < BATCH; ++t) {
-        if (m0 + t < cnt) {
-          const float w = s_w[m0 + t];
-          den += w;
-#pragma unroll
-          for (int u = 0; u < NV; ++u) {
-            float f[8];
-            unpack8(x[t][u], f);
-#pragma unroll
-            for (int e = 0; e < 8; ++e) acc[u][e] += w * f[e];
-          }
-        }
-      }
+      __syncthreads();
+      add_members(0, cnt);
     }
   }
   if (den <= a.eps || !merged) {

@@ -847,9 +847,15 @@ struct SimArgs {
   int mask_pitch;            // halfwords per row, even
   const float *salience;     // [B, max_vis] or nullptr: with member_meta, the merge weights the grouping copies
   int2 *member_meta;         // [B, max_vis-keep_k] or nullptr (see csr_block)
+  uint32_t *member_bits;     // [B, keep_k, bit_words], zero, or nullptr: bit j of a slot's row is set where visual token j merges into it
+  int bit_words;
   uint32_t *status;
   long long wait_limit;      // clock cycles a wait may take before the block gives up
 };
+
+__device__ __forceinline__ void set_member_bit(const SimArgs &a, int b, int slot, int v) {
+  atomicOr(a.member_bits + ((size_t)b * a.keep_k + slot) * a.bit_words + (v >> 5), 1u << (v & 31));
+}
 
 struct SimBook {
   uint64_t full[SIM_MAX_STAGES], empty[SIM_MAX_STAGES], acc_full[2], acc_empty[2], mma_done;
@@ -1476,9 +1482,10 @@ sim_kernel(const __grid_constant__ CUtensorMap tmap_h, const __grid_constant__ C
       const size_t o = (size_t)b * (a.max_vis - a.keep_k) + dp;
       a.assign[o] = (sim > a.threshold) ? slot : -1;
       if (a.best_sim) a.best_sim[o] = sim;
+      if (a.member_bits && sim > a.threshold) set_member_bit(a, b, slot, gather ? min(max(__ldg(a.drop_idx + o), 0), d.nv - 1) : v);
     }
     if (warp == 2 && lane == 0) bk->is_last = finalize ? 1 : 0;
-    __threadfence();
+    if (a.seg) __threadfence();
   }
   tc_fence_before();
   __syncthreads();
@@ -1791,9 +1798,10 @@ sim_pair_kernel(const __grid_constant__ CUtensorMap tmap_h, const __grid_constan
       const size_t o = (size_t)b * (a.max_vis - a.keep_k) + dp;
       a.assign[o] = (sim > a.threshold) ? slot : -1;
       if (a.best_sim) a.best_sim[o] = sim;
+      if (a.member_bits && sim > a.threshold) set_member_bit(a, b, slot, v);
     }
     if (warp == 2 && lane == 0) bk->is_last = finalize ? 1 : 0;
-    __threadfence();
+    if (a.seg) __threadfence();
   }
   tc_fence_before();
   __syncthreads();

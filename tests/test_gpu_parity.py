@@ -128,6 +128,20 @@ def test_merge_blocks_that_scan_for_their_members(ctx, nvs, k):
     run_step(ctx, batch, A.Params(keep_k=k))
 
 
+@pytest.mark.parametrize("nvs,k,tokens", [([4200, 33], 20, 9000), ([4097, 64], 16, 9000), ([640, 610], 310, 1400)],
+                         ids=["two_passes_long_lists", "one_member_past_a_pass", "grouped_instead"])
+def test_rows_of_member_bits(nvs, k, tokens):
+    """A slot's members as a row of bits: more words than a warp takes per pass (4096 tokens), more members than its list holds
+    (64), a sequence whose last token alone lies in the second pass, and a context (310 kept slots, width 256, few tokens) whose
+    scratch has no room for the rows, so that the similarity kernel groups the members."""
+    batch = W.tiny(B=len(nvs), n_vis=nvs, text_lens=[9 + b for b in range(len(nvs))], H=2, keep_k=k, seed=310 + k, centres=11)
+    small = A.asap_init(0, max_total_tokens=tokens, max_B=len(nvs), max_H=2, max_D=256)
+    try:
+        run_step(small, batch, A.Params(keep_k=k))
+    finally:
+        A.asap_free(small)
+
+
 def test_many_row_tiles_and_three_slot_tiles(ctx):
     """A batch large enough that the similarity kernel runs unsliced with more blocks than SMs
     (15 sequences x 19 row tiles) and three slot tiles (600 kept slots).  Odd and even numbers of row
