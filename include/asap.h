@@ -132,7 +132,7 @@ typedef struct {
  * here once per context, move those decisions for measurements (results are the same up to rounding order):
  *   ASAP_SIM_PAIR_MIN_BLOCKS    blocks from which the similarity takes two row tiles per block (default: half the SMs, an eighth in
  *                               asap_consolidate; 1 above 256 kept slots)
- *   ASAP_SIM_PAIR_STAGES        tile stages of that form (default: what fits 192 KB)
+ *   ASAP_SIM_PAIR_STAGES        64-column steps of tiles in flight of that form (default: what fits 192 KB)
  *   ASAP_SIM_CLUSTER            0: sliced similarity launches add their partial products through global memory
  *                               instead of a thread-block cluster's shared memory (default 1, if the device can
  *                               place such a cluster) */

@@ -326,6 +326,24 @@ asap_status launch_rank(asap_ctx *ctx, const asap_inputs *in, const asap_params 
   return after_launch(ctx, "head_sum");
 }
 
+// Slots of sim_pair_kernel's rings in 192 KB of tiles (one row tile of 16 KB, or one tile of kept rows): three for the kept
+// rows, four while they are small, the rest for the rows.  Two slots of kept rows and more of rows: 8 x 1536 with 340 kept 49 ->
+// 58 us, 64 x 2880 with 576 kept 775 -> 827.
+struct PairRings {
+  int rows, kept;
+  size_t bytes;
+};
+PairRings pair_rings(const asap_ctx *ctx, int n_tile) {
+  PairRings r;
+  r.kept = ctx->sim_pair_stages > 0 ? (ctx->sim_pair_stages < SIMP_MAX_KEPT ? ctx->sim_pair_stages : SIMP_MAX_KEPT) : n_tile <= 64 ? 4 : 3;
+  r.rows = (192 * 1024 - r.kept * n_tile * 128) / SIM_A_BYTES;
+  if (ctx->sim_pair_stages > 0 && r.rows > 2 * ctx->sim_pair_stages) r.rows = 2 * ctx->sim_pair_stages;
+  if (r.rows > SIMP_MAX_ROWS) r.rows = SIMP_MAX_ROWS;
+  r.rows &= ~1;               // (a slot always holds the same row tile of the pair: its readers see every fill of it)
+  r.bytes = (size_t)r.rows * SIM_A_BYTES + (size_t)r.kept * n_tile * 128;
+  return r;
+}
+
 // true when a similarity kernel will run for this call (it then writes assign / best_sim of every
 // dropped token itself)
 bool merging(const asap_inputs *in, const asap_params *p) { return p->merge_enable && in->max_vis > p->keep_k; }
@@ -477,14 +495,11 @@ asap_status launch_merge_front(asap_ctx *ctx, const asap_inputs *in, const asap_
       const int pg = (k + 255) / 256;
       const int ptile = (((k + pg - 1) / pg) + 15) & ~15;
       const long long min_blocks = ctx->sim_pair_min_blocks > 0 ? ctx->sim_pair_min_blocks : k > 256 ? 1 : (ctx->num_sms + 1) / 2;
-      const int pstage = 2 * SIM_A_BYTES + ptile * 128;
-      int pstages = ctx->sim_pair_stages > 0 ? ctx->sim_pair_stages : (192 * 1024) / pstage;
-      if (pstages > SIM_MAX_STAGES) pstages = SIM_MAX_STAGES;
-      const size_t psmem = (size_t)pstages * pstage + SIM_BOOK_BYTES + 1024;
-      if (!gather_rows && D % 64 == 0 && (long long)pairs * B * pg >= min_blocks &&
-          (size_t)B * pairs <= ctx->cap_tiles && pstages >= 2 && psmem <= 227 * 1024 &&
-          (size_t)B * pairs * (size_t)(pg * 512 + 256) * sizeof(float) <= ctx->sim_part_bytes &&
-          (size_t)(SIMP_THREADS / 32 + 1) * k * sizeof(int) <= (size_t)pstages * pstage) {
+      const PairRings rings = pair_rings(ctx, ptile);
+      const size_t psmem = rings.bytes + SIM_BOOK_BYTES + 1024;
+      if (!gather_rows && D % 64 == 0 && (long long)pairs * B * pg >= min_blocks && (size_t)B * pairs <= ctx->cap_tiles &&
+          (size_t)B * pairs * (size_t)(pg * 768) * sizeof(float) <= ctx->sim_part_bytes &&
+          (bits || (size_t)(SIMP_THREADS / 32 + 1) * k * sizeof(int) <= rings.bytes)) {
         uint32_t pcols = 32;
         while ((int)pcols < 2 * ptile) pcols <<= 1;
         CUtensorMap map_h, map_kept;
@@ -493,7 +508,7 @@ asap_status launch_merge_front(asap_ctx *ctx, const asap_inputs *in, const asap_
           return fail(ctx, ASAP_ERR_CUDA, "cuTensorMapEncodeTiled failed for hidden / kept rows");
         SimArgs sa;
         sa.desc = ctx->desc; sa.D = D; sa.max_vis = in->max_vis; sa.keep_k = k; sa.n_tile = ptile;
-        sa.n_nt = 1; sa.stages = pstages; sa.a_stages = 0; sa.splits = 1; sa.max_mt = pairs; sa.tmem_cols = pcols;
+        sa.n_nt = 1; sa.stages = rings.kept; sa.a_stages = rings.rows; sa.splits = 1; sa.max_mt = pairs; sa.tmem_cols = pcols;
         sa.wide = 1; sa.groups = pg; sa.cluster = 0; sa.threshold = p->sim_threshold;
         sa.drop_idx = nullptr; sa.role = ctx->role;
         sa.hidden = static_cast<const __nv_bfloat16 *>(in->hidden); sa.kept_inv = ctx->kept_inv; sa.assign = out->assign;
@@ -636,11 +651,9 @@ asap_status launch_consolidate_front(asap_ctx *ctx, const asap_inputs *in, const
     const int pg = (k + 255) / 256;
     const int ptile = (((k + pg - 1) / pg) + 15) & ~15;
     const long long min_blocks = ctx->sim_pair_min_blocks > 0 ? ctx->sim_pair_min_blocks : k > 256 ? 1 : ctx->num_sms / 8;
-    const int pstage = 2 * SIM_A_BYTES + ptile * 128;
-    int pstages = ctx->sim_pair_stages > 0 ? ctx->sim_pair_stages : (192 * 1024) / pstage;
-    if (pstages > SIM_MAX_STAGES) pstages = SIM_MAX_STAGES;
-    const size_t psmem = (size_t)pstages * pstage + SIM_BOOK_BYTES + 1024;
-    if (D % 64 == 0 && (long long)pairs * B * pg >= min_blocks && pstages >= 2 && psmem <= 227 * 1024) {
+    const PairRings rings = pair_rings(ctx, ptile);
+    const size_t psmem = rings.bytes + SIM_BOOK_BYTES + 1024;
+    if (D % 64 == 0 && (long long)pairs * B * pg >= min_blocks) {
       uint32_t pcols = 32;
       while ((int)pcols < 2 * ptile) pcols <<= 1;
       CUtensorMap map_a, map_b;
@@ -649,7 +662,7 @@ asap_status launch_consolidate_front(asap_ctx *ctx, const asap_inputs *in, const
         return fail(ctx, ASAP_ERR_CUDA, "cuTensorMapEncodeTiled failed for the kept rows");
       SimArgs sa;
       sa.desc = ctx->desc; sa.D = D; sa.max_vis = in->max_vis; sa.keep_k = k; sa.n_tile = ptile;
-      sa.n_nt = 1; sa.stages = pstages; sa.a_stages = 0; sa.splits = 1; sa.max_mt = pairs; sa.tmem_cols = pcols;
+      sa.n_nt = 1; sa.stages = rings.kept; sa.a_stages = rings.rows; sa.splits = 1; sa.max_mt = pairs; sa.tmem_cols = pcols;
       sa.wide = 1; sa.groups = pg; sa.cluster = 0; sa.threshold = p->sim_threshold;
       sa.drop_idx = nullptr; sa.role = nullptr; sa.drop_all = nullptr; sa.hidden = nullptr; sa.kept_inv = ctx->kept_inv;
       sa.assign = nullptr; sa.best_sim = nullptr; sa.seg = nullptr; sa.members = nullptr; sa.counters = nullptr;

@@ -1526,17 +1526,20 @@ sim_kernel(const __grid_constant__ CUtensorMap tmap_h, const __grid_constant__ C
 // pair of row tiles (blockIdx.x = pair * groups + group).  The blocks of a pair are neighbours in
 // launch order and stream the same rows at the same pace, so the rows come from memory once and
 // from L2 for the other groups.  Accumulators: row tile t at tensor-memory column t * n_tile.
-// Every block adds up its rows' squares from shared memory only if it is group 0, and publishes
-// its rows' best (value, slot); the block that finishes a pair last takes the maximum over the
+// Rows and kept rows have rings of their own: the rows come from memory and want as many bytes in flight as there is room for,
+// the kept rows come from L2.  Every block adds up its rows' squares over its group's share of the 64-column blocks, and
+// publishes its rows' best (value, slot) and that sum (one ring, and all the squares in group 0: 8 x 2304 with 320 kept 58 -> 49.5
+// us, 8 x 1536 with 340 56 -> 49, 12 x 577-2881 with 145 56.5 -> 50, 64 x 2880 793 -> 775); the block that finishes a pair last takes the maximum over the
 // groups (lowest slot among equals), looks up which rows were dropped and writes their assignment.
 // The block that finishes a sample's last pair groups the dropped tokens by destination.
 // Matrix mode (a.smat set): the row operand is the dense kept-row array too (`tmap_h` maps it with a 128-row box)
 // and every block writes its 256 x n_tile piece of the sample's keep_k x keep_k cosine matrix; nothing else.
 // =======================================================================================
-constexpr int SIMP_THREADS = 320;                // copy warp, MMA warp, two groups of four epilogue warps
+constexpr int SIMP_THREADS = 352;                // copy warp (rows), MMA warp, two groups of four epilogue warps, copy warp (kept rows)
+constexpr int SIMP_MAX_ROWS = 12, SIMP_MAX_KEPT = 4;   // slots of the two rings
 
 struct SimPairBook {
-  uint64_t full[SIM_MAX_STAGES], empty[SIM_MAX_STAGES], acc_full, mma_done;
+  uint64_t full[SIMP_MAX_ROWS], empty[SIMP_MAX_ROWS], full_b[SIMP_MAX_KEPT], empty_b[SIMP_MAX_KEPT], acc_full, mma_done, norm_go;
   uint32_t tmem_base;
   int abort_flag;
   int is_last;
@@ -1570,20 +1573,28 @@ sim_pair_kernel(const __grid_constant__ CUtensorMap tmap_h, const __grid_constan
 
   const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
   uint8_t *base_ptr = smem_raw + (base - smem_u32(smem_raw));
-  // a stage: [ row tile 0 | row tile 1 | kept rows ] of one 64-column block
+  // a ring of row tiles (row tile 0, row tile 1, row tile 0 of the next 64 columns, ...) and one of the kept rows' tiles
   const int b_bytes = a.n_tile * 128;
-  const int stage_bytes = 2 * SIM_A_BYTES + b_bytes;
-  SimPairBook *bk = reinterpret_cast<SimPairBook *>(base_ptr + (size_t)a.stages * stage_bytes);
+  const int ring_bytes = a.a_stages * SIM_A_BYTES + a.stages * b_bytes;
+  const uint32_t base_b = base + a.a_stages * SIM_A_BYTES;
+  SimPairBook *bk = reinterpret_cast<SimPairBook *>(base_ptr + (size_t)ring_bytes);
 
-  // the epilogue warps of group 0 read their row tile from the stages (for the row norms)
-  const int n_readers = (gz == 0 && !a.smat) ? (two ? 8 : 4) : 0;   // (matrix mode takes the norms from kept_inv)
+  // the epilogue warps read this group's range of 64-column blocks of their row tile (for the row norms; matrix mode takes them
+  // from kept_inv)
+  const int n_kb = a.D / 64;
+  const int norm_lo = n_kb * gz / a.groups, norm_hi = n_kb * (gz + 1) / a.groups;
   if (threadIdx.x == 0) {
-    for (int s = 0; s < a.stages; ++s) {
+    for (int s = 0; s < a.a_stages; ++s) {
       mbar_init(smem_u32(&bk->full[s]), 1);
-      mbar_init(smem_u32(&bk->empty[s]), 1 + n_readers);   // the MMAs that read the stage + the warps that do
+      mbar_init(smem_u32(&bk->empty[s]), a.smat ? 1 : 5);  // the MMAs that read the tile + the warps that do, or their issuer for them
+    }
+    for (int s = 0; s < a.stages; ++s) {
+      mbar_init(smem_u32(&bk->full_b[s]), 1);
+      mbar_init(smem_u32(&bk->empty_b[s]), 1);
     }
     mbar_init(smem_u32(&bk->acc_full), 1);
     mbar_init(smem_u32(&bk->mma_done), 1);
+    mbar_init(smem_u32(&bk->norm_go), 1);
     bk->abort_flag = 0;
     bk->is_last = 0;
     fence_barrier_init();
@@ -1598,62 +1609,63 @@ sim_pair_kernel(const __grid_constant__ CUtensorMap tmap_h, const __grid_constan
   pdl_enter();
   const uint32_t tmem_base = bk->tmem_base;
   WaitCtx wc{&bk->abort_flag, a.status, STATUS_SIM_TIMEOUT, a.wait_limit};
-  const int n_kb = a.D / 64;
   // the groups of a pair walk the 64-column blocks from the same starting point (they share the rows
   // through L2); different pairs start elsewhere and spread over the memory channels
   const int rot = (pr * 5 + b * 3) % n_kb;
 
-  if (warp == 0) {
-    // ---- copy warp (converged, see tma_load_2d_w)
+  const int n_t = two ? 2 : 1;
+  if (warp == 0 || warp == 10) {
+    // ---- copy warps, one per ring (converged, see tma_load_2d_w)
     const uint32_t leader = warp_leader();
-    if (leader) {
-      tma_prefetch_desc(&tmap_h);
-      tma_prefetch_desc(&tmap_kept);
-    }
-    const int row_a = a.smat ? b * a.keep_k + pr * 256 : d.row0 + d.v0 + pr * 256;
-    const int row_b = b * a.keep_k + gz * a.n_tile;
-    const int tx_bytes = two ? stage_bytes : stage_bytes - SIM_A_BYTES;
+    const bool rows = warp == 0;
+    const CUtensorMap *map = rows ? &tmap_h : &tmap_kept;
+    if (leader) tma_prefetch_desc(map);
+    const int slots = rows ? a.a_stages : a.stages, bytes = rows ? SIM_A_BYTES : b_bytes, tiles = rows ? n_t : 1;
+    const int row = !rows ? b * a.keep_k + gz * a.n_tile : a.smat ? b * a.keep_k + pr * 256 : d.row0 + d.v0 + pr * 256;
+    const uint32_t ring = rows ? base : base_b;
+    uint64_t *full0 = rows ? bk->full : bk->full_b, *empty0 = rows ? bk->empty : bk->empty_b;
     int issued = 0, kb = rot;
     RingPos r;
     for (int it = 0; it < n_kb; ++it) {
-      const uint32_t full = smem_u32(&bk->full[r.slot]);
-      if (it >= a.stages) mbar_wait_warp(smem_u32(&bk->empty[r.slot]), r.phase ^ 1u, wc);
-      if (__shfl_sync(0xffffffffu, bk->abort_flag, 0)) break;
-      const uint32_t dst = base + r.slot * stage_bytes;
-      mbar_expect_tx_w(full, tx_bytes, leader);
-      tma_load_2d_w(dst, &tmap_h, full, kb * 64, row_a, leader);
-      if (two) tma_load_2d_w(dst + SIM_A_BYTES, &tmap_h, full, kb * 64, row_a + 128, leader);
-      tma_load_2d_w(dst + 2 * SIM_A_BYTES, &tmap_kept, full, kb * 64, row_b, leader);
-      issued = it + 1;
-      r.step(a.stages);
+      int t = 0;
+      for (; t < tiles; ++t) {
+        if (issued >= slots) mbar_wait_warp(smem_u32(&empty0[r.slot]), r.phase ^ 1u, wc);
+        if (__shfl_sync(0xffffffffu, bk->abort_flag, 0)) break;
+        const uint32_t full = smem_u32(&full0[r.slot]);
+        mbar_expect_tx_w(full, bytes, leader);
+        tma_load_2d_w(ring + r.slot * bytes, map, full, kb * 64, row + t * 128, leader);
+        ++issued;
+        r.step(slots);
+      }
+      if (t < tiles) break;
       if (++kb == n_kb) kb = 0;
     }
-    // drain: the last fill of every stage must have landed before the block leaves
-    for (int s = 0; s < a.stages; ++s) {
-      if (issued > s) {
-        const int last = ((issued - 1 - s) / a.stages) * a.stages + s;
-        mbar_wait_drain(smem_u32(&bk->full[s]), (last / a.stages) & 1, TC_WAIT_LIMIT);
-      }
-    }
+    // drain: the last fill of every slot must have landed before the block leaves
+    for (int s = 0; s < slots; ++s)
+      if (issued > s) mbar_wait_drain(smem_u32(&full0[s]), ((issued - 1 - s) / slots) & 1, TC_WAIT_LIMIT);
     __syncwarp();
   } else if (warp == 1) {
     // ---- MMA issuer (converged, as in sim_kernel)
     const uint32_t leader = warp_leader();
     const uint32_t tm = __shfl_sync(0xffffffffu, tmem_base, 0);
     const uint32_t idesc = umma_idesc_bf16(128, a.n_tile);
-    const uint64_t desc0 = umma_desc_sw128(base);
-    const int n_t = two ? 2 : 1;
-    RingPos r;
-    for (int it = 0; it < n_kb; ++it, r.step(a.stages)) {
-      const int s = r.slot;
-      mbar_wait_warp(smem_u32(&bk->full[s]), r.phase, wc);
-      tc_fence_after();
-      const uint64_t da = desc0 + (uint32_t)(s * stage_bytes) / 16, db = da + 2 * SIM_A_BYTES / 16;
-      for (int t = 0; t < n_t; ++t)
+    const uint64_t desc0 = umma_desc_sw128(base), bdesc0 = umma_desc_sw128(base_b);
+    RingPos ra, rb;
+    for (int it = 0; it < n_kb; ++it, rb.step(a.stages)) {
+      mbar_wait_warp(smem_u32(&bk->full_b[rb.slot]), rb.phase, wc);
+      const uint64_t db = bdesc0 + (uint32_t)(rb.slot * b_bytes) / 16;
+      for (int t = 0; t < n_t; ++t, ra.step(a.a_stages)) {
+        mbar_wait_warp(smem_u32(&bk->full[ra.slot]), ra.phase, wc);
+        tc_fence_after();
+        if (it == norm_lo && t == 0 && leader) mbar_arrive(smem_u32(&bk->norm_go));
+        const uint64_t da = desc0 + ra.slot * (SIM_A_BYTES / 16);
 #pragma unroll
         for (int kk = 0; kk < 4; ++kk)
-          tc_mma_bf16_w(tm + t * a.n_tile, da + t * (SIM_A_BYTES / 16) + kk * 2, db + kk * 2, idesc, (it > 0 || kk > 0) ? 1u : 0u, leader);
-      tc_commit_w(smem_u32(&bk->empty[s]), leader);
+          tc_mma_bf16_w(tm + t * a.n_tile, da + kk * 2, db + kk * 2, idesc, (it > 0 || kk > 0) ? 1u : 0u, leader);
+        tc_commit_w(smem_u32(&bk->empty[ra.slot]), leader);
+        if (!a.smat && (it < norm_lo || it >= norm_hi) && leader) mbar_arrive_n(smem_u32(&bk->empty[ra.slot]), 4);
+      }
+      tc_commit_w(smem_u32(&bk->empty_b[rb.slot]), leader);
     }
     tc_commit_w(smem_u32(&bk->acc_full), leader);
     // every MMA this warp issued has completed before tensor memory is given back
@@ -1668,16 +1680,17 @@ sim_pair_kernel(const __grid_constant__ CUtensorMap tmap_h, const __grid_constan
     const int v = pr * 256 + prow;                       // visual token
     const bool active = grp == 0 || two;
     const float *kinv = a.kept_inv + (size_t)b * a.keep_k;
-    // ---- squared norm of this thread's row (group 0 only; the other groups just free the stages)
+    // ---- squared norm of this thread's row: this group's share of the 64-column blocks
     float ssq[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-    const bool norms = gz == 0 && active && !a.smat;
-    RingPos r;
-    for (int it = 0; it < (norms ? n_kb : 0); ++it, r.step(a.stages)) {
-      const int s = r.slot;
-      mbar_wait(smem_u32(&bk->full[s]), r.phase, wc);
+    const bool norms = active && !a.smat;
+    // (a parity tells two neighbouring fills of a slot apart, no more: the warps join in when the issuer, who waits for every
+    // tile, has reached the range, so that all earlier fills are complete)
+    if (norms) mbar_wait(smem_u32(&bk->norm_go), 0, wc);
+    for (int it = norm_lo; it < (norms ? norm_hi : 0); ++it) {
+      const int u = it * n_t + grp, s = u % a.a_stages;
+      mbar_wait(smem_u32(&bk->full[s]), (u / a.a_stages) & 1, wc);
       if (!bk->abort_flag) {
-        const uint4 *row = reinterpret_cast<const uint4 *>(base_ptr + (size_t)s * stage_bytes +
-                                                           grp * SIM_A_BYTES + lrow * 128);
+        const uint4 *row = reinterpret_cast<const uint4 *>(base_ptr + (size_t)s * SIM_A_BYTES + lrow * 128);
 #pragma unroll
         for (int c = 0; c < 8; ++c) {
           const uint4 x = row[c ^ (lrow & 7)];
@@ -1759,11 +1772,11 @@ sim_pair_kernel(const __grid_constant__ CUtensorMap tmap_h, const __grid_constan
     tc_fence_before();
     bool finalize = !a.smat;
     if (a.groups > 1 && !a.smat) {
-      // per pair: [group][best of 256 rows | slot of 256 rows], then the 256 squared norms
-      float *pp = a.part + ((size_t)b * a.max_mt + pr) * (size_t)(a.groups * 512 + 256);
-      pp[gz * 512 + prow] = best;
-      reinterpret_cast<int *>(pp)[gz * 512 + 256 + prow] = best_slot;
-      if (gz == 0) pp[a.groups * 512 + prow] = ss;
+      // per pair: [group][best of 256 rows | slot of 256 rows | its share of their squared norms]
+      float *pp = a.part + ((size_t)b * a.max_mt + pr) * (size_t)(a.groups * 768);
+      pp[gz * 768 + prow] = best;
+      reinterpret_cast<int *>(pp)[gz * 768 + 256 + prow] = best_slot;
+      pp[gz * 768 + 512 + prow] = ss;
       __threadfence();
       asm volatile("bar.sync 1, 256;" ::: "memory");
       if (warp == 2 && lane == 0) {
@@ -1778,12 +1791,13 @@ sim_pair_kernel(const __grid_constant__ CUtensorMap tmap_h, const __grid_constan
         __threadfence();
         best = -INFINITY;
         best_slot = 0;
+        ss = 0.f;
         for (int g2 = 0; g2 < a.groups; ++g2) {           // ascending slots: the first maximum stays
-          const float val = __ldcg(pp + g2 * 512 + prow);
-          const int slot = __ldcg(reinterpret_cast<const int *>(pp) + g2 * 512 + 256 + prow);
+          const float val = __ldcg(pp + g2 * 768 + prow);
+          const int slot = __ldcg(reinterpret_cast<const int *>(pp) + g2 * 768 + 256 + prow);
+          ss += __ldcg(pp + g2 * 768 + 512 + prow);
           if (val > best) { best = val; best_slot = slot; }
         }
-        ss = __ldcg(pp + a.groups * 512 + prow);
       }
     }
     int dp = -1;

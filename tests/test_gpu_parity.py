@@ -142,6 +142,14 @@ def test_rows_of_member_bits(nvs, k, tokens):
         A.asap_free(small)
 
 
+@pytest.mark.parametrize("k,H", [(600, 1), (600, 3), (340, 5), (1100, 1)], ids=["fewer_steps_than_groups", "two_steps_each", "uneven", "five_groups"])
+def test_row_norms_shared_by_the_groups(ctx, k, H):
+    """Every group of kept slots adds up the squares of its range of the columns: two 64-column steps for three or five groups (some
+    have none), and ranges of different lengths; pairs of row tiles whose second tile is empty or holds one row."""
+    batch = W.tiny(B=2, n_vis=[1300, 1409], text_lens=[12, 30], H=H, keep_k=k, seed=330 + H, centres=50)
+    run_step(ctx, batch, A.Params(keep_k=k))
+
+
 def test_many_row_tiles_and_three_slot_tiles(ctx):
     """A batch large enough that the similarity kernel runs unsliced with more blocks than SMs
     (15 sequences x 19 row tiles) and three slot tiles (600 kept slots).  Odd and even numbers of row
