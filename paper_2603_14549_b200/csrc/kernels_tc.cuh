@@ -1533,7 +1533,9 @@ sim_kernel(const __grid_constant__ CUtensorMap tmap_h, const __grid_constant__ C
 // groups (lowest slot among equals), looks up which rows were dropped and writes their assignment.
 // The block that finishes a sample's last pair groups the dropped tokens by destination.
 // Matrix mode (a.smat set): the row operand is the dense kept-row array too (`tmap_h` maps it with a 128-row box)
-// and every block writes its 256 x n_tile piece of the sample's keep_k x keep_k cosine matrix; nothing else.
+// and every block writes its 256 x n_tile piece of the sample's keep_k x keep_k cosine matrix; nothing else.  The matrix is
+// symmetric: blocks that lie below the diagonal as a whole leave, and the blocks of the mirrored places write their pieces too
+// (24 x 576 slots: 6 of 9 blocks per sequence are left, one round of blocks instead of two: 100 -> 64 us).
 // =======================================================================================
 constexpr int SIMP_THREADS = 352;                // copy warp (rows), MMA warp, two groups of four epilogue warps, copy warp (kept rows)
 constexpr int SIMP_MAX_ROWS = 12, SIMP_MAX_KEPT = 4;   // slots of the two rings
@@ -1564,6 +1566,10 @@ sim_pair_kernel(const __grid_constant__ CUtensorMap tmap_h, const __grid_constan
   const int nd = d.nv - a.keep_k;
   const int n_rows = a.smat ? a.keep_k : d.nv;           // matrix mode: the row operand is the dense kept-row array
   if (pr * 256 >= n_rows) return;
+  if (a.smat && (gz + 1) * a.n_tile <= pr * 256) {       // below the diagonal: written by the block of the mirrored place
+    pdl_wait();
+    return;
+  }
   if (*reinterpret_cast<volatile uint32_t *>(a.status) & STATUS_SIM_TIMEOUT) {
     pdl_wait();
     return;
@@ -1730,15 +1736,15 @@ sim_pair_kernel(const __grid_constant__ CUtensorMap tmap_h, const __grid_constan
         tmem_wait_ld();
         if (a.smat) {
           // matrix mode: S[p][q] = <h_p, h_q> * (1/||h_p|| * 1/||h_q||) for this thread's kept row p
+          float sv[16];
+#pragma unroll
+          for (int e = 0; e < 16; ++e) sv[e] = __uint_as_float(r[e]) * (inv_p * bk->kinv[c + e]);   // (a column past the last slot has kinv 0 in shared memory)
           if (v < a.keep_k) {
             float *srow = a.smat + ((size_t)b * a.keep_k + v) * a.keep_k + slot0 + c;
-            float sv[16];
             uint32_t above = 0u;
 #pragma unroll
-            for (int e = 0; e < 16; ++e) {                // (a column past the last slot has kinv 0 in shared memory)
-              sv[e] = __uint_as_float(r[e]) * (inv_p * bk->kinv[c + e]);
+            for (int e = 0; e < 16; ++e)
               if (c + e < ncol && slot0 + c + e != v && sv[e] > a.threshold) above |= 1u << e;
-            }
             if (c + 16 <= ncol && (reinterpret_cast<size_t>(srow) & 15) == 0) {
 #pragma unroll
               for (int e = 0; e < 16; e += 4)         // 16-byte stores: a quarter of the store requests
@@ -1756,6 +1762,22 @@ sim_pair_kernel(const __grid_constant__ CUtensorMap tmap_h, const __grid_constan
               mrow[hw] = (uint16_t)above;
               if (slot0 + c + 16 >= a.keep_k && !(hw & 1)) mrow[hw + 1] = 0;
             }
+          }
+          // S[q][p] where the block of that place has left it to this one (the same for the 16 columns, and for each half of the
+          // warp's rows): a warp's 32 rows are neighbours in row q
+          const bool mirrored = (v / a.n_tile + 1) * a.n_tile <= ((slot0 + c) & ~255);
+          const uint32_t halves = __ballot_sync(0xffffffffu, mirrored);
+          if (halves) {
+            uint32_t word = 0u;
+#pragma unroll
+            for (int e = 0; e < 16; ++e) {
+              if (mirrored && c + e < ncol) a.smat[((size_t)b * a.keep_k + slot0 + c + e) * a.keep_k + v] = sv[e];
+              const uint32_t w = __ballot_sync(0xffffffffu, mirrored && sv[e] > a.threshold);
+              if ((lane & 15) == e) word = w;
+            }
+            const int half = lane >> 4;                   // lane writes its half of the warp's rows for column lane & 15
+            if (a.mask16 && ((halves >> (16 * half)) & 1u) && c + (lane & 15) < ncol)
+              a.mask16[((size_t)b * a.keep_k + slot0 + c + (lane & 15)) * a.mask_pitch + ((v & ~31) >> 4) + half] = (uint16_t)(word >> (16 * half));
           }
           continue;
         }

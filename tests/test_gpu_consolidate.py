@@ -380,3 +380,36 @@ def test_a_chain_costs_little_more_than_clusters():
         assert ms[1] < 6.0 * ms[0]
     finally:
         A.asap_free(c)
+
+
+@pytest.mark.parametrize("k", [257, 272, 513, 577, 784, 1040])
+def test_cosine_matrix_is_whole_where_half_its_blocks_are_multiplied(ctx, k):
+    """Blocks below the diagonal leave, the blocks of the mirrored places write their pieces: every entry of the matrix against 64
+    bits (two groups of slots to five, ragged ones, a last pair of one row and of one row tile), and every bit of the routing's
+    matrix against that entry, padding of the last word included."""
+    batch = W.tiny(B=2, n_vis=[k + 40, k + 3], text_lens=[5, 9], H=2, keep_k=k, seed=500 + k, centres=k // 8)
+    inp = A.make_inputs(batch, DEV)
+    mv, t = inp.max_vis, 0.3
+    keep = torch.stack([torch.arange(k, dtype=torch.int32) + 3, torch.arange(k, dtype=torch.int32)])
+    drop = torch.full((2, mv - k), -1, dtype=torch.int32)
+    drop[0] = torch.cat([torch.arange(3), torch.arange(k + 3, k + 40)]).int()
+    drop[1, :3] = torch.arange(k, k + 3).int()
+    out = A.alloc_outputs(inp, k, fill=True)
+    scratch = torch.full((A.asap_consolidate_scratch_bytes(2, k),), 255, dtype=torch.uint8, device=DEV)
+    A.asap_consolidate(ctx, inp, A.Params(keep_k=k, sim_threshold=t), torch.rand(2, mv, device=DEV), torch.rand(2, mv, device=DEV),
+                       keep.to(DEV), drop.to(DEV), scratch, out, torch.zeros(2, dtype=torch.int32, device=DEV))
+    torch.cuda.synchronize()
+    A.asap_check(ctx)
+    raw, kw = scratch.cpu(), (k + 31) // 32
+    at = (2 * k * k * 4 + 255) // 256 * 256
+    S = raw[:2 * k * k * 4].view(torch.float32).view(2, k, k)
+    words = raw[at:at + 2 * k * kw * 4].view(torch.int32).view(2, k, kw)
+    got = ((words.unsqueeze(-1) >> torch.arange(32, dtype=torch.int32)) & 1).bool().view(2, k, kw * 32)
+    for b in range(2):
+        lo = int(batch.cu_seqlens[b]) + int(batch.vis_start[b])
+        h = batch.hidden[lo + keep[b].long()].double()
+        h = h / h.norm(dim=1, keepdim=True)
+        assert float((S[b].double() - h @ h.T).abs().max()) < 1e-5      # 256 products: 2^-23 each at most
+        want = torch.zeros(k, kw * 32, dtype=torch.bool)
+        want[:, :k] = (S[b] > t) & ~torch.eye(k, dtype=torch.bool)
+        assert torch.equal(got[b], want)
