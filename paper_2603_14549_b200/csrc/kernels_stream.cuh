@@ -849,12 +849,13 @@ kept_gather_kernel(const __nv_bfloat16 *__restrict__ hidden, const SampleDesc *_
                    int bit_words) {
   pdl_enter();
   const int b = blockIdx.y;
-  const SampleDesc d = desc[b];
-  if (!d.valid) return;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int slot = blockIdx.x * (GATHER_THREADS / 32) + warp;
   if (slot >= keep_k) return;
-  const int j = min(max(keep_idx[(size_t)b * keep_k + slot], 0), d.nv - 1);
+  const int kept = ld_prev(keep_idx + (size_t)b * keep_k + slot);      // (beside the descriptor, not behind it)
+  const SampleDesc d = desc[b];
+  if (!d.valid) return;
+  const int j = min(max(kept, 0), d.nv - 1);
   const uint4 *src = reinterpret_cast<const uint4 *>(hidden + (size_t)(d.row0 + d.v0 + j) * D);
   uint4 *dst = reinterpret_cast<uint4 *>(kept_rows + ((size_t)b * keep_k + slot) * D);
   const int nvec = D / 8;
@@ -1529,15 +1530,41 @@ merge_compact_kernel(MergeArgs a) {
   __shared__ int s_j[BITS ? (MERGE_THREADS / 32) * MERGE_WARP_LIST : MERGE_LIST];
   __shared__ float s_w[BITS ? 1 : MERGE_LIST];
   const int b = blockIdx.y;
-  const SampleDesc d = a.desc[b];
-  if (!d.valid) return;
   const int nvec = a.D / 8;
   const int k = a.keep_k;
-  if ((int)blockIdx.x >= k) {
+  // The look-ups of a kept row that need no other are under way together with the descriptor: behind it they cost every block another
+  // round trip before its first row.
+  const int lane = threadIdx.x & 31;
+  const int slot = blockIdx.x;
+  int kept = 0, m_lo = 0, m_hi = 0;
+  // BITS: the lanes of a warp own neighbouring words, so that one scan over the lanes gives every member's place
+  const uint32_t *bit_row = BITS ? a.member_bits + ((size_t)b * k + slot) * a.bit_words : nullptr;
+  uint32_t mw[MERGE_BIT_WORDS];
+  int per = 0;
+  auto load_words = [&](int w0) {
+    per = (min(a.bit_words - w0, 32 * MERGE_BIT_WORDS) + 31) >> 5;
+#pragma unroll
+    for (int g = 0; g < MERGE_BIT_WORDS; ++g) {
+      const int w = w0 + lane * per + g;
+      mw[g] = g < per && w < a.bit_words ? (uint32_t)ld_prev(reinterpret_cast<const int *>(bit_row + w)) : 0u;
+    }
+  };
+  if (slot < k) {
+    kept = ld_prev(a.keep_idx + (size_t)b * k + slot);
+    if (BITS) {
+      load_words(0);
+    } else if (a.merge_enable) {
+      m_lo = ld_prev(a.seg + (size_t)b * (k + 1) + slot);
+      m_hi = ld_prev(a.seg + (size_t)b * (k + 1) + slot + 1);
+    }
+  }
+  const SampleDesc d = a.desc[b];
+  if (!d.valid) return;
+  if (slot >= k) {
     if (blockIdx.z) return;
     // ---------------------------------------------------------------- copy rows, one per warp
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int c = ((int)blockIdx.x - k) * MERGE_COPY_ROWS + warp;     // index among prefix + suffix rows
+    const int warp = threadIdx.x >> 5;
+    const int c = (slot - k) * MERGE_COPY_ROWS + warp;                // index among prefix + suffix rows
     if (c >= d.n - d.nv) return;
     const int srow = c < d.v0 ? c : c + d.nv;
     const int orow = d.out_row0 + (c < d.v0 ? c : c + k);
@@ -1560,8 +1587,7 @@ merge_compact_kernel(MergeArgs a) {
     return;
   }
   // ------------------------------------------------------------------ one kept row
-  const int slot = blockIdx.x;
-  const int vi = min(max(a.keep_idx[(size_t)b * k + slot], 0), d.nv - 1);   // visual index
+  const int vi = min(max(kept, 0), d.nv - 1);           // visual index
   const size_t grow = (size_t)(d.row0 + d.v0 + vi);
   const int orow = d.out_row0 + d.v0 + slot;
   const int v0 = blockIdx.z * (NV * MERGE_THREADS) + threadIdx.x;       // grid z: pieces of NV * 256 vectors of the row
@@ -1572,25 +1598,8 @@ merge_compact_kernel(MergeArgs a) {
   const uint4 *src = reinterpret_cast<const uint4 *>(a.hidden + grow * a.D);
   uint4 *dst = reinterpret_cast<uint4 *>(a.out_hidden + (size_t)orow * a.D);
   const int nd_max = a.max_vis - k;
-  int m_lo = 0, m_hi = 0;
-  if (!BITS && a.merge_enable) {
-    m_lo = min(max(a.seg[(size_t)b * (k + 1) + slot], 0), nd_max);
-    m_hi = min(max(a.seg[(size_t)b * (k + 1) + slot + 1], m_lo), nd_max);
-  }
-  // BITS: the lanes of a warp own neighbouring words, so that one scan over the lanes gives every member's place
-  const int lane = threadIdx.x & 31, words = (d.nv + 31) >> 5;
-  const uint32_t *bit_row = BITS ? a.member_bits + ((size_t)b * k + slot) * a.bit_words : nullptr;
-  uint32_t mw[MERGE_BIT_WORDS];
-  int per = 0;
-  auto load_words = [&](int w0) {
-    per = (min(words - w0, 32 * MERGE_BIT_WORDS) + 31) >> 5;
-#pragma unroll
-    for (int g = 0; g < MERGE_BIT_WORDS; ++g) {
-      const int w = w0 + lane * per + g;
-      mw[g] = g < per && w < words ? (uint32_t)ld_prev(reinterpret_cast<const int *>(bit_row + w)) : 0u;
-    }
-  };
-  if (BITS) load_words(0);
+  m_lo = min(max(m_lo, 0), nd_max);
+  m_hi = min(max(m_hi, m_lo), nd_max);
   uint4 self[NV];
 #pragma unroll
   for (int u = 0; u < NV; ++u) {
@@ -1657,7 +1666,7 @@ merge_compact_kernel(MergeArgs a) {
   if (BITS) {
     const int list0 = (threadIdx.x >> 5) * MERGE_WARP_LIST;
     // (a pass over more members than the list holds reads the words again: kept, they cost the pass its registers)
-    for (int w0 = 0, c0 = 0; w0 < words;) {
+    for (int w0 = 0, c0 = 0; w0 < a.bit_words;) {
       if (w0 | c0) load_words(w0);
       int mine = 0;
 #pragma unroll
