@@ -316,8 +316,11 @@ asap_status launch_rank(asap_ctx *ctx, const asap_inputs *in, const asap_params 
   sa.partial = ctx->score_partial; sa.work = ctx->cnt_work; sa.status = ctx->status; sa.wait_limit = ctx->wait_limit;
   mark(ctx, "score", st);
   const int items = B * in->H;
-  launch_pdl(score_kernel, dim3(items < ctx->num_sms ? items : ctx->num_sms), dim3(SC_THREADS), SC_SMEM_BYTES, st,
-             map_q, map_k, sa);
+  const dim3 blocks(items < ctx->num_sms ? items : ctx->num_sms);
+  if (in->min_vis < in->max_vis && items > ctx->num_sms && B <= SC_ORDER_MAX)
+    launch_pdl(score_kernel<true>, blocks, dim3(SC_THREADS), SC_SMEM_BYTES, st, map_q, map_k, sa);
+  else
+    launch_pdl(score_kernel<false>, blocks, dim3(SC_THREADS), SC_SMEM_BYTES, st, map_q, map_k, sa);
   ASAP_TRY(after_launch(ctx, "score"));
   if (!with_head_sum) return ASAP_OK;
   mark(ctx, "head_sum", st);
@@ -842,7 +845,8 @@ asap_status asap_init(asap_ctx **ctx_out, int device, size_t max_total_tokens, i
   if (e == cudaSuccess) e = cudaMemset(ctx->arena + o_tiles, 0, ctx->cap_tiles * sizeof(unsigned int));
   if (e == cudaSuccess) e = cudaMemset(ctx->status, 0, sizeof(uint32_t));
   // kernels whose dynamic shared memory exceeds the 48 KB default
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(score_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SC_SMEM_BYTES);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(score_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, SC_SMEM_BYTES);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(score_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, SC_SMEM_BYTES);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(sim_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(sim_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(sim_pair_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
