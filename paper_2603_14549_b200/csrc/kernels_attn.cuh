@@ -525,7 +525,7 @@ attn_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__ 
           const int di = i - j0, hi = hi_adm - j0;  // columns of the diagonal and of the last admitted key
 #pragma unroll 1
           for (int c0 = 0; c0 < 128; c0 += 32) {
-            if (j0 + c0 + 31 <= i_lo && j0 + c0 + 31 < it.n) continue;       // nothing to do for any row of the warp
+            if (j0 + c0 + 31 < it.n && (j0 + c0 + 31 <= i_lo || (kind.crossed && j0 + c0 > i_lo))) continue;   // nothing to do, or done below
             uint32_t r[32];
             tmem_ld32(s_addr + c0, r);
             tmem_wait_ld();
@@ -543,11 +543,6 @@ attn_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__ 
             tmem_st32(s_addr + c0, r);
           }
           tmem_wait_st();
-          if (kind.crossed) {
-            __syncwarp();
-            if (lane == 0) mbar_arrive(smem_u32(&bk->m_empty[g]));
-            ++mc;
-          }
         }
         // ---- this row's 128 logits, once
         uint32_t xr[128];
@@ -557,6 +552,29 @@ attn_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__ 
         tc_fence_before();
         __syncwarp();
         if (lane == 0) mbar_arrive(smem_u32(&bk->s_empty));
+        if (kind.crossed) {
+          // columns past all rows of the warp (the tile lies on the diagonal, so its first 32 never do): m_j for a row of the span,
+          // AT_NEVER for any other.  Put right in tensor memory like the 32 columns that the diagonal crosses, 450 clocks per 32, they
+          // held up the S that both row tiles share for 2000 to 2600 clocks (1 x 643 rows 20.5 -> 19.7 us, 16 x 627-739 167 -> 163.5).
+          const float off = vis_row ? 0.f : AT_NEVER, in = vis_row ? 1.f : 0.f;
+          const uint64_t off2 = f2_pack(off, off), in2 = f2_pack(in, in);
+#pragma unroll
+          for (int c0 = 32; c0 < 128; c0 += 32) {
+            if (j0 + c0 <= i_lo || j0 + c0 + 31 >= it.n) continue;
+#pragma unroll
+            for (int c = c0; c < c0 + 32; c += 4) {
+              const ulonglong2 m4 = *reinterpret_cast<const ulonglong2 *>(bk->m_tile[g] + c);
+              float x[4];
+              f2_unpack(f2_add(f2_fma(in2, m4.x, f2_pack(__uint_as_float(xr[c]), __uint_as_float(xr[c + 1]))), off2), x[0], x[1]);
+              f2_unpack(f2_add(f2_fma(in2, m4.y, f2_pack(__uint_as_float(xr[c + 2]), __uint_as_float(xr[c + 3]))), off2), x[2], x[3]);
+#pragma unroll
+              for (int e = 0; e < 4; ++e) xr[c + e] = __float_as_uint(x[e]);
+            }
+          }
+          __syncwarp();
+          if (lane == 0) mbar_arrive(smem_u32(&bk->m_empty[g]));
+          ++mc;
+        }
         if (kt > 0) {
           mbar_wait(smem_u32(&bk->pv_done[g]), (sc - 1) & 1, wc);      // O is complete up to here, and P may be overwritten
           tc_fence_after();
