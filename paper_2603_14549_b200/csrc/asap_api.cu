@@ -594,10 +594,13 @@ asap_status launch_merge_back(asap_ctx *ctx, const asap_inputs *in, const asap_p
   ma.out_pos = out->out_pos; ma.src_row = out->src_row;
   const int copy_rows = in->max_seq - in->min_vis;   // prefix + suffix rows of the longest sequence, at most
   int nv = (D / 8 + MERGE_THREADS - 1) / MERGE_THREADS;
-  dim3 grid(k + (copy_rows + MERGE_COPY_ROWS - 1) / MERGE_COPY_ROWS, B);
+  // Without member bits (after the routing, most kept rows have no members): a row per warp where that still fills the machine.
+  const int per_block = MERGE_THREADS / 32, blocks8 = (k + per_block - 1) / per_block;
+  ma.block_rows = !bits && (long long)blocks8 * B >= 2LL * ctx->num_sms ? per_block : 1;
+  dim3 grid((ma.block_rows > 1 ? blocks8 : k) + (copy_rows + MERGE_COPY_ROWS - 1) / MERGE_COPY_ROWS, B);
   // Rows cut into pieces of 2048 elements while all of them still run in one wave (1 x 192 slots: merge 10.4 -> 9.0 us, the
   // step 41.6 -> 40.5); beyond that the shorter pieces cost more than they balance (16 x 64 slots 28.8 -> 31.8 us).
-  if (nv > 1 && (long long)grid.x * grid.y * nv <= 3LL * ctx->num_sms) { grid.z = nv; nv = 1; }
+  if (nv > 1 && ma.block_rows == 1 && (long long)grid.x * grid.y * nv <= 3LL * ctx->num_sms) { grid.z = nv; nv = 1; }
   mark(ctx, "merge_compact", st);
   auto launch = [&](auto bits_c) {
     constexpr bool BITS = decltype(bits_c)::value != 0;
