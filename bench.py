@@ -92,17 +92,15 @@ def algorithmic(batch, keep_k, rank_visual=False):
     every operand it consumes read once, every result written once (bf16 = 2 bytes)."""
     D = batch.D
     out = {name: {"bytes": 0, "flops": 0} for name in
-           ("qsum", "mass_salience", "salience", "score", "head_sum", "select", "kept_gather", "sim", "merge_compact",
+           ("mass", "salience", "score", "head_sum", "select", "kept_gather", "sim", "merge_compact",
             "prepare", "role_map")}
     for b in range(batch.B):
         n = int(batch.cu_seqlens[b + 1] - batch.cu_seqlens[b])
         nv, tl = int(batch.vis_len[b]), int(batch.text_len[b])
         t0 = int(batch.text_start[b])
         row = D * 2
-        out["qsum"]["bytes"] += nv * row
-        out["qsum"]["flops"] += nv * D
-        out["mass_salience"]["bytes"] += nv * row + nv * 12
-        out["mass_salience"]["flops"] += 2 * nv * D
+        out["mass"]["bytes"] += 2 * nv * row + batch.H * nv * 4
+        out["mass"]["flops"] += 3 * nv * D
         out["salience"]["bytes"] += batch.H * nv * 4 + nv * 12      # per-head masses in, mass / salience / mask out
         # ranking rows = text span: queries once, every key they may attend to once
         out["score"]["bytes"] += tl * row + (t0 + tl) * row + nv * 4
@@ -581,7 +579,7 @@ def run_cuda(args):
         sk = {name: ms / max(n, 1) * 1e3 for name, (n, ms) in A.asap_profile_read(ctx).items()}
         A.asap_profile(ctx, False)
         hs_bytes = sum(batch.H * int(v) * 4 + int(v) * 4 for v in batch.vis_len)
-        mh_bytes = sum(int(v) * batch.D * 2 + 2 * batch.H * int(v) * 4 for v in batch.vis_len)
+        mh_bytes = sum(int(v) * batch.D * 4 + 2 * batch.H * int(v) * 4 for v in batch.vis_len)
         staged = {"calls": "asap_score, asap_select, asap_merge, asap_score(per_head_mask)", "kernel_us": sk,
                   "head_sum_GBs": hs_bytes / sk["head_sum"] / 1e3 if sk.get("head_sum") else None,
                   "mass_heads_GBs": mh_bytes / sk["mass_heads"] / 1e3 if sk.get("mass_heads") else None}

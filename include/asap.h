@@ -280,7 +280,7 @@ asap_status asap_select_static(const asap_inputs *in, const asap_params *p, cons
  * the events; at most 16384 are used between two reads, later launches go untimed).
  * asap_profile(ctx, 0) stops that.  Either call clears the accumulated times. */
 typedef struct {
-  char name[32];     /* kernel name: "qsum", "mass_salience", "score", "select", "sim", ... */
+  char name[32];     /* kernel name: "mass", "score", "select", "sim", ... */
   uint64_t launches; /* launches timed since profiling was enabled */
   double total_ms;   /* sum over those launches of (next event - this kernel's event) */
 } asap_kernel_time;

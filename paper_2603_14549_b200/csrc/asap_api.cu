@@ -37,12 +37,12 @@ struct asap_ctx {
   int device = 0, num_sms = 1;
   size_t cap_tokens = 0, cap_keep_rows = 0;
   int cap_B = 0, cap_H = 0, cap_D = 0;
-  size_t cap_chunks = 0;      // rows of the query-sum partial buffer
   uint8_t *arena = nullptr;   // one allocation, carved below
   SampleDesc *desc = nullptr;
-  float *qsum_partial = nullptr, *qbar = nullptr, *score_partial = nullptr,
-        *kept_inv = nullptr;
-  unsigned int *cnt_qsum = nullptr, *cnt_mass = nullptr, *cnt_sim = nullptr,
+  uint32_t *member_bits = nullptr;  // rows of member bits of the merge, member_cap words
+  size_t member_cap = 0;
+  float *score_partial = nullptr, *kept_inv = nullptr;
+  unsigned int *cnt_sim = nullptr,
                *cnt_tiles = nullptr, *cnt_work = nullptr;
   float *mass_partial = nullptr;    // [B, H, max_vis] per-head attention masses
   float *head_norm = nullptr;       // [B, H, 2] minimum and 1 / range of a head's masses (per-head masks)
@@ -129,8 +129,6 @@ asap_status validate(asap_ctx *ctx, const asap_inputs *in, const asap_params *p,
     return fail(ctx, ASAP_ERR_WORKSPACE, "B * max_vis exceeds max_total_tokens");
   if ((size_t)in->B * (size_t)p->keep_k > ctx->cap_keep_rows)
     return fail(ctx, ASAP_ERR_WORKSPACE, "B * keep_k exceeds max_keep_rows");
-  const size_t chunks = (size_t)in->B * ((in->max_vis + QSUM_ROWS - 1) / QSUM_ROWS);
-  if (chunks > ctx->cap_chunks) return fail(ctx, ASAP_ERR_WORKSPACE, "query-sum scratch too small for B * max_vis");
   if (!in->cu_seqlens || !in->vis_start || !in->vis_len || !in->text_start || !in->text_len)
     return fail(ctx, ASAP_ERR_INVALID, "null per-sample array");
   if ((in->rank_start == nullptr) != (in->rank_len == nullptr))
@@ -246,53 +244,38 @@ asap_status launch_prepare(asap_ctx *ctx, const asap_inputs *in, const asap_para
   return after_launch(ctx, "prepare");
 }
 
-// Steps 1a-1b: query sum, attention mass, salience, mask vector.  The query-sum kernel also carries the device-side validation and
-// writes the descriptors.
-
-// Rows a block of the query-sum kernel adds up: 32, doubled (up to 128) while the grid still has two blocks per
-// SM -- every chunk costs a partial row written and read back (32 rows: 12 % on top of the queries themselves).
-int qsum_rows_per_chunk(const asap_ctx *ctx, const asap_inputs *in) {
-  const long long col_blocks = (in->D + QSUM_COLS - 1) / QSUM_COLS;
-  int rows = QSUM_ROWS;
-  while (rows < 4 * QSUM_ROWS &&
-         (long long)((in->max_vis + 2 * rows - 1) / (2 * rows)) * col_blocks * in->B >= 2LL * ctx->num_sms)
-    rows *= 2;
-  return rows;
+SalienceArgs salience_args(const asap_ctx *ctx, const asap_inputs *in, const asap_params *p, const asap_outputs *out) {
+  SalienceArgs a;
+  a.H = in->H; a.scale = 1.0 / ((double)in->H * sqrt((double)in->head_dim)); a.lambda_max = p->lambda_max; a.eps = p->eps;
+  a.heads = ctx->mass_partial; a.norm = p->per_head_mask ? ctx->head_norm : nullptr; a.mass = out->mass; a.salience = out->salience;
+  a.mask_log = out->mask_log; a.rank_score = out->rank_score;
+  return a;
 }
 
+// Steps 1a-1b: attention mass, salience, mask vector.  The kernel also carries the device-side validation and writes the
+// descriptors.  With a mask per head the head means, which nothing before the merge needs, come later: beside the selection, or in
+// asap_score at its end.
 asap_status launch_mass(asap_ctx *ctx, const asap_inputs *in, const asap_params *p, const asap_outputs *out,
                         int32_t *out_cu, int out_capacity, cudaStream_t st) {
-  const int D = in->D, B = in->B;
-  const int qrows = qsum_rows_per_chunk(ctx, in);
-  const int max_chunks = (in->max_vis + qrows - 1) / qrows;
-  const int col_blocks = (D + QSUM_COLS - 1) / QSUM_COLS;
-  PrepareArgs pa = prepare_args(ctx, in, p, out_cu, out_capacity);
-  pa.write_desc = 1;
-  mark(ctx, "qsum", st);
-  launch_pdl(qsum_kernel, dim3(max_chunks, col_blocks, B), dim3(QSUM_THREADS), 0, st,
-             static_cast<const __nv_bfloat16 *>(in->q), pa, D, max_chunks, qrows, ctx->qsum_partial, ctx->qbar,
-             ctx->cnt_qsum);
-  ASAP_TRY(after_launch(ctx, "qsum"));
-
-  const int row_blocks = (in->max_vis + MASS_ROWS - 1) / MASS_ROWS;
-  if (p->per_head_mask) {
-    // (the head means, which nothing before the merge needs, come later: beside the selection, or in asap_score at its end)
-    mark(ctx, "mass_heads", st);
-    launch_pdl(mass_heads_kernel, dim3(row_blocks, B), dim3(MASS_THREADS), (size_t)D * sizeof(float), st,
-               static_cast<const __nv_bfloat16 *>(in->k), ctx->desc, D, in->H, in->max_vis,
-               1.0f / sqrtf((float)in->head_dim), ctx->qbar, ctx->mass_partial);
-    ASAP_TRY(after_launch(ctx, "mass_heads"));
-    mark(ctx, "mask_heads", st);
-    launch_pdl(mask_heads_kernel, dim3(in->H, B), dim3(MASS_THREADS), 0, st, ctx->desc, in->H, in->max_vis, p->lambda_max, p->eps,
-               ctx->mass_partial, out->mask_log_heads, ctx->head_norm);
-    return after_launch(ctx, "mask_heads");
-  }
-  const float scale = 1.0f / ((float)in->H * sqrtf((float)in->head_dim));
-  mark(ctx, "mass_salience", st);
-  launch_pdl(mass_salience_kernel, dim3(row_blocks, B), dim3(MASS_THREADS), (size_t)D * sizeof(float), st,
-             static_cast<const __nv_bfloat16 *>(in->k), ctx->desc, D, in->max_vis, scale, p->lambda_max, p->eps,
-             ctx->qbar, out->mass, out->salience, out->mask_log, out->rank_score, ctx->cnt_mass);
-  return after_launch(ctx, "mass_salience");
+  CUtensorMap map_q, map_k;
+  if (!make_map(ctx, &map_q, in->q, (uint64_t)in->total_tokens, (uint64_t)in->D, 128) ||
+      !make_map(ctx, &map_k, in->k, (uint64_t)in->total_tokens, (uint64_t)in->D, 128))
+    return fail(ctx, ASAP_ERR_CUDA, "cuTensorMapEncodeTiled failed for q / k");
+  MassArgs ma;
+  ma.pa = prepare_args(ctx, in, p, out_cu, out_capacity);
+  ma.pa.write_desc = 1;
+  ma.max_vis = in->max_vis; ma.scale = p->per_head_mask ? 1.0f / sqrtf((float)in->head_dim) : 1.0f;
+  ma.heads = ctx->mass_partial; ma.mask_log_heads = p->per_head_mask ? out->mask_log_heads : nullptr; ma.norm = ctx->head_norm;
+  ma.H = in->H; ma.lambda_max = p->lambda_max; ma.eps = p->eps; ma.status = ctx->status; ma.wait_limit = ctx->wait_limit;
+  const int items = in->B * in->H;
+  mark(ctx, p->per_head_mask ? "mass_heads" : "mass", st);
+  launch_pdl(p->per_head_mask ? mass_kernel<true> : mass_kernel<false>, dim3(items < ctx->num_sms ? items : ctx->num_sms),
+             dim3(MASS_THREADS), MASS_SMEM_BYTES, st, map_q, map_k, ma);
+  ASAP_TRY(after_launch(ctx, "mass"));
+  if (p->per_head_mask) return ASAP_OK;
+  mark(ctx, "salience", st);
+  launch_pdl(salience_kernel, dim3(in->B), dim3(SAL_THREADS), 0, st, ctx->desc, in->max_vis, salience_args(ctx, in, p, out));
+  return after_launch(ctx, "salience");
 }
 
 // Steps 1c-2: Eq. 4 probabilities of the ranking rows, summed per head; optionally the head sum.
@@ -317,10 +300,8 @@ asap_status launch_rank(asap_ctx *ctx, const asap_inputs *in, const asap_params 
   mark(ctx, "score", st);
   const int items = B * in->H;
   const dim3 blocks(items < ctx->num_sms ? items : ctx->num_sms);
-  if (in->min_vis < in->max_vis && items > ctx->num_sms && B <= SC_ORDER_MAX)
-    launch_pdl(score_kernel<true>, blocks, dim3(SC_THREADS), SC_SMEM_BYTES, st, map_q, map_k, sa);
-  else
-    launch_pdl(score_kernel<false>, blocks, dim3(SC_THREADS), SC_SMEM_BYTES, st, map_q, map_k, sa);
+  const bool sorted = in->min_vis < in->max_vis && items > ctx->num_sms && B <= SC_ORDER_MAX;
+  launch_pdl(sorted ? score_kernel<true> : score_kernel<false>, blocks, dim3(SC_THREADS), SC_SMEM_BYTES, st, map_q, map_k, sa);
   ASAP_TRY(after_launch(ctx, "score"));
   if (!with_head_sum) return ASAP_OK;
   mark(ctx, "head_sum", st);
@@ -368,24 +349,15 @@ asap_status check_merge_room(asap_ctx *ctx, const asap_inputs *in, const asap_pa
 size_t route_fixed_words(const asap_params *p) { return 5 * (size_t)p->keep_k; }
 size_t route_tail_words(const asap_inputs *in, const asap_params *p) { return (size_t)(in->max_vis - p->keep_k) + (size_t)in->max_vis; }
 
-// Words of a slot's row of member bits (bit j: visual token j merges into the slot), and whether a batch's rows fit the query
-// sum's partials, which nothing reads any more by then (they do while keep_k <= max_D: B * ceil(max_vis / 32) is at most the rows
-// of that buffer).  If not, the similarity kernel's last block per sequence groups the dropped tokens by destination: a chain of
+// Words of a slot's row of member bits (bit j: visual token j merges into the slot), and whether a batch's rows fit
+// their scratch (they do while keep_k <= max_D).  If not, the similarity kernel's last block per sequence groups the dropped tokens by destination: a chain of
 // eight barriers, 10 to 17 us behind the last product of a sequence.  The bits cost an atomic per dropped token and a scan of one
 // row per merge block.  Measured per step, grouped -> bits: 8 x 2304 with 320 kept 193 -> 185 us, 12 x 577-2881 with 145 kept 230 ->
 // 221.5, 8 x 1536 with 340 kept 219 -> 213.5; against blocks that looked for their members among all dropped tokens' destinations,
 // 16 x 576 with 64 kept 113 -> 110, 1 x 576 with 192 kept 39.7 -> 39.6.
 int member_words(const asap_inputs *in) { return (in->max_vis + 31) / 32; }
 bool merge_bits(const asap_ctx *ctx, const asap_inputs *in, const asap_params *p) {
-  return merging(in, p) && (size_t)in->B * p->keep_k * member_words(in) <= ctx->cap_chunks * (size_t)ctx->cap_D;
-}
-
-SalienceArgs salience_args(const asap_ctx *ctx, const asap_inputs *in, const asap_params *p, const asap_outputs *out) {
-  SalienceArgs a;
-  a.H = in->H; a.scale = 1.0 / ((double)in->H * sqrt((double)in->head_dim)); a.lambda_max = p->lambda_max; a.eps = p->eps;
-  a.heads = ctx->mass_partial; a.norm = p->per_head_mask ? ctx->head_norm : nullptr; a.mass = out->mass; a.salience = out->salience;
-  a.mask_log = out->mask_log; a.rank_score = out->rank_score;
-  return a;
+  return merging(in, p) && (size_t)in->B * p->keep_k * member_words(in) <= ctx->member_cap;
 }
 
 // `fused_head_sum`: the ranking scores are still per-head sums in scratch (the score kernel ran
@@ -410,7 +382,7 @@ asap_status launch_merge_front(asap_ctx *ctx, const asap_inputs *in, const asap_
                                cudaStream_t st) {
   const int B = in->B, D = in->D, k = p->keep_k;
   if (merging(in, p)) {
-    uint32_t *bits = merge_bits(ctx, in, p) ? reinterpret_cast<uint32_t *>(ctx->qsum_partial) : nullptr;
+    uint32_t *bits = merge_bits(ctx, in, p) ? ctx->member_bits : nullptr;
     mark(ctx, "kept_gather", st);
     launch_pdl(kept_gather_kernel, dim3(dim3((k + GATHER_THREADS / 32 - 1) / (GATHER_THREADS / 32), B)), dim3(GATHER_THREADS), 0, st, 
         static_cast<const __nv_bfloat16 *>(in->hidden), ctx->desc, D, k, keep_idx, ctx->kept_rows, ctx->kept_inv, bits,
@@ -589,7 +561,7 @@ asap_status launch_merge_back(asap_ctx *ctx, const asap_inputs *in, const asap_p
   ma.D = D; ma.max_vis = in->max_vis; ma.keep_k = k; ma.merge_enable = do_merge ? 1 : 0; ma.eps = p->eps;
   ma.salience = salience; ma.keep_idx = keep_idx; ma.drop_idx = drop_idx; ma.seg = ctx->seg;
   ma.members = ctx->members; ma.member_meta = (do_merge && grouped_with_weights) ? ctx->member_meta : nullptr;
-  ma.member_bits = bits ? reinterpret_cast<const uint32_t *>(ctx->qsum_partial) : nullptr; ma.bit_words = member_words(in);
+  ma.member_bits = bits ? ctx->member_bits : nullptr; ma.bit_words = member_words(in);
   ma.out_hidden = static_cast<__nv_bfloat16 *>(out->out_hidden);
   ma.out_pos = out->out_pos; ma.src_row = out->src_row;
   const int copy_rows = in->max_seq - in->min_vis;   // prefix + suffix rows of the longest sequence, at most
@@ -782,7 +754,6 @@ asap_status asap_init(asap_ctx **ctx_out, int device, size_t max_total_tokens, i
   ctx->num_sms = prop.multiProcessorCount;
   ctx->cap_tokens = max_total_tokens; ctx->cap_B = max_B; ctx->cap_H = max_H; ctx->cap_D = max_D;
   ctx->cap_keep_rows = max_keep_rows;
-  ctx->cap_chunks = max_total_tokens / QSUM_ROWS + 2 * (size_t)max_B;
 
   void *fn = nullptr;
   cudaDriverEntryPointQueryResult qres;
@@ -794,17 +765,17 @@ asap_status asap_init(asap_ctx **ctx_out, int device, size_t max_total_tokens, i
   ctx->encode = reinterpret_cast<EncodeTiledFn>(fn);
 
   const size_t T = max_total_tokens, Bc = (size_t)max_B, Hc = (size_t)max_H, Dc = (size_t)max_D;
-  const size_t col_blocks = (Dc + QSUM_COLS - 1) / QSUM_COLS;
   size_t off = 0;
   auto carve = [&](size_t bytes) { size_t o = off; off = align_up(off + bytes, 256); return o; };
   const size_t o_desc = carve(Bc * sizeof(SampleDesc));
-  const size_t o_qpart = carve(ctx->cap_chunks * Dc * sizeof(float));
-  const size_t o_qbar = carve(Bc * Dc * sizeof(float));
+  ctx->member_cap = (T / 32 + 2 * Bc) * Dc;           // (every batch with keep_k <= max_D: B * ceil(max_vis / 32) <= T / 32 + B)
+  const size_t o_bits = carve(ctx->member_cap * sizeof(uint32_t));
   const size_t o_spart = carve(Hc * T * sizeof(float));
   const size_t o_mpart = carve(Hc * T * sizeof(float));
   const size_t o_hnorm = carve(Bc * Hc * 2 * sizeof(float));
   const size_t o_kinv = carve(max_keep_rows * sizeof(float));
-  const size_t o_cnt = carve((Bc * col_blocks + 2 * Bc + 4) * sizeof(unsigned int));
+  const size_t n_cnt = Bc + 4;
+  const size_t o_cnt = carve(n_cnt * sizeof(unsigned int));
   const size_t o_role = carve(T * sizeof(int32_t));
   const size_t o_seg = carve((max_keep_rows + Bc) * sizeof(int32_t));
   const size_t o_mem = carve(T * sizeof(int32_t));
@@ -821,8 +792,7 @@ asap_status asap_init(asap_ctx **ctx_out, int device, size_t max_total_tokens, i
     return fail(nullptr, ASAP_ERR_CUDA, "cudaMalloc of %zu scratch bytes: %s", off, cudaGetErrorString(e));
   }
   ctx->desc = reinterpret_cast<SampleDesc *>(ctx->arena + o_desc);
-  ctx->qsum_partial = reinterpret_cast<float *>(ctx->arena + o_qpart);
-  ctx->qbar = reinterpret_cast<float *>(ctx->arena + o_qbar);
+  ctx->member_bits = reinterpret_cast<uint32_t *>(ctx->arena + o_bits);
   ctx->score_partial = reinterpret_cast<float *>(ctx->arena + o_spart);
   ctx->mass_partial = reinterpret_cast<float *>(ctx->arena + o_mpart);
   if (const char *env = getenv("ASAP_SIM_PAIR_MIN_BLOCKS")) ctx->sim_pair_min_blocks = atoll(env);
@@ -830,11 +800,9 @@ asap_status asap_init(asap_ctx **ctx_out, int device, size_t max_total_tokens, i
   if (const char *env = getenv("ASAP_SIM_CLUSTER")) ctx->sim_cluster = atoi(env);
   ctx->head_norm = reinterpret_cast<float *>(ctx->arena + o_hnorm);
   ctx->kept_inv = reinterpret_cast<float *>(ctx->arena + o_kinv);
-  ctx->counters_off = o_cnt; ctx->counters_bytes = (Bc * col_blocks + 2 * Bc + 4) * sizeof(unsigned int);
+  ctx->counters_off = o_cnt; ctx->counters_bytes = n_cnt * sizeof(unsigned int);
   ctx->tiles_off = o_tiles; ctx->tiles_bytes = ctx->cap_tiles * sizeof(unsigned int);
-  ctx->cnt_qsum = reinterpret_cast<unsigned int *>(ctx->arena + o_cnt);
-  ctx->cnt_mass = ctx->cnt_qsum + Bc * col_blocks;
-  ctx->cnt_sim = ctx->cnt_mass + Bc;
+  ctx->cnt_sim = reinterpret_cast<unsigned int *>(ctx->arena + o_cnt);
   ctx->cnt_work = ctx->cnt_sim + Bc;
   ctx->role = reinterpret_cast<int32_t *>(ctx->arena + o_role);
   ctx->seg = reinterpret_cast<int32_t *>(ctx->arena + o_seg);
@@ -844,12 +812,14 @@ asap_status asap_init(asap_ctx **ctx_out, int device, size_t max_total_tokens, i
   ctx->cnt_tiles = reinterpret_cast<unsigned int *>(ctx->arena + o_tiles);
   ctx->sim_part = reinterpret_cast<float *>(ctx->arena + o_simpart);
   ctx->status = reinterpret_cast<uint32_t *>(ctx->arena + o_status);
-  e = cudaMemset(ctx->arena + o_cnt, 0, (Bc * col_blocks + 2 * Bc + 4) * sizeof(unsigned int));
+  e = cudaMemset(ctx->arena + o_cnt, 0, n_cnt * sizeof(unsigned int));
   if (e == cudaSuccess) e = cudaMemset(ctx->arena + o_tiles, 0, ctx->cap_tiles * sizeof(unsigned int));
   if (e == cudaSuccess) e = cudaMemset(ctx->status, 0, sizeof(uint32_t));
   // kernels whose dynamic shared memory exceeds the 48 KB default
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(score_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, SC_SMEM_BYTES);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(score_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, SC_SMEM_BYTES);
+  for (auto kernel : {score_kernel<false>, score_kernel<true>})
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SC_SMEM_BYTES);
+  for (auto kernel : {mass_kernel<false>, mass_kernel<true>})
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, MASS_SMEM_BYTES);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(sim_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(sim_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(sim_pair_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
@@ -1043,15 +1013,16 @@ asap_status asap_check(asap_ctx *ctx, void *stream) {
   if (e != cudaSuccess) return fail(ctx, ASAP_ERR_CUDA, "asap_check: %s", cudaGetErrorString(e));
   if (word == 0) { ctx->err[0] = 0; return ASAP_OK; }
   cudaMemsetAsync(ctx->status, 0, sizeof(uint32_t), st);
-  if (word & (STATUS_SCORE_TIMEOUT | STATUS_SIM_TIMEOUT | STATUS_ATTN_TIMEOUT)) {
+  if (word & (STATUS_MASS_TIMEOUT | STATUS_SCORE_TIMEOUT | STATUS_SIM_TIMEOUT | STATUS_ATTN_TIMEOUT)) {
     // blocks that gave up did not finish the hand-shakes that leave the counters at zero
     cudaMemsetAsync(ctx->arena + ctx->counters_off, 0, ctx->counters_bytes, st);
     cudaMemsetAsync(ctx->arena + ctx->tiles_off, 0, ctx->tiles_bytes, st);
   }
   cudaStreamSynchronize(st);
-  return fail(ctx, ASAP_ERR_DEVICE, "device status 0x%x:%s%s%s%s%s", word,
+  return fail(ctx, ASAP_ERR_DEVICE, "device status 0x%x:%s%s%s%s%s%s", word,
               (word & STATUS_BAD_SAMPLE) ? " a per-sample span failed validation (sample skipped);" : "",
               (word & STATUS_OUT_CAPACITY) ? " shortened batch exceeds out_rows_capacity (nothing written);" : "",
+              (word & STATUS_MASS_TIMEOUT) ? " a wait timed out in the mass kernel;" : "",
               (word & STATUS_SCORE_TIMEOUT) ? " a wait timed out in the score kernel;" : "",
               (word & STATUS_SIM_TIMEOUT) ? " a wait timed out in the similarity kernel;" : "",
               (word & STATUS_ATTN_TIMEOUT) ? " a wait timed out in the attention kernel;" : "");

@@ -30,6 +30,7 @@ enum : uint32_t {
   STATUS_OUT_CAPACITY = 2u,    // shortened batch does not fit out_rows_capacity
   STATUS_SCORE_TIMEOUT = 4u,   // a bounded wait ran out in the score kernel
   STATUS_SIM_TIMEOUT = 8u,     // a bounded wait ran out in the similarity kernel
+  STATUS_MASS_TIMEOUT = 32u,   // a bounded wait ran out in the mass kernel
 };
 
 // Programmatic dependent launch: wait until the previous kernel of the stream has completed and

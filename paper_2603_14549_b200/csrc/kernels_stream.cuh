@@ -1,8 +1,6 @@
 // The memory-bound and latency-bound kernels of the ASAP prune step:
 //   prepare        device-side validation, per-sample descriptors, output row offsets (one warp of a kernel that runs anyway)
-//   qsum           sum of the visual query rows                       (Eq. 1, summed over i first)
-//   mass_salience  s_j, then s_hat_j and m_j                          (Eq. 1, Eq. 2, Eq. 3)
-//   mass_heads, mask_heads, salience_heads   the same with a mask per head
+//   mass           sum of the visual queries, s_j, then s_hat_j and m_j   (Eq. 1, Eq. 2, Eq. 3), with one mask or one per head
 //   salience_block s_hat_j from per-head masses the score kernel produced (part of the selection launch)
 //   select         stable radix top-k of the ranking scores           (Fig. 3)
 //   role_map       kept slot / dropped position of every visual token
@@ -13,6 +11,8 @@
 //   gather_rows    KV-cache compaction with the row map of the hand-off
 #pragma once
 
+#include <cuda.h>
+
 #include "common.cuh"
 
 namespace asap {
@@ -22,7 +22,7 @@ namespace asap {
 // =======================================================================================
 struct PrepareArgs {
   int32_t B, total_tokens, min_vis, max_vis, max_seq, max_rank, keep_k, out_capacity;
-  int32_t write_desc;        // query-sum and score kernel: the first block also runs prepare_warp
+  int32_t write_desc;        // mass and score kernel: the first block also runs prepare_warp
   const int32_t *cu_seqlens, *vis_start, *vis_len, *text_start, *text_len, *rank_start, *rank_len;
   SampleDesc *desc;          // [B]
   int32_t *out_cu_seqlens;   // [B+1] or nullptr
@@ -95,276 +95,26 @@ __global__ void prepare_kernel(PrepareArgs a) {
 }
 
 // =======================================================================================
-// qsum: qbar[b, c] = sum over visual rows i of q[i, c]   (fp32, fixed summation order)
-// grid (chunks, column blocks, B); a block sums QSUM_ROWS rows of 2048 columns and the block
-// that finishes last for (b, column block) adds the chunk partials in chunk order.
+// mass_kernel: Eq. 1 with the sum over the queries taken first, per head:  s_j^h = qbar^h . k_j^h,  qbar^h = sum of the visual
+// queries of head h.  Persistent blocks, an item is one (sample, head): a copy warp streams the head's visual queries and then
+// its keys, 128 rows a tile, through a ring of shared memory and runs ahead into the next item; eight warps add the query rows up,
+// exchange their sums and multiply the key rows.  A half-warp holds a row of the head (256 bytes).
+//   PER_HEAD   (one salience and one mask per head) heads gets s_j^h / sqrt(d); then Eq. 2 and Eq. 3 of the head, whose
+//              (minimum, 1 / range) stay in `norm` [B, H, 2] for the head means.
+//   otherwise  heads gets the masses as they are, for salience_kernel.  (As the tail of the block that finishes a sample's last
+//              head it held that block's ring up: 31 samples of 611 rows 108 us.)
+// Bound by memory: queries and keys are read once and nothing else of size moves.  Three kernels did this (a query sum with
+// partial rows through memory, masses with all heads of a row per warp, masks; per step, before -> now): 8 x 1536 rows, 32 heads, a
+// mask per head 70 -> 45 us of kernels (4.5 TB/s), the step 206.5 -> 189; 31 x 611 83 -> 70 (5.2 TB/s without the salience), the step
+// 270 -> 252; 3 x 174-186 with 16 heads, a mask per head 49.5 -> 39.7.  The same work with rows held in registers, eight in flight per
+// thread, and a cluster of blocks per item: 59 us on the first (loads, sums and exchanges in turn).
 // =======================================================================================
-constexpr int QSUM_ROWS = 32;
-constexpr int QSUM_THREADS = 256;
-constexpr int QSUM_COLS = QSUM_THREADS * 8;
-
-__global__ void __launch_bounds__(QSUM_THREADS)
-qsum_kernel(const __nv_bfloat16 *__restrict__ q, PrepareArgs pa, int D,
-            int max_chunks, int rows_per_chunk /* a multiple of QSUM_ROWS */, float *__restrict__ partial /*[B, max_chunks, D]*/,
-            float *__restrict__ qbar /*[B, D]*/, unsigned int *__restrict__ counters) {
-  pdl_enter();
-  const int b = blockIdx.z, cb = blockIdx.y, chunk = blockIdx.x;
-  // When this is the first kernel of the step, block (0,0,0) also does the device-side validation
-  // and writes the descriptors every later kernel reads; each block derives its own copy.
-  if (pa.write_desc && blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0 && threadIdx.x < 32) prepare_warp(pa);
-  const SampleDesc d = make_desc(pa, b);
-  if (!d.valid) return;
-  const int nchunks = (d.nv + rows_per_chunk - 1) / rows_per_chunk;
-  if (chunk >= nchunks) return;
-  const int col = cb * QSUM_COLS + threadIdx.x * 8;
-  const bool active = col < D;
-  float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-  if (active) {
-    const int r_lo = chunk * rows_per_chunk;
-    const int r_hi = min(d.nv, r_lo + rows_per_chunk);
-    const uint4 *base =
-        reinterpret_cast<const uint4 *>(q + (size_t)(d.row0 + d.v0) * D + col);
-    const size_t pitch = (size_t)D / 8;
-    int r = r_lo;
-    for (; r + 8 <= r_hi; r += 8) {       // eight independent 16-byte loads in flight per thread
-      uint4 v[8];
-#pragma unroll
-      for (int u = 0; u < 8; ++u) v[u] = __ldg(base + (size_t)(r + u) * pitch);
-#pragma unroll
-      for (int u = 0; u < 8; ++u) {
-        float f[8];
-        unpack8(v[u], f);
-#pragma unroll
-        for (int e = 0; e < 8; ++e) acc[e] += f[e];
-      }
-    }
-    for (; r < r_hi; ++r) {
-      uint4 v = __ldg(base + (size_t)r * pitch);
-      float f[8];
-      unpack8(v, f);
-#pragma unroll
-      for (int e = 0; e < 8; ++e) acc[e] += f[e];
-    }
-    float4 *dst = reinterpret_cast<float4 *>(partial + ((size_t)b * max_chunks + chunk) * D + col);
-    dst[0] = make_float4(acc[0], acc[1], acc[2], acc[3]);
-    dst[1] = make_float4(acc[4], acc[5], acc[6], acc[7]);
-  }
-  // last block for (b, cb) reduces the chunk partials
-  __shared__ int s_last;
-  __threadfence();
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    unsigned int *c = counters + (size_t)b * gridDim.y + cb;
-    unsigned int old = atomicAdd(c, 1u);
-    s_last = (old == (unsigned int)(nchunks - 1));
-    if (s_last) *c = 0u;   // ready for the next call
-  }
-  __syncthreads();
-  if (!s_last || !active) return;
-  __threadfence();
-  float tot[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-#pragma unroll 4
-  for (int c = 0; c < nchunks; ++c) {
-    const float4 *src =
-        reinterpret_cast<const float4 *>(partial + ((size_t)b * max_chunks + c) * D + col);
-    float4 a0 = __ldcg(src), a1 = __ldcg(src + 1);
-    tot[0] += a0.x; tot[1] += a0.y; tot[2] += a0.z; tot[3] += a0.w;
-    tot[4] += a1.x; tot[5] += a1.y; tot[6] += a1.z; tot[7] += a1.w;
-  }
-  float4 *dst = reinterpret_cast<float4 *>(qbar + (size_t)b * D + col);
-  dst[0] = make_float4(tot[0], tot[1], tot[2], tot[3]);
-  dst[1] = make_float4(tot[4], tot[5], tot[6], tot[7]);
-}
-
-// =======================================================================================
-// mass_salience: s_j = qbar . k_j / (H sqrt(d))  (Eq. 1 with the sum over queries taken first
-// and the mean over heads folded in); the block that finishes last for a sample then does the
-// min-max normalisation (Eq. 2) and the mask vector (Eq. 3).
-// grid (row blocks, B); 8 warps x 4 rows each.
-// =======================================================================================
-constexpr int MASS_THREADS = 256;
-constexpr int MASS_ROWS_PER_WARP = 4;                   // (mass_heads deals exactly four rows out over its lanes)
-constexpr int MASS_ROWS = (MASS_THREADS / 32) * MASS_ROWS_PER_WARP;
-
-__global__ void __launch_bounds__(MASS_THREADS)
-mass_salience_kernel(const __nv_bfloat16 *__restrict__ k, const SampleDesc *__restrict__ desc,
-                     int D, int max_vis, float scale, float lambda_max, float eps,
-                     const float *__restrict__ qbar, float *__restrict__ mass,
-                     float *__restrict__ salience, float *__restrict__ mask_log,
-                     float *__restrict__ rank_score, unsigned int *__restrict__ counters) {
-  pdl_enter();
-  extern __shared__ float s_q[];   // [D]
-  __shared__ float s_red[2 * (MASS_THREADS / 32)];
-  __shared__ int s_last;
-  const int b = blockIdx.y;
-  const SampleDesc d = desc[b];
-  float *mass_b = mass + (size_t)b * max_vis;
-  if (!d.valid) {
-    for (int j = blockIdx.x * MASS_THREADS + threadIdx.x; j < max_vis; j += gridDim.x * MASS_THREADS) {
-      mass_b[j] = 0.f; salience[(size_t)b * max_vis + j] = 0.f; mask_log[(size_t)b * max_vis + j] = 0.f;
-      rank_score[(size_t)b * max_vis + j] = 0.f;   // the score kernel skips the sample
-    }
-    return;
-  }
-  const int nblocks = (d.nv + MASS_ROWS - 1) / MASS_ROWS;
-  if ((int)blockIdx.x >= nblocks) return;
-  for (int c = threadIdx.x * 4; c < D; c += MASS_THREADS * 4)
-    *reinterpret_cast<float4 *>(s_q + c) = __ldcg(reinterpret_cast<const float4 *>(qbar + (size_t)b * D + c));
-  __syncthreads();
-
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int j0 = blockIdx.x * MASS_ROWS + warp * MASS_ROWS_PER_WARP;
-  const int nvec = D / 8;
-  float acc[MASS_ROWS_PER_WARP];
-  const uint4 *rowp[MASS_ROWS_PER_WARP];
-#pragma unroll
-  for (int r = 0; r < MASS_ROWS_PER_WARP; ++r) {
-    acc[r] = 0.f;
-    const int j = min(j0 + r, d.nv - 1);   // clamp: duplicates are discarded below
-    rowp[r] = reinterpret_cast<const uint4 *>(k + (size_t)(d.row0 + d.v0 + j) * D);
-  }
-  for (int v0 = lane; v0 < nvec; v0 += 64) {   // two vectors x four rows in flight per lane
-    uint4 kv[2][MASS_ROWS_PER_WARP];
-#pragma unroll
-    for (int t = 0; t < 2; ++t)
-#pragma unroll
-      for (int r = 0; r < MASS_ROWS_PER_WARP; ++r)
-        if (v0 + 32 * t < nvec) kv[t][r] = __ldg(rowp[r] + v0 + 32 * t);
-#pragma unroll
-    for (int t = 0; t < 2; ++t) {
-      const int v = v0 + 32 * t;
-      if (v < nvec) {
-        const float4 qa = *reinterpret_cast<const float4 *>(s_q + v * 8);
-        const float4 qb = *reinterpret_cast<const float4 *>(s_q + v * 8 + 4);
-#pragma unroll
-        for (int r = 0; r < MASS_ROWS_PER_WARP; ++r) {
-          float f[8];
-          unpack8(kv[t][r], f);
-          acc[r] += f[0] * qa.x + f[1] * qa.y + f[2] * qa.z + f[3] * qa.w + f[4] * qb.x + f[5] * qb.y +
-                    f[6] * qb.z + f[7] * qb.w;
-        }
-      }
-    }
-  }
-#pragma unroll
-  for (int r = 0; r < MASS_ROWS_PER_WARP; ++r) {
-    const float tot = warp_sum(acc[r]);
-    if (lane == 0 && j0 + r < d.nv) mass_b[j0 + r] = tot * scale;
-  }
-
-  // ---- last block of the sample: Eq. 2 and Eq. 3 over the whole image span ----
-  __threadfence();
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    unsigned int old = atomicAdd(counters + b, 1u);
-    s_last = (old == (unsigned int)(nblocks - 1));
-    if (s_last) counters[b] = 0u;
-  }
-  __syncthreads();
-  if (!s_last) return;
-  __threadfence();
-  float lo = INFINITY, hi = -INFINITY;
-  for (int j = threadIdx.x; j < d.nv; j += MASS_THREADS) {
-    const float s = __ldcg(mass_b + j);
-    lo = fminf(lo, s); hi = fmaxf(hi, s);
-  }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    lo = fminf(lo, __shfl_xor_sync(0xffffffffu, lo, o));
-    hi = fmaxf(hi, __shfl_xor_sync(0xffffffffu, hi, o));
-  }
-  if (lane == 0) { s_red[warp] = lo; s_red[MASS_THREADS / 32 + warp] = hi; }
-  __syncthreads();
-  lo = s_red[0]; hi = s_red[MASS_THREADS / 32];
-#pragma unroll
-  for (int w = 1; w < MASS_THREADS / 32; ++w) {
-    lo = fminf(lo, s_red[w]); hi = fmaxf(hi, s_red[MASS_THREADS / 32 + w]);
-  }
-  const float inv = 1.0f / ((hi - lo) + eps);
-  float *sal_b = salience + (size_t)b * max_vis, *msk_b = mask_log + (size_t)b * max_vis;
-  for (int j = threadIdx.x; j < max_vis; j += MASS_THREADS) {
-    if (j < d.nv) {
-      const float sh = (__ldcg(mass_b + j) - lo) * inv;
-      sal_b[j] = sh;
-      msk_b[j] = logf(fmaxf(lambda_max * sh, eps));
-    } else {
-      mass_b[j] = 0.f; sal_b[j] = 0.f; msk_b[j] = 0.f;
-    }
-  }
-}
-
-// =======================================================================================
-// mass_heads: Eq. 1 kept per head (the variant with one salience and one mask per head).
-//   s_j^h = qbar^h . k_j^h / sqrt(d): one warp per visual key row; a 16-byte vector of the row lies
-//   inside one head (16 vectors per head), so the two halves of the warp reduce two heads per pass.
-// grid (row blocks, B); 8 warps x 4 rows each.  s_heads: scratch [B, H, max_vis].  Dynamic shared memory: D floats.
-// mask_heads: one block per (head, sample): the min-max normalisation (Eq. 2) and the mask vector (Eq. 3) of that head; the
-// head's (minimum, 1 / range) stay in `norm` [B, H, 2] for the head means.
-// salience_heads_block: one block per sample: mass = mean_h s^h (equal to the default mass), salience =
-// mean_h s_hat^h (the Eq. 5 weight), mask_log = Eq. 3 of that mean.
-// (One block per sample did all of this at the end of mass_heads: 8 sequences x 1536 tokens x 32 heads 81 -> 40 us, the step 277 -> 226.
-// The mass kernel itself waits for memory: the next vectors are on their way while these are reduced, 29.0 -> 26.4 us, the step 223.6 -> 218.4.)
-// =======================================================================================
-__global__ void __launch_bounds__(MASS_THREADS)
-mass_heads_kernel(const __nv_bfloat16 *__restrict__ k, const SampleDesc *__restrict__ desc, int D, int H,
-                  int max_vis, float scale, const float *__restrict__ qbar, float *__restrict__ s_heads) {
-  pdl_enter();
-  extern __shared__ float s_q[];   // [D]
-  const int b = blockIdx.y;
-  const SampleDesc d = desc[b];
-  float *sh_b = s_heads + (size_t)b * H * max_vis;
-  if (!d.valid) return;
-  const int nblocks = (d.nv + MASS_ROWS - 1) / MASS_ROWS;
-  if ((int)blockIdx.x >= nblocks) return;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int j0 = blockIdx.x * MASS_ROWS + warp * MASS_ROWS_PER_WARP;
-  const int nvec = D / 8;
-  const uint4 *rowp[MASS_ROWS_PER_WARP];
-#pragma unroll
-  for (int r = 0; r < MASS_ROWS_PER_WARP; ++r) {
-    const int j = min(j0 + r, d.nv - 1);   // clamp: duplicates are discarded below
-    rowp[r] = reinterpret_cast<const uint4 *>(k + (size_t)(d.row0 + d.v0 + j) * D);
-  }
-  uint4 kv[MASS_ROWS_PER_WARP], next[MASS_ROWS_PER_WARP];
-#pragma unroll
-  for (int r = 0; r < MASS_ROWS_PER_WARP; ++r)
-    if (lane < nvec) kv[r] = __ldg(rowp[r] + lane);
-  for (int c = threadIdx.x * 4; c < D; c += MASS_THREADS * 4)
-    *reinterpret_cast<float4 *>(s_q + c) = __ldcg(reinterpret_cast<const float4 *>(qbar + (size_t)b * D + c));
-  __syncthreads();
-  const bool up8 = lane & 8, up4 = lane & 4;
-  const int r_out = (up8 ? 2 : 0) + (up4 ? 1 : 0);   // the row whose sum this lane ends with
-  for (int v0 = 0; v0 < nvec; v0 += 32) {      // one pass = 32 vectors = two heads
-    const int v = v0 + lane;
-#pragma unroll
-    for (int r = 0; r < MASS_ROWS_PER_WARP; ++r)
-      if (v + 32 < nvec) next[r] = __ldg(rowp[r] + v + 32);
-    const int h = (v0 >> 4) + (lane >> 4);      // head of this half of the warp
-    float part[MASS_ROWS_PER_WARP] = {0.f, 0.f, 0.f, 0.f};
-    if (v < nvec) {
-      const float4 qa = *reinterpret_cast<const float4 *>(s_q + v * 8);
-      const float4 qb = *reinterpret_cast<const float4 *>(s_q + v * 8 + 4);
-#pragma unroll
-      for (int r = 0; r < MASS_ROWS_PER_WARP; ++r) {
-        float f[8];
-        unpack8(kv[r], f);
-        part[r] = f[0] * qa.x + f[1] * qa.y + f[2] * qa.z + f[3] * qa.w + f[4] * qb.x + f[5] * qb.y + f[6] * qb.z +
-                  f[7] * qb.w;
-      }
-    }
-    // sums over 16 lanes, the rows dealt out on the way: five shuffles for four rows instead of sixteen
-    float s0 = up8 ? part[2] : part[0], s1 = up8 ? part[3] : part[1];
-    s0 += __shfl_xor_sync(0xffffffffu, up8 ? part[0] : part[2], 8);
-    s1 += __shfl_xor_sync(0xffffffffu, up8 ? part[1] : part[3], 8);
-    float sum = up4 ? s1 : s0;
-    sum += __shfl_xor_sync(0xffffffffu, up4 ? s0 : s1, 4);
-    sum += __shfl_xor_sync(0xffffffffu, sum, 2);
-    sum += __shfl_xor_sync(0xffffffffu, sum, 1);
-    if ((lane & 3) == 0 && h < H && j0 + r_out < d.nv) sh_b[(size_t)h * max_vis + j0 + r_out] = sum * scale;
-#pragma unroll
-    for (int r = 0; r < MASS_ROWS_PER_WARP; ++r) kv[r] = next[r];
-  }
-}
+constexpr int MASS_THREADS = 288;                // copy warp, eight adding warps
+constexpr int MASS_ADDERS = 256;
+constexpr int MASS_STAGES = 5;                   // (with the rest below the 195 KB that the neighbouring kernels use)
+constexpr int MASS_TILE_BYTES = 2 * 128 * 128;   // 128 rows x 128 bf16 as two 64-column blocks
+constexpr int MASS_SMEM_BYTES = MASS_STAGES * MASS_TILE_BYTES + 1024;
+constexpr long long MASS_WAIT_LIMIT = 1500000000LL;   // clock cycles, roughly one second
 
 struct SalienceArgs {
   int H;
@@ -375,45 +125,53 @@ struct SalienceArgs {
   float *mass, *salience, *mask_log, *rank_score;   // [B, max_vis]
 };
 
-__global__ void __launch_bounds__(MASS_THREADS)
-mask_heads_kernel(const SampleDesc *__restrict__ desc, int H, int max_vis, float lambda_max, float eps,
-                  const float *__restrict__ s_heads, float *__restrict__ mask_log_heads, float *__restrict__ norm) {
-  pdl_enter();
-  __shared__ float s_red[2 * (MASS_THREADS / 32)];
-  const int h = blockIdx.x, b = blockIdx.y;
-  const SampleDesc d = desc[b];
-  float *mh = mask_log_heads + ((size_t)b * H + h) * max_vis;
-  if (!d.valid) {
-    for (int j = threadIdx.x; j < max_vis; j += MASS_THREADS) mh[j] = 0.f;
-    return;
-  }
-  const float *sh = s_heads + ((size_t)b * H + h) * max_vis;
-  float lo = INFINITY, hi = -INFINITY;
-  for (int j = threadIdx.x; j < d.nv; j += MASS_THREADS) {
-    const float s = __ldcg(sh + j);
-    lo = fminf(lo, s); hi = fmaxf(hi, s);
-  }
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+struct MassArgs {
+  PrepareArgs pa;            // write_desc: the first block validates the batch and writes the descriptors
+  int max_vis;
+  float scale;               // of `heads`
+  float *heads;              // [B, H, max_vis]
+  float *mask_log_heads;     // PER_HEAD: [B, H, max_vis]
+  float *norm;               // PER_HEAD: [B, H, 2]
+  int H;
+  float lambda_max, eps;
+  uint32_t *status;
+  long long wait_limit;
+};
+
+// barrier of the adding warps alone
+__device__ __forceinline__ void mass_bar() { asm volatile("bar.sync 1, 256;" ::: "memory"); }
+
+// The masses' own sums over the heads: sixteen in pairs, the sixteens and the scale in 64 bits.  One after the other in 32 bits, 32
+// heads lose more than the masses themselves do (error against 64 bits 9.3e-8 instead of 5.0e-8 with their exact sum).
+template <int N>
+__device__ __forceinline__ float pair_sum(float (&v)[N]) {
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    lo = fminf(lo, __shfl_xor_sync(0xffffffffu, lo, o));
-    hi = fmaxf(hi, __shfl_xor_sync(0xffffffffu, hi, o));
-  }
-  if (lane == 0) { s_red[warp] = lo; s_red[MASS_THREADS / 32 + warp] = hi; }
-  __syncthreads();
+  for (int o = 1; o < N; o <<= 1)
 #pragma unroll
-  for (int w = 0; w < MASS_THREADS / 32; ++w) {
-    lo = fminf(lo, s_red[w]); hi = fmaxf(hi, s_red[MASS_THREADS / 32 + w]);
-  }
-  const float inv = 1.0f / ((hi - lo) + eps);
-  if (threadIdx.x == 0) {
-    norm[((size_t)b * H + h) * 2] = lo;
-    norm[((size_t)b * H + h) * 2 + 1] = inv;
-  }
-  for (int j = threadIdx.x; j < max_vis; j += MASS_THREADS)
-    mh[j] = j < d.nv ? logf(fmaxf(lambda_max * ((__ldcg(sh + j) - lo) * inv), eps)) : 0.f;
+    for (int e = 0; e < N; e += 2 * o) v[e] += v[e + o];
+  return v[0];
 }
 
+// Column j of `p` [H, max_vis]: the sum over the heads, scaled.
+__device__ __forceinline__ float head_total(const float *p, int H, int max_vis, double scale) {
+  double sum = 0.0;
+  int hh = 0;
+  for (; hh + 16 <= H; hh += 16) {          // sixteen loads in flight
+    float v[16];
+#pragma unroll
+    for (int e = 0; e < 16; ++e) v[e] = __ldcg(p + (size_t)(hh + e) * max_vis);
+    sum += (double)pair_sum(v);
+  }
+  if (hh < H) {
+    float v[16];
+#pragma unroll
+    for (int e = 0; e < 16; ++e) v[e] = hh + e < H ? __ldcg(p + (size_t)(hh + e) * max_vis) : 0.f;
+    sum += (double)pair_sum(v);
+  }
+  return (float)(sum * scale);
+}
+// salience_heads_block: one block per sample: mass = mean_h s^h (equal to the default mass), salience =
+// mean_h s_hat^h (the Eq. 5 weight), mask_log = Eq. 3 of that mean.
 __device__ __forceinline__ void salience_heads_block(const SampleDesc &d, int b, int max_vis, const SalienceArgs &a) {
   float *mass_b = a.mass + (size_t)b * max_vis, *sal_b = a.salience + (size_t)b * max_vis, *msk_b = a.mask_log + (size_t)b * max_vis;
   const float *sh_b = a.heads + (size_t)b * a.H * max_vis, *norm = a.norm + (size_t)b * a.H * 2;
@@ -456,7 +214,7 @@ salience_heads_kernel(const SampleDesc *__restrict__ desc, int max_vis, Salience
 // salience_block: the tail of Eq. 1 and Eq. 2-3 when the per-head masses qbar^h . k_j^h were
 // produced by the score kernel (from the query and key tiles it streams).  One block per sample, beside
 // the block that selects (grid y of the selection launch): s_j = scale * sum_h heads[b, h, j], then the min-max normalisation and
-// the mask vector over the image span; padding past the span is zeroed as mass_salience does.
+// the mask vector over the image span; padding past the span is zeroed.
 // =======================================================================================
 constexpr int SAL_THREADS = 1024;
 
@@ -478,17 +236,6 @@ __device__ __forceinline__ float4 head_sum4(const float *p, int H, int max_vis) 
     t.x += v.x; t.y += v.y; t.z += v.z; t.w += v.w;
   }
   return t;
-}
-
-// The masses' own sums over the heads: sixteen in pairs, the sixteens and the scale in 64 bits.  One after the other in 32 bits, 32
-// heads lose more than the masses themselves do (error against 64 bits 9.3e-8 instead of 5.0e-8 with their exact sum).
-template <int N>
-__device__ __forceinline__ float pair_sum(float (&v)[N]) {
-#pragma unroll
-  for (int o = 1; o < N; o <<= 1)
-#pragma unroll
-    for (int e = 0; e < N; e += 2 * o) v[e] += v[e + o];
-  return v[0];
 }
 
 __device__ __forceinline__ void salience_block(const SampleDesc &d, int b, int max_vis, const SalienceArgs &a) {
@@ -529,21 +276,7 @@ __device__ __forceinline__ void salience_block(const SampleDesc &d, int b, int m
     }
   }
   for (int j = vec ? d.nv : (int)threadIdx.x; j < d.nv; j += SAL_THREADS) {
-    double sum = 0.0;
-    int hh = 0;
-    for (; hh + 16 <= H; hh += 16) {          // sixteen loads in flight
-      float v[16];
-#pragma unroll
-      for (int e = 0; e < 16; ++e) v[e] = __ldcg(hb + (size_t)(hh + e) * max_vis + j);
-      sum += (double)pair_sum(v);
-    }
-    if (hh < H) {
-      float v[16];
-#pragma unroll
-      for (int e = 0; e < 16; ++e) v[e] = hh + e < H ? __ldcg(hb + (size_t)(hh + e) * max_vis + j) : 0.f;
-      sum += (double)pair_sum(v);
-    }
-    const float tot = (float)(sum * a.scale);
+    const float tot = head_total(hb + j, H, max_vis, a.scale);
     mass_b[j] = tot;
     lo = fminf(lo, tot); hi = fmaxf(hi, tot);
   }
@@ -568,6 +301,181 @@ __device__ __forceinline__ void salience_block(const SampleDesc &d, int b, int m
       msk_b[j] = logf(fmaxf(lambda_max * sh, eps));
     } else {
       mass_b[j] = 0.f; sal_b[j] = 0.f; msk_b[j] = 0.f;
+    }
+  }
+}
+
+// one block per sample, where the score kernel needs the mask vector (ranking rows in the image span)
+__global__ void __launch_bounds__(SAL_THREADS)
+salience_kernel(const SampleDesc *__restrict__ desc, int max_vis, SalienceArgs a) {
+  pdl_enter();
+  salience_block(desc[blockIdx.x], blockIdx.x, max_vis, a);
+}
+
+template <bool PER_HEAD>
+__global__ void __launch_bounds__(MASS_THREADS, 1)
+mass_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__ CUtensorMap tmap_k, MassArgs a) {
+  extern __shared__ __align__(1024) uint8_t m_smem[];
+  __shared__ uint64_t s_full[MASS_STAGES], s_empty[MASS_STAGES];
+  __shared__ float s_part[MASS_ADDERS / 32][128], s_sum[128], s_red[2 * (MASS_ADDERS / 32)];
+  __shared__ int s_abort;
+  const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
+  const uint32_t base = (smem_u32(m_smem) + 1023u) & ~1023u;
+  const uint8_t *tiles = m_smem + (base - smem_u32(m_smem));
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < MASS_STAGES; ++s) {
+      mbar_init(smem_u32(&s_full[s]), 1);
+      mbar_init(smem_u32(&s_empty[s]), MASS_ADDERS / 32);
+    }
+    s_abort = 0;
+    fence_barrier_init();
+  }
+  __syncthreads();
+  pdl_enter();
+  if (threadIdx.x == 0 && (*reinterpret_cast<volatile uint32_t *>(a.status) & STATUS_MASS_TIMEOUT)) s_abort = 1;
+  __syncthreads();
+  WaitCtx wc{&s_abort, a.status, STATUS_MASS_TIMEOUT, a.wait_limit};
+  const int H = a.H, n_items = a.pa.B * H;
+  if (warp == 0) {
+    // ---- copies (converged, see tma_load_2d_w)
+    const uint32_t leader = warp_leader();
+    const uint64_t keep = l2_evict_normal(), drop = l2_evict_first();     // (the score kernel comes for the keys)
+    if (leader) {
+      tma_prefetch_desc(&tmap_q);
+      tma_prefetch_desc(&tmap_k);
+    }
+    RingPos r;
+    int issued = 0;
+    for (int item = blockIdx.x; item < n_items; item += gridDim.x) {
+      const int b = item / H, h = item - b * H;
+      const SampleDesc d = make_desc(a.pa, b);
+      const int n = d.valid ? (d.nv + 127) / 128 : 0;
+      int u = 0;
+      for (; u < 2 * n; ++u) {
+        if (issued >= MASS_STAGES) mbar_wait_warp(smem_u32(&s_empty[r.slot]), r.phase ^ 1u, wc);
+        if (__shfl_sync(0xffffffffu, s_abort, 0)) break;
+        const uint32_t bar = smem_u32(&s_full[r.slot]), dst = base + r.slot * MASS_TILE_BYTES;
+        const int row = d.row0 + d.v0 + (u < n ? u : u - n) * 128;
+        const CUtensorMap *map = u < n ? &tmap_q : &tmap_k;
+        mbar_expect_tx_w(bar, MASS_TILE_BYTES, leader);
+        tma_load_2d_hint_w(dst, map, bar, h * 128, row, u < n ? drop : keep, leader);
+        tma_load_2d_hint_w(dst + MASS_TILE_BYTES / 2, map, bar, h * 128 + 64, row, u < n ? drop : keep, leader);
+        ++issued;
+        r.step(MASS_STAGES);
+      }
+      if (u < 2 * n) break;
+    }
+    for (int s = 0; s < MASS_STAGES; ++s)                 // every copy has landed before the block may leave
+      if (issued > s) mbar_wait_drain(smem_u32(&s_full[s]), ((issued - 1 - s) / MASS_STAGES) & 1, MASS_WAIT_LIMIT);
+    __syncwarp();
+    return;
+  }
+  const int tid = threadIdx.x - 32, aw = warp - 1;        // among the adding warps
+  if (a.pa.write_desc && blockIdx.x == 0 && aw == 0) prepare_warp(a.pa);
+  const int c = lane & 15, row0 = (tid >> 4) * 8;         // this thread's 16-byte chunk of the head, its half-warp's eight rows of a tile
+  const bool up8 = lane & 8, up4 = lane & 4, up2 = lane & 2;
+  RingPos r;
+  for (int item = blockIdx.x; item < n_items; item += gridDim.x) {
+    const int b = item / H, h = item - b * H;
+    const SampleDesc d = make_desc(a.pa, b);
+    float *mh = PER_HEAD ? a.mask_log_heads + (size_t)item * a.max_vis : nullptr;
+    float *out = a.heads + (size_t)item * a.max_vis;
+    if (!d.valid) {
+      if (PER_HEAD)
+        for (int j = tid; j < a.max_vis; j += MASS_ADDERS) mh[j] = 0.f;
+      continue;
+    }
+    const int n = (d.nv + 127) / 128;
+    auto chunk = [&](int row) {                            // (row r of a block: its chunk c at position c ^ (r & 7))
+      return *reinterpret_cast<const uint4 *>(tiles + r.slot * MASS_TILE_BYTES + (c >> 3) * (MASS_TILE_BYTES / 2) + row * 128 + (((c & 7) ^ (row & 7)) << 4));
+    };
+    auto release = [&]() {
+      __syncwarp();
+      if (lane == 0) mbar_arrive(smem_u32(&s_empty[r.slot]));
+      r.step(MASS_STAGES);
+    };
+    // ---- the queries' sum
+    uint64_t acc[4] = {0ull, 0ull, 0ull, 0ull};
+    for (int u = 0; u < n; ++u) {
+      mbar_wait(smem_u32(&s_full[r.slot]), r.phase, wc);
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        uint4 x = chunk(row0 + i);
+        if (u * 128 + row0 + i >= d.nv) x = make_uint4(0u, 0u, 0u, 0u);
+        acc[0] = f2_add(acc[0], f2_pack(bf16_lo(x.x), bf16_hi(x.x)));
+        acc[1] = f2_add(acc[1], f2_pack(bf16_lo(x.y), bf16_hi(x.y)));
+        acc[2] = f2_add(acc[2], f2_pack(bf16_lo(x.z), bf16_hi(x.z)));
+        acc[3] = f2_add(acc[3], f2_pack(bf16_lo(x.w), bf16_hi(x.w)));
+      }
+      release();
+    }
+    float f[8];
+#pragma unroll
+    for (int e = 0; e < 4; ++e) f2_unpack(acc[e], f[2 * e], f[2 * e + 1]);
+#pragma unroll
+    for (int e = 0; e < 8; ++e) f[e] += __shfl_xor_sync(0xffffffffu, f[e], 16);
+    if (lane < 16) {
+#pragma unroll
+      for (int e = 0; e < 8; ++e) s_part[aw][c * 8 + e] = f[e];
+    }
+    mass_bar();
+    if (tid < 128) {
+      float t = 0.f;
+#pragma unroll
+      for (int w = 0; w < MASS_ADDERS / 32; ++w) t += s_part[w][tid];
+      s_sum[tid] = t;
+    }
+    mass_bar();
+    float qs[8];
+#pragma unroll
+    for (int e = 0; e < 8; ++e) qs[e] = s_sum[c * 8 + e];
+    // ---- the keys
+    float lo = INFINITY, hi = -INFINITY;
+    for (int u = 0; u < n; ++u) {
+      mbar_wait(smem_u32(&s_full[r.slot]), r.phase, wc);
+      float s[8];
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        float g[8];
+        unpack8(chunk(row0 + i), g);
+        s[i] = (g[0] * qs[0] + g[1] * qs[1] + g[2] * qs[2] + g[3] * qs[3]) + (g[4] * qs[4] + g[5] * qs[5] + g[6] * qs[6] + g[7] * qs[7]);
+      }
+      release();
+      // sums over 16 lanes, the rows dealt out on the way: eight shuffles for eight rows
+#pragma unroll
+      for (int i = 0; i < 4; ++i) s[i] = (up8 ? s[4 + i] : s[i]) + __shfl_xor_sync(0xffffffffu, up8 ? s[i] : s[4 + i], 8);
+#pragma unroll
+      for (int i = 0; i < 2; ++i) s[i] = (up4 ? s[2 + i] : s[i]) + __shfl_xor_sync(0xffffffffu, up4 ? s[i] : s[2 + i], 4);
+      float t = (up2 ? s[1] : s[0]) + __shfl_xor_sync(0xffffffffu, up2 ? s[0] : s[1], 2);
+      t += __shfl_xor_sync(0xffffffffu, t, 1);
+      const int j = u * 128 + row0 + (up8 ? 4 : 0) + (up4 ? 2 : 0) + (up2 ? 1 : 0);
+      if (j < d.nv) {
+        t *= a.scale;
+        if (!(lane & 1)) out[j] = t;
+        lo = fminf(lo, t); hi = fmaxf(hi, t);
+      }
+    }
+    if (PER_HEAD) {
+      // ---- Eq. 2 and Eq. 3 of the head
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) {
+        lo = fminf(lo, __shfl_xor_sync(0xffffffffu, lo, o));
+        hi = fmaxf(hi, __shfl_xor_sync(0xffffffffu, hi, o));
+      }
+      if (lane == 0) { s_red[aw] = lo; s_red[MASS_ADDERS / 32 + aw] = hi; }
+      mass_bar();
+#pragma unroll
+      for (int w = 0; w < MASS_ADDERS / 32; ++w) {
+        lo = fminf(lo, s_red[w]); hi = fmaxf(hi, s_red[MASS_ADDERS / 32 + w]);
+      }
+      const float inv = 1.0f / ((hi - lo) + a.eps);
+      if (tid == 0) {
+        a.norm[(size_t)item * 2] = lo;
+        a.norm[(size_t)item * 2 + 1] = inv;
+      }
+      for (int j = tid; j < a.max_vis; j += MASS_ADDERS)
+        mh[j] = j < d.nv ? logf(fmaxf(a.lambda_max * ((out[j] - lo) * inv), a.eps)) : 0.f;
+      // (two barriers come before s_red is written again)
     }
   }
 }

@@ -150,6 +150,21 @@ def test_row_norms_shared_by_the_groups(ctx, k, H):
     run_step(ctx, batch, A.Params(keep_k=k))
 
 
+@pytest.mark.parametrize("per_head", [False, True], ids=["mean", "heads"])
+@pytest.mark.parametrize("nvs,H", [([127, 128, 129, 641], 2), ([40, 300, 90, 256] * 10, 4)], ids=["tile_edges", "many_items_per_block"])
+def test_masses_with_visual_ranking_rows(nvs, H, per_head):
+    """The mass kernel streams a head's queries, then its keys, 128 rows a tile: spans that end on a tile edge and beside it, and more
+    (sequence, head) items than blocks, so that the ring runs on from one item to the next."""
+    B = len(nvs)
+    batch = W.tiny(B=B, n_vis=nvs, text_lens=[5 + b % 7 for b in range(B)], H=H, keep_k=24, seed=350 + B, centres=6)
+    big = A.asap_init(0, max_total_tokens=batch.total + B * 641, max_B=B, max_H=H, max_D=H * 128)
+    try:
+        run_step(big, batch, A.Params(keep_k=24, per_head_mask=per_head, lambda_max=0.7), batch.text_start - 9, batch.text_len + 9,
+                 samples=range(B) if B < 5 else [0, 1, 2, B - 2, B - 1])
+    finally:
+        A.asap_free(big)
+
+
 def test_many_row_tiles_and_three_slot_tiles(ctx):
     """A batch large enough that the similarity kernel runs unsliced with more blocks than SMs
     (15 sequences x 19 row tiles) and three slot tiles (600 kept slots).  Odd and even numbers of row

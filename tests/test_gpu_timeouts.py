@@ -49,6 +49,25 @@ def test_score_kernel_gives_up_and_the_context_recovers(ctx):
     _same(good, again, ("rank_score", "keep_idx", "drop_idx", "assign", "out_hidden", "out_pos", "src_row", "out_cu_seqlens"))
 
 
+@pytest.mark.parametrize("per_head", [False, True], ids=["mean", "heads"])
+def test_mass_kernel_gives_up_and_the_context_recovers(ctx, per_head):
+    batch = W.tiny(B=3, n_vis=[300, 260, 140], text_lens=[20, 150, 7], H=2, keep_k=40, seed=611, centres=6)
+    inp = A.make_inputs(batch, DEV, batch.text_start - 3, batch.text_len + 3)
+    p = A.Params(keep_k=40, per_head_mask=per_head)
+    outs = [A.alloc_outputs(inp, 40, fill=True, per_head=per_head) for _ in range(3)]
+    A.asap_prune_step(ctx, inp, p, outs[0])
+    torch.cuda.synchronize(); A.asap_check(ctx)
+    A.asap_debug_wait_limit(ctx, 1)
+    A.asap_prune_step(ctx, inp, p, outs[1])          # returns normally; its results are void
+    torch.cuda.synchronize()
+    with pytest.raises(A.AsapError) as e:
+        A.asap_check(ctx)
+    assert e.value.status == -6 and "timed out in the mass kernel" in str(e.value)
+    A.asap_prune_step(ctx, inp, p, outs[2])
+    torch.cuda.synchronize(); A.asap_check(ctx)
+    _same(outs[0], outs[2], ("mass", "salience", "rank_score", "keep_idx", "drop_idx", "assign", "out_hidden", "out_pos", "src_row", "out_cu_seqlens"))
+
+
 def test_similarity_kernel_gives_up_and_the_context_recovers(ctx):
     batch = W.tiny(B=2, n_vis=[400, 330], text_lens=[9, 12], H=2, keep_k=150, seed=602, centres=9)
     inp = A.make_inputs(batch, DEV)
