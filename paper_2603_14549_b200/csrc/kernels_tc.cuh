@@ -294,15 +294,17 @@ score_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__
       const int n_rp = (d.nr + pair_rows - 1) / pair_rows;
       for (int rp = 0; rp < n_rp; ++rp, ++qc) {
         const RowPair T = score_row_pair(d, rp, a.mask_enable, pair_rows);
-        if (qc >= 1) mbar_wait_warp(smem_u32(&bk->q_empty), (qc - 1) & 1, wc);
-        if (!__shfl_sync(0xffffffffu, bk->abort_flag, 0)) {
-          mbar_expect_tx_w(smem_u32(&bk->q_full), T.nrt * SC_TILE_BYTES, leader);
-          for (int hf = 0; hf < 2; ++hf)
-            for (int rt = 0; rt < T.nrt; ++rt)
-              tma_load_2d_w(q_smem + hf * SC_Q_HALF_BYTES + rt * SC_HALF_BYTES, &tmap_q, smem_u32(&bk->q_full),
-                            h * 128 + hf * 64, d.row0 + T.R0 + rt * 128, leader);
-          q_issued = qc + 1;
-        }
+        auto load_queries = [&]() {
+          if (qc >= 1) mbar_wait_warp(smem_u32(&bk->q_empty), (qc - 1) & 1, wc);
+          if (!__shfl_sync(0xffffffffu, bk->abort_flag, 0)) {
+            mbar_expect_tx_w(smem_u32(&bk->q_full), T.nrt * SC_TILE_BYTES, leader);
+            for (int hf = 0; hf < 2; ++hf)
+              for (int rt = 0; rt < T.nrt; ++rt)
+                tma_load_2d_w(q_smem + hf * SC_Q_HALF_BYTES + rt * SC_HALF_BYTES, &tmap_q, smem_u32(&bk->q_full),
+                              h * 128 + hf * 64, d.row0 + T.R0 + rt * 128, leader);
+            q_issued = qc + 1;
+          }
+        };
         const int nq = with_mass && rp == 0 ? (d.nv + 127) / 128 : 0;      // tiles of visual queries (never more than n_kt)
         // A query tile lands on a barrier of its own (alternating: the sum warps see only these, in order, so they cannot
         // mistake a ring slot's phase; two query tiles are never in flight on the same one, see below) and its slot's
@@ -326,7 +328,12 @@ score_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__
           }
           ++kc;
         };
+        // The pair's queries overwrite the last pair's, whose MMAs must have ended; the ring's tiles only wait for their slots.
+        // Two key tiles and what follows them go first, no more: four tiles find a slot without these queries' products (16 x 576
+        // 110.2 -> 108.9 us, 8 x 1536 with a mask per head 189.7 -> 188.1, score of 64 x 2880 986 -> 966).  A block's first pair waits for nothing.
+        const int q_at = qc == 0 ? 0 : min(2, T.n_kt + T.n_p2 - 1);
         for (int u = 0; u < T.n_kt + T.n_p2; ++u) {
+          if (u == q_at) load_queries();
           load_tile(false, T.past && u == T.n_kt - 1, d.row0 + (u < T.n_kt ? u : T.t_hi - (u - T.n_kt)) * 128, u < T.n_kt ? keep : drop);
           // (query tiles are two ring positions apart, so the one after the next takes the slot of this one, whose
           // release says that it has been added up; between two items at least four other tiles pass)
