@@ -863,8 +863,8 @@ head_sum_kernel(const SampleDesc *__restrict__ desc, int H, int max_vis,
 //                   products and partial squared norms; the block that finishes last for the
 //                   row tile adds the slices in slice order and does the same epilogue.
 // Rows past the last dropped token (the ragged tail of the last tile) repeat that token and are
-// not written.  The block that finishes a sample's last row tile groups the dropped tokens by
-// destination.
+// not written.  The thread that assigns a token sets its bit in the slot's row of member bits (a.member_bits), or, where
+// those have no room, the block that finishes a sample's last row tile groups the dropped tokens by destination.
 //   one pass:       (a.wide, gathered rows, or up to 384 slots of a batch too large for sim_pair_kernel) the accumulators of
 //                   all slot tiles are live at once and a stage is one 64-column block of the rows
 //                   plus the matching block of EVERY slot tile, so the visual rows are read from
@@ -896,7 +896,7 @@ constexpr int SIM_B_STAGES = 4;
 struct SimArgs {
   const SampleDesc *desc;
   int D, max_vis, keep_k, n_tile, n_nt, stages, splits, max_mt;
-  int a_stages;              // gathered form: slots of the row ring (`stages` counts those of the kept-row ring)
+  int a_stages;              // gathered form and pair kernel: slots of the row ring (`stages` counts those of the kept-row ring)
   int wide;                  // 1: one pass, all slot tiles' accumulators live at once
   int groups;                // > 1: slot tiles dealt to `groups` blocks per row tile (n_nt counts one group's tiles)
   int cluster;               // 1: the `splits` slices of a row tile form a thread-block cluster (grid z) and add their
@@ -1571,7 +1571,7 @@ sim_kernel(const __grid_constant__ CUtensorMap tmap_h, const __grid_constant__ C
   if (a.smat) return;
   if (!a.seg || (!bk->is_last && (a.splits > 1 || a.groups > 1))) return;   // (or a slice / group that did not finalize its row tile)
   __syncthreads();
-  // the block that finishes the sample's last row tile groups the dropped tokens by destination
+  // (no member bits) the block that finishes the sample's last row tile groups the dropped tokens by destination
   if (threadIdx.x == 0) {
     __threadfence();
     const unsigned int n_mt = (unsigned int)((n_rows + 127) / 128);
@@ -1606,7 +1606,7 @@ sim_kernel(const __grid_constant__ CUtensorMap tmap_h, const __grid_constant__ C
 // publishes its rows' best (value, slot) and that sum (one ring, and all the squares in group 0: 8 x 2304 with 320 kept 58 -> 49.5
 // us, 8 x 1536 with 340 56 -> 49, 12 x 577-2881 with 145 56.5 -> 50, 64 x 2880 793 -> 775); the block that finishes a pair last takes the maximum over the
 // groups (lowest slot among equals), looks up which rows were dropped and writes their assignment.
-// The block that finishes a sample's last pair groups the dropped tokens by destination.
+// The assignment leaves as member bits or a grouping, as in sim_kernel.
 // Matrix mode (a.smat set): the row operand is the dense kept-row array too (`tmap_h` maps it with a 128-row box)
 // and every block writes its 256 x n_tile piece of the sample's keep_k x keep_k cosine matrix; nothing else.  The matrix is
 // symmetric: blocks that lie below the diagonal as a whole leave, and the blocks of the mirrored places write their pieces too
