@@ -5,7 +5,7 @@
 //   select         stable radix top-k of the ranking scores           (Fig. 3)
 //   role_map       kept slot / dropped position of every visual token
 //   kept_gather    kept rows gathered for the similarity GEMM, with their inverse norms (Sec. 4.2)
-//   csr_block      dropped tokens grouped by destination slot (tail of the similarity kernel)
+//   csr_block      dropped tokens grouped by destination slot (tail of the similarity kernel where member bits have no room)
 //   route          Sec. 4.2 inside the kept set, from the bit matrix of similar pairs
 //   merge_compact  Eq. 5 and the hand-off of Fig. 3
 //   gather_rows    KV-cache compaction with the row map of the hand-off
@@ -307,9 +307,12 @@ __device__ __forceinline__ void salience_block(const SampleDesc &d, int b, int m
 
 // one block per sample, where the score kernel needs the mask vector (ranking rows in the image span)
 __global__ void __launch_bounds__(SAL_THREADS)
-salience_kernel(const SampleDesc *__restrict__ desc, int max_vis, SalienceArgs a) {
+salience_kernel(const SampleDesc *desc, int max_vis, SalienceArgs a) {
   pdl_enter();
-  salience_block(desc[blockIdx.x], blockIdx.x, max_vis, a);
+  SampleDesc d = {};                       // (the directly preceding kernel wrote the descriptors)
+  d.nv = ld_prev(&desc[blockIdx.x].nv);
+  d.valid = ld_prev(&desc[blockIdx.x].valid);
+  salience_block(d, blockIdx.x, max_vis, a);
 }
 
 template <bool PER_HEAD>
@@ -795,7 +798,7 @@ kept_gather_kernel(const __nv_bfloat16 *__restrict__ hidden, const SampleDesc *_
 // =======================================================================================
 // csr_block: group the dropped tokens of one sample by destination slot (counting sort, stable
 // in dropped order so the merge adds its members in a fixed order).  Run by one whole block of W
-// warps (six, or ten in the gathered and the two-row-tile forms): warp w owns the w-th contiguous
+// warps (six, ten in the gathered and eleven in the two-row-tile form): warp w owns the w-th contiguous
 // chunk of dropped positions, counts its chunk into its own histogram, and after a scan over (slot,
 // warp) writes its chunk's positions behind those of the warps before it.  s_cnt needs (W + 1) * keep_k ints, s_scan 33 ints.
 // seg [B, keep_k+1], members [B, max_vis-keep_k] (dropped POSITIONS, ascending inside a slot).
@@ -1389,11 +1392,10 @@ route_kernel(RouteArgs a) {
 }
 
 // =======================================================================================
-// merge_compact: grid (keep_k + copy-row groups, B).
-//   blockIdx.x <  keep_k : the block owns one kept visual row.  Its members (the dropped tokens
-//                          assigned to that slot) are first listed in shared memory with their
-//                          weights, then their rows are streamed four at a time and accumulated
-//                          in fp32 in CSR order:  (s_hat_i h_i + sum_j s_hat_j h_j) / (s_hat_i +
+// merge_compact: grid (keep_k, or an eighth of it, + copy-row groups, B).
+//   blockIdx.x <  keep_k : the block owns one kept visual row (or eight, see below).  Its members (the dropped tokens
+//                          assigned to that slot) are first listed in shared memory, then their rows are streamed
+//                          up to four at a time and accumulated in fp32 in ascending order:  (s_hat_i h_i + sum_j s_hat_j h_j) / (s_hat_i +
 //                          sum_j s_hat_j)   (Eq. 5), rounded to bf16 once.  No members, merging
 //                          off, or total weight <= eps: the row is copied.
 //   blockIdx.x >= keep_k : each warp copies one prefix / suffix row.
