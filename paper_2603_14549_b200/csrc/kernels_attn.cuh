@@ -114,7 +114,7 @@ __device__ __forceinline__ bool attn_last_above(const int (&n_kt)[2], const int 
 // about 3000 clocks where either alone needs 2048.  Measured per call (before: a block per pair of row tiles, a kernel that
 // transposed V, a validation kernel, two threads per query row with a shared running maximum, S and P on the same columns):
 //   1 x 643 rows, 32 heads            29.0 ->   19.7 us
-//   16 x 627-739 rows, 32 heads        304 ->    176 us
+//   16 x 627-739 rows, 32 heads        304 ->    171 us
 //   64 x 2947-3171 rows, 32 heads     14.2 ->    8.9 ms   (9.3 TFLOP)
 // Of that on the largest: persistent blocks with V as an MN-major operand 14.1 -> 12.3, an S of its own 11.7 -> 9.8, the mask
 // above the diagonal as one more k-step and the issuing warp converged -> 9.0 ms.  A polynomial for an eighth or a quarter of
