@@ -63,6 +63,90 @@ def test_query_sums_inside_the_score_kernel(ctx, nvs, texts, H):
         A.asap_free(big)
 
 
+@pytest.mark.parametrize("B,H,skipped,visual", [
+    (64, 4, [], 0),                    # 256 items, the most sequences that are drawn by size; the first round ends with a sequence
+    (65, 4, [0, 64], 0),               # one sequence more: drawn in order
+    (60, 5, [0, 1, 2, 29, 30, 59], 0), # the first round ends inside sequence 29, which is skipped
+    (37, 12, [11, 12, 13], 0),         # inside sequence 12; three rounds
+    (11, 40, [0, 3, 10], 0),           # inside sequence 3
+    (60, 5, list(range(31)), 0),       # every item of the first round is skipped
+    (60, 5, [0, 1, 2, 29, 30, 59], 2), # masses in front, at most four tiles per item: the ring takes several items at once
+], ids=["most", "one_more", "skipped", "rounds", "wide", "first_round_skipped", "rows"])
+def test_items_drawn_by_size(B, H, skipped, visual):
+    """Image spans of different lengths in more (sequence, head) items than blocks: after the first round the items are drawn by
+    size.  Each head of each sequence comes once, whichever sequences are skipped (every sequence's scores against the oracle),
+    and the call repeats bit for bit."""
+    nvs = [16 + (37 * b) % 150 for b in range(B)]
+    batch = W.tiny(B=B, n_vis=nvs, text_lens=[3 + (11 * b) % 40 for b in range(B)], H=H, keep_k=8, seed=370 + B, centres=5)
+    rank = (batch.text_start - visual, batch.text_len + visual) if visual else (None, None)
+    inp = A.make_inputs(batch, DEV, *rank)
+    for b in skipped:
+        inp.text_len[b] = 9999
+        if visual:
+            inp.rank_len[b] = 9999
+    p = A.Params(keep_k=8)
+    c = A.asap_init(0, max_total_tokens=batch.total + B * 166, max_B=B, max_H=H, max_D=H * 128)
+    try:
+        outs = []
+        for _ in range(20):
+            out = A.alloc_outputs(inp, 8, fill=True)
+            A.asap_prune_step(c, inp, p, out)
+            torch.cuda.synchronize()
+            if skipped:
+                with pytest.raises(A.AsapError) as e:
+                    A.asap_check(c)
+                assert e.value.status == -6 and "timed out" not in str(e.value)
+            else:
+                A.asap_check(c)
+            outs.append(out)
+    finally:
+        A.asap_free(c)
+    valid = [b for b in range(B) if b not in skipped]
+    for out in outs[1:]:
+        for f in ("mass", "salience", "rank_score", "keep_idx", "assign", "out_hidden"):
+            assert torch.equal(getattr(out, f), getattr(outs[0], f)), f
+    for b in valid:
+        compare_sample(batch, b, p, outs[0], *rank)
+    assert not skipped or float(outs[0].rank_score[skipped].abs().max()) == 0.0
+
+
+def test_items_drawn_by_size_on_two_streams():
+    """Two contexts whose score kernels contend for the SMs: blocks of the second start one by one as blocks of the first leave, some
+    only when the others have drawn all items of the first rounds.  Every result is that of the call by itself."""
+    B, H = 40, 8
+    batches, inps, ctxs, want = [], [], [], []
+    p = A.Params(keep_k=12)
+    for i in range(2):
+        nvs = [20 + (53 * b + 300 * i * (b % 3)) % 700 for b in range(B)]
+        batches.append(W.tiny(B=B, n_vis=nvs, text_lens=[4 + (b * 7) % 90 for b in range(B)], H=H, keep_k=12, seed=380 + i, centres=5))
+        inps.append(A.make_inputs(batches[i], DEV))
+    streams = [torch.cuda.Stream() for _ in range(2)]
+    for i in range(2):
+        ctxs.append(A.asap_init(0, max_total_tokens=batches[i].total + B * 720, max_B=B, max_H=H, max_D=H * 128))
+    try:
+        for i in range(2):
+            out = A.alloc_outputs(inps[i], 12, fill=True)
+            A.asap_prune_step(ctxs[i], inps[i], p, out)
+            torch.cuda.synchronize()
+            A.asap_check(ctxs[i])
+            want.append(out)
+        outs = [[A.alloc_outputs(inps[i], 12, fill=True) for _ in range(16)] for i in range(2)]
+        torch.cuda.synchronize()
+        for n in range(16):
+            for i in range(2):
+                A.asap_prune_step(ctxs[i], inps[i], p, outs[i][n], streams[i])
+        torch.cuda.synchronize()
+        for i in range(2):
+            A.asap_check(ctxs[i], streams[i])
+            for out in outs[i]:
+                for f in ("mass", "salience", "rank_score", "keep_idx", "drop_idx", "assign", "out_hidden", "out_pos", "src_row"):
+                    n = int(want[i].out_cu_seqlens[-1]) if f in ("out_hidden", "out_pos", "src_row") else None
+                    assert torch.equal(getattr(out, f)[:n], getattr(want[i], f)[:n]), f
+    finally:
+        for c in ctxs:
+            A.asap_free(c)
+
+
 @pytest.mark.parametrize("per_head,visual", [(False, 0), (False, 5), (True, 0), (True, 5)], ids=["text", "rows", "heads", "heads_rows"])
 @pytest.mark.parametrize("text", [3, 37, 127, 128, 245, 491])
 def test_a_sequence_does_not_see_its_neighbours(ctx, text, per_head, visual):
