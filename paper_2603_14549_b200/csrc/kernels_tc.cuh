@@ -139,8 +139,17 @@ __device__ __forceinline__ RowPair score_row_pair(const SampleDesc &d, int rp, i
   return r;
 }
 
+// Work of one item: the exponentials of pass 1 (a row tile counts whole) and of pass 2, for each pair of row tiles.  In 64 bits and then
+// capped: half a million ranking rows over as many keys are past 31 bits, and score_order leaves out what is negative.
+__host__ __device__ constexpr int score_work(int n_kt, int nrt, int n_p2, int n2, int n_rp) {
+  const long long w = ((long long)n_kt * nrt * 128 + (long long)n_p2 * (n2 + 16)) * n_rp;
+  return w < 0x7fffffff ? (int)w : 0x7fffffff;
+}
+static_assert(score_work(5, 1, 4, 64, 1) == 960 && score_work(4096, 2, 448, 240, 2185) == 0x7fffffff &&
+              score_work(1 << 24, 2, 449, 240, 0x7fffffff / 240 + 1) == 0x7fffffff, "a sequence's work is positive at every length");
+
 // Sequences first .. B - 1 (at most SC_ORDER_MAX in all) by descending work of one of their items, a stable order, by one warp;
-// returns the place of sequence `first`.  Work: the exponentials of pass 1 (a row tile counts whole) and of pass 2.
+// returns the place of sequence `first`.
 __device__ __forceinline__ int score_order(const ScoreArgs &a, int first, int *work, uint8_t *order, int pair_rows, int lane) {
   int mine[SC_ORDER_MAX / 32];
 #pragma unroll
@@ -151,8 +160,7 @@ __device__ __forceinline__ int score_order(const ScoreArgs &a, int first, int *w
       const SampleDesc d = make_desc(a.pa, b);
       if (d.valid) {
         const RowPair T = score_row_pair(d, 0, a.mask_enable, pair_rows);
-        mine[e] = T.n_kt * T.nrt * 128 + T.n_p2 * (T.n2 + 16);
-        if (d.nr > pair_rows) mine[e] *= (d.nr + pair_rows - 1) / pair_rows;
+        mine[e] = score_work(T.n_kt, T.nrt, T.n_p2, T.n2, (d.nr + pair_rows - 1) / pair_rows);
       } else {
         mine[e] = 0;
       }
