@@ -113,9 +113,9 @@ __device__ __forceinline__ bool attn_last_above(const int (&n_kt)[2], const int 
 // the same cap); below that the hand-overs between the tensor pipe and the softmax warps: a key tile of both row tiles takes
 // about 3000 clocks where either alone needs 2048.  Measured per call (before: a block per pair of row tiles, a kernel that
 // transposed V, a validation kernel, two threads per query row with a shared running maximum, S and P on the same columns):
-//   1 x 643 rows, 32 heads            29.0 ->   19.7 us
-//   16 x 627-739 rows, 32 heads        304 ->    171 us
-//   64 x 2947-3171 rows, 32 heads     14.2 ->    8.9 ms   (9.3 TFLOP)
+//   1 x 643 rows, 32 heads            29.0 ->   19.6 us
+//   16 x 627-739 rows, 32 heads        304 ->    173 us
+//   64 x 2947-3171 rows, 32 heads     14.2 ->    8.7 ms   (9.3 TFLOP)
 // Of that on the largest: persistent blocks with V as an MN-major operand 14.1 -> 12.3, an S of its own 11.7 -> 9.8, the mask
 // above the diagonal as one more k-step and the issuing warp converged -> 9.0 ms.  A polynomial for an eighth or a quarter of
 // the exponentials changed nothing (8.9-9.0), for three eighths it cost 4 %.
@@ -554,8 +554,8 @@ attn_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__ 
         if (lane == 0) mbar_arrive(smem_u32(&bk->s_empty));
         if (kind.crossed) {
           // columns past all rows of the warp (the tile lies on the diagonal, so its first 32 never do): m_j for a row of the span,
-          // AT_NEVER for any other.  Put right in tensor memory like the 32 columns that the diagonal crosses, 450 clocks per 32, they
-          // held up the S that both row tiles share for 2000 to 2600 clocks (1 x 643 rows 20.5 -> 19.7 us, 16 x 627-739 167 -> 163.5).
+          // AT_NEVER for any other (see `chosen` below for logits that are not finite).  Put right in tensor memory like the 32 columns that the diagonal crosses, 450 clocks per 32, they
+          // held up the S that both row tiles share for 2000 to 2600 clocks (per call 1 x 643 rows 20.1 -> 19.5 us, 16 x 627-739 174.7 -> 171.3).
           const float off = vis_row ? 0.f : AT_NEVER, in = vis_row ? 1.f : 0.f;
           const uint64_t off2 = f2_pack(off, off), in2 = f2_pack(in, in);
 #pragma unroll
@@ -579,7 +579,7 @@ attn_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__ 
           mbar_wait(smem_u32(&bk->pv_done[g]), (sc - 1) & 1, wc);      // O is complete up to here, and P may be overwritten
           tc_fence_after();
         }
-        bool move = kt == 0, again = kt == 0;
+        bool move = kt == 0, again = kt == 0, chosen = !kind.crossed;
         float tile_sum;
 #pragma unroll 1
         while (true) {
@@ -627,7 +627,20 @@ attn_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__ 
           f2_unpack(f2_add(sum2[0], sum2[1]), s0, s1);
           tile_sum = s0 + s1;
           move = !(tile_sum < AT_SUM_LIMIT);
-          if (again || !__any_sync(0xffffffffu, move)) break;   // (relative to the true maximum no sum exceeds 128)
+          if (!__any_sync(0xffffffffu, move)) break;
+          if (!chosen) {
+            // An addend hides the logit of a key that the row does not admit only if that logit is finite.  The tile is done again
+            // with -inf in its place.  (Per call, 16 x 627-739 rows: without this 172.3 us, with it 173.1, with the choice in every tile,
+            // two instructions a column, 178.4.)
+            chosen = true;
+            move = kt == 0;                         // the first tile's reference is taken again, other references stay
+            const int hi = hi_adm - j0;
+#pragma unroll
+            for (int c = 32; c < 128; ++c)
+              if (c > hi) xr[c] = __float_as_uint(-INFINITY);
+            continue;
+          }
+          if (again) break;                         // (relative to the true maximum no sum exceeds 128)
           again = true;
         }
         l_run += tile_sum;

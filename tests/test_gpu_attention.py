@@ -120,6 +120,34 @@ def test_a_sequence_does_not_see_its_neighbours(ctx, nv, text, skipped):
     assert torch.equal(out[:n0].cpu(), good.cpu())
 
 
+@pytest.mark.parametrize("value", [float("nan"), float("inf")], ids=["nan", "inf"])
+@pytest.mark.parametrize("per_head", [False, True], ids=["mean", "heads"])
+@pytest.mark.parametrize("nv,text,key", [(121, 4, 100), (40, 70, 90), (40, 85, 127), (60, 61, 66), (147, 106, 200), (130, 120, 250)])
+def test_a_row_does_not_see_a_key_that_it_does_not_admit(ctx, nv, text, key, per_head, value):
+    """A key that is not finite, later in the SAME sequence and in the key tile that a row's diagonal crosses: the rows of that row
+    tile that do not admit it (system and text rows before it, rows of the span when it lies behind the span) keep every bit."""
+    batch = W.tiny(B=1, n_vis=[nv], text_lens=[text], H=2, keep_k=8, seed=618)
+    v = W.draw_values(batch, 88).to(DEV)
+    m, _ = _mask_vectors(batch, 1.0)
+    if per_head:
+        m = torch.stack([m, 0.5 * m], dim=1)
+    scratch = torch.empty(A.asap_attention_scratch_bytes(batch.total, batch.D), dtype=torch.uint8, device=DEV)
+    outs = []
+    for spoil in (False, True):
+        if spoil:
+            batch.k[key, :, 5] = value
+        out = torch.zeros_like(v)
+        A.asap_attention(ctx, A.make_inputs(batch, DEV), A.Params(keep_k=8, per_head_mask=per_head), m.contiguous().to(DEV), v, scratch, out)
+        torch.cuda.synchronize(); A.asap_check(ctx)
+        outs.append(out.cpu())
+    v0, rows = int(batch.vis_start[0]), torch.arange(batch.total)
+    admits = (rows >= key) | ((rows >= v0) & (rows < v0 + nv) & (v0 <= key < v0 + nv))
+    look = ~admits & (rows // 128 == key // 128)
+    assert int(look.sum()) > 2
+    assert torch.isfinite(outs[0].float()).all()
+    assert torch.equal(outs[0][look], outs[1][look])
+
+
 def test_mask_off_is_causal_attention_and_only_visual_rows_differ(ctx):
     batch = W.tiny(B=2, n_vis=[200, 333], text_lens=[17, 5], H=2, keep_k=8, seed=610)
     v = W.draw_values(batch, 78)
