@@ -465,6 +465,8 @@ asap_status launch_merge_front(asap_ctx *ctx, const asap_inputs *in, const asap_
     //              256 slots     28 65 -> 76, 36 64 to 78 -> 84 to 85, 48 99 to 104 -> 93 to 98, 72 97 to 131 -> 105 to 123, 96 139 -> 118
     //   width 2048   64 slots    48 32 to 37 -> 36 to 40, 96 62 -> 62; 160 slots 18 36 -> 37, 24 40 -> 38, 36 43 to 54 -> 41 to 43,
     //              72 67 to 74 -> 60 to 67; 256 slots 24 46 -> 43, 36 38 to 55 -> 44 to 50, 72 60 to 92 -> 65 to 81
+    // Not beyond the batches whose partial results fit their buffer when the groups share the rows' squared norms: with a norm for each
+    // group counted too, 230 x 3100 with 770 kept of width 128 fell to the tiled form, its launch 971 us instead of 705.
     {
       const int pairs = (in->max_vis + 255) / 256;
       const int pg = (k + 255) / 256;
@@ -473,7 +475,7 @@ asap_status launch_merge_front(asap_ctx *ctx, const asap_inputs *in, const asap_
       const PairRings rings = pair_rings(ctx, ptile);
       const size_t psmem = rings.bytes + SIM_BOOK_BYTES + 1024;
       if (!gather_rows && D % 64 == 0 && (long long)pairs * B * pg >= min_blocks && (size_t)B * pairs <= ctx->cap_tiles &&
-          (size_t)B * pairs * (size_t)(pg * 768) * sizeof(float) <= ctx->sim_part_bytes &&
+          (size_t)B * pairs * (size_t)(pg * 512 + 256) * sizeof(float) <= ctx->sim_part_bytes &&
           (bits || (size_t)(SIMP_THREADS / 32 + 1) * k * sizeof(int) <= rings.bytes)) {
         uint32_t pcols = 32;
         while ((int)pcols < 2 * ptile) pcols <<= 1;
@@ -784,7 +786,8 @@ asap_status asap_init(asap_ctx **ctx_out, int device, size_t max_total_tokens, i
   ctx->cap_tiles = T / 128 + Bc;                       // row tiles of 128 visual rows in any batch that fits
   ctx->sim_part_bytes = (size_t)32 << 20;
   const size_t o_tiles = carve(ctx->cap_tiles * sizeof(unsigned int));
-  const size_t o_simpart = carve(ctx->sim_part_bytes);
+  // (half as much again: sim_pair_kernel's groups leave 768 floats per pair each, where its limit counts 512, and 256 per pair)
+  const size_t o_simpart = carve(ctx->sim_part_bytes / 2 * 3);
   const size_t o_status = carve(sizeof(uint32_t));
   e = cudaMalloc(&ctx->arena, off);
   if (e != cudaSuccess) {

@@ -14,7 +14,7 @@ from oracle import asap_oracle as O
 from paper_2603_14549_b200 import binding as A
 from paper_2603_14549_b200 import workloads as W
 from tests.helpers import bits
-from tests.parity import merged_tolerance
+from tests.parity import compare_sample, merged_tolerance
 
 pytestmark = pytest.mark.gpu
 DEV = "cuda:0"
@@ -150,6 +150,36 @@ def test_many_kept_slots_of_a_long_sequence():
         _merge_matches_oracle(c, [15000, 5100], 5000, H=2, seed=934)
     finally:
         A.asap_free(c)
+
+
+def test_pair_form_at_the_end_of_its_partial_results():
+    """2990 pairs of row tiles with four groups of slots each: close to the most that the form takes, and more than its partial results
+    had room for before the groups left a share of the row norms each.  115 copies of two sequences give the same bits, and the first
+    two are the oracle's."""
+    two = W.tiny(B=2, n_vis=[3100, 3081], text_lens=[8, 5], H=1, keep_k=770, seed=937, centres=60)
+    n, reps = two.total, 115
+    rep = lambda t: t.repeat(reps, *([1] * (t.dim() - 1)))
+    cu = torch.cat([torch.zeros(1, dtype=torch.int32)] + [two.cu_seqlens[1:] + r * n for r in range(reps)]).to(torch.int32)
+    batch = W.Batch(name="tiny", B=2 * reps, H=1, head_dim=128, D=128, keep_k=770, cu_seqlens=cu,
+                    **{f: rep(getattr(two, f)) for f in ("vis_start", "vis_len", "text_start", "text_len", "q", "k", "hidden", "pos_ids")})
+    p = A.Params(keep_k=770)
+    c = A.asap_init(0, max_total_tokens=batch.total + batch.B * 20, max_B=batch.B, max_H=1, max_D=128, max_keep_rows=batch.B * 770)
+    try:
+        inp = A.make_inputs(batch, DEV)
+        out = A.alloc_outputs(inp, 770, fill=True)
+        A.asap_prune_step(c, inp, p, out)
+        torch.cuda.synchronize()
+        A.asap_check(c)
+    finally:
+        A.asap_free(c)
+    for b in range(2):
+        compare_sample(batch, b, p, out)
+    for f in ("rank_score", "keep_idx", "assign", "best_sim"):
+        t = getattr(out, f)
+        assert torch.equal(t.view(reps, -1), t[:2].reshape(1, -1).expand(reps, -1)), f
+    rows = int(out.out_cu_seqlens[2])
+    h = out.out_hidden[:reps * rows].view(reps, -1)
+    assert torch.equal(h, h[:1].expand(reps, -1))
 
 
 def test_pair_form_gives_up_and_the_context_recovers(ctx_pair_form):
