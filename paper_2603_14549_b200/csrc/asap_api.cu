@@ -552,10 +552,11 @@ asap_status launch_merge_front(asap_ctx *ctx, const asap_inputs *in, const asap_
   return ASAP_OK;
 }
 
-// Steps 4b-5: weighted merge and compaction (the first consumer of the salience).
+// Steps 4b-5: weighted merge and compaction (the first consumer of the salience).  `members`: the most that a sequence's slots have
+// together.
 asap_status launch_merge_back(asap_ctx *ctx, const asap_inputs *in, const asap_params *p,
                               const float *salience, const int32_t *keep_idx, const int32_t *drop_idx,
-                              const asap_outputs *out, cudaStream_t st, bool grouped_with_weights = false, bool bits = false) {
+                              const asap_outputs *out, int members, cudaStream_t st, bool grouped_with_weights = false, bool bits = false) {
   const int B = in->B, D = in->D, k = p->keep_k;
   const bool do_merge = merging(in, p);
   MergeArgs ma;
@@ -568,9 +569,16 @@ asap_status launch_merge_back(asap_ctx *ctx, const asap_inputs *in, const asap_p
   ma.out_pos = out->out_pos; ma.src_row = out->src_row;
   const int copy_rows = in->max_seq - in->min_vis;   // prefix + suffix rows of the longest sequence, at most
   int nv = (D / 8 + MERGE_THREADS - 1) / MERGE_THREADS;
-  // Without member bits (after the routing, most kept rows have no members): a row per warp where that still fills the machine.
+  // Without member bits: eight kept rows per block where that still fills the machine.  Rows without members (nearly all after the
+  // routing, all with merging off) are then copied by a warp each; the others are merged one after the other, so only up to two members a
+  // slot on average.  Measured, one row per block -> eight, as asap_merge by members per slot: 1 (64 x 1152 tokens, 576 kept, width 2048)
+  // 418 -> 362 us, 1 (32 x 2304, width 5120) 873 -> 846, 1 (64 x 576, width 4096) 287 -> 291, 2 (64 x 1152, 384 kept) 312 -> 279, 3 (64 x
+  // 1152, 288 kept) 289 -> 269 but 292 -> 301 (2 x 8192) and 486 -> 501 (1 x 16384), 4 (4 x 5760) 255 -> 264, 7 (8 x 8192) 592 -> 606,
+  // 9 (8 x 5760) 301 -> 325, 15 (4 x 16384, 1024 kept) 587 -> 630; none (24 x 2880) 83 -> 56.  Consolidation, 24 x 2304 tokens with 576 kept
+  // of width 5120: none absorbed 206 -> 194, 72 slots that absorb one each 218 -> 210, 288 233 -> 230, 192 that absorb two 235 -> 236,
+  // 64 that absorb eight 241 -> 246; of width 4096 (24 x 2880) merge 79 -> 62, 98 -> 87, 94 -> 82, 89 -> 81.
   const int per_block = MERGE_THREADS / 32, blocks8 = (k + per_block - 1) / per_block;
-  ma.block_rows = !bits && (long long)blocks8 * B >= 2LL * ctx->num_sms ? per_block : 1;
+  ma.block_rows = !bits && members <= 2LL * k && (long long)blocks8 * B >= 2LL * ctx->num_sms ? per_block : 1;
   dim3 grid((ma.block_rows > 1 ? blocks8 : k) + (copy_rows + MERGE_COPY_ROWS - 1) / MERGE_COPY_ROWS, B);
   // Rows cut into pieces of 2048 elements while all of them still run in one wave (1 x 192 slots: merge 10.4 -> 9.0 us, the
   // step 41.6 -> 40.5); beyond that the shorter pieces cost more than they balance (16 x 64 slots 28.8 -> 31.8 us).
@@ -599,7 +607,7 @@ asap_status launch_merge(asap_ctx *ctx, const asap_inputs *in, const asap_params
                          const float *salience, const int32_t *keep_idx, const int32_t *drop_idx,
                          const asap_outputs *out, cudaStream_t st) {
   ASAP_TRY(launch_merge_front(ctx, in, p, salience, keep_idx, drop_idx, out, st));
-  return launch_merge_back(ctx, in, p, salience, keep_idx, drop_idx, out, st, true, merge_bits(ctx, in, p));
+  return launch_merge_back(ctx, in, p, salience, keep_idx, drop_idx, out, merging(in, p) ? in->max_vis - p->keep_k : 0, st, true, merge_bits(ctx, in, p));
 }
 
 // Sec. 4.2 inside the kept set: kept rows gathered, their keep_k x keep_k cosine matrix, routing.
@@ -958,7 +966,7 @@ asap_status asap_consolidate(asap_ctx *ctx, const asap_inputs *in, const asap_pa
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   ASAP_TRY(launch_prepare(ctx, in, p, out->out_cu_seqlens, out->out_rows_capacity, st));
   ASAP_TRY(launch_consolidate_front(ctx, in, p, mass, salience, keep_idx, drop_idx, scratch, out, n_absorbed, st));
-  return finish(ctx, launch_merge_back(ctx, in, p, salience, out->keep_idx, out->drop_idx, out, st), st);
+  return finish(ctx, launch_merge_back(ctx, in, p, salience, out->keep_idx, out->drop_idx, out, p->keep_k, st), st);
 }
 
 asap_status asap_prune_step(asap_ctx *ctx, const asap_inputs *in, const asap_params *p, const asap_outputs *out,

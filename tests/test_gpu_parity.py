@@ -226,6 +226,18 @@ def test_rows_of_member_bits(nvs, k, tokens):
         A.asap_free(small)
 
 
+@pytest.mark.parametrize("nv", [576, 577], ids=["eight_rows_a_block", "one_more_member"])
+def test_grouped_members_of_many_slots(nv):
+    """Width 128 has no room for the bits of 192 kept slots: grouped members, up to two a slot on average with eight slots per block,
+    beyond that with one."""
+    batch = W.tiny(B=13, n_vis=[nv] + [576 - 20 * b for b in range(12)], text_lens=[4 + b for b in range(13)], H=1, keep_k=192, seed=340, centres=40)
+    c = A.asap_init(0, max_total_tokens=13 * 592, max_B=13, max_H=1, max_D=128)
+    try:
+        run_step(c, batch, A.Params(keep_k=192))
+    finally:
+        A.asap_free(c)
+
+
 @pytest.mark.parametrize("k,H", [(600, 1), (600, 3), (340, 5), (1100, 1)], ids=["fewer_steps_than_groups", "two_steps_each", "uneven", "five_groups"])
 def test_row_norms_shared_by_the_groups(ctx, k, H):
     """Every group of kept slots adds up the squares of its range of the columns: two 64-column steps for three or five groups (some
