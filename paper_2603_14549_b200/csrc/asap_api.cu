@@ -355,9 +355,19 @@ size_t route_tail_words(const asap_inputs *in, const asap_params *p) { return (s
 // row per merge block.  Measured per step, grouped -> bits: 8 x 2304 with 320 kept 193 -> 185 us, 12 x 577-2881 with 145 kept 230 ->
 // 221.5, 8 x 1536 with 340 kept 219 -> 213.5; against blocks that looked for their members among all dropped tokens' destinations,
 // 16 x 576 with 64 kept 113 -> 110, 1 x 576 with 192 kept 39.7 -> 39.6.
+// A row of more than 4096 tokens is read in several passes, a round trip each, by every merge block: those past the first cost the merge
+// about 1 us per 3 blocks an SM has room for, a sequence's grouping about 3 us per 1024 tokens, and the line is where the two meet.
+// As asap_merge, width 4096, grouped -> bits: 4 x 16384 with 512, 1024, 2048 and 4096 kept 381 -> 351 us, 587 -> 572, 1011 -> 1029,
+// 1862 -> 1871; 8 x 8192 with 512, 1024, 2048 370 -> 360, 592 -> 592, 1081 -> 1076; 8 x 5760 with 576, 1152 301 -> 295, 500 -> 504; 1 x
+// 57344 with 512, 2048, 4096 428 -> 328, 948 -> 863, 1650 -> 1628; width 2048, 32 x 8192 with 256 531 -> 502, 16 x 16384 with 512 761 -> 763.
+// (sim_pair_kernel's rings have to hold the grouping's counters: above some 4096 slots the bits keep a batch in that form.)
 int member_words(const asap_inputs *in) { return (in->max_vis + 31) / 32; }
 bool merge_bits(const asap_ctx *ctx, const asap_inputs *in, const asap_params *p) {
-  return merging(in, p) && (size_t)in->B * p->keep_k * member_words(in) <= ctx->member_cap;
+  if (!merging(in, p) || (size_t)in->B * p->keep_k * member_words(in) > ctx->member_cap) return false;
+  const int k = p->keep_k, pg = (k + 255) / 256, ptile = (((k + pg - 1) / pg) + 15) & ~15;
+  const long long later_passes = (member_words(in) - 1) / (32 * MERGE_BIT_WORDS);
+  return (long long)in->B * k * later_passes * 1024 <= 9LL * ctx->num_sms * in->max_vis ||
+         (size_t)(SIMP_THREADS / 32 + 1) * k * sizeof(int) > pair_rings(ctx, ptile).bytes;
 }
 
 // `fused_head_sum`: the ranking scores are still per-head sums in scratch (the score kernel ran

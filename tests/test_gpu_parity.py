@@ -226,6 +226,13 @@ def test_rows_of_member_bits(nvs, k, tokens):
         A.asap_free(small)
 
 
+@pytest.mark.parametrize("k", [680, 700], ids=["bits", "grouped"])
+def test_long_rows_of_member_bits(ctx, k):
+    """Rows of bits in two passes: from some 690 slots of eight sequences of 4224 tokens on (148 SMs) the members are grouped instead."""
+    batch = W.tiny(B=8, n_vis=[4224] + [4000 - 100 * b for b in range(7)], text_lens=[4 + b for b in range(8)], H=1, keep_k=k, seed=341, centres=90)
+    run_step(ctx, batch, A.Params(keep_k=k), samples=[0, 7])
+
+
 @pytest.mark.parametrize("nv", [576, 577], ids=["eight_rows_a_block", "one_more_member"])
 def test_grouped_members_of_many_slots(nv):
     """Width 128 has no room for the bits of 192 kept slots: grouped members, up to two a slot on average with eight slots per block,
