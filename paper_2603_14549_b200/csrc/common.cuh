@@ -56,6 +56,14 @@ __device__ __forceinline__ int2 ld_prev(const int2 *p) {
   asm volatile("ld.global.v2.s32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "l"(p));
   return v;
 }
+// (descriptors lie at multiples of 32 bytes: an array of them starts at a multiple of 256)
+static_assert(sizeof(SampleDesc) == 32, "a descriptor is two 16-byte loads");
+__device__ __forceinline__ SampleDesc ld_prev(const SampleDesc *p) {
+  SampleDesc d;
+  asm volatile("ld.global.v4.s32 {%0, %1, %2, %3}, [%4];" : "=r"(d.row0), "=r"(d.n), "=r"(d.v0), "=r"(d.nv) : "l"(p));
+  asm volatile("ld.global.v4.s32 {%0, %1, %2, %3}, [%4];" : "=r"(d.r0), "=r"(d.nr), "=r"(d.out_row0), "=r"(d.valid) : "l"(&p->r0));
+  return d;
+}
 
 __device__ __forceinline__ float bf16_lo(uint32_t w) { return __uint_as_float(w << 16); }
 __device__ __forceinline__ float bf16_hi(uint32_t w) { return __uint_as_float(w & 0xffff0000u); }

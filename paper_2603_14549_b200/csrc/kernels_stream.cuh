@@ -309,10 +309,7 @@ __device__ __forceinline__ void salience_block(const SampleDesc &d, int b, int m
 __global__ void __launch_bounds__(SAL_THREADS)
 salience_kernel(const SampleDesc *desc, int max_vis, SalienceArgs a) {
   pdl_enter();
-  SampleDesc d = {};                       // (the directly preceding kernel wrote the descriptors)
-  d.nv = ld_prev(&desc[blockIdx.x].nv);
-  d.valid = ld_prev(&desc[blockIdx.x].valid);
-  salience_block(d, blockIdx.x, max_vis, a);
+  salience_block(ld_prev(desc + blockIdx.x), blockIdx.x, max_vis, a);
 }
 
 template <bool PER_HEAD>
@@ -525,7 +522,7 @@ __device__ __forceinline__ int block_exclusive_scan(int v, int *s_warp /*[32]*/,
 }
 
 __global__ void __launch_bounds__(SELECT_THREADS)
-select_kernel(const float *__restrict__ rank_score, const SampleDesc *__restrict__ desc,
+select_kernel(const float *__restrict__ rank_score, const SampleDesc *desc,
               int max_vis, int keep_k, int32_t *__restrict__ keep_idx, int32_t *__restrict__ drop_idx,
               int32_t *__restrict__ role /*[B, max_vis]*/, int32_t *__restrict__ assign /*nullable*/,
               float *__restrict__ best_sim /*nullable*/, int sim_follows,
@@ -534,8 +531,9 @@ select_kernel(const float *__restrict__ rank_score, const SampleDesc *__restrict
               SalienceArgs sal /* blockIdx.y == 1 */) {
   pdl_enter();
   if (blockIdx.y == 1) {
-    if (sal.norm) salience_heads_block(desc[blockIdx.x], blockIdx.x, max_vis, sal);
-    else salience_block(desc[blockIdx.x], blockIdx.x, max_vis, sal);
+    const SampleDesc d = ld_prev(desc + blockIdx.x);
+    if (sal.norm) salience_heads_block(d, blockIdx.x, max_vis, sal);
+    else salience_block(d, blockIdx.x, max_vis, sal);
     return;
   }
   extern __shared__ uint32_t s_key[];   // [max_vis]
@@ -544,7 +542,7 @@ select_kernel(const float *__restrict__ rank_score, const SampleDesc *__restrict
   __shared__ uint32_t s_prefix, s_lo[32], s_hi[32];
   __shared__ int s_remaining, s_bucket;
   const int b = blockIdx.x;
-  const SampleDesc d = desc[b];
+  const SampleDesc d = ld_prev(desc + b);
   const int nd_max = max_vis - keep_k;
   int32_t *keep_b = keep_idx + (size_t)b * keep_k;
   int32_t *drop_b = drop_idx + (size_t)b * nd_max;
@@ -715,14 +713,14 @@ select_kernel(const float *__restrict__ rank_score, const SampleDesc *__restrict
 }
 
 // role map from caller-provided keep / drop lists (entry point asap_merge)
-__global__ void role_map_kernel(const SampleDesc *__restrict__ desc, int max_vis, int keep_k,
+__global__ void role_map_kernel(const SampleDesc *desc, int max_vis, int keep_k,
                                 const int32_t *__restrict__ keep_idx,
                                 const int32_t *__restrict__ drop_idx, int32_t *__restrict__ role,
                                 int32_t *__restrict__ assign, float *__restrict__ best_sim,
                                 int sim_follows) {
   pdl_enter();
   const int b = blockIdx.y;
-  const SampleDesc d = desc[b];
+  const SampleDesc d = ld_prev(desc + b);
   const int nd_max = max_vis - keep_k;
   {
     const int first = (d.valid && sim_follows) ? d.nv - keep_k : 0;
@@ -753,7 +751,7 @@ __global__ void role_map_kernel(const SampleDesc *__restrict__ desc, int max_vis
 constexpr int GATHER_THREADS = 256;
 
 __global__ void __launch_bounds__(GATHER_THREADS)
-kept_gather_kernel(const __nv_bfloat16 *__restrict__ hidden, const SampleDesc *__restrict__ desc,
+kept_gather_kernel(const __nv_bfloat16 *__restrict__ hidden, const SampleDesc *desc,
                    int D, int keep_k, const int32_t *__restrict__ keep_idx,
                    __nv_bfloat16 *__restrict__ kept_rows /*[B*keep_k, D]*/,
                    float *__restrict__ kept_inv /*[B*keep_k]*/, uint32_t *__restrict__ member_bits /*[B*keep_k, bit_words], nullable*/,
@@ -764,7 +762,7 @@ kept_gather_kernel(const __nv_bfloat16 *__restrict__ hidden, const SampleDesc *_
   const int slot = blockIdx.x * (GATHER_THREADS / 32) + warp;
   if (slot >= keep_k) return;
   const int kept = ld_prev(keep_idx + (size_t)b * keep_k + slot);      // (beside the descriptor, not behind it)
-  const SampleDesc d = desc[b];
+  const SampleDesc d = ld_prev(desc + b);
   if (!d.valid) return;
   const int j = min(max(kept, 0), d.nv - 1);
   const uint4 *src = reinterpret_cast<const uint4 *>(hidden + (size_t)(d.row0 + d.v0 + j) * D);
