@@ -50,6 +50,16 @@ __device__ __forceinline__ SampleDesc make_desc(const PrepareArgs &a, int b) {
   return d;
 }
 
+// Whether the shortened batch fits the output, by one warp: if not, nothing may be written (see prepare_warp).
+__device__ __forceinline__ bool output_fits(const PrepareArgs &a) {
+  int len = 0;
+  for (int b = threadIdx.x & 31; b < a.B; b += 32) {
+    const SampleDesc d = make_desc(a, b);
+    if (d.valid) len += d.n - d.nv + a.keep_k;
+  }
+  return __reduce_add_sync(0xffffffffu, len) <= a.out_capacity;
+}
+
 // Run by one warp: validates every sequence, writes the descriptors, the output row offsets and the status bits.
 // (A whole block with one thread adding the offsets up took 6 us for 8 sequences: a chain of round trips.)
 __device__ __forceinline__ void prepare_warp(const PrepareArgs &a) {
@@ -372,6 +382,7 @@ mass_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__ 
   }
   const int tid = threadIdx.x - 32, aw = warp - 1;        // among the adding warps
   if (a.pa.write_desc && blockIdx.x == 0 && aw == 0) prepare_warp(a.pa);
+  const bool fits = !PER_HEAD || output_fits(a.pa);       // (the masks of the heads are outputs; the first tiles are on their way)
   const int c = lane & 15, row0 = (tid >> 4) * 8;         // this thread's 16-byte chunk of the head, its half-warp's eight rows of a tile
   const bool up8 = lane & 8, up4 = lane & 4, up2 = lane & 2;
   RingPos r;
@@ -474,7 +485,7 @@ mass_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__ 
         a.norm[(size_t)item * 2 + 1] = inv;
       }
       for (int j = tid; j < a.max_vis; j += MASS_ADDERS)
-        mh[j] = j < d.nv ? logf(fmaxf(a.lambda_max * ((out[j] - lo) * inv), a.eps)) : 0.f;
+        mh[j] = fits && j < d.nv ? logf(fmaxf(a.lambda_max * ((out[j] - lo) * inv), a.eps)) : 0.f;
       // (two barriers come before s_red is written again)
     }
   }

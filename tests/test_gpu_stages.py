@@ -208,6 +208,25 @@ def test_output_capacity_overflow_is_reported(ctx):
     assert float(out.out_hidden.float().abs().sum()) == 0.0   # nothing was written
 
 
+@pytest.mark.parametrize("per_head,visual", [(True, 0), (True, 3), (False, 3)], ids=["heads", "heads_rows", "rows"])
+def test_output_capacity_overflow_leaves_padding_in_every_output(ctx, per_head, visual):
+    """The masses of such a batch come from a kernel of their own, which does not see the shortened length: the sequences' outputs are
+    those of skipped sequences all the same, the masks of the heads among them."""
+    batch = W.tiny(B=3, n_vis=[150, 50, 140], text_lens=[5, 9, 7], H=2, keep_k=10, seed=308)
+    inp = A.make_inputs(batch, DEV, *((batch.text_start - visual, batch.text_len + visual) if visual else ()))
+    out = A.alloc_outputs(inp, 10, fill=True, per_head=per_head)
+    out.out_hidden = out.out_hidden[:20]
+    A.asap_prune_step(ctx, inp, A.Params(keep_k=10, per_head_mask=per_head), out)
+    torch.cuda.synchronize()
+    with pytest.raises(A.AsapError) as e:
+        A.asap_check(ctx)
+    assert e.value.status == -6 and "capacity" in str(e.value)
+    for f in ("mass", "salience", "mask_log", "rank_score", "best_sim", "out_hidden") + (("mask_log_heads",) if per_head else ()):
+        assert torch.all(getattr(out, f) == 0), f
+    for f in ("keep_idx", "drop_idx", "assign"):
+        assert torch.all(getattr(out, f) == -1), f
+
+
 def test_repeated_calls_are_deterministic(ctx):
     batch = W.tiny(B=2, n_vis=[300, 170], text_lens=[33, 8], H=2, keep_k=40, seed=307, centres=5)
     inp = A.make_inputs(batch, DEV)
