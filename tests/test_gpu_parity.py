@@ -202,12 +202,13 @@ def test_masses_in_the_score_kernel_lose_no_precision(ctx, nvs, H):
     assert math.sqrt(err / tot) < 1.04e-7
 
 
-@pytest.mark.parametrize("nvs,k", [([1028, 1029], 4), ([2500, 1030], 3), ([40, 16], 16), ([2060], 7)],
-                         ids=["one_pass", "three_passes", "nothing_dropped", "three_passes_one"])
-def test_merge_blocks_that_scan_for_their_members(ctx, nvs, k):
-    """Few kept slots: the merge blocks look their members up among all dropped tokens, 1024 per pass -- exactly
-    one full pass, ragged later passes, far more members per slot than a list of the grouped form holds, and a
-    sequence without a dropped token."""
+@pytest.mark.parametrize("nvs,k", [([65, 66], 1), ([129, 130, 32, 33], 1), ([4096, 4097, 4129], 1), ([1028, 1029], 4), ([2500, 1030], 3),
+                                   ([40, 16], 16), ([2060], 7)],
+                         ids=["a_full_list", "two_lists_and_word_edges", "a_full_pass", "words_of_few", "several_lists", "nothing_dropped", "one"])
+def test_few_slots_with_many_members(ctx, nvs, k):
+    """A slot's members come from its row of bits, 32 visual tokens a word, 4096 a pass, and are merged 64 at a time.  With one slot
+    everything else is its member: 64 and 65, 128 and 129 members, spans that end on a word or one past it, on a pass, one and 33 past it;
+    a sequence without a dropped token."""
     batch = W.tiny(B=len(nvs), n_vis=nvs, text_lens=[9 + b for b in range(len(nvs))], H=2, keep_k=k, seed=120 + k, centres=k + 1)
     run_step(ctx, batch, A.Params(keep_k=k))
 

@@ -271,9 +271,9 @@ def test_kv_cache_compaction_follows_the_row_map(ctx):
 
 
 def test_prune_step_can_be_captured_into_a_cuda_graph(ctx):
-    """The step allocates nothing, never synchronises, and its side stream forks from and joins back
-    into the caller's stream inside the call, so a stream capture records it whole; a replay on new
-    input contents (same buffers) gives what a direct call gives, bit for bit."""
+    """The step allocates nothing, never synchronises and stays on the caller's stream, so a stream
+    capture records it whole; a replay on new input contents (same buffers) gives what a direct call
+    gives, bit for bit."""
     batch = W.tiny(B=3, n_vis=[300, 170, 520], text_lens=[9, 30, 4], H=2, keep_k=48, seed=306, centres=8)
     other = W.tiny(B=3, n_vis=[300, 170, 520], text_lens=[9, 30, 4], H=2, keep_k=48, seed=307, centres=8)
     inp = A.make_inputs(batch, DEV)
