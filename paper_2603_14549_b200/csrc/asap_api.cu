@@ -502,7 +502,7 @@ asap_status launch_merge_front(asap_ctx *ctx, const asap_inputs *in, const asap_
         sa.best_sim = out->best_sim; sa.seg = bits ? nullptr : ctx->seg; sa.members = ctx->members; sa.counters = ctx->cnt_sim;
         sa.tile_counters = ctx->cnt_tiles; sa.part = ctx->sim_part; sa.ss_part = nullptr; sa.smat = nullptr; sa.mask16 = nullptr; sa.mask_pitch = 0;
         sa.drop_all = drop_idx; sa.salience = salience; sa.member_meta = salience ? ctx->member_meta : nullptr;
-    sa.member_bits = bits; sa.bit_words = member_words(in);
+        sa.member_bits = bits; sa.bit_words = member_words(in);
         sa.status = ctx->status; sa.wait_limit = ctx->wait_limit;
         mark(ctx, "sim", st);
         launch_pdl(sim_pair_kernel, dim3(pairs * pg, B), dim3(SIMP_THREADS), psmem, st, map_h, map_kept, sa);

@@ -189,7 +189,10 @@ __device__ __forceinline__ int score_order(const ScoreArgs &a, int first, int *w
 }
 
 // SORTED: items past the first round are drawn by size, so that the blocks end together (score of 12 images of 577 to 2881 rows
-// 115 -> 98 us).  Taken for image spans of different lengths in more items than blocks.  The order is worked out by a query-sum
+// 109 -> 97 us, of 64 of 280 to 1400 rows with 16 heads 157 -> 149).  Taken for image spans of different lengths in more items than blocks,
+// up to 64 sequences: beyond, a block has so many items that the last one counts little (in order against by size: 96 of 280 to 1400
+// rows 220 and 224 us, 128 of them 283 and 286, 128 of 140 to 700 rows with 32 heads 352 and 364).  A block's first item is its own number, see
+// the draw.  The order is worked out by a query-sum
 // warp that has its first item behind it: by the copy warp it cost 2 to 4 us, and in the kernel for batches that do not want
 // it, its code alone 1 to 3 us (1 x 576 39.5 -> 40.6 us, 16 x 576 110.3 -> 113.4).
 template <bool SORTED>
