@@ -49,6 +49,30 @@ def test_score_kernel_gives_up_and_the_context_recovers(ctx):
     _same(good, again, ("rank_score", "keep_idx", "drop_idx", "assign", "out_hidden", "out_pos", "src_row", "out_cu_seqlens"))
 
 
+def test_score_kernel_that_draws_by_size_gives_up_and_the_context_recovers():
+    """The same where items past the first round wait for their order too (image spans of different lengths, 240 items)."""
+    B = 60
+    batch = W.tiny(B=B, n_vis=[30 + (41 * b) % 170 for b in range(B)], text_lens=[3 + b % 9 for b in range(B)], H=4, keep_k=10, seed=612, centres=6)
+    c = A.asap_init(0, max_total_tokens=batch.total + B * 200, max_B=B, max_H=4, max_D=512)
+    try:
+        inp = A.make_inputs(batch, DEV)
+        p = A.Params(keep_k=10)
+        outs = [A.alloc_outputs(inp, 10, fill=True) for _ in range(3)]
+        A.asap_prune_step(c, inp, p, outs[0])
+        torch.cuda.synchronize(); A.asap_check(c)
+        A.asap_debug_wait_limit(c, 1)
+        A.asap_prune_step(c, inp, p, outs[1])            # returns normally; its results are void
+        torch.cuda.synchronize()
+        with pytest.raises(A.AsapError) as e:
+            A.asap_check(c)
+        assert e.value.status == -6 and "timed out in the score kernel" in str(e.value)
+        A.asap_prune_step(c, inp, p, outs[2])
+        torch.cuda.synchronize(); A.asap_check(c)
+        _same(outs[0], outs[2], ("mass", "rank_score", "keep_idx", "drop_idx", "assign", "out_hidden", "out_pos", "src_row", "out_cu_seqlens"))
+    finally:
+        A.asap_free(c)
+
+
 @pytest.mark.parametrize("per_head", [False, True], ids=["mean", "heads"])
 def test_mass_kernel_gives_up_and_the_context_recovers(ctx, per_head):
     batch = W.tiny(B=3, n_vis=[300, 260, 140], text_lens=[20, 150, 7], H=2, keep_k=40, seed=611, centres=6)
